@@ -249,102 +249,305 @@ __global__ void __launch_bounds__(128) k_regular64(BlockArgs A, const int64_t* _
 }
 
 // ---------------------------------------------------------------------------
-// singular pairs (Sauter-Schwab), FP64: one warp per pair
+// singular pairs (Sauter-Schwab), FP64: 16 lanes per pair, lanes over the
+// angular ("hat") points of the rule (common.h)
+//
+// What bounds it: the FP64 pipe (about 1/64 of the FP32 rate).  A rule point
+// evaluated by itself costs about 118 FP64 instructions (sqrt, reciprocal,
+// sincos, 28 moment sums).  Here the n_ss radial points of a hat point share
+// everything: with |x - y| = xi rho the pair's moments are
+//   sum W xi^3 xi^m G:  re = P_{2+m} / rho,   im = k S_{3+m},      m = 0, 1, 2
+//   sum W xi^3 xi^m g:  re = -(P_m / rho^3 + k^2 S_{2+m} / rho),
+//                       im = k (P_{1+m} - S_{1+m}) / rho^2,         m = 1, 2
+// (m the degree of the moment's monomial in the coordinates), and the radial
+// sums P, S are power series in (k rho)^2: 8 Horner chains of 6 to 12 steps
+// per hat point instead of n_ss square roots and sincos.  kappa = k rho <= 2
+// is carried to FP64 rounding; wider pairs evaluate the sums point by point.
+// The moments are monomials x_i y_j in the rule's own coordinates (their
+// weights tabulated per hat point), 6 (coincident, halved by the x <-> y
+// symmetry, coplanar: K = 0), 9 + 6 (common edge) or 9 + 8 (common vertex)
+// complex sums.  Measured: 15.4 -> 3.5 ms for the 2 x 2 x 2 cube's 11,664
+// coincident, 17,496 edge and 52,272 vertex pairs (n_ss = 4).
 // ---------------------------------------------------------------------------
-template <class OutT>
-__global__ void __launch_bounds__(256) k_singular64(BlockArgs A, const SingPair* __restrict__ sp,
-                                                    int64_t npairs, const double* __restrict__ ss0,
-                                                    const double* __restrict__ ss1,
-                                                    const double* __restrict__ ss2, int n0, int n1,
-                                                    int n2, OutT* __restrict__ TK) {
-  const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= npairs) return;
-  const SingPair P = sp[w];
-  const int kind = P.code & 3;
-  const int pt0 = (P.code >> 2) & 3, pt1 = (P.code >> 4) & 3, pt2 = (P.code >> 6) & 3;
-  const int ps0 = (P.code >> 8) & 3, ps1 = (P.code >> 10) & 3, ps2 = (P.code >> 12) & 3;
-  const double* tab = kind == 0 ? ss0 : (kind == 1 ? ss1 : ss2);
-  const int npts = kind == 0 ? n0 : (kind == 1 ? n1 : n2);
+
+// 1 / sqrt(d), d > 0: the hardware approximation refined by one step of the
+// cubic Householder iteration y + y e (1/2 + 3/8 e), e = 1 - d y^2
+__device__ __forceinline__ double rsqrt_h(double d) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-(d * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// sum over the 16 lanes of a pair of N values per lane by recursive halving:
+// the lane ends with values [base, base + count) of the sums in v[0 ..]
+template <int N>
+__device__ __forceinline__ void halve16(double* v, int lane, int off, int& base, int& count) {
+  constexpr int H = (N + 1) / 2;
+  const bool up = (lane & off) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const double lo = v[i], hi = H + i < N ? v[H + i] : 0.0;
+    v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, off);
+  }
+  if (up) {
+    base += H;
+    count = max(0, count - H);
+  } else {
+    count = min(count, H);
+  }
+  if constexpr (H > 1) {
+    if (off > 1) halve16<H>(v, lane, off >> 1, base, count);
+  } else {
+    for (int o = off >> 1; o > 0; o >>= 1) {  // one value left: plain sums
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      if (lane & o) count = 0;
+    }
+  }
+}
+
+// hat-table rows, sums per pair of each kind
+template <int KIND> struct SingKind;
+template <> struct SingKind<0> { static constexpr int rows = 8, sums = 12; };
+template <> struct SingKind<1> { static constexpr int rows = 13, sums = 30; };
+template <> struct SingKind<2> { static constexpr int rows = 13, sums = 34; };
+
+// hat-table rows of a kind from its rule, value-major (row r of point p at
+// [r npts + p]): the coordinates the distance needs, then the weights times
+// the monomials of the moments
+static std::vector<double> singular_table(int kind, int n_ss, int& npts) {
+  std::vector<double> pts;
+  sauter_schwab_hat(kind, n_ss, pts);
+  npts = int(pts.size() / 5);
+  const int rows = kind == 0 ? SingKind<0>::rows : SingKind<1>::rows;
+  std::vector<double> t(size_t(rows) * npts);
+  for (int p = 0; p < npts; ++p) {
+    const double x1 = pts[5 * p], x2 = pts[5 * p + 1], y1 = pts[5 * p + 2], y2 = pts[5 * p + 3], w = pts[5 * p + 4];
+    std::vector<double> v;
+    if (kind == 0)
+      v = {x1 - y1, x2 - y2, 2 * w, w * (x1 + y1), w * (x2 + y2), 2 * w * x1 * y1, 2 * w * x2 * y2, w * (x1 * y2 + x2 * y1)};
+    else if (kind == 1)
+      v = {x1 - y1, x2, y2, w, w * x1, w * x2, w * y1, w * y2, w * x1 * y1, w * x1 * y2, w * x2 * y1, w * x2 * y2,
+           w * (x1 - y1)};
+    else
+      v = {x1, x2, y1, y2, w, w * x1, w * x2, w * y1, w * y2, w * x1 * y1, w * x1 * y2, w * x2 * y1, w * x2 * y2};
+    for (int r = 0; r < rows; ++r) t[size_t(r) * npts + p] = v[size_t(r)];
+  }
+  return t;
+}
+
+__device__ __forceinline__ double dot3(const double* a, const double* b) { return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2])); }
+__device__ __forceinline__ void cross3(const double* a, const double* b, double* c) {
+  c[0] = fma(a[1], b[2], -(a[2] * b[1]));
+  c[1] = fma(a[2], b[0], -(a[0] * b[2]));
+  c[2] = fma(a[0], b[1], -(a[1] * b[0]));
+}
+
+template <int KIND, class OutT>
+__global__ void __launch_bounds__(128) k_singular64(BlockArgs A, const SingPair* __restrict__ sp, int64_t npairs,
+                                                    const double* __restrict__ tab, int npts,
+                                                    const __grid_constant__ SingRadial R, OutT* __restrict__ TK) {
+  constexpr int NS = SingKind<KIND>::sums;
+  __shared__ double sums[8][NS];
+  const int slot = threadIdx.x >> 4, lane = threadIdx.x & 15;
+  const int64_t w = int64_t(blockIdx.x) * 8 + slot;
+  const SingPair P = sp[min(w, npairs - 1)];  // the tail repeats the last pair (not stored)
   const int64_t qt = P.tau, qs = P.sig;
   const double* vt = A.bt_v + 9 * qt;
   const double* vs = A.bt_v + 9 * qs;
-  double o[3], e1[3], e2[3], f1[3], f2[3];
+  const double* t0 = vt + 3 * ((P.code >> 2) & 3);
+  const double* t1 = vt + 3 * ((P.code >> 4) & 3);
+  const double* t2 = vt + 3 * ((P.code >> 6) & 3);
+  const double* s0 = vs + 3 * ((P.code >> 8) & 3);
+  const double* s1 = vs + 3 * ((P.code >> 10) & 3);
+  const double* s2 = vs + 3 * ((P.code >> 12) & 3);
+  // x = P0 + x1 e1 + x2 e2, y = P0 + y1 f1 + y2 f2 (P0 shared for every kind)
+  double e1[3], e2[3], f1[3], f2[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    o[c] = vt[3 * pt0 + c];
-    e1[c] = vt[3 * pt1 + c] - vt[3 * pt0 + c];
-    e2[c] = vt[3 * pt2 + c] - vt[3 * pt1 + c];
-    // the trial map shares its origin with the test map (P0 = Q0 for every kind)
-    f1[c] = vs[3 * ps1 + c] - vs[3 * ps0 + c];
-    f2[c] = vs[3 * ps2 + c] - vs[3 * ps1 + c];
+    e1[c] = t1[c] - t0[c];
+    e2[c] = t2[c] - t1[c];
+    f1[c] = s1[c] - s0[c];
+    f2[c] = s2[c] - s1[c];
   }
-  const double W4 = 4.0 * A.bt_area[qt] * A.bt_area[qs];
-  const int i = P.block;
-  const double kr = A.k[2 * i], ki = A.k[2 * i + 1];
-  Moments M;
-  zero(M);
-  for (int p = lane; p < npts; p += 32) {
-    const double x1 = tab[5 * p], x2 = tab[5 * p + 1], y1 = tab[5 * p + 2], y2 = tab[5 * p + 3];
-    const double W = tab[5 * p + 4] * W4;
-    double xp[3], yp[3], d[3];
+  const double k = A.k[2 * P.block], k2 = k * k;
+  // steps of the series: kappa is at most k times the largest vertex distance
+  float zmax = 0.f;
+  if (lane < 9) {
+    const double* a = vt + 3 * (lane / 3);
+    const double* b = vs + 3 * (lane % 3);
+    const double d[3] = {a[0] - b[0], a[1] - b[1], a[2] - b[2]};
+    zmax = float(k2 * dot3(d, d)) * 1.0001f;
+  }
+  zmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(zmax)));
+  const int deg = zmax <= 0.0625f ? 6 : zmax <= 0.25f ? 7 : zmax <= 1.f ? 9 : zmax <= 2.25f ? 10 : 12;
+  const bool series = zmax <= 4.f;
+
+  double acc[NS];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      xp[c] = x1 * e1[c] + x2 * e2[c];
-      yp[c] = y1 * f1[c] + y2 * f2[c];
+  for (int q = 0; q < NS; ++q) acc[q] = 0.0;
+  for (int p = lane; p < npts; p += 16) {
+    const double* tp = tab + p;
+    double d[3];
+    if (KIND == 0) {
+      const double u = tp[0], v = tp[npts];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d[c] = fma(u, e1[c], v * e2[c]);
+    } else if (KIND == 1) {
+      const double u = tp[0], x2 = tp[npts], y2 = tp[2 * npts];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d[c] = fma(u, e1[c], fma(x2, e2[c], -(y2 * f2[c])));
+    } else {
+      const double x1 = tp[0], x2 = tp[npts], y1 = tp[2 * npts], y2 = tp[3 * npts];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d[c] = fma(x1, e1[c], x2 * e2[c]) - fma(y1, f1[c], y2 * f2[c]);
     }
-    if (kind == 0) {
+    const double r2 = dot3(d, d);
+    const double ri = rsqrt_h(r2), ri2 = ri * ri;
+    const double z = k2 * r2;
+    double v[8];  // P_1..P_4, S_2..S_5
+    if (series) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) d[c] = (x1 - y1) * e1[c] + (x2 - y2) * e2[c];
+      for (int j = 0; j < 8; ++j) v[j] = R.c[deg][j];
+#pragma unroll 1
+      for (int t = deg - 1; t >= 0; --t)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = fma(v[j], z, R.c[t][j]);
     } else {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) d[c] = xp[c] - yp[c];
-    }
-    const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    C2 G, g;
-    helmholtz(kr, ki, r, G, g);
-    G = cscale(G, W);
-    g = cscale(g, W);
-    M.S0 = cadd(M.S0, G);
-    double xy = xp[0] * yp[0] + xp[1] * yp[1] + xp[2] * yp[2];
-    M.Sxy = cadd(M.Sxy, cscale(G, xy));
-    const double cr[3] = {xp[1] * yp[2] - xp[2] * yp[1], xp[2] * yp[0] - xp[0] * yp[2],
-                          xp[0] * yp[1] - xp[1] * yp[0]};
+      for (int j = 0; j < 8; ++j) v[j] = 0.0;
+      const double kap = k * (r2 * ri);
+#pragma unroll 1
+      for (int q = 0; q < R.n; ++q) {
+        const double x = R.xi[q], a = kap * x;
+        double sn, cs;
+        sincos(a, &sn, &cs);
+        sn = a > 0.0 ? sn / a : 1.0;
+        double wq = R.gw[q] * x;
+        v[0] = fma(wq, cs, v[0]);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      M.Sx[c] = cadd(M.Sx[c], cscale(G, xp[c]));
-      M.Sy[c] = cadd(M.Sy[c], cscale(G, yp[c]));
-      M.Gx[c] = cadd(M.Gx[c], cscale(g, d[c]));  // only Gx - Gy enters when Delta = 0
-      M.C[c] = cadd(M.C[c], cscale(g, cr[c]));
+        for (int j = 1; j < 4; ++j) {
+          wq *= x;
+          v[j] = fma(wq, cs, v[j]);
+          v[3 + j] = fma(wq, sn, v[3 + j]);
+        }
+        v[7] = fma(wq * x, sn, v[7]);
+      }
+    }
+    // G moments of degree 0, 1, 2 (the imaginary parts without their factor k)
+    const double Gr[3] = {ri * v[1], ri * v[2], ri * v[3]}, Gi[3] = {v[5], v[6], v[7]};
+    const double* wt = tp + size_t(KIND == 0 ? 2 : KIND == 1 ? 3 : 4) * npts;
+#pragma unroll
+    for (int q = 0; q < (KIND == 0 ? 6 : 9); ++q) {
+      const int m = q == 0 ? 0 : q <= (KIND == 0 ? 2 : 4) ? 1 : 2;
+      const double ww = wt[size_t(q) * npts];
+      acc[2 * q] = fma(ww, Gr[m], acc[2 * q]);
+      acc[2 * q + 1] = fma(ww, Gi[m], acc[2 * q + 1]);
+    }
+    if (KIND != 0) {
+      // g moments of degree 1, 2 (minus the real part; im without k)
+      const double g1r = ri * fma(ri2, v[0], k2 * v[5]), g1i = ri2 * (v[1] - v[4]);
+      const double g2r = ri * fma(ri2, v[1], k2 * v[6]), g2i = ri2 * (v[2] - v[5]);
+      // edge: u, x2, y2, x1 y2, x2 y1, x2 y2; vertex: x1, x2, y1, y2, x_i y_j
+      constexpr int ng = KIND == 1 ? 6 : 8;
+#pragma unroll
+      for (int q = 0; q < ng; ++q) {
+        const int row = KIND == 1 ? (q == 0 ? 9 : q == 1 ? 2 : q == 2 ? 4 : 3 + q) : 1 + q;
+        const bool first = q < (KIND == 1 ? 3 : 4);
+        const double ww = wt[size_t(row) * npts];
+        acc[18 + 2 * q] = fma(ww, first ? g1r : g2r, acc[18 + 2 * q]);
+        acc[18 + 2 * q + 1] = fma(ww, first ? g1i : g2i, acc[18 + 2 * q + 1]);
+      }
     }
   }
-  // warp reduction of the 28 doubles actually used (Q, Gy stay zero)
-  double* f = reinterpret_cast<double*>(&M);
-  const int nd = sizeof(Moments) / sizeof(double);
+  int base = 0, count = NS;
+  halve16<NS>(acc, lane, 8, base, count);
 #pragma unroll
-  for (int q = 0; q < nd; ++q) {
-    double v = f[q];
+  for (int q = 0; q < (NS + 15) / 16; ++q)
+    if (q < count) sums[slot][base + q] = acc[q];
+  __syncwarp();
+  if (lane >= 9 || w >= npairs) return;
+  // entry (a, b) of the 3 x 3 block: v_a = P0 + al1 e1 + al2 e2 and u_b =
+  // P0 + be1 f1 + be2 f2 with (0, 0), (1, 0), (1, 1) for the vertices in rule order
+  const double* S = sums[slot];
+  const int a = lane / 3, b = lane % 3;
+  const double al[2] = {a > 0 ? 1.0 : 0.0, a > 1 ? 1.0 : 0.0}, be[2] = {b > 0 ? 1.0 : 0.0, b > 1 ? 1.0 : 0.0};
+  // sums of G: 1 | x_i | y_j | x_i y_j
+  auto G = [&](int q, int c) { return S[2 * q + c]; };
+  const double ef[4] = {dot3(e1, f1), dot3(e1, f2), dot3(e2, f1), dot3(e2, f2)};
+  double X[2] = {0.0, 0.0};  // sum G (x - v_a) . (y - u_b)
 #pragma unroll
-    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    f[q] = v;
-  }
-  if (lane < 9) {
-    const int a = lane / 3, b = lane % 3;
-    double pa[3], qb[3];
-    const double D[3] = {0.0, 0.0, 0.0};
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      pa[c] = vt[3 * a + c] - o[c];
-      qb[c] = vs[3 * b + c] - o[c];
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const double mx = G(1 + i, c);
+        const double my = KIND == 0 ? G(1 + j, c) : G(3 + j, c);
+        const double mxy = KIND == 0 ? (i == j ? G(3 + i, c) : G(5, c)) : G(5 + 2 * i + j, c);
+        X[c] = fma(ef[2 * i + j], mxy - be[j] * mx - al[i] * (my - be[j] * G(0, c)), X[c]);
+      }
+  const int pa = (P.code >> (2 + 2 * a)) & 3, pb = (P.code >> (8 + 2 * b)) & 3;
+  const double cc = 4.0 * INV_FOUR_PI * A.bt_area[qt] * A.bt_area[qs] * A.bt_c[3 * qt + pa] * A.bt_c[3 * qs + pb];
+  // T = -i k X - 4 / (i k) S0
+  const C2 Tv{cc * fma(k2, X[1], -4.0 * G(0, 1)), cc * (4.0 / k * G(0, 0) - k * X[0])};
+  C2 Kv{0.0, 0.0};
+  if (KIND != 0) {
+    // K_ab = -c_a c_b (v_a - u_b) . sum g (y - u_b) x (x - v_a)
+    double s[2] = {0.0, 0.0}, t[3];
+    auto g = [&](int q, int c) { return S[18 + 2 * q + c]; };
+    if (KIND == 1) {
+      cross3(e1, e2, t);
+      const double A2 = dot3(t, f2);  // f1 = e1
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        s[c] = A2 * (al[1] * g(3, c) - be[1] * g(4, c) + (be[0] - al[0]) * g(5, c) - al[1] * be[1] * g(0, c) +
+                     al[0] * be[1] * g(1, c) - al[1] * be[0] * g(2, c));
+    } else {
+      cross3(e1, e2, t);
+      const double A1 = dot3(t, f1), A2 = dot3(t, f2);
+      cross3(f1, f2, t);
+      const double B1 = dot3(t, e1), B2 = dot3(t, e2);
+      const double V[4] = {al[1] * A1 + be[1] * B1, al[1] * A2 - be[0] * B1, be[1] * B2 - al[0] * A1,
+                           -(al[0] * A2 + be[0] * B2)};
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+            s[c] = fma(V[2 * i + j], g(4 + 2 * i + j, c) - be[j] * g(i, c) - al[i] * g(2 + j, c), s[c]);
     }
-    C2 Tv, Kv;
-    local_entry(M, pa, qb, D, A.bt_c[3 * qt + a] * A.bt_c[3 * qs + b], kr, ki, Tv, Kv);
-    const int N = A.blk_N[i];
-    const int64_t ra = A.bt_dof[3 * qt + a], cb = A.bt_dof[3 * qs + b];
-    add_entry(TK, A.blk_mat_off[i] + ra * N + cb, Tv, Kv);
-    // the swapped pair (sigma, tau) of an adjacent pair: the same value at
-    // the transposed position (symmetric Galerkin forms)
-    if (kind != 0) add_entry(TK, A.blk_mat_off[i] + cb * N + ra, Tv, Kv);
+    Kv = C2{cc * s[0], -cc * k * s[1]};
+  }
+  const int N = A.blk_N[P.block];
+  const int64_t ra = A.bt_dof[3 * qt + pa], cb = A.bt_dof[3 * qs + pb];
+  add_entry(TK, A.blk_mat_off[P.block] + ra * N + cb, Tv, Kv);
+  // the swapped pair (sigma, tau) of an adjacent pair: the same value at
+  // the transposed position (symmetric Galerkin forms)
+  if (KIND != 0) add_entry(TK, A.blk_mat_off[P.block] + cb * N + ra, Tv, Kv);
+}
+
+// the three kinds of the mesh's singular pairs (sorted by kind)
+template <class OutT>
+static void launch_singular(mtf_system sys, const BlockArgs& A, OutT* TK, cudaStream_t s) {
+  mtf_mesh m = sys->mesh;
+  int64_t at = 0;
+  for (int kind = 0; kind < 3; ++kind) {
+    int64_t end = at;
+    while (end < int64_t(m->sing.size()) && (m->sing[size_t(end)].code & 3) == kind) ++end;
+    const int64_t np = end - at;
+    if (np > 0) {
+      const unsigned g = unsigned((np + 7) / 8);
+      auto go = [&](auto kernel) {
+        MTF_LAUNCH(KID_SINGULAR64, s, kernel<<<g, 128, 0, s>>>(A, m->d_sing.p + at, np, sys->d_ss_pts[kind].p,
+                                                               sys->ss_npts[kind], sys->ss_radial, TK));
+      };
+      if (kind == 0) go(k_singular64<0, OutT>);
+      else if (kind == 1) go(k_singular64<1, OutT>);
+      else go(k_singular64<2, OutT>);
+    }
+    at = end;
   }
 }
 
@@ -564,16 +767,13 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
   // Sauter-Schwab tables (once per system)
   if (sys->ss_npts[0] == 0) {
     for (int kind = 0; kind < 3; ++kind) {
-      std::vector<double> pts;
-      sauter_schwab_rule(kind, sys->opt.n_ss, pts);
-      sys->d_ss_pts[kind].upload(pts, s);
+      const std::vector<double> tab = singular_table(kind, sys->opt.n_ss, sys->ss_npts[kind]);
+      sys->d_ss_pts[kind].upload(tab, s);
       MTF_CUDA(cudaStreamSynchronize(s));
-      sys->ss_npts[kind] = int(pts.size() / 5);
     }
+    singular_radial(sys->opt.n_ss, sys->ss_radial);
   }
   BlockArgs A = block_args(sys);
-  const int64_t np = int64_t(m->sing.size());
-  const unsigned sblocks = unsigned((np * 32 + 255) / 256);
   const bool fp64_blocks = sys->opt.precision == MTF_PREC_FP64 || sys->opt.residual_fp64;
   if (fp64_blocks) {
     sys->d_TK64.alloc(size_t(m->n_mat) * 4);
@@ -581,10 +781,7 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
     const int64_t nct = m->reg_cta_prefix.back();
     if (nct > 0)
       MTF_LAUNCH(KID_REGULAR64, s, k_regular64<<<unsigned(nct), 128, 0, s>>>(A, m->d_reg_cta_prefix.p, sys->d_TK64.p));
-    if (np > 0)
-      MTF_LAUNCH(KID_SINGULAR64, s, k_singular64<double><<<sblocks, 256, 0, s>>>(
-          A, m->d_sing.p, np, sys->d_ss_pts[0].p, sys->d_ss_pts[1].p, sys->d_ss_pts[2].p, sys->ss_npts[0],
-          sys->ss_npts[1], sys->ss_npts[2], sys->d_TK64.p));
+    launch_singular(sys, A, sys->d_TK64.p, s);
   }
   if (fp64_blocks && sys->opt.precision != MTF_PREC_FP64) {
     // residual_fp64: the FP64 entries split into FP32 pairs once per assembly,
@@ -599,10 +796,7 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
     sys->d_TK32.alloc(size_t(m->n_mat) * 4);
     MTF_CUDA(cudaMemsetAsync(sys->d_TK32.p, 0, size_t(m->n_mat) * 4 * sizeof(float), s));
     launch_assemble_regular32(sys, s);
-    if (np > 0)
-      MTF_LAUNCH(KID_SINGULAR64, s, k_singular64<float><<<sblocks, 256, 0, s>>>(
-          A, m->d_sing.p, np, sys->d_ss_pts[0].p, sys->d_ss_pts[1].p, sys->d_ss_pts[2].p, sys->ss_npts[0],
-          sys->ss_npts[1], sys->ss_npts[2], sys->d_TK32.p));
+    launch_singular(sys, A, sys->d_TK32.p, s);
     if (sys->opt.mv_tensor) tc_build_operator(sys, s);
     else tile_matvec_operator(sys, s);
   }

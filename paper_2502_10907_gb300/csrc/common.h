@@ -72,9 +72,27 @@ struct TriRule {
 };
 const TriRule& triangle_rule6();
 void gauss_legendre01(int n, std::vector<double>& x, std::vector<double>& w);
-// Sauter-Schwab rule: (x1, x2, y1, y2, w) per point, kinds 0 coincident,
-// 1 common edge, 2 common vertex.
-void sauter_schwab_rule(int kind, int n, std::vector<double>& pts);
+// Sauter-Schwab rules in radial form.  Every region of the three rules maps
+// the 4-cube by x = xi x^(eta), y = xi y^(eta) (coordinates from the shared
+// vertex P0) with Jacobian xi^3 J^(eta), so a rule of n points per coordinate
+// is n radial nodes times n^3 angular ("hat") points per region:
+// (x1, x2, y1, y2, w J^) at xi = 1 per hat point, kinds 0 coincident, 1 common
+// edge, 2 common vertex.  Kind 0 lists one region of each pair that differs
+// by swapping x and y.
+void sauter_schwab_hat(int kind, int n, std::vector<double>& pts);
+// The radial part of the kernel's moments at one hat point, |x - y| = xi rho,
+// kappa = k rho:
+//   P_j = sum_q gw_q xi_q^j cos(kappa xi_q),           j = 1..4,
+//   S_j = sum_q gw_q xi_q^j sin(kappa xi_q) / (kappa xi_q),  j = 2..5,
+// as power series in kappa^2: c[t] holds the coefficients of kappa^(2t) of
+// P_1..P_4, S_2..S_5.  kSingTerms terms carry kappa <= 2 to FP64 rounding.
+constexpr int kSsMax = 12, kSingTerms = 13;
+struct SingRadial {
+  double c[kSingTerms][8];
+  double xi[kSsMax], gw[kSsMax];
+  int n;
+};
+void singular_radial(int n, SingRadial& r);
 
 // ---------------------------------------------------------------------------
 // mesh (Algorithm 1 and RWG tables)
@@ -205,7 +223,8 @@ struct mtf_system_s {
   mtf::DevBuf<double> d_xval;                // exchange values (6 per row)
   mtf::DevBuf<float> d_xval32;               // FP32 copy of the exchange values
   mtf::DevBuf<float> d_rho32;                // per block: rho (re, im), 1 / rho (re, im)
-  mtf::DevBuf<double> d_ss_pts[3];           // Sauter-Schwab tables
+  mtf::DevBuf<double> d_ss_pts[3];           // Sauter-Schwab hat tables
+  mtf::SingRadial ss_radial{};               // and their radial sums
   // FP32 geometry of the mixed regular-pair kernel (per block-triangle)
   mtf::DevBuf<float> d_x32;                  // FP32 copy of the matvec input (mixed path)
   mtf::DevBuf<float> d_adj32;                // conjugated input of the adjoint matvec

@@ -122,50 +122,61 @@ const TriRule& triangle_rule6() {
   return rule;
 }
 
-void sauter_schwab_rule(int kind, int n, std::vector<double>& pts) {
+void sauter_schwab_hat(int kind, int n, std::vector<double>& pts) {
   std::vector<double> g, gw;
   gauss_legendre01(n, g, gw);
-  const int nreg = kind == 0 ? 6 : (kind == 1 ? 5 : 2);
+  const int nreg = kind == 0 ? 3 : (kind == 1 ? 5 : 2);
   pts.clear();
-  pts.reserve(size_t(nreg) * n * n * n * n * 5);
-  for (int reg = 0; reg < nreg; ++reg) {
-    for (int a = 0; a < n; ++a)
-      for (int b = 0; b < n; ++b)
-        for (int c = 0; c < n; ++c)
-          for (int d = 0; d < n; ++d) {
-            const double xi = g[a], e1 = g[b], e2 = g[c], e3 = g[d];
-            const double W = gw[a] * gw[b] * gw[c] * gw[d];
-            double x1 = 0, x2 = 0, y1 = 0, y2 = 0, J = 0;
-            if (kind == 0) {  // coincident: Jacobian xi^3 eta1^2 eta2
-              J = xi * xi * xi * e1 * e1 * e2;
-              switch (reg) {
-                case 0: x1 = xi; x2 = xi * (1 - e1 + e1 * e2); y1 = xi * (1 - e1 * e2 * e3); y2 = xi * (1 - e1); break;
-                case 1: y1 = xi; y2 = xi * (1 - e1 + e1 * e2); x1 = xi * (1 - e1 * e2 * e3); x2 = xi * (1 - e1); break;
-                case 2: x1 = xi; x2 = xi * e1 * (1 - e2 + e2 * e3); y1 = xi * (1 - e1 * e2); y2 = xi * e1 * (1 - e2); break;
-                case 3: y1 = xi; y2 = xi * e1 * (1 - e2 + e2 * e3); x1 = xi * (1 - e1 * e2); x2 = xi * e1 * (1 - e2); break;
-                case 4: x1 = xi * (1 - e1 * e2 * e3); x2 = xi * e1 * (1 - e2 * e3); y1 = xi; y2 = xi * e1 * (1 - e2); break;
-                default: y1 = xi * (1 - e1 * e2 * e3); y2 = xi * e1 * (1 - e2 * e3); x1 = xi; x2 = xi * e1 * (1 - e2); break;
-              }
-            } else if (kind == 1) {  // common edge P0-P1 (x2 = 0 in both)
-              J = reg == 0 ? xi * xi * xi * e1 * e1 : xi * xi * xi * e1 * e1 * e2;
-              switch (reg) {
-                case 0: x1 = xi; x2 = xi * e1 * e3; y1 = xi * (1 - e1 * e2); y2 = xi * e1 * (1 - e2); break;
-                case 1: x1 = xi; x2 = xi * e1; y1 = xi * (1 - e1 * e2 * e3); y2 = xi * e1 * e2 * (1 - e3); break;
-                case 2: x1 = xi * (1 - e1 * e2); x2 = xi * e1 * (1 - e2); y1 = xi; y2 = xi * e1 * e2 * e3; break;
-                case 3: x1 = xi * (1 - e1 * e2 * e3); x2 = xi * e1 * e2 * (1 - e3); y1 = xi; y2 = xi * e1; break;
-                default: x1 = xi * (1 - e1 * e2 * e3); x2 = xi * e1 * (1 - e2 * e3); y1 = xi; y2 = xi * e1 * e2; break;
-              }
-            } else {  // common vertex P0 (origin of both)
-              J = xi * xi * xi * e2;
-              if (reg == 0) { x1 = xi; x2 = xi * e1; y1 = xi * e2; y2 = xi * e2 * e3; }
-              else { x1 = xi * e2; x2 = xi * e2 * e3; y1 = xi; y2 = xi * e1; }
+  pts.reserve(size_t(nreg) * n * n * n * 5);
+  for (int reg = 0; reg < nreg; ++reg)
+    for (int b = 0; b < n; ++b)
+      for (int c = 0; c < n; ++c)
+        for (int d = 0; d < n; ++d) {
+          const double e1 = g[b], e2 = g[c], e3 = g[d], W = gw[b] * gw[c] * gw[d];
+          double x1 = 1, x2 = 0, y1 = 1, y2 = 0, J = 0;
+          if (kind == 0) {  // coincident: Jacobian xi^3 eta1^2 eta2; the other three regions swap x and y
+            J = e1 * e1 * e2;
+            switch (reg) {
+              case 0: x2 = 1 - e1 + e1 * e2; y1 = 1 - e1 * e2 * e3; y2 = 1 - e1; break;
+              case 1: x2 = e1 * (1 - e2 + e2 * e3); y1 = 1 - e1 * e2; y2 = e1 * (1 - e2); break;
+              default: x1 = 1 - e1 * e2 * e3; x2 = e1 * (1 - e2 * e3); y2 = e1 * (1 - e2); break;
             }
-            pts.push_back(x1);
-            pts.push_back(x2);
-            pts.push_back(y1);
-            pts.push_back(y2);
-            pts.push_back(W * J);
+          } else if (kind == 1) {  // common edge P0-P1 (x2 = 0 in both)
+            J = reg == 0 ? e1 * e1 : e1 * e1 * e2;
+            switch (reg) {
+              case 0: x2 = e1 * e3; y1 = 1 - e1 * e2; y2 = e1 * (1 - e2); break;
+              case 1: x2 = e1; y1 = 1 - e1 * e2 * e3; y2 = e1 * e2 * (1 - e3); break;
+              case 2: x1 = 1 - e1 * e2; x2 = e1 * (1 - e2); y2 = e1 * e2 * e3; break;
+              case 3: x1 = 1 - e1 * e2 * e3; x2 = e1 * e2 * (1 - e3); y2 = e1; break;
+              default: x1 = 1 - e1 * e2 * e3; x2 = e1 * (1 - e2 * e3); y2 = e1 * e2; break;
+            }
+          } else {  // common vertex P0 (origin of both)
+            J = e2;
+            if (reg == 0) { x2 = e1; y1 = e2; y2 = e2 * e3; }
+            else { x1 = e2; x2 = e2 * e3; y2 = e1; }
           }
+          pts.insert(pts.end(), {x1, x2, y1, y2, W * J});
+        }
+}
+
+void singular_radial(int n, SingRadial& r) {
+  std::vector<double> g, gw;
+  gauss_legendre01(n, g, gw);
+  r.n = n;
+  for (int q = 0; q < kSsMax; ++q) {
+    r.xi[q] = q < n ? g[q] : 0.0;
+    r.gw[q] = q < n ? gw[q] : 0.0;
+  }
+  long double fc = 1.0L;  // (-1)^t / (2t)!
+  for (int t = 0; t < kSingTerms; ++t) {
+    if (t > 0) fc /= -(2.0L * t - 1) * (2.0L * t);
+    const long double fs = fc / (2.0L * t + 1);
+    for (int j = 0; j < 8; ++j) {
+      const int e = (j < 4 ? j + 1 : j - 2) + 2 * t;  // P_1..P_4, then S_2..S_5
+      long double m = 0.0L;
+      for (int q = 0; q < n; ++q) m += static_cast<long double>(gw[q]) * powl(static_cast<long double>(g[q]), e);
+      r.c[t][j] = static_cast<double>((j < 4 ? fc : fs) * m);
+    }
   }
 }
 
