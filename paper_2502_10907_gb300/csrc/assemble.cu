@@ -22,10 +22,13 @@
 #include <cmath>
 
 #include "common.h"
+#include "pair_tile.cuh"
 
 namespace mtf {
 
 __constant__ double c_tri_s[6], c_tri_t[6], c_tri_w[6];  // 6-point rule
+// per orbit (a, a, 1 - 2a): w, w a, w (1 - 3a); per point: w, w s, w t
+__constant__ double c_orbit[2][3], c_point[6][3];
 
 #define INV_FOUR_PI 0.079577471545947667884
 
@@ -37,16 +40,6 @@ __device__ __forceinline__ C2 cscale(C2 a, double s) { return {a.re * s, a.im * 
 __device__ __forceinline__ C2 cadd(C2 a, C2 b) { return {a.re + b.re, a.im + b.im}; }
 __device__ __forceinline__ C2 csub(C2 a, C2 b) { return {a.re - b.re, a.im - b.im}; }
 
-struct Moments {
-  C2 S0, Sx[3], Sy[3], Sxy, Q, Gx[3], Gy[3], C[3];
-};
-
-__device__ __forceinline__ void zero(Moments& M) {
-  C2 z{0, 0};
-  M.S0 = M.Sxy = M.Q = z;
-  for (int c = 0; c < 3; ++c) M.Sx[c] = M.Sy[c] = M.Gx[c] = M.Gy[c] = M.C[c] = z;
-}
-
 // G = exp(i k r) / (4 pi r) and g = G (i k - 1/r) / r for complex k.
 __device__ __forceinline__ void helmholtz(double kr, double ki, double r, C2& G, C2& g) {
   const double rinv = 1.0 / r;
@@ -57,52 +50,6 @@ __device__ __forceinline__ void helmholtz(double kr, double ki, double r, C2& G,
   G = {amp * cs, amp * sn};
   const C2 f{-ki - rinv, kr};  // i k - 1/r
   g = cscale(cmul(G, f), rinv);
-}
-
-// 3x3 local T and K of one pair from its moments; (a, b) = (row, col).
-__device__ __forceinline__ void local_entry(const Moments& M, const double* pa, const double* qb,
-                                            const double* D, double cc, double kr, double ki, C2& T,
-                                            C2& K) {
-  const double pq = pa[0] * qb[0] + pa[1] * qb[1] + pa[2] * qb[2];
-  C2 X = M.Sxy;
-  for (int c = 0; c < 3; ++c) {
-    X = csub(X, cscale(M.Sx[c], qb[c]));
-    X = csub(X, cscale(M.Sy[c], pa[c]));
-  }
-  X = cadd(X, cscale(M.S0, pq));
-  // -i k X  and  -4/(i k) S0 = 4 i conj(k) / |k|^2 S0
-  const C2 mik{ki, -kr};
-  const double k2 = kr * kr + ki * ki;
-  const C2 f4{4.0 * ki / k2, 4.0 * kr / k2};
-  T = cscale(cadd(cmul(mik, X), cmul(f4, M.S0)), cc);
-  // K
-  double u[3], qxp[3], DxGy_re[3], DxGy_im[3], GxxD_re[3], GxxD_im[3];
-  for (int c = 0; c < 3; ++c) u[c] = qb[c] - pa[c] - D[c];
-  qxp[0] = qb[1] * pa[2] - qb[2] * pa[1];
-  qxp[1] = qb[2] * pa[0] - qb[0] * pa[2];
-  qxp[2] = qb[0] * pa[1] - qb[1] * pa[0];
-  // Delta x Gy and Gx x Delta
-  DxGy_re[0] = D[1] * M.Gy[2].re - D[2] * M.Gy[1].re;
-  DxGy_re[1] = D[2] * M.Gy[0].re - D[0] * M.Gy[2].re;
-  DxGy_re[2] = D[0] * M.Gy[1].re - D[1] * M.Gy[0].re;
-  DxGy_im[0] = D[1] * M.Gy[2].im - D[2] * M.Gy[1].im;
-  DxGy_im[1] = D[2] * M.Gy[0].im - D[0] * M.Gy[2].im;
-  DxGy_im[2] = D[0] * M.Gy[1].im - D[1] * M.Gy[0].im;
-  GxxD_re[0] = M.Gx[1].re * D[2] - M.Gx[2].re * D[1];
-  GxxD_re[1] = M.Gx[2].re * D[0] - M.Gx[0].re * D[2];
-  GxxD_re[2] = M.Gx[0].re * D[1] - M.Gx[1].re * D[0];
-  GxxD_im[0] = M.Gx[1].im * D[2] - M.Gx[2].im * D[1];
-  GxxD_im[1] = M.Gx[2].im * D[0] - M.Gx[0].im * D[2];
-  GxxD_im[2] = M.Gx[0].im * D[1] - M.Gx[1].im * D[0];
-  C2 s{0, 0};
-  for (int c = 0; c < 3; ++c) {
-    s = cadd(s, cscale(M.C[c], u[c]));
-    s.re -= pa[c] * DxGy_re[c] + qb[c] * GxxD_re[c];
-    s.im -= pa[c] * DxGy_im[c] + qb[c] * GxxD_im[c];
-    const C2 Dm = cadd(csub(M.Gx[c], M.Gy[c]), cscale(M.Q, D[c]));
-    s = cadd(s, cscale(Dm, qxp[c]));
-  }
-  K = cscale(s, -cc);
 }
 
 __device__ __forceinline__ void add_entry(double* TK, int64_t idx, C2 T, C2 K) {
@@ -117,7 +64,19 @@ __device__ __forceinline__ void add_entry(float* TK, int64_t idx, C2 T, C2 K) {
 }
 
 // ---------------------------------------------------------------------------
-// regular (vertex-disjoint) pairs, FP64: one thread per ordered pair
+// regular (vertex-disjoint) pairs, FP64: one thread per unordered pair, CTAs
+// over 16 x 16 tiles of a block's triangles (pair_tile.cuh)
+//
+// What bounds it: the FP64 pipe.  Both orderings of a pair have transposed
+// 3 x 3 blocks (the Galerkin forms are symmetric), so each pair is evaluated
+// once and added at the upper position (m < n); k_mirror fills the lower
+// triangle.  A kernel evaluation takes the reciprocal square root by a
+// Householder step and exp(i k (r - r0)) by its Taylor series (r0 the
+// centroid distance; the phase exp(i k r0) is applied once per pair), of the
+// length the pair's extent asks for.  The 6-point rule's two orbits share
+// their weight, so the moments over (1, s, t) take 14 operations per channel
+// and 6 points.  Measured on the split sphere of 7 rings (1.04 M ordered
+// pairs): 7.95 -> 2.41 ms.
 // ---------------------------------------------------------------------------
 struct BlockArgs {
   const double* bt_v;
@@ -133,118 +92,319 @@ struct BlockArgs {
   int nblk;
 };
 
+// (cos x, sin x / x) series in x^2: coefficients of x^(2t)
+__constant__ double c_cos[13] = {1.0, -1.0 / 2, 1.0 / 24, -1.0 / 720, 1.0 / 40320, -1.0 / 3628800, 1.0 / 479001600,
+                                 -1.0 / 87178291200.0, 1.0 / 20922789888000.0, -1.0 / 6402373705728000.0,
+                                 1.0 / 2432902008176640000.0, -1.0 / 1124000727777607680000.0,
+                                 1.0 / 620448401733239439360000.0};
+__constant__ double c_sin[13] = {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880, -1.0 / 39916800,
+                                 1.0 / 6227020800.0, -1.0 / 1307674368000.0, 1.0 / 355687428096000.0,
+                                 -1.0 / 121645100408832000.0, 1.0 / 51090942171709440000.0,
+                                 -1.0 / 25852016738884976640000.0, 1.0 / 15511210043330985984000000.0};
+
+// terms beyond the first of the series above that carry |x| <= xmax to FP64
+// rounding (next term below 1e-16); -1: too wide for them
+__device__ __forceinline__ int series_degree(float xmax) {
+  return xmax <= 0.25f ? 6 : xmax <= 0.5f ? 7 : xmax <= 1.f ? 9 : xmax <= 1.5f ? 10 : xmax <= 2.f ? 12 : -1;
+}
+
+// 1 / sqrt(d), d > 0: the hardware approximation refined by one step of the
+// cubic Householder iteration y + y e (1/2 + 3/8 e), e = 1 - d y^2
+__device__ __forceinline__ double rsqrt_h(double d) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-(d * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+__device__ __forceinline__ double dot3(const double* a, const double* b) { return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2])); }
+__device__ __forceinline__ void cross3(const double* a, const double* b, double* c) {
+  c[0] = fma(a[1], b[2], -(a[2] * b[1]));
+  c[1] = fma(a[2], b[0], -(a[0] * b[2]));
+  c[2] = fma(a[0], b[1], -(a[1] * b[0]));
+}
+
+// triangles of one side of a tile: quadrature points, vertices, c_a 2 A
+struct Side64 {
+  double x[18][kPairTile], v[9][kPairTile], cen[3][kPairTile], c[3][kPairTile];
+  float rad[kPairTile];
+  int dof[3][kPairTile], vid[3][kPairTile];
+};
+
+__device__ __forceinline__ void load_side(const BlockArgs& A, int64_t first, int n, Side64& S) {
+  for (int t = threadIdx.x; t < kPairTile * 6; t += blockDim.x) {
+    const int q = t / 6, p = t % 6;
+    if (q >= n) continue;
+    const double* v = A.bt_v + 9 * (first + q);
+    for (int c = 0; c < 3; ++c)
+      S.x[3 * p + c][q] = v[c] + c_tri_s[p] * (v[3 + c] - v[c]) + c_tri_t[p] * (v[6 + c] - v[c]);
+  }
+  for (int q = threadIdx.x; q < n; q += blockDim.x) {
+    const double* v = A.bt_v + 9 * (first + q);
+    for (int c = 0; c < 9; ++c) S.v[c][q] = v[c];
+    for (int c = 0; c < 3; ++c) {
+      S.cen[c][q] = (v[c] + v[3 + c] + v[6 + c]) * (1.0 / 3.0);
+      S.c[c][q] = A.bt_c[3 * (first + q) + c] * (2.0 * A.bt_area[first + q]);
+      S.dof[c][q] = A.bt_dof[3 * (first + q) + c];
+      S.vid[c][q] = A.bt_vid[3 * (first + q) + c];
+    }
+    float r = 0.f;
+    for (int a = 0; a < 3; ++a) {
+      float d2 = 0.f;
+      for (int c = 0; c < 3; ++c) {
+        const float d = float(v[3 * a + c] - S.cen[c][q]);
+        d2 = fmaf(d, d, d2);
+      }
+      r = fmaxf(r, d2);
+    }
+    S.rad[q] = sqrtf(r) * 1.0001f;
+  }
+}
+
 __global__ void __launch_bounds__(128) k_regular64(BlockArgs A, const int64_t* __restrict__ cta_prefix,
                                                    double* __restrict__ TK) {
-  const int64_t cta = blockIdx.x;
-  int lo = 0, hi = A.nblk - 1;
-  while (lo < hi) {  // largest i with cta_prefix[i] <= cta
-    const int mid = (lo + hi + 1) >> 1;
-    if (cta_prefix[mid] <= cta) lo = mid; else hi = mid - 1;
-  }
-  const int i = lo;
-  const int T = A.blk_T[i];
-  const int64_t pair = (cta - cta_prefix[i]) * 128 + threadIdx.x;
-  if (pair >= int64_t(T) * T) return;
-  const int64_t qt = A.blk_bt_off[i] + pair / T;
-  const int64_t qs = A.blk_bt_off[i] + pair % T;
-  int shared = 0;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) shared += A.bt_vid[3 * qt + a] == A.bt_vid[3 * qs + b];
-  if (shared) return;  // singular pairs are handled by k_singular64
-
-  double vt[9], vs[9];
-#pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    vt[c] = A.bt_v[9 * qt + c];
-    vs[c] = A.bt_v[9 * qs + c];
-  }
-  double ot[3], os[3], D[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    ot[c] = (vt[c] + vt[3 + c] + vt[6 + c]) * (1.0 / 3.0);
-    os[c] = (vs[c] + vs[3 + c] + vs[6 + c]) * (1.0 / 3.0);
-    D[c] = ot[c] - os[c];
-  }
-  const double At2 = 2.0 * A.bt_area[qt], As2 = 2.0 * A.bt_area[qs];
-  const double kr = A.k[2 * i], ki = A.k[2 * i + 1];
-  double yq[6][3], wq[6];
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      yq[q][c] = vs[c] + c_tri_s[q] * (vs[3 + c] - vs[c]) + c_tri_t[q] * (vs[6 + c] - vs[c]) - os[c];
-    wq[q] = As2 * c_tri_w[q];
-  }
-  Moments M;
-  zero(M);
+  __shared__ Side64 X, Y;
+  const PairTile P = pair_tile(blockIdx.x, cta_prefix, A.nblk);
+  const int i = P.blk, T = A.blk_T[i];
+  load_side(A, A.blk_bt_off[i] + P.t0, min(kPairTile, T - P.t0), X);
+  load_side(A, A.blk_bt_off[i] + P.s0, min(kPairTile, T - P.s0), Y);
+  __syncthreads();
+  const double k = A.k[2 * i], m4k2 = -4.0 / (k * k);
+  const int N = A.blk_N[i];
+  double* M = TK + 4 * A.blk_mat_off[i];
+  const int b = threadIdx.x & (kPairTile - 1);
 #pragma unroll 1
-  for (int p = 0; p < 6; ++p) {
-    double xp[3], e[3];
+  for (int a = threadIdx.x / kPairTile; a < kPairTile; a += 128 / kPairTile) {
+    // unordered pairs, once each; singular ones are k_singular64's
+    bool live = P.t0 + a < P.s0 + b && P.s0 + b < T;
+    if (live) {
+      bool shared = false;
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) shared |= X.vid[p][a] == Y.vid[q][b];
+      live = !shared;
+    }
+    float ext = live ? float(k) * (X.rad[a] + Y.rad[b]) : 0.f;
+    ext = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ext)));
+    const int deg = series_degree(ext);
+    if (!live) continue;
+    const double D[3] = {X.cen[0][a] - Y.cen[0][b], X.cen[1][a] - Y.cen[1][b], X.cen[2][a] - Y.cen[2][b]};
+    const double kr0 = k * sqrt(dot3(D, D));
+    // sums over the rule of G exp(-i k r0) 4 pi and of -g: [row: 1, s, t of x][1, s, t of y] (re, im)
+    double G[3][3][2], H[3][3][2];
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) G[p][q][0] = G[p][q][1] = H[p][q][0] = H[p][q][1] = 0.0;
+#pragma unroll 1
+    for (int p = 0; p < 6; ++p) {
+      const double x0 = X.x[3 * p][a], x1 = X.x[3 * p + 1][a], x2 = X.x[3 * p + 2][a];
+      double m[3][4], bc[4];  // y moments of (re G, im G, re H, im H); bc: part common to s and t
+#pragma unroll
+      for (int f = 0; f < 4; ++f) m[0][f] = m[1][f] = m[2][f] = bc[f] = 0.0;
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        double v[3][4], ri[3], ph[3], sn[3], cs[3];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const int q = 3 * o + e;
+          const double d[3] = {x0 - Y.x[3 * q][b], x1 - Y.x[3 * q + 1][b], x2 - Y.x[3 * q + 2][b]};
+          const double r2 = dot3(d, d);
+          ri[e] = rsqrt_h(r2);
+          ph[e] = fma(k, r2 * ri[e], -kr0);
+        }
+        if (deg >= 0) {
+          double z[3];
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            z[e] = ph[e] * ph[e];
+            cs[e] = c_cos[deg];
+            sn[e] = c_sin[deg];
+          }
+#pragma unroll 1
+          for (int t = deg - 1; t >= 0; --t)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+              cs[e] = fma(cs[e], z[e], c_cos[t]);
+              sn[e] = fma(sn[e], z[e], c_sin[t]);
+            }
+#pragma unroll
+          for (int e = 0; e < 3; ++e) sn[e] *= ph[e];
+        } else {
+#pragma unroll
+          for (int e = 0; e < 3; ++e) sincos(ph[e], &sn[e], &cs[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          v[e][0] = ri[e] * cs[e];
+          v[e][1] = ri[e] * sn[e];
+          const double al = k * ri[e], be = ri[e] * ri[e];  // -g = G (1/r - i k) / r
+          v[e][2] = fma(be, v[e][0], al * v[e][1]);
+          v[e][3] = fma(be, v[e][1], -(al * v[e][0]));
+        }
+        // orbit o: barycentric coordinates a, a, 1 - 2a; s = 1 - 2a at its point 1, t at its point 2
+        const double w = c_orbit[o][0], wa = c_orbit[o][1], wc = c_orbit[o][2];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          const double sum = v[0][f] + v[1][f] + v[2][f];
+          m[0][f] = fma(w, sum, m[0][f]);
+          bc[f] = fma(wa, sum, bc[f]);
+          m[1][f] = fma(wc, v[1][f], m[1][f]);
+          m[2][f] = fma(wc, v[2][f], m[2][f]);
+        }
+      }
+      const double wx[3] = {c_point[p][0], c_point[p][1], c_point[p][2]};
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          const double t = q == 0 ? m[0][f] : m[q][f] + bc[f];
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            double& dst = f < 2 ? G[r][q][f] : H[r][q][f - 2];
+            dst = fma(wx[r], t, dst);
+          }
+        }
+    }
+    // the common phase, and 1 / (4 pi)
+    double s0, c0;
+    sincos(kr0, &s0, &c0);
+    s0 *= INV_FOUR_PI;
+    c0 *= INV_FOUR_PI;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const double gr = G[p][q][0], hr = H[p][q][0];
+        G[p][q][0] = gr * c0 - G[p][q][1] * s0;
+        G[p][q][1] = gr * s0 + G[p][q][1] * c0;
+        H[p][q][0] = hr * c0 - H[p][q][1] * s0;
+        H[p][q][1] = hr * s0 + H[p][q][1] * c0;
+      }
+    // x = v_0 + s E_1 + t E_2, y = u_0 + s' F_1 + t' F_2:
+    //   T_ab = c_a c_b [-i k sum G (x - v_a).(y - u_b) - 4 / (i k) sum G]
+    //   K_ab = -c_a c_b (v_a - u_b) . sum g (y - u_b) x (x - v_a)
+    double E[2][3], F[2][3], De[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      xp[c] = vt[c] + c_tri_s[p] * (vt[3 + c] - vt[c]) + c_tri_t[p] * (vt[6 + c] - vt[c]) - ot[c];
-      e[c] = xp[c] + D[c];
+      De[c] = X.v[c][a] - Y.v[c][b];
+      E[0][c] = X.v[3 + c][a] - X.v[c][a];
+      E[1][c] = X.v[6 + c][a] - X.v[c][a];
+      F[0][c] = Y.v[3 + c][b] - Y.v[c][b];
+      F[1][c] = Y.v[6 + c][b] - Y.v[c][b];
     }
-    const double wp = At2 * c_tri_w[p];
-    C2 R{0, 0}, Qp{0, 0}, Ry[3], Qy[3];
+    // ef = E_i . F_j, V_ij(a, b) = det(v_a - u_b, F_j, E_i) from D_ij = det(De, F_j, E_i),
+    // Av_j = det(E_1, E_2, F_j), Bv_i = det(F_1, F_2, E_i)
+    double ef[2][2], Dv[2][2], Av[2], Bv[2], t3[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) Ry[c] = Qy[c] = C2{0, 0};
+    for (int p = 0; p < 2; ++p)
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const double d0 = e[0] - yq[q][0], d1 = e[1] - yq[q][1], d2 = e[2] - yq[q][2];
-      const double r = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-      C2 G, g;
-      helmholtz(kr, ki, r, G, g);
-      G = cscale(G, wq[q]);
-      g = cscale(g, wq[q]);
-      R = cadd(R, G);
-      Qp = cadd(Qp, g);
+      for (int q = 0; q < 2; ++q) {
+        ef[p][q] = dot3(E[p], F[q]);
+        cross3(F[q], E[p], t3);
+        Dv[p][q] = dot3(De, t3);
+        if (p == 1) Av[q] = -dot3(E[0], t3);
+        if (q == 1) Bv[p] = dot3(F[0], t3);
+      }
+    // sum over (i, j) of ef G_ij, with the S0 term of T folded in: X_ab = Xs - Hx_b - Hy_a + ef_ab S0
+    double Xs[2], Hx[2][2], Hy[2][2];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        Ry[c] = cadd(Ry[c], cscale(G, yq[q][c]));
-        Qy[c] = cadd(Qy[c], cscale(g, yq[q][c]));
+    for (int c = 0; c < 2; ++c) {
+      Xs[c] = m4k2 * G[0][0][c];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) Hx[q][c] = fma(ef[0][q], G[1][0][c], ef[1][q] * G[2][0][c]);
+#pragma unroll
+      for (int p = 0; p < 2; ++p) Hy[p][c] = fma(ef[p][0], G[0][1][c], ef[p][1] * G[0][2][c]);
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) Xs[c] = fma(ef[p][q], G[1 + p][1 + q][c], Xs[c]);
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const int mrow = X.dof[p][a];
+      const double cp = X.c[p][a];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        double x2c[2], kk[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          double t = Xs[c];
+          if (q > 0) t -= Hx[q - 1][c];
+          if (p > 0) t -= Hy[p - 1][c];
+          if (p > 0 && q > 0) t = fma(ef[p - 1][q - 1], G[0][0][c], t);
+          x2c[c] = t;
+        }
+        double V[2][2];
+#pragma unroll
+        for (int ii = 0; ii < 2; ++ii)
+#pragma unroll
+          for (int jj = 0; jj < 2; ++jj) {
+            double t = Dv[ii][jj];
+            if (p == 2 - ii) t += ii == 0 ? Av[jj] : -Av[jj];  // v_a = v_0 + E of the other index
+            if (q == 2 - jj) t += jj == 0 ? Bv[ii] : -Bv[ii];
+            V[ii][jj] = t;
+          }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          double s = 0.0;
+#pragma unroll
+          for (int ii = 0; ii < 2; ++ii)
+#pragma unroll
+            for (int jj = 0; jj < 2; ++jj) {
+              double n = H[1 + ii][1 + jj][c];
+              if (q == jj + 1) n -= H[1 + ii][0][c];
+              if (p == ii + 1) n -= H[0][1 + jj][c];
+              if (p == ii + 1 && q == jj + 1) n += H[0][0][c];
+              s = fma(V[ii][jj], n, s);
+            }
+          kk[c] = s;
+        }
+        const double cc = cp * Y.c[q][b];
+        const int ncol = Y.dof[q][b];
+        const int64_t at = mrow < ncol ? int64_t(mrow) * N + ncol : int64_t(ncol) * N + mrow;
+        add_entry(M, at, C2{cc * (k * x2c[1]), -(cc * (k * x2c[0]))}, C2{cc * kk[0], cc * kk[1]});
       }
     }
-    R = cscale(R, wp);
-    Qp = cscale(Qp, wp);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      Ry[c] = cscale(Ry[c], wp);
-      Qy[c] = cscale(Qy[c], wp);
-    }
-    M.S0 = cadd(M.S0, R);
-    M.Q = cadd(M.Q, Qp);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      M.Sx[c] = cadd(M.Sx[c], cscale(R, xp[c]));
-      M.Sy[c] = cadd(M.Sy[c], Ry[c]);
-      M.Sxy = cadd(M.Sxy, cscale(Ry[c], xp[c]));
-      M.Gx[c] = cadd(M.Gx[c], cscale(Qp, xp[c]));
-      M.Gy[c] = cadd(M.Gy[c], Qy[c]);
-    }
-    // C += x' x Qy
-    M.C[0] = cadd(M.C[0], csub(cscale(Qy[2], xp[1]), cscale(Qy[1], xp[2])));
-    M.C[1] = cadd(M.C[1], csub(cscale(Qy[0], xp[2]), cscale(Qy[2], xp[0])));
-    M.C[2] = cadd(M.C[2], csub(cscale(Qy[1], xp[0]), cscale(Qy[0], xp[1])));
   }
-  const int N = A.blk_N[i];
-  const int64_t base = A.blk_mat_off[i];
-#pragma unroll 1
-  for (int a = 0; a < 3; ++a) {
-    double pa[3];
-    for (int c = 0; c < 3; ++c) pa[c] = vt[3 * a + c] - ot[c];
-    const double ca = A.bt_c[3 * qt + a];
-    const int m = A.bt_dof[3 * qt + a];
-#pragma unroll 1
-    for (int b = 0; b < 3; ++b) {
-      double qb[3];
-      for (int c = 0; c < 3; ++c) qb[c] = vs[3 * b + c] - os[c];
-      C2 Tv, Kv;
-      local_entry(M, pa, qb, D, ca * A.bt_c[3 * qs + b], kr, ki, Tv, Kv);
-      add_entry(TK, base + int64_t(m) * N + A.bt_dof[3 * qs + b], Tv, Kv);
+}
+
+struct __align__(16) Entry64 {
+  double x, y, z, w;
+};
+
+// lower triangle of every block from the upper one (M symmetric), 32 x 32
+// entries per CTA through shared memory; with amax, also the block's largest
+// |re|, |im| of T and K (float bits), which the FP16 operator tiles scale by
+template <class V4>
+__global__ void __launch_bounds__(256) k_mirror(V4* __restrict__ TK, const int64_t* __restrict__ tile_prefix, int nblk,
+                                                const int32_t* __restrict__ blk_N,
+                                                const int64_t* __restrict__ blk_mat_off, unsigned* __restrict__ amax) {
+  __shared__ V4 t[32][33];
+  const PairTile P = pair_tile(blockIdx.x, tile_prefix, nblk, 32);
+  const int N = blk_N[P.blk];
+  V4* M = TK + blk_mat_off[P.blk];
+  const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  float mx = 0.f;
+#pragma unroll
+  for (int y = ly; y < 32; y += 8) {
+    const int r = P.t0 + y, c = P.s0 + lx;
+    if (r < N && c < N && r <= c) {
+      const V4 v = M[int64_t(r) * N + c];
+      t[y][lx] = v;
+      mx = fmaxf(mx, fmaxf(fmaxf(fabsf(float(v.x)), fabsf(float(v.y))), fmaxf(fabsf(float(v.z)), fabsf(float(v.w)))));
     }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int y = ly; y < 32; y += 8) {
+    const int r = P.s0 + y, c = P.t0 + lx;  // transposed tile
+    if (r < N && c < N && c < r) M[int64_t(r) * N + c] = t[lx][y];
+  }
+  if (amax) {
+    mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+    if (lx == 0) atomicMax(amax + P.blk, __float_as_uint(mx));
   }
 }
 
@@ -269,15 +429,6 @@ __global__ void __launch_bounds__(128) k_regular64(BlockArgs A, const int64_t* _
 // complex sums.  Measured: 15.4 -> 3.5 ms for the 2 x 2 x 2 cube's 11,664
 // coincident, 17,496 edge and 52,272 vertex pairs (n_ss = 4).
 // ---------------------------------------------------------------------------
-
-// 1 / sqrt(d), d > 0: the hardware approximation refined by one step of the
-// cubic Householder iteration y + y e (1/2 + 3/8 e), e = 1 - d y^2
-__device__ __forceinline__ double rsqrt_h(double d) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-(d * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
 
 // sum over the 16 lanes of a pair of N values per lane by recursive halving:
 // the lane ends with values [base, base + count) of the sums in v[0 ..]
@@ -334,13 +485,6 @@ static std::vector<double> singular_table(int kind, int n_ss, int& npts) {
     for (int r = 0; r < rows; ++r) t[size_t(r) * npts + p] = v[size_t(r)];
   }
   return t;
-}
-
-__device__ __forceinline__ double dot3(const double* a, const double* b) { return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2])); }
-__device__ __forceinline__ void cross3(const double* a, const double* b, double* c) {
-  c[0] = fma(a[1], b[2], -(a[2] * b[1]));
-  c[1] = fma(a[2], b[0], -(a[0] * b[2]));
-  c[2] = fma(a[0], b[1], -(a[1] * b[0]));
 }
 
 template <int KIND, class OutT>
@@ -522,17 +666,23 @@ __global__ void __launch_bounds__(128) k_singular64(BlockArgs A, const SingPair*
   }
   const int N = A.blk_N[P.block];
   const int64_t ra = A.bt_dof[3 * qt + pa], cb = A.bt_dof[3 * qs + pb];
-  add_entry(TK, A.blk_mat_off[P.block] + ra * N + cb, Tv, Kv);
-  // the swapped pair (sigma, tau) of an adjacent pair: the same value at
-  // the transposed position (symmetric Galerkin forms)
-  if (KIND != 0) add_entry(TK, A.blk_mat_off[P.block] + cb * N + ra, Tv, Kv);
+  // upper position (k_mirror fills the lower one).  Both orderings of an
+  // adjacent pair have this value at transposed positions: once here, twice on
+  // the diagonal; a coincident pair holds every (a, b) with (b, a) itself.
+  const int64_t mat = A.blk_mat_off[P.block];
+  if (KIND == 0) {
+    if (ra <= cb) add_entry(TK, mat + ra * N + cb, Tv, Kv);
+  } else {
+    const double two = ra == cb ? 2.0 : 1.0;
+    add_entry(TK, mat + (ra < cb ? ra * N + cb : cb * N + ra), cscale(Tv, two), cscale(Kv, two));
+  }
 }
 
 // the three kinds of the mesh's singular pairs (sorted by kind)
 template <class OutT>
 static void launch_singular(mtf_system sys, const BlockArgs& A, OutT* TK, cudaStream_t s) {
   mtf_mesh m = sys->mesh;
-  int64_t at = 0;
+  int64_t at = 0;  // the list is sorted by kind
   for (int kind = 0; kind < 3; ++kind) {
     int64_t end = at;
     while (end < int64_t(m->sing.size()) && (m->sing[size_t(end)].code & 3) == kind) ++end;
@@ -732,6 +882,20 @@ static void upload_rule_constants(cudaStream_t s) {
   MTF_CUDA(cudaMemcpyToSymbolAsync(c_tri_s, r.s, sizeof(r.s), 0, cudaMemcpyHostToDevice, s));
   MTF_CUDA(cudaMemcpyToSymbolAsync(c_tri_t, r.t, sizeof(r.t), 0, cudaMemcpyHostToDevice, s));
   MTF_CUDA(cudaMemcpyToSymbolAsync(c_tri_w, r.w, sizeof(r.w), 0, cudaMemcpyHostToDevice, s));
+  double orbit[2][3], point[6][3];
+  for (int o = 0; o < 2; ++o) {
+    const double w = r.w[3 * o], a = r.s[3 * o];
+    orbit[o][0] = w;
+    orbit[o][1] = w * a;
+    orbit[o][2] = w * (1.0 - 3.0 * a);
+  }
+  for (int p = 0; p < 6; ++p) {
+    point[p][0] = r.w[p];
+    point[p][1] = r.w[p] * r.s[p];
+    point[p][2] = r.w[p] * r.t[p];
+  }
+  MTF_CUDA(cudaMemcpyToSymbolAsync(c_orbit, orbit, sizeof(orbit), 0, cudaMemcpyHostToDevice, s));
+  MTF_CUDA(cudaMemcpyToSymbolAsync(c_point, point, sizeof(point), 0, cudaMemcpyHostToDevice, s));
 }
 
 static BlockArgs block_args(mtf_system sys) {
@@ -779,9 +943,11 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
     sys->d_TK64.alloc(size_t(m->n_mat) * 4);
     MTF_CUDA(cudaMemsetAsync(sys->d_TK64.p, 0, size_t(m->n_mat) * 4 * sizeof(double), s));
     const int64_t nct = m->reg_cta_prefix.back();
-    if (nct > 0)
-      MTF_LAUNCH(KID_REGULAR64, s, k_regular64<<<unsigned(nct), 128, 0, s>>>(A, m->d_reg_cta_prefix.p, sys->d_TK64.p));
+    MTF_LAUNCH(KID_REGULAR64, s, k_regular64<<<unsigned(nct), 128, 0, s>>>(A, m->d_reg_cta_prefix.p, sys->d_TK64.p));
     launch_singular(sys, A, sys->d_TK64.p, s);
+    MTF_LAUNCH(KID_MIRROR, s, k_mirror<Entry64><<<unsigned(m->mirror_cta_prefix.back()), 256, 0, s>>>(
+        reinterpret_cast<Entry64*>(sys->d_TK64.p), m->d_mirror_cta_prefix.p, m->nd, m->d_blk_N.p, m->d_blk_mat_off.p,
+        nullptr));
   }
   if (fp64_blocks && sys->opt.precision != MTF_PREC_FP64) {
     // residual_fp64: the FP64 entries split into FP32 pairs once per assembly,
@@ -797,6 +963,9 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
     MTF_CUDA(cudaMemsetAsync(sys->d_TK32.p, 0, size_t(m->n_mat) * 4 * sizeof(float), s));
     launch_assemble_regular32(sys, s);
     launch_singular(sys, A, sys->d_TK32.p, s);
+    MTF_LAUNCH(KID_MIRROR, s, k_mirror<float4><<<unsigned(m->mirror_cta_prefix.back()), 256, 0, s>>>(
+        reinterpret_cast<float4*>(sys->d_TK32.p), m->d_mirror_cta_prefix.p, m->nd, m->d_blk_N.p, m->d_blk_mat_off.p,
+        sys->opt.mv_tensor ? tc_operator_amax(sys, s) : nullptr));
     if (sys->opt.mv_tensor) tc_build_operator(sys, s);
     else tile_matvec_operator(sys, s);
   }

@@ -170,8 +170,10 @@ struct mtf_mesh_s {
   mtf::DevBuf<int64_t> d_blk_mat_off;        // per block
   mtf::DevBuf<int32_t> d_blk_N, d_blk_T;
   mtf::DevBuf<int64_t> d_blk_bt_off, d_blk_dof_off, d_blk_row_off;
-  std::vector<int64_t> reg_cta_prefix;       // regular-pair CTA prefix over blocks
-  mtf::DevBuf<int64_t> d_reg_cta_prefix;
+  // CTA prefixes over blocks of the regular-pair tiles (16 triangles per side)
+  // and of the mirror tiles (32 rows per side)
+  std::vector<int64_t> reg_cta_prefix, mirror_cta_prefix;
+  mtf::DevBuf<int64_t> d_reg_cta_prefix, d_mirror_cta_prefix;
   mtf::DevBuf<int32_t> d_row_blk;            // exchange row -> block
   // streaming work units of the FP32 matvec ({T, K} entries) and of the
   // OSRC apply (T~ entries)
@@ -236,7 +238,7 @@ struct mtf_system_s {
   mtf::DevBuf<float> d_os_coef16;            // per block: s_i (rho, 1/rho) for the FP16 copy
   mtf::DevBuf<float> d_os_part;              // per-row piece sums of the OSRC apply
   mtf::DevBuf<double> d_cen;
-  mtf::DevBuf<float> d_qx, d_qw, d_pv, d_cc;
+  mtf::DevBuf<float> d_qx, d_pv, d_cc;
   int32_t ss_npts[3] = {0, 0, 0};
   // streaming matvec: per-row piece sums and the error word (d_mv_ctl[2])
   mtf::DevBuf<float> d_mv_part;
@@ -257,7 +259,7 @@ enum KernelId {
   KID_REGULAR64 = 0, KID_SINGULAR64, KID_XVALUES, KID_RHS, KID_MATVEC64, KID_DOTS, KID_AXPY,
   KID_NORM, KID_SUB, KID_FARFIELD, KID_SPLIT, KID_REGULAR32, KID_MATVEC32, KID_OSRC, KID_MLP,
   KID_MISC, KID_MVCOMBINE, KID_OSCOMBINE, KID_MVTC, KID_MVTC_PREP, KID_MVTC_COMBINE, KID_TC_TILE,
-  KID_BCHOL, KID_BXFORM, KID_BSTORE, KID_TT, KID_TT_MMA, KID_TCA_PREP, KID_BGRAM, KID_COUNT
+  KID_BCHOL, KID_BXFORM, KID_BSTORE, KID_TT, KID_TT_MMA, KID_TCA_PREP, KID_BGRAM, KID_MIRROR, KID_COUNT
 };
 void prof_begin(int kid, cudaStream_t s);
 void prof_end(int kid, cudaStream_t s);
@@ -399,6 +401,9 @@ void probe_peaks(double* rates, cudaStream_t s);
 void osrc_form_tc(mtf_system sys, cudaStream_t s);
 // tensor-core matvec (mv_tc.cu): the FP16 hi / lo tiled operator copy built
 // after every mixed assembly (opt.mv_tensor), and y = M x from it
+// per-block largest |re|, |im| of the stored entries (cleared; filled by the
+// assembly before tc_build_operator)
+unsigned* tc_operator_amax(mtf_system sys, cudaStream_t s);
 void tc_build_operator(mtf_system sys, cudaStream_t s);
 bool tc_matvec_enabled(mtf_system sys);
 void launch_matvec_tc(mtf_system sys, const float* x, int64_t ldx, float* y, int64_t ldy, int nrhs, cudaStream_t s);

@@ -284,6 +284,7 @@ void upload_mesh(mtf_mesh m, cudaStream_t s) {
   std::vector<int64_t> mo, bo, dofo, rowo;
   std::vector<int32_t> N, T, row_blk;
   m->reg_cta_prefix.assign(1, 0);
+  m->mirror_cta_prefix.assign(1, 0);
   for (int i = 0; i < m->nd; ++i) {
     mo.push_back(m->blk[i].mat_off);
     bo.push_back(m->blk[i].bt_off);
@@ -291,8 +292,9 @@ void upload_mesh(mtf_mesh m, cudaStream_t s) {
     rowo.push_back(m->blk[i].row_off);
     N.push_back(m->blk[i].N);
     T.push_back(m->blk[i].T);
-    const int64_t pairs = int64_t(m->blk[i].T) * m->blk[i].T;
-    m->reg_cta_prefix.push_back(m->reg_cta_prefix.back() + (pairs + 127) / 128);
+    const int64_t nt = (m->blk[i].T + 15) / 16, nr = (m->blk[i].N + 31) / 32;  // tiles per side (pair_tile.cuh)
+    m->reg_cta_prefix.push_back(m->reg_cta_prefix.back() + nt * (nt + 1) / 2);
+    m->mirror_cta_prefix.push_back(m->mirror_cta_prefix.back() + nr * (nr + 1) / 2);
     for (int r = 0; r < m->blk[i].N; ++r) row_blk.push_back(i);
   }
   m->d_blk_mat_off.upload(mo, s);
@@ -302,6 +304,7 @@ void upload_mesh(mtf_mesh m, cudaStream_t s) {
   m->d_blk_N.upload(N, s);
   m->d_blk_T.upload(T, s);
   m->d_reg_cta_prefix.upload(m->reg_cta_prefix, s);
+  m->d_mirror_cta_prefix.upload(m->mirror_cta_prefix, s);
   m->d_row_blk.upload(row_blk, s);
   MTF_CUDA(cudaStreamSynchronize(s));
 }

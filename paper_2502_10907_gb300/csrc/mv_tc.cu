@@ -108,21 +108,6 @@ __device__ __forceinline__ void tc_split(float v, __half& hi, __half& lo) {
   lo = __float2half_rn(v - __half2float(hi));
 }
 
-// amax[i] = max over block i's stored T and K entries of |re|, |im|
-__global__ void k_tc_blkmax(const float4* __restrict__ TK, const int64_t* __restrict__ blk_mat_off,
-                            const int32_t* __restrict__ blk_N, unsigned* __restrict__ amax) {
-  const int i = blockIdx.y;
-  const int64_t N = blk_N[i];
-  const float4* e = TK + blk_mat_off[i];
-  float m = 0.f;
-  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < N * N; t += int64_t(gridDim.x) * blockDim.x) {
-    const float4 v = e[t];
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-  }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax + i, __float_as_uint(m));
-}
-
 // Tiled hi / lo copy: thread = (tile, row, group g of 4 complex columns);
 // writes 8 halves (16 bytes) into each of the 4 parts.
 __global__ void __launch_bounds__(256) k_tc_tile_a(const float4* __restrict__ TK, const int4* __restrict__ tile_info,
@@ -720,8 +705,16 @@ void tc_set_plan(mtf_system sys, int waves, int min_len, int grid, bool prefer_f
   if (t.osr.planned) tc_osr_plan_tables(sys, t, s);  // same tile order, new units
 }
 
+unsigned* tc_operator_amax(mtf_system sys, cudaStream_t s) {
+  if (!sys->tc) sys->tc = new TcMatvec();
+  TcMatvec& t = *sys->tc;
+  tc_plan_tables(sys, t, s);
+  MTF_CUDA(cudaMemsetAsync(t.amax.p, 0, size_t(sys->mesh->nd) * sizeof(unsigned), s));
+  return t.amax.p;
+}
+
 // FP16 hi / lo tiled copy of the FP32-stored {T, K}, rebuilt after every
-// mixed-precision assembly
+// mixed-precision assembly (scaled by tc_operator_amax)
 void tc_build_operator(mtf_system sys, cudaStream_t s) {
   if (!sys->opt.mv_tensor) return;
   if (!sys->tc) sys->tc = new TcMatvec();
@@ -733,9 +726,6 @@ void tc_build_operator(mtf_system sys, cudaStream_t s) {
     t.A.alloc(nh);
     t.amap_ptr = nullptr;
   }
-  MTF_CUDA(cudaMemsetAsync(t.amax.p, 0, size_t(m->nd) * sizeof(unsigned), s));
-  MTF_LAUNCH(KID_TC_TILE, s, k_tc_blkmax<<<dim3(256, unsigned(m->nd)), 256, 0, s>>>(
-      reinterpret_cast<const float4*>(sys->d_TK32.p), m->d_blk_mat_off.p, m->d_blk_N.p, t.amax.p));
   const int64_t nthr = t.plan.n_tiles * kTcRows * 8;
   MTF_LAUNCH(KID_TC_TILE, s, k_tc_tile_a<<<unsigned((nthr + 255) / 256), 256, 0, s>>>(
       reinterpret_cast<const float4*>(sys->d_TK32.p), t.tile_info.p, m->d_blk_mat_off.p, m->d_blk_N.p, t.amax.p,

@@ -40,3 +40,24 @@ def test_singular_pairs_over_kappa_and_rule_size(api, k0, n_ss):
         T, K = (t.cpu().numpy() for t in s.block(i))
         Tr, Kr = assemble_block(sk, i, k0 * np.sqrt(eps[i]), n_ss=n_ss)
         assert rel(T, Tr) < 1e-12 and rel(K, Kr) < 1e-12, (i, rel(T, Tr), rel(K, Kr))
+
+
+# tiles of 16 triangles: blocks of 8, 20, 24, 32 and 80 triangles (fewer than a tile, ragged, whole tiles) and every
+# length of the phase series, up to pairs that fall back to sincos (k times the radii above 2)
+@pytest.mark.parametrize("mesh, k0", [("cube1", 0.3), ("ico0", 0.5), ("ico0", 4.0), ("split2", 0.9), ("ico1", 2.0),
+                                      ("ico1", 6.0), ("uv", 1.3)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_regular_pairs_over_tiles_and_phases(api, mesh, k0, precision):
+    """FP64: 1e-12 as above.  Mixed: FP32 products of about 60 rounded operations per evaluation, summed over the
+    pairs of an entry: 64 x 2^-24 = 4e-6 norm-wise."""
+    m = {"cube1": lambda: mi.cube_partition((1, 1, 2), 1), "ico0": lambda: mi.icosphere(0), "ico1": lambda: mi.icosphere(1),
+         "split2": lambda: mi.split_sphere(2), "uv": lambda: mi.uv_sphere(5, 7)}[mesh]()
+    eps = np.concatenate([[1.0], np.linspace(1.5, 2.5, m.n_domains - 1)])
+    sk = skeleton_of(m)
+    s = api.System(api.Mesh.from_inputs(m), k0, eps, np.ones(m.n_domains), precision=precision)
+    tol = 4e-6 if precision else 1e-12
+    for i in range(m.n_domains):
+        T, K = (t.cpu().numpy() for t in s.block(i))
+        Tr, Kr = assemble_block(sk, i, k0 * np.sqrt(eps[i]))
+        assert rel(T, Tr) < tol and rel(K, Kr) < tol, (i, rel(T, Tr), rel(K, Kr))
+        assert np.array_equal(T, T.T) and np.array_equal(K, K.T)
