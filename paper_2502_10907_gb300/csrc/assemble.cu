@@ -22,6 +22,7 @@
 #include <cmath>
 
 #include "common.h"
+#include "kernel64.cuh"
 #include "pair_tile.cuh"
 
 namespace mtf {
@@ -30,8 +31,6 @@ __constant__ double c_tri_s[6], c_tri_t[6], c_tri_w[6];  // 6-point rule
 // per orbit (a, a, 1 - 2a): w, w a, w (1 - 3a); per point: w, w s, w t
 __constant__ double c_orbit[2][3], c_point[6][3];
 
-#define INV_FOUR_PI 0.079577471545947667884
-
 struct C2 {
   double re, im;
 };
@@ -39,18 +38,6 @@ __device__ __forceinline__ C2 cmul(C2 a, C2 b) { return {a.re * b.re - a.im * b.
 __device__ __forceinline__ C2 cscale(C2 a, double s) { return {a.re * s, a.im * s}; }
 __device__ __forceinline__ C2 cadd(C2 a, C2 b) { return {a.re + b.re, a.im + b.im}; }
 __device__ __forceinline__ C2 csub(C2 a, C2 b) { return {a.re - b.re, a.im - b.im}; }
-
-// G = exp(i k r) / (4 pi r) and g = G (i k - 1/r) / r for complex k.
-__device__ __forceinline__ void helmholtz(double kr, double ki, double r, C2& G, C2& g) {
-  const double rinv = 1.0 / r;
-  double sn, cs;
-  sincos(kr * r, &sn, &cs);
-  double amp = INV_FOUR_PI * rinv;
-  if (ki != 0.0) amp *= exp(-ki * r);
-  G = {amp * cs, amp * sn};
-  const C2 f{-ki - rinv, kr};  // i k - 1/r
-  g = cscale(cmul(G, f), rinv);
-}
 
 __device__ __forceinline__ void add_entry(double* TK, int64_t idx, C2 T, C2 K) {
   double* e = TK + 4 * idx;
@@ -91,38 +78,6 @@ struct BlockArgs {
   const double* k;  // (re, im) per block
   int nblk;
 };
-
-// (cos x, sin x / x) series in x^2: coefficients of x^(2t)
-__constant__ double c_cos[13] = {1.0, -1.0 / 2, 1.0 / 24, -1.0 / 720, 1.0 / 40320, -1.0 / 3628800, 1.0 / 479001600,
-                                 -1.0 / 87178291200.0, 1.0 / 20922789888000.0, -1.0 / 6402373705728000.0,
-                                 1.0 / 2432902008176640000.0, -1.0 / 1124000727777607680000.0,
-                                 1.0 / 620448401733239439360000.0};
-__constant__ double c_sin[13] = {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880, -1.0 / 39916800,
-                                 1.0 / 6227020800.0, -1.0 / 1307674368000.0, 1.0 / 355687428096000.0,
-                                 -1.0 / 121645100408832000.0, 1.0 / 51090942171709440000.0,
-                                 -1.0 / 25852016738884976640000.0, 1.0 / 15511210043330985984000000.0};
-
-// terms beyond the first of the series above that carry |x| <= xmax to FP64
-// rounding (next term below 1e-16); -1: too wide for them
-__device__ __forceinline__ int series_degree(float xmax) {
-  return xmax <= 0.25f ? 6 : xmax <= 0.5f ? 7 : xmax <= 1.f ? 9 : xmax <= 1.5f ? 10 : xmax <= 2.f ? 12 : -1;
-}
-
-// 1 / sqrt(d), d > 0: the hardware approximation refined by one step of the
-// cubic Householder iteration y + y e (1/2 + 3/8 e), e = 1 - d y^2
-__device__ __forceinline__ double rsqrt_h(double d) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-(d * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-__device__ __forceinline__ double dot3(const double* a, const double* b) { return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2])); }
-__device__ __forceinline__ void cross3(const double* a, const double* b, double* c) {
-  c[0] = fma(a[1], b[2], -(a[2] * b[1]));
-  c[1] = fma(a[2], b[0], -(a[0] * b[2]));
-  c[2] = fma(a[0], b[1], -(a[1] * b[0]));
-}
 
 // triangles of one side of a tile: quadrature points, vertices, c_a 2 A
 struct Side64 {
@@ -788,81 +743,6 @@ __global__ void k_rhs(const int32_t* __restrict__ dof_bt, int N0, int nrhs, int6
   bc[2 * (N0 + m) + 1] = 2.0 * sN.im;
 }
 
-// ---------------------------------------------------------------------------
-// far field (Stratton-Chu in Omega_0): one CTA per (direction, rhs)
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_farfield(const double* __restrict__ x, int64_t n_total, int N0,
-                                                  int T0, const double* __restrict__ bt_v,
-                                                  const double* __restrict__ bt_c,
-                                                  const double* __restrict__ bt_area,
-                                                  const int32_t* __restrict__ bt_dof, double k0,
-                                                  const double* __restrict__ obs, int nobs,
-                                                  double* __restrict__ fout) {
-  const int o = blockIdx.x, col = blockIdx.y;
-  const double xh[3] = {obs[3 * o], obs[3 * o + 1], obs[3 * o + 2]};
-  const double* xc = x + 2 * int64_t(col) * n_total;
-  double acc[12];
-  for (int c = 0; c < 12; ++c) acc[c] = 0.0;  // wa (re,im)x3, wb (re,im)x3
-  for (int it = threadIdx.x; it < T0 * 6; it += blockDim.x) {
-    const int q = it / 6, qp = it % 6;
-    const double* v = bt_v + 9 * int64_t(q);
-    double y[3];
-    for (int c = 0; c < 3; ++c) y[c] = v[c] + c_tri_s[qp] * (v[3 + c] - v[c]) + c_tri_t[qp] * (v[6 + c] - v[c]);
-    double sn, cs;
-    sincos(-k0 * (xh[0] * y[0] + xh[1] * y[1] + xh[2] * y[2]), &sn, &cs);
-    const double w = 2.0 * bt_area[q] * c_tri_w[qp];
-    for (int a = 0; a < 3; ++a) {
-      const int m = bt_dof[3 * q + a];
-      const double ca = bt_c[3 * q + a] * w;
-      const C2 uD{xc[2 * m], xc[2 * m + 1]}, uN{xc[2 * (N0 + m)], xc[2 * (N0 + m) + 1]};
-      const C2 fD = cmul(uD, C2{cs * ca, sn * ca}), fN = cmul(uN, C2{cs * ca, sn * ca});
-      for (int c = 0; c < 3; ++c) {
-        const double f = y[c] - v[3 * a + c];
-        acc[2 * c] += fD.re * f;
-        acc[2 * c + 1] += fD.im * f;
-        acc[6 + 2 * c] += fN.re * f;
-        acc[6 + 2 * c + 1] += fN.im * f;
-      }
-    }
-  }
-  __shared__ double red[8][12];
-  for (int c = 0; c < 12; ++c) {
-    double v = acc[c];
-    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    acc[c] = v;
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0)
-    for (int c = 0; c < 12; ++c) red[warp][c] = acc[c];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s[12];
-    for (int c = 0; c < 12; ++c) {
-      s[c] = 0;
-      for (int w = 0; w < int(blockDim.x >> 5); ++w) s[c] += red[w][c];
-    }
-    // E = i k0/(4 pi) [xh x wa + (xh x wb) x xh]
-    double out[6];
-    for (int ri = 0; ri < 2; ++ri) {
-      const double wa[3] = {s[ri], s[2 + ri], s[4 + ri]};
-      const double wb[3] = {s[6 + ri], s[8 + ri], s[10 + ri]};
-      const double t1[3] = {xh[1] * wa[2] - xh[2] * wa[1], xh[2] * wa[0] - xh[0] * wa[2],
-                            xh[0] * wa[1] - xh[1] * wa[0]};
-      const double u[3] = {xh[1] * wb[2] - xh[2] * wb[1], xh[2] * wb[0] - xh[0] * wb[2],
-                           xh[0] * wb[1] - xh[1] * wb[0]};
-      const double t2[3] = {u[1] * xh[2] - u[2] * xh[1], u[2] * xh[0] - u[0] * xh[2],
-                            u[0] * xh[1] - u[1] * xh[0]};
-      for (int c = 0; c < 3; ++c) out[2 * c + ri] = t1[c] + t2[c];
-    }
-    double* f = fout + 2 * 3 * (int64_t(col) * nobs + o);
-    const double sc = k0 * INV_FOUR_PI;
-    for (int c = 0; c < 3; ++c) {  // multiply by i sc
-      f[2 * c] = -sc * out[2 * c + 1];
-      f[2 * c + 1] = sc * out[2 * c];
-    }
-  }
-}
-
 template <class MatT>
 __global__ void k_split_block(const MatT* __restrict__ TK, int64_t n, double* __restrict__ T,
                               double* __restrict__ K) {
@@ -997,117 +877,6 @@ void launch_rhs(mtf_system sys, int nrhs, const double* d_dirs, const double* d_
   const int64_t nth = int64_t(N0) * nrhs;
   MTF_LAUNCH(KID_RHS, s, k_rhs<<<unsigned((nth + 127) / 128), 128, 0, s>>>(m->d_dof_bt.p, N0, nrhs, m->n_total, m->d_bt_v.p,
                                                       m->d_bt_c.p, m->d_bt_area.p, sys->k0, d_dirs, d_pols, b));
-  MTF_CUDA(cudaGetLastError());
-}
-
-// ---------------------------------------------------------------------------
-// near field (Stratton-Chu, Eq. 8): for a point x in Omega_i,
-//   U(x) = H_k(a)(x) + E_k(b)(x),  a = gamma_D U,  b = gamma_N U (N slot / rho_i),
-//   H_k a = int grad_x G x a,  E_k b = i k int G b - 1/(i k) int grad_x G div b,
-// with k = k_i, the RWG fields of block i's coefficients and div psi_a = 2 c_a.
-// One CTA per (point, rhs); the 6-point rule on every triangle of block i.
-// blk: per block {first block-triangle, triangles, N, dof offset}.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_nearfield(const double* __restrict__ x, int64_t n_total,
-                                                   const double* __restrict__ bt_v,
-                                                   const double* __restrict__ bt_c,
-                                                   const double* __restrict__ bt_area,
-                                                   const int32_t* __restrict__ bt_dof,
-                                                   const int64_t* __restrict__ blk, const double* __restrict__ kk,
-                                                   const double* __restrict__ rho, const double* __restrict__ pts,
-                                                   const int32_t* __restrict__ dom, int npts,
-                                                   double* __restrict__ fout) {
-  const int p = blockIdx.x, col = blockIdx.y;
-  const int i = dom[p];
-  const double X[3] = {pts[3 * p], pts[3 * p + 1], pts[3 * p + 2]};
-  const int64_t q0 = blk[4 * i], T = blk[4 * i + 1], N = blk[4 * i + 2], off = blk[4 * i + 3];
-  const double kr = kk[2 * i], ki = kk[2 * i + 1];
-  const double rr = rho[2 * i], ri = rho[2 * i + 1], rn = rr * rr + ri * ri;
-  const C2 irho{rr / rn, -ri / rn};
-  const C2 ik{-ki, kr};
-  const double kn = kr * kr + ki * ki;
-  const C2 minv_ik{ki / kn, kr / kn};  // -1 / (i k)
-  const double* xc = x + 2 * int64_t(col) * n_total;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int64_t it = threadIdx.x; it < T * 6; it += blockDim.x) {
-    const int64_t q = q0 + it / 6;
-    const int qp = int(it % 6);
-    const double* v = bt_v + 9 * q;
-    double y[3], d[3];
-    for (int c = 0; c < 3; ++c) {
-      y[c] = v[c] + c_tri_s[qp] * (v[3 + c] - v[c]) + c_tri_t[qp] * (v[6 + c] - v[c]);
-      d[c] = X[c] - y[c];
-    }
-    const double R = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    C2 G, g;
-    helmholtz(kr, ki, R, G, g);  // grad_x G = g d
-    const double w = 2.0 * bt_area[q] * c_tri_w[qp];
-    C2 av[3] = {{0, 0}, {0, 0}, {0, 0}}, bv[3] = {{0, 0}, {0, 0}, {0, 0}}, divb{0, 0};
-    for (int a = 0; a < 3; ++a) {
-      const int64_t m = bt_dof[3 * q + a];
-      const double ca = bt_c[3 * q + a];
-      const C2 uD{xc[2 * (off + m)], xc[2 * (off + m) + 1]};
-      const C2 uN = cmul(C2{xc[2 * (off + N + m)], xc[2 * (off + N + m) + 1]}, irho);
-      for (int c = 0; c < 3; ++c) {
-        const double f = ca * (y[c] - v[3 * a + c]);
-        av[c] = cadd(av[c], cscale(uD, f));
-        bv[c] = cadd(bv[c], cscale(uN, f));
-      }
-      divb = cadd(divb, cscale(uN, 2.0 * ca));
-    }
-    const C2 ikG = cmul(ik, G);
-    const C2 e2 = cmul(minv_ik, cmul(g, divb));
-    for (int c = 0; c < 3; ++c) {
-      const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
-      const C2 cr = csub(cscale(av[c2], d[c1]), cscale(av[c1], d[c2]));  // (d x a)_c
-      const C2 e = cadd(cadd(cmul(g, cr), cmul(ikG, bv[c])), cscale(e2, d[c]));
-      acc[2 * c] += w * e.re;
-      acc[2 * c + 1] += w * e.im;
-    }
-  }
-  __shared__ double red[8][6];
-  for (int c = 0; c < 6; ++c) {
-    double v = acc[c];
-    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    acc[c] = v;
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0)
-    for (int c = 0; c < 6; ++c) red[warp][c] = acc[c];
-  __syncthreads();
-  if (threadIdx.x < 6) {
-    double t = 0;
-    for (int wi = 0; wi < int(blockDim.x >> 5); ++wi) t += red[wi][threadIdx.x];
-    fout[(int64_t(col) * npts + p) * 6 + threadIdx.x] = t;
-  }
-}
-
-void launch_nearfield(mtf_system sys, const double* x, int nrhs, const double* d_pts, const int32_t* d_dom,
-                      int npts, double* f, cudaStream_t s) {
-  mtf_mesh m = sys->mesh;
-  upload_rule_constants(s);
-  std::vector<int64_t> blk(static_cast<size_t>(4 * m->nd));
-  for (int i = 0; i < m->nd; ++i) {
-    blk[size_t(4 * i)] = m->blk[i].bt_off;
-    blk[size_t(4 * i + 1)] = m->blk[i].T;
-    blk[size_t(4 * i + 2)] = m->blk[i].N;
-    blk[size_t(4 * i + 3)] = m->blk[i].dof_off;
-  }
-  DevBuf<int64_t> d_blk;
-  d_blk.upload(blk, s);
-  MTF_LAUNCH(KID_FARFIELD, s, k_nearfield<<<dim3(unsigned(npts), unsigned(nrhs)), 256, 0, s>>>(
-      x, m->n_total, m->d_bt_v.p, m->d_bt_c.p, m->d_bt_area.p, m->d_bt_dof.p, d_blk.p, sys->d_k.p, sys->d_rho.p,
-      d_pts, d_dom, npts, f));
-  MTF_CUDA(cudaStreamSynchronize(s));  // d_blk is released on return
-}
-
-void launch_farfield(mtf_system sys, const double* x, int nrhs, const double* d_obs, int nobs, double* f,
-                     cudaStream_t s) {
-  mtf_mesh m = sys->mesh;
-  upload_rule_constants(s);
-  dim3 grid{unsigned(nobs), unsigned(nrhs), 1u};
-  MTF_LAUNCH(KID_FARFIELD, s, k_farfield<<<grid, 256, 0, s>>>(x, m->n_total, m->blk[0].N, m->blk[0].T, m->d_bt_v.p, m->d_bt_c.p,
-                                   m->d_bt_area.p, m->d_bt_dof.p, sys->k0, d_obs, nobs, f));
   MTF_CUDA(cudaGetLastError());
 }
 

@@ -667,13 +667,7 @@ mtf_status mtf_nearfield(mtf_system sys, const void* x, int32_t nrhs, const doub
                       std::isfinite(points[3 * p + 1]) && std::isfinite(points[3 * p + 2]),
                   MTF_ERR_ARG, "point with a subdomain out of range or a non-finite coordinate");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    DevBuf<double> dp;
-    DevBuf<int32_t> dd;
-    dp.alloc(size_t(3) * n_pts);
-    dd.alloc(size_t(n_pts));
-    MTF_CUDA(cudaMemcpyAsync(dp.p, points, size_t(3) * n_pts * sizeof(double), cudaMemcpyHostToDevice, s));
-    MTF_CUDA(cudaMemcpyAsync(dd.p, domains, size_t(n_pts) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    launch_nearfield(sys, static_cast<const double*>(x), nrhs, dp.p, dd.p, n_pts, static_cast<double*>(f_out), s);
+    launch_nearfield(sys, static_cast<const double*>(x), nrhs, points, domains, n_pts, static_cast<double*>(f_out), s);
   });
 }
 
@@ -683,10 +677,7 @@ mtf_status mtf_farfield(mtf_system sys, const void* x, int32_t nrhs, const doubl
     MTF_REQUIRE(sys && x && obs_dirs && f_out, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(nrhs >= 1 && n_obs >= 1, MTF_ERR_ARG, "need nrhs >= 1 and n_obs >= 1");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    DevBuf<double> d_obs;
-    upload_small(d_obs, obs_dirs, size_t(n_obs) * 3, s);
-    launch_farfield(sys, static_cast<const double*>(x), nrhs, d_obs.p, n_obs, static_cast<double*>(f_out), s);
-    MTF_CUDA(cudaStreamSynchronize(s));
+    launch_farfield(sys, static_cast<const double*>(x), nrhs, obs_dirs, n_obs, static_cast<double*>(f_out), s);
   });
 }
 

@@ -106,6 +106,8 @@ struct BlockInfo {
   int64_t row_off = 0;    // first exchange row (sum_{j<i} N_j)
 };
 
+constexpr int kFieldTris = 32;  // triangles per chunk of the field kernels
+
 // Singular pair record (device): block-triangle ids and the Sauter-Schwab
 // vertex orders (local vertex indices 0..2 packed in 2 bits each).
 struct SingPair {
@@ -175,6 +177,12 @@ struct mtf_mesh_s {
   std::vector<int64_t> reg_cta_prefix, mirror_cta_prefix;
   mtf::DevBuf<int64_t> d_reg_cta_prefix, d_mirror_cta_prefix;
   mtf::DevBuf<int32_t> d_row_blk;            // exchange row -> block
+  // field evaluation: chunks of kFieldTris triangles of a block (first chunk
+  // of every block, and the end) and the dofs of each: {corner (3 t + a) |
+  // second corner << 8 (0xff: outside the chunk), local dof}
+  std::vector<int32_t> fld_chunk;
+  mtf::DevBuf<int32_t> d_fld_first;
+  mtf::DevBuf<int2> d_fld_dofs;
   // streaming work units of the FP32 matvec ({T, K} entries) and of the
   // OSRC apply (T~ entries)
   mtf::StreamUnits mv_units, os_units;
@@ -370,13 +378,10 @@ void launch_matvec(mtf_system sys, const double* x, int64_t ldx, double* y, int6
                    cudaStream_t s);
 void launch_rhs(mtf_system sys, int nrhs, const double* d_dirs, const double* d_pols, double* b,
                 cudaStream_t s);
-void launch_farfield(mtf_system sys, const double* x, int nrhs, const double* d_obs, int nobs,
-                     double* f, cudaStream_t s);
-// U(x) by the representation formula (Eq. 8) at npts points (device, 3 each)
-// in the subdomains d_dom (device), from the solutions x; f: device complex128
-// (nrhs x npts x 3)
-void launch_nearfield(mtf_system sys, const double* x, int nrhs, const double* d_pts, const int32_t* d_dom,
-                      int npts, double* f, cudaStream_t s);
+void launch_farfield(mtf_system sys, const double* x, int nrhs, const double* obs, int nobs, double* f,
+                     cudaStream_t s);
+void launch_nearfield(mtf_system sys, const double* x, int nrhs, const double* pts, const int32_t* dom, int npts,
+                      double* f, cudaStream_t s);
 void launch_get_block(mtf_system sys, int i, double* t_out, double* k_out, cudaStream_t s);
 mtf_status solve(mtf_system sys, int nrhs, const double* b_dev, double* x_dev, mtf_solve_stats* st,
                  cudaStream_t s);

@@ -297,6 +297,26 @@ void upload_mesh(mtf_mesh m, cudaStream_t s) {
     m->mirror_cta_prefix.push_back(m->mirror_cta_prefix.back() + nr * (nr + 1) / 2);
     for (int r = 0; r < m->blk[i].N; ++r) row_blk.push_back(i);
   }
+  // chunks of the field kernels
+  std::vector<int2> fdofs;
+  std::vector<int32_t> ffirst(1, 0);
+  m->fld_chunk.assign(1, 0);
+  for (int i = 0; i < m->nd; ++i) {
+    for (int t0 = 0; t0 < m->blk[i].T; t0 += mtf::kFieldTris) {
+      std::vector<int2> d;
+      for (int c = 0; c < 3 * std::min(mtf::kFieldTris, m->blk[i].T - t0); ++c) {
+        const int32_t dof = m->bt_dof[size_t(3 * (m->blk[i].bt_off + t0) + c)];
+        auto e = std::find_if(d.begin(), d.end(), [&](const int2& v) { return v.y == dof; });
+        if (e == d.end()) d.push_back(make_int2(c | 0xff << 8, dof));
+        else e->x = (e->x & 0xff) | c << 8;
+      }
+      fdofs.insert(fdofs.end(), d.begin(), d.end());
+      ffirst.push_back(int32_t(fdofs.size()));
+    }
+    m->fld_chunk.push_back(int32_t(ffirst.size()) - 1);
+  }
+  m->d_fld_first.upload(ffirst, s);
+  m->d_fld_dofs.upload(fdofs, s);
   m->d_blk_mat_off.upload(mo, s);
   m->d_blk_bt_off.upload(bo, s);
   m->d_blk_dof_off.upload(dofo, s);
