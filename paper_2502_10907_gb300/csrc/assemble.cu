@@ -331,15 +331,20 @@ struct __align__(16) Entry64 {
 
 // lower triangle of every block from the upper one (M symmetric), 32 x 32
 // entries per CTA through shared memory; with amax, also the block's largest
-// |re|, |im| of T and K (float bits), which the FP16 operator tiles scale by
+// |re|, |im| of T and K (float bits), which the FP16 operator tiles scale by;
+// with rot, a copy of the whole block as (K - i T, K + i T), the form the FP64
+// matvec multiplies with (apply.cu)
 template <class V4>
 __global__ void __launch_bounds__(256) k_mirror(V4* __restrict__ TK, const int64_t* __restrict__ tile_prefix, int nblk,
                                                 const int32_t* __restrict__ blk_N,
-                                                const int64_t* __restrict__ blk_mat_off, unsigned* __restrict__ amax) {
+                                                const int64_t* __restrict__ blk_mat_off, unsigned* __restrict__ amax,
+                                                V4* __restrict__ rot) {
   __shared__ V4 t[32][33];
   const PairTile P = pair_tile(blockIdx.x, tile_prefix, nblk, 32);
   const int N = blk_N[P.blk];
   V4* M = TK + blk_mat_off[P.blk];
+  V4* Q = rot ? rot + blk_mat_off[P.blk] : nullptr;
+  auto rotated = [](const V4& v) { return V4{v.z + v.y, v.w - v.x, v.z - v.y, v.w + v.x}; };
   const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
   float mx = 0.f;
 #pragma unroll
@@ -348,6 +353,7 @@ __global__ void __launch_bounds__(256) k_mirror(V4* __restrict__ TK, const int64
     if (r < N && c < N && r <= c) {
       const V4 v = M[int64_t(r) * N + c];
       t[y][lx] = v;
+      if (rot) Q[int64_t(r) * N + c] = rotated(v);
       mx = fmaxf(mx, fmaxf(fmaxf(fabsf(float(v.x)), fabsf(float(v.y))), fmaxf(fabsf(float(v.z)), fabsf(float(v.w)))));
     }
   }
@@ -355,7 +361,10 @@ __global__ void __launch_bounds__(256) k_mirror(V4* __restrict__ TK, const int64
 #pragma unroll
   for (int y = ly; y < 32; y += 8) {
     const int r = P.s0 + y, c = P.t0 + lx;  // transposed tile
-    if (r < N && c < N && c < r) M[int64_t(r) * N + c] = t[lx][y];
+    if (r < N && c < N && c < r) {
+      M[int64_t(r) * N + c] = t[lx][y];
+      if (rot) Q[int64_t(r) * N + c] = rotated(t[lx][y]);
+    }
   }
   if (amax) {
     mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
@@ -384,33 +393,6 @@ __global__ void __launch_bounds__(256) k_mirror(V4* __restrict__ TK, const int64
 // complex sums.  Measured: 15.4 -> 3.5 ms for the 2 x 2 x 2 cube's 11,664
 // coincident, 17,496 edge and 52,272 vertex pairs (n_ss = 4).
 // ---------------------------------------------------------------------------
-
-// sum over the 16 lanes of a pair of N values per lane by recursive halving:
-// the lane ends with values [base, base + count) of the sums in v[0 ..]
-template <int N>
-__device__ __forceinline__ void halve16(double* v, int lane, int off, int& base, int& count) {
-  constexpr int H = (N + 1) / 2;
-  const bool up = (lane & off) != 0;
-#pragma unroll
-  for (int i = 0; i < H; ++i) {
-    const double lo = v[i], hi = H + i < N ? v[H + i] : 0.0;
-    v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, off);
-  }
-  if (up) {
-    base += H;
-    count = max(0, count - H);
-  } else {
-    count = min(count, H);
-  }
-  if constexpr (H > 1) {
-    if (off > 1) halve16<H>(v, lane, off >> 1, base, count);
-  } else {
-    for (int o = off >> 1; o > 0; o >>= 1) {  // one value left: plain sums
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-      if (lane & o) count = 0;
-    }
-  }
-}
 
 // hat-table rows, sums per pair of each kind
 template <int KIND> struct SingKind;
@@ -560,7 +542,7 @@ __global__ void __launch_bounds__(128) k_singular64(BlockArgs A, const SingPair*
     }
   }
   int base = 0, count = NS;
-  halve16<NS>(acc, lane, 8, base, count);
+  halve_sum<NS>(acc, lane, 8, base, count);
 #pragma unroll
   for (int q = 0; q < (NS + 15) / 16; ++q)
     if (q < count) sums[slot][base + q] = acc[q];
@@ -822,12 +804,13 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
   if (fp64_blocks) {
     sys->d_TK64.alloc(size_t(m->n_mat) * 4);
     MTF_CUDA(cudaMemsetAsync(sys->d_TK64.p, 0, size_t(m->n_mat) * 4 * sizeof(double), s));
+    if (sys->opt.precision == MTF_PREC_FP64) sys->d_rot64.alloc(size_t(m->n_mat) * 4);
     const int64_t nct = m->reg_cta_prefix.back();
     MTF_LAUNCH(KID_REGULAR64, s, k_regular64<<<unsigned(nct), 128, 0, s>>>(A, m->d_reg_cta_prefix.p, sys->d_TK64.p));
     launch_singular(sys, A, sys->d_TK64.p, s);
     MTF_LAUNCH(KID_MIRROR, s, k_mirror<Entry64><<<unsigned(m->mirror_cta_prefix.back()), 256, 0, s>>>(
         reinterpret_cast<Entry64*>(sys->d_TK64.p), m->d_mirror_cta_prefix.p, m->nd, m->d_blk_N.p, m->d_blk_mat_off.p,
-        nullptr));
+        nullptr, reinterpret_cast<Entry64*>(sys->d_rot64.p)));
   }
   if (fp64_blocks && sys->opt.precision != MTF_PREC_FP64) {
     // residual_fp64: the FP64 entries split into FP32 pairs once per assembly,
@@ -845,7 +828,7 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
     launch_singular(sys, A, sys->d_TK32.p, s);
     MTF_LAUNCH(KID_MIRROR, s, k_mirror<float4><<<unsigned(m->mirror_cta_prefix.back()), 256, 0, s>>>(
         reinterpret_cast<float4*>(sys->d_TK32.p), m->d_mirror_cta_prefix.p, m->nd, m->d_blk_N.p, m->d_blk_mat_off.p,
-        sys->opt.mv_tensor ? tc_operator_amax(sys, s) : nullptr));
+        sys->opt.mv_tensor ? tc_operator_amax(sys, s) : nullptr, nullptr));
     if (sys->opt.mv_tensor) tc_build_operator(sys, s);
     else tile_matvec_operator(sys, s);
   }

@@ -177,6 +177,9 @@ struct mtf_mesh_s {
   std::vector<int64_t> reg_cta_prefix, mirror_cta_prefix;
   mtf::DevBuf<int64_t> d_reg_cta_prefix, d_mirror_cta_prefix;
   mtf::DevBuf<int32_t> d_row_blk;            // exchange row -> block
+  // first CTA of every block of the FP64 matvec with 8, 16, 32 rows per CTA
+  std::vector<int32_t> mv_cta_prefix[3];
+  mtf::DevBuf<int32_t> d_mv_cta_prefix[3];
   // field evaluation: chunks of kFieldTris triangles of a block (first chunk
   // of every block, and the end) and the dofs of each: {corner (3 t + a) |
   // second corner << 8 (0xff: outside the chunk), local dof}
@@ -227,6 +230,7 @@ struct mtf_system_s {
   mtf::DevBuf<double> d_k, d_rho;            // (re, im) per block
   mtf::DevBuf<double> d_wdir, d_wpol, d_brhs;  // mtf_solve: wave parameters and right-hand sides (kept)
   mtf::DevBuf<double> d_TK64;                // FP64: 4 doubles per dense entry
+  mtf::DevBuf<double> d_rot64;               // FP64 systems: the entries as (K - i T, K + i T) for the matvec
   mtf::DevBuf<float> d_TK64hl;               // residual_fp64: the FP64 entries as FP32 pairs (all hi, then all lo)
   mtf::DevBuf<float> d_TK32;                 // mixed: 4 floats per dense entry
   mtf::DevBuf<float> d_TK32t;                // the same, tiled per stream unit (streaming matvec)

@@ -41,4 +41,32 @@ __device__ __forceinline__ void cross3(const double* a, const double* b, double*
   c[2] = fma(a[0], b[1], -(a[1] * b[0]));
 }
 
+// sums of N values per lane over groups of 2 off lanes by recursive halving:
+// the lane ends with values [base, base + count) of the sums in v[0 ..]
+// (start with base = 0, count = N)
+template <int N>
+__device__ __forceinline__ void halve_sum(double* v, int lane, int off, int& base, int& count) {
+  constexpr int H = (N + 1) / 2;
+  const bool up = (lane & off) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const double lo = v[i], hi = H + i < N ? v[H + i] : 0.0;
+    v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, off);
+  }
+  if (up) {
+    base += H;
+    count = max(0, count - H);
+  } else {
+    count = min(count, H);
+  }
+  if constexpr (H > 1) {
+    if (off > 1) halve_sum<H>(v, lane, off >> 1, base, count);
+  } else {
+    for (int o = off >> 1; o > 0; o >>= 1) {  // one value left: plain sums
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      if (lane & o) count = 0;
+    }
+  }
+}
+
 }  // namespace mtf

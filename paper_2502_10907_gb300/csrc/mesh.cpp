@@ -297,6 +297,12 @@ void upload_mesh(mtf_mesh m, cudaStream_t s) {
     m->mirror_cta_prefix.push_back(m->mirror_cta_prefix.back() + nr * (nr + 1) / 2);
     for (int r = 0; r < m->blk[i].N; ++r) row_blk.push_back(i);
   }
+  for (int q = 0; q < 3; ++q) {  // rows per CTA of the FP64 matvec
+    m->mv_cta_prefix[q].assign(1, 0);
+    for (int i = 0; i < m->nd; ++i)
+      m->mv_cta_prefix[q].push_back(m->mv_cta_prefix[q].back() + (m->blk[i].N + (8 << q) - 1) / (8 << q));
+    m->d_mv_cta_prefix[q].upload(m->mv_cta_prefix[q], s);
+  }
   // chunks of the field kernels
   std::vector<int2> fdofs;
   std::vector<int32_t> ffirst(1, 0);
