@@ -58,6 +58,8 @@ __device__ __forceinline__ void load_rotated(const void* entries, int64_t e, dou
 template <class MatT, int NC, int R>
 __global__ void __launch_bounds__(256, R * NC >= 4 ? 2 : 4) k_matvec(const MvArgs A, const double* __restrict__ x, int64_t ldx,
                                                 double* __restrict__ y, int64_t ldy, int c0) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
   constexpr int NV = R * NC * 4;
   __shared__ double2 us[NC][kMvCols][2];  // u+, u- of a tile of columns
   __shared__ double sums[8][NV];
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(256, R * NC >= 4 ? 2 : 4) k_matvec(const MvArg
 template <class MatT, int NC, int R>
 static void mv64_launch(mtf_system sys, const MvArgs& A, unsigned grid, const double* x, int64_t ldx, double* y,
                         int64_t ldy, int c0, cudaStream_t s) {
-  MTF_LAUNCH(KID_MATVEC64, s, k_matvec<MatT, NC, R><<<grid, 256, 0, s>>>(A, x, ldx, y, ldy, c0));
+  MTF_LAUNCH(KID_MATVEC64, s, launch_pdl(k_matvec<MatT, NC, R>, dim3(grid), dim3(256), 0, s, A, x, ldx, y, ldy, c0));
 }
 
 // passes of up to 4 right-hand sides

@@ -26,11 +26,63 @@ namespace mtf {
 constexpr size_t kStaticScratchDoubles = size_t(2) * 1024 * 1024;
 static __device__ __align__(256) double g_static_scratch[kStaticScratchDoubles];
 
-// kernels shared with the allocating solver (defined in solver.cu)
-__global__ void k_dots(const double* __restrict__ V, const double* __restrict__ w, int64_t n, int ldv,
-                       double* __restrict__ h, int ldh);
+// h[c*(ldh) + i] = <V_i^c, w^c> = sum conj(V) w  for i < j, one CTA per (i, c)
+__global__ void __launch_bounds__(256) k_dots(const double* __restrict__ V, const double* __restrict__ w,
+                                              int64_t n, int ldv, double* __restrict__ h, int ldh) {
+  const int i = blockIdx.x, c = blockIdx.y;
+  const double2* v = reinterpret_cast<const double2*>(V) + (int64_t(c) * ldv + i) * n;
+  const double2* x = reinterpret_cast<const double2*>(w) + int64_t(c) * n;
+  double sr = 0, si = 0;
+  for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
+    const double2 a = v[k], b = x[k];
+    sr += a.x * b.x + a.y * b.y;
+    si += a.x * b.y - a.y * b.x;
+  }
+  __shared__ double red[2][8];
+  for (int s = 16; s > 0; s >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, s);
+    si += __shfl_xor_sync(0xffffffffu, si, s);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = sr;
+    red[1][threadIdx.x >> 5] = si;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0, b = 0;
+    for (int q = 0; q < int(blockDim.x >> 5); ++q) {
+      a += red[0][q];
+      b += red[1][q];
+    }
+    h[2 * (int64_t(c) * ldh + i)] = a;
+    h[2 * (int64_t(c) * ldh + i) + 1] = b;
+  }
+}
+
+// w^c += sign * sum_{i<j} V_i^c h_i^c
 __global__ void k_axpy_multi(const double* __restrict__ V, const double* __restrict__ h, int j, int64_t n,
-                             int ldv, int ldh, double sign, double* __restrict__ w, int nrhs);
+                             int ldv, int ldh, double sign, double* __restrict__ w, int nrhs) {
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= n * nrhs) return;
+  const int c = int(t / n);
+  const int64_t k = t % n;
+  const double2* v = reinterpret_cast<const double2*>(V) + int64_t(c) * ldv * n + k;
+  const double* hc = h + 2 * int64_t(c) * ldh;
+  double sr = 0, si = 0;
+  for (int i = 0; i < j; ++i) {
+    const double2 a = v[int64_t(i) * n];
+    const double hr = hc[2 * i], hi = hc[2 * i + 1];
+    sr += a.x * hr - a.y * hi;
+    si += a.x * hi + a.y * hr;
+  }
+  double2* x = reinterpret_cast<double2*>(w) + int64_t(c) * n + k;
+  double2 o = *x;
+  o.x += sign * sr;
+  o.y += sign * si;
+  *x = o;
+}
+
+// kernels shared with the allocating solver (defined in solver.cu)
 __global__ void k_norm_scale(const double* __restrict__ w, int64_t n, double* __restrict__ nrm,
                              double* __restrict__ out, int64_t out_stride);
 __global__ void k_sub(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,

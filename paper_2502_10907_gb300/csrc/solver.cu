@@ -4,7 +4,9 @@
 // is one multi-column matvec.  Orthogonalisation is classical Gram-Schmidt
 // applied twice (CGS2) in FP64 on the device; the small Hessenberg least-
 // squares problems (Givens rotations) run on the host from the (j+2) new
-// Hessenberg entries per right-hand side copied back each iteration.  A
+// Hessenberg entries per right-hand side copied back each iteration, while
+// the device runs the next one (an iteration queued past convergence is
+// discarded).  A
 // restart cycle ends on convergence of every right-hand side, on the restart
 // length or on the iteration cap; each cycle starts from the true residual
 // b - M x, which is also the stopping test.
@@ -15,6 +17,7 @@
 #include <complex>
 
 #include "common.h"
+#include "kernel64.cuh"
 
 namespace mtf {
 
@@ -24,70 +27,20 @@ struct GmresWork {
   int nrhs = 0, m = 0;
   int64_t n = 0;
   DevBuf<double> V, Z, w, r, b, y;
-  DevBuf<double> h;  // [hA (m+1) x nrhs][hB (m+1) x nrhs][norm nrhs] complex
+  // two slots of [hA (m+1) x nrhs][hB (m+1) x nrhs][norm nrhs] complex [sum of
+  // squares nrhs]: step j of a cycle uses slot j mod 2 with j + 1 in place of
+  // m + 1, the norms outside the steps use slot 0 in full
+  DevBuf<double> h;
   double* h_host = nullptr;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
   ~GmresWork() {
     if (h_host) cudaFreeHost(h_host);
+    for (auto& e : ev)
+      if (e) cudaEventDestroy(e);
   }
 };
 
 void destroy_gmres(GmresWork* w) { delete w; }
-
-// h[c*(ldh) + i] = <V_i^c, w^c> = sum conj(V) w  for i < j, one CTA per (i, c)
-__global__ void __launch_bounds__(256) k_dots(const double* __restrict__ V, const double* __restrict__ w,
-                                              int64_t n, int ldv, double* __restrict__ h, int ldh) {
-  const int i = blockIdx.x, c = blockIdx.y;
-  const double2* v = reinterpret_cast<const double2*>(V) + (int64_t(c) * ldv + i) * n;
-  const double2* x = reinterpret_cast<const double2*>(w) + int64_t(c) * n;
-  double sr = 0, si = 0;
-  for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
-    const double2 a = v[k], b = x[k];
-    sr += a.x * b.x + a.y * b.y;
-    si += a.x * b.y - a.y * b.x;
-  }
-  __shared__ double red[2][8];
-  for (int s = 16; s > 0; s >>= 1) {
-    sr += __shfl_xor_sync(0xffffffffu, sr, s);
-    si += __shfl_xor_sync(0xffffffffu, si, s);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = sr;
-    red[1][threadIdx.x >> 5] = si;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0, b = 0;
-    for (int q = 0; q < int(blockDim.x >> 5); ++q) {
-      a += red[0][q];
-      b += red[1][q];
-    }
-    h[2 * (int64_t(c) * ldh + i)] = a;
-    h[2 * (int64_t(c) * ldh + i) + 1] = b;
-  }
-}
-
-// w^c += sign * sum_{i<j} V_i^c h_i^c
-__global__ void k_axpy_multi(const double* __restrict__ V, const double* __restrict__ h, int j, int64_t n,
-                             int ldv, int ldh, double sign, double* __restrict__ w, int nrhs) {
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n * nrhs) return;
-  const int c = int(t / n);
-  const int64_t k = t % n;
-  const double2* v = reinterpret_cast<const double2*>(V) + int64_t(c) * ldv * n + k;
-  const double* hc = h + 2 * int64_t(c) * ldh;
-  double sr = 0, si = 0;
-  for (int i = 0; i < j; ++i) {
-    const double2 a = v[int64_t(i) * n];
-    const double hr = hc[2 * i], hi = hc[2 * i + 1];
-    sr += a.x * hr - a.y * hi;
-    si += a.x * hi + a.y * hr;
-  }
-  double2* x = reinterpret_cast<double2*>(w) + int64_t(c) * n + k;
-  double2 o = *x;
-  o.x += sign * sr;
-  o.y += sign * si;
-  *x = o;
-}
 
 // nrm[c] = ||w^c||, out^c = w^c / nrm[c] (zero if nrm is 0); one CTA per c
 __global__ void __launch_bounds__(1024) k_norm_scale(const double* __restrict__ w, int64_t n,
@@ -123,209 +76,121 @@ __global__ void k_sub(const double* __restrict__ a, const double* __restrict__ b
 
 static inline unsigned nblk(int64_t n, int t) { return unsigned((n + t - 1) / t); }
 
-// Segmented kernels of the batched Arnoldi step: the row range is cut into
-// segments of kSeg entries so that every step keeps the whole GPU busy;
-// per-segment partial sums are accumulated with FP64 atomics (the
-// accumulators are cleared before each use).
-constexpr int kSeg = 2048;
+// Gram-Schmidt kernels of the FP64 Arnoldi step.  Bound: the FP64 pipe (4
+// instructions per entry and basis vector) once every SM has work; on small
+// systems (2,000 unknowns) the former kernels ran on 60 to 80 of the 152 SMs.
+// Measured there at 300 basis vectors: dots 20 -> 12 us, update 22 -> 12 us (with launch events).
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0;
-  if (threadIdx.x < 32) {
-    t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    for (int s = 16; s > 0; s >>= 1) t += __shfl_xor_sync(0xffffffffu, t, s);
-  }
-  return t;  // valid in thread 0
-}
-
-// h[c*ldh + i] += sum_k conj(V_i^c[k]) w^c[k] over one segment of length seg;
-// grid (segments, i, c)
-__global__ void __launch_bounds__(256) k_dots_seg(const double* __restrict__ V, const double* __restrict__ w,
-                                                  int64_t n, int ldv, double* __restrict__ h, int ldh, int64_t seg) {
-  const int i = blockIdx.y, c = blockIdx.z;
-  const int64_t k0 = int64_t(blockIdx.x) * seg;
-  const int64_t k1 = min(n, k0 + seg);
-  const double2* v = reinterpret_cast<const double2*>(V) + (int64_t(c) * ldv + i) * n;
+// h[c ldh + i] += sum over a segment of conj(V_i^c) w^c: one warp per (pair of
+// basis vectors, segment, right-hand side), the pairs of a segment in
+// consecutive warps (w's segment stays in L1); segments so that about 16
+// warps per SM run whatever the number of basis vectors is
+__global__ void __launch_bounds__(256) k_dots64(const double* __restrict__ V, const double* __restrict__ w, int64_t n,
+                                                int ldv, int rows, int nseg, int64_t seg, int nrhs,
+                                                double* __restrict__ h, int ldh) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  const int pairs = (rows + 1) / 2;
+  const int64_t id = (int64_t(blockIdx.x) * 256 + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (id >= int64_t(pairs) * nseg * nrhs) return;
+  const int i0 = 2 * int(id % pairs), g = int(id / pairs % nseg), c = int(id / (int64_t(pairs) * nseg));
+  const int64_t k0 = g * seg, k1 = min(n, k0 + seg);
+  const double2* v0 = reinterpret_cast<const double2*>(V) + (int64_t(c) * ldv + i0) * n;
+  const double2* v1 = i0 + 1 < rows ? v0 + n : v0;
   const double2* x = reinterpret_cast<const double2*>(w) + int64_t(c) * n;
-  double sr = 0, si = 0;
-#pragma unroll 8
-  for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-    const double2 a = v[k], b = x[k];
-    sr += a.x * b.x + a.y * b.y;
-    si += a.x * b.y - a.y * b.x;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int64_t k = k0 + lane; k < k1; k += 32) {
+    const double2 a = v0[k], b = v1[k], t = x[k];
+    v[0] = fma(a.x, t.x, fma(a.y, t.y, v[0]));
+    v[1] = fma(a.x, t.y, fma(-a.y, t.x, v[1]));
+    v[2] = fma(b.x, t.x, fma(b.y, t.y, v[2]));
+    v[3] = fma(b.x, t.y, fma(-b.y, t.x, v[3]));
   }
-  __shared__ double red[32];
-  sr = block_sum(sr, red);
-  si = block_sum(si, red);
-  if (threadIdx.x == 0) {
-    atomicAdd(h + 2 * (int64_t(c) * ldh + i), sr);
-    atomicAdd(h + 2 * (int64_t(c) * ldh + i) + 1, si);
-  }
-}
-
-// h[c*ldh + i] += sum_{k in segment} conj(V_i^c[k]) w^c[k]: CTA = one column
-// segment (<= 2048 entries of w staged in shared memory) x 16 basis vectors
-// (2 per warp, interleaved for 16 loads in flight); grid (segments,
-// ceil(rows/16), c).
-__global__ void __launch_bounds__(256) k_dots_stage(const double* __restrict__ V, const double* __restrict__ w,
-                                                    int64_t n, int ldv, int rows, double* __restrict__ h, int ldh,
-                                                    int64_t seg) {
-  extern __shared__ double2 ws[];
-  const int c = blockIdx.z;
-  const int64_t k0 = int64_t(blockIdx.x) * seg;
-  const int len = int(min(n, k0 + seg) - k0);
-  const double2* wc = reinterpret_cast<const double2*>(w) + int64_t(c) * n + k0;
-  for (int t = threadIdx.x; t < len; t += blockDim.x) ws[t] = wc[t];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i0 = blockIdx.y * 16 + warp * 2;
-  if (i0 >= rows) return;
-  const bool two = i0 + 1 < rows;
-  const double2* v0 = reinterpret_cast<const double2*>(V) + (int64_t(c) * ldv + i0) * n + k0;
-  const double2* v1 = two ? v0 + n : v0;
-  double r0 = 0, q0 = 0, r1 = 0, q1 = 0;
-#pragma unroll 8
-  for (int t = lane; t < len; t += 32) {
-    const double2 a = v0[t], b = v1[t], x = ws[t];
-    r0 += a.x * x.x + a.y * x.y;
-    q0 += a.x * x.y - a.y * x.x;
-    r1 += b.x * x.x + b.y * x.y;
-    q1 += b.x * x.y - b.y * x.x;
-  }
-#pragma unroll
-  for (int s2 = 16; s2 > 0; s2 >>= 1) {
-    r0 += __shfl_xor_sync(0xffffffffu, r0, s2);
-    q0 += __shfl_xor_sync(0xffffffffu, q0, s2);
-    r1 += __shfl_xor_sync(0xffffffffu, r1, s2);
-    q1 += __shfl_xor_sync(0xffffffffu, q1, s2);
-  }
-  if (lane == 0) {
-    atomicAdd(h + 2 * (int64_t(c) * ldh + i0), r0);
-    atomicAdd(h + 2 * (int64_t(c) * ldh + i0) + 1, q0);
-    if (two) {
-      atomicAdd(h + 2 * (int64_t(c) * ldh + i0 + 1), r1);
-      atomicAdd(h + 2 * (int64_t(c) * ldh + i0 + 1) + 1, q1);
-    }
-  }
+  int base = 0, count = 4;
+  halve_sum<4>(v, lane, 16, base, count);
+  if (count > 0 && i0 + base / 2 < rows) atomicAdd(h + 2 * (int64_t(c) * ldh + i0) + base, v[0]);
 }
 
 static void launch_dots(const double* V, const double* w, int64_t n, int ldv, int rows, double* h, int ldh, int nrhs,
                         cudaStream_t s) {
-  const int64_t rg = (rows + 15) / 16;
-  const int64_t minseg = (n + 2047) / 2048;
-  const int64_t nseg = std::max<int64_t>(minseg, std::min<int64_t>((n + 511) / 512, 1200 / (rg * nrhs)));
+  const int64_t pairs = (rows + 1) / 2;
+  const int64_t nseg = std::max<int64_t>(1, std::min<int64_t>((n + 63) / 64, 2432 / (pairs * nrhs)));
   const int64_t seg = (n + nseg - 1) / nseg;
-  dim3 g{unsigned(nseg), unsigned(rg), unsigned(nrhs)};
-  MTF_LAUNCH(KID_DOTS, s, k_dots_stage<<<g, 256, size_t(seg) * sizeof(double2), s>>>(V, w, n, ldv, rows, h, ldh, seg));
+  MTF_LAUNCH(KID_DOTS, s, launch_pdl(k_dots64, dim3(nblk(pairs * nseg * nrhs, 8)), dim3(256), 0, s, V, w, n, ldv, rows,
+                                     int(nseg), seg, nrhs, h, ldh));
 }
 
-// w^c -= sum_{i<j} V_i^c h_i^c ; optionally ss[c] += ||w^c||^2 (after update).
-// CTA = 32 consecutive rows x 8 groups of basis vectors (i = g mod 8), the
-// group partial sums combined in shared memory; grid (ceil(n/32), c).
-__global__ void __launch_bounds__(256) k_axpy_grp(const double* __restrict__ V, const double* __restrict__ h, int j,
-                                                  int64_t n, int ldv, int ldh, double sign, double* __restrict__ w,
-                                                  double* __restrict__ ss) {
+// w^c += sign sum_{i<j} V_i^c h_i^c ; optionally ss[c] += ||w^c||^2 (after update).
+// CTA = 8 consecutive rows (a 128-byte run of every vector) x 32 groups of
+// basis vectors (i = group mod 32): 8 lanes and 4 groups per warp
+__global__ void __launch_bounds__(256) k_axpy64(const double* __restrict__ V, const double* __restrict__ h, int j,
+                                                int64_t n, int ldv, int ldh, double sign, double* __restrict__ w,
+                                                double* __restrict__ ss) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
   const int c = blockIdx.y;
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int64_t k = int64_t(blockIdx.x) * 32 + lane;
-  __shared__ double2 part[8][32];
-  __shared__ double red[32];
-  extern __shared__ double2 hs[];  // h of this rhs (j entries)
+  const int r = threadIdx.x & 7, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t k = int64_t(blockIdx.x) * 8 + r;
+  __shared__ double2 part[8][8];
   const double2* hc = reinterpret_cast<const double2*>(h) + int64_t(c) * ldh;
-  for (int t = threadIdx.x; t < j; t += blockDim.x) hs[t] = hc[t];
-  __syncthreads();
+  const double2* v = reinterpret_cast<const double2*>(V) + int64_t(c) * ldv * n + min(k, n - 1);
   double sr = 0, si = 0;
-  if (k < n) {
-    const double2* v = reinterpret_cast<const double2*>(V) + int64_t(c) * ldv * n + k;
 #pragma unroll 8
-    for (int i = grp; i < j; i += 8) {
-      const double2 a = v[int64_t(i) * n];
-      const double2 hv = hs[i];
-      sr += a.x * hv.x - a.y * hv.y;
-      si += a.x * hv.y + a.y * hv.x;
-    }
+  for (int i = threadIdx.x >> 3; i < j; i += 32) {
+    const double2 a = v[int64_t(i) * n], t = hc[i];
+    sr = fma(a.x, t.x, fma(-a.y, t.y, sr));
+    si = fma(a.x, t.y, fma(a.y, t.x, si));
   }
-  part[grp][lane] = make_double2(sr, si);
-  __syncthreads();
-  double sq = 0;
-  if (grp == 0 && k < n) {
-    double tr = 0, ti = 0;
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      tr += part[g][lane].x;
-      ti += part[g][lane].y;
-    }
-    double2* x = reinterpret_cast<double2*>(w) + int64_t(c) * n + k;
-    double2 o = *x;
-    o.x += sign * tr;
-    o.y += sign * ti;
-    *x = o;
-    sq = o.x * o.x + o.y * o.y;
+  for (int o = 8; o < 32; o <<= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, o);
+    si += __shfl_xor_sync(0xffffffffu, si, o);
   }
-  if (ss) {
-    if (grp == 0) {
-      for (int s2 = 16; s2 > 0; s2 >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, s2);
-      if (lane == 0) atomicAdd(ss + c, sq);
+  if (lane < 8) part[warp][r] = make_double2(sr, si);
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double sq = 0;
+    if (k < n) {
+      double tr = 0, ti = 0;
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {
+        tr += part[g][r].x;
+        ti += part[g][r].y;
+      }
+      double2* x = reinterpret_cast<double2*>(w) + int64_t(c) * n + k;
+      double2 o = *x;
+      o.x = fma(sign, tr, o.x);
+      o.y = fma(sign, ti, o.y);
+      *x = o;
+      sq = fma(o.x, o.x, o.y * o.y);
     }
-  }
-  (void)red;
-}
-
-__global__ void __launch_bounds__(256) k_axpy_sq(const double* __restrict__ V, const double* __restrict__ h, int j,
-                                                 int64_t n, int ldv, int ldh, double sign, double* __restrict__ w,
-                                                 double* __restrict__ ss) {
-  const int c = blockIdx.y;
-  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  double sq = 0;
-  if (k < n) {
-    const double2* v = reinterpret_cast<const double2*>(V) + int64_t(c) * ldv * n + k;
-    const double* hc = h + 2 * int64_t(c) * ldh;
-    double sr = 0, si = 0;
-#pragma unroll 8
-    for (int i = 0; i < j; ++i) {
-      const double2 a = v[int64_t(i) * n];
-      const double hr = hc[2 * i], hi = hc[2 * i + 1];
-      sr += a.x * hr - a.y * hi;
-      si += a.x * hi + a.y * hr;
+    if (ss) {
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) sq += __shfl_xor_sync(0xffu, sq, o);
+      if (threadIdx.x == 0) atomicAdd(ss + c, sq);
     }
-    double2* x = reinterpret_cast<double2*>(w) + int64_t(c) * n + k;
-    double2 o = *x;
-    o.x += sign * sr;
-    o.y += sign * si;
-    *x = o;
-    sq = o.x * o.x + o.y * o.y;
-  }
-  if (ss) {
-    __shared__ double red[32];
-    sq = block_sum(sq, red);
-    if (threadIdx.x == 0) atomicAdd(ss + c, sq);
   }
 }
 
-// ss[c] += ||w^c||^2
-__global__ void __launch_bounds__(256) k_sqnorm(const double* __restrict__ w, int64_t n, double* __restrict__ ss) {
-  const int c = blockIdx.y;
-  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  double sq = 0;
-  if (k < n) {
-    const double2 a = reinterpret_cast<const double2*>(w)[int64_t(c) * n + k];
-    sq = a.x * a.x + a.y * a.y;
-  }
-  __shared__ double red[32];
-  sq = block_sum(sq, red);
-  if (threadIdx.x == 0) atomicAdd(ss + c, sq);
+static void launch_axpy(const double* V, const double* h, int j, int64_t n, int ldv, int ldh, double sign, double* w,
+                        double* ss, int nrhs, cudaStream_t s) {
+  MTF_LAUNCH(KID_AXPY, s, launch_pdl(k_axpy64, dim3(nblk(n, 8), unsigned(nrhs)), dim3(256), 0, s, V, h, j, n, ldv, ldh,
+                                     sign, w, ss));
 }
 
-// out^c = w^c / sqrt(ss[c]) (zero if 0); nrm[c] = (sqrt(ss[c]), 0)
+// out^c = w^c / sqrt(ss[c]) (zero if 0); nrm[c] = (sqrt(ss[c]), 0); clears the
+// nclear accumulators of the next step
 __global__ void __launch_bounds__(256) k_scale(const double* __restrict__ w, int64_t n, const double* __restrict__ ss,
-                                               double* __restrict__ nrm, double* __restrict__ out,
-                                               int64_t out_stride) {
+                                               double* __restrict__ nrm, double* __restrict__ out, int64_t out_stride,
+                                               double* __restrict__ clear, int64_t nclear) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
   const int c = blockIdx.y;
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (c == 0)
+    for (int64_t q = k; q < nclear; q += int64_t(gridDim.x) * blockDim.x) clear[q] = 0.0;
   const double t = sqrt(ss[c]);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     nrm[2 * c] = t;
@@ -347,12 +212,9 @@ static mtf_status gmres_core(mtf_system sys, int nrhs, const double* b_dev, doub
   const int64_t n = msh->n_total;
   const int m = std::max(1, sys->opt.restart);
   GmresWork& G = *sys->gw;
-  double* hA = G.h.p;
-  double* hB = G.h.p + 2 * size_t(m + 1) * nrhs;
   double* hN = G.h.p + 4 * size_t(m + 1) * nrhs;
-  double* hostA = G.h_host;
-  double* hostB = G.h_host + 2 * size_t(m + 1) * nrhs;
   double* hostN = G.h_host + 4 * size_t(m + 1) * nrhs;
+  const size_t slot = G.h.n / 2;
   const int ldv = m + 1;
   const size_t vec_bytes = size_t(n) * nrhs * 2 * sizeof(double);
 
@@ -403,8 +265,11 @@ static mtf_status gmres_core(mtf_system sys, int nrhs, const double* b_dev, doub
     ++restarts;
     std::vector<int> active(nrhs);
     for (int c = 0; c < nrhs; ++c) active[c] = !done[c];
-    for (int j = 0; j < m && total < max_iter; ++j) {
-      // flexible right preconditioning: z_j = P v_j, w = M z_j
+    // step j: z_j = P v_j (flexible right preconditioning), w = M z_j, CGS2
+    // h_A = V^H w, w -= V h_A, h_B = V^H w, w -= V h_B (with ||w||^2),
+    // v_{j+1} = w / ||w||, all on the device; its coefficients go to the
+    // pinned slot j mod 2
+    auto launch_step = [&](int j) {
       if (pre) {
         launch_osrc_apply(sys, G.V.p + 2 * size_t(j) * n, int64_t(ldv) * n, G.Z.p + 2 * size_t(j) * n,
                           int64_t(m) * n, nrhs, s);
@@ -412,35 +277,39 @@ static mtf_status gmres_core(mtf_system sys, int nrhs, const double* b_dev, doub
       } else {
         launch_matvec_kind(sys, mvkind, G.V.p + 2 * size_t(j) * n, int64_t(ldv) * n, G.r.p, n, nrhs, s);
       }
-      // CGS2: h_A = V^H w, w -= V h_A, h_B = V^H w, w -= V h_B (with ||w||^2)
-      MTF_CUDA(cudaMemsetAsync(G.h.p, 0, G.h.n * sizeof(double), s));
-      // segments per dot so that ~1200 CTAs run whatever j is
-      const int64_t nseg = std::max<int64_t>(1, std::min<int64_t>((n + 1023) / 1024,
-                                                                  1200 / (int64_t(j + 1) * nrhs)));
-      const int64_t seg = (n + nseg - 1) / nseg;
-      dim3 gd(unsigned(nseg), unsigned(j + 1), unsigned(nrhs));
-      dim3 ga(nblk(n, 256), unsigned(nrhs));
-      dim3 gg(nblk(n, 32), unsigned(nrhs));
-      double* ss = hN + 2 * nrhs;  // sum of squares scratch after the norms
-      const size_t hsm = size_t(j + 1) * sizeof(double2);
-      (void)gd;
-      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hA, m + 1, nrhs, s);
-      MTF_LAUNCH(KID_AXPY, s, k_axpy_grp<<<gg, 256, hsm, s>>>(G.V.p, hA, j + 1, n, ldv, m + 1, -1.0, G.r.p, nullptr));
-      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hB, m + 1, nrhs, s);
-      MTF_LAUNCH(KID_AXPY, s, k_axpy_grp<<<gg, 256, hsm, s>>>(G.V.p, hB, j + 1, n, ldv, m + 1, -1.0, G.r.p, ss));
-      // v_{j+1} = w / ||w||
-      MTF_LAUNCH(KID_NORM, s, k_scale<<<ga, 256, 0, s>>>(G.r.p, n, ss, hN, G.V.p + 2 * size_t(j + 1) * n, int64_t(ldv) * n));
-      MTF_CUDA(cudaMemcpyAsync(G.h_host, G.h.p, G.h.n * sizeof(double), cudaMemcpyDeviceToHost, s));
-      MTF_CUDA(cudaStreamSynchronize(s));
+      const size_t L = size_t(j) + 1;
+      double* hA = G.h.p + (j & 1) * slot;
+      double* hB = hA + 2 * L * nrhs;
+      double* nrm = hB + 2 * L * nrhs;
+      double* ss = nrm + 2 * nrhs;  // sum of squares scratch after the norms
+      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hA, j + 1, nrhs, s);
+      launch_axpy(G.V.p, hA, j + 1, n, ldv, j + 1, -1.0, G.r.p, nullptr, nrhs, s);
+      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hB, j + 1, nrhs, s);
+      launch_axpy(G.V.p, hB, j + 1, n, ldv, j + 1, -1.0, G.r.p, ss, nrhs, s);
+      MTF_LAUNCH(KID_NORM, s, launch_pdl(k_scale, dim3(nblk(n, 256), unsigned(nrhs)), dim3(256), 0, s, G.r.p, n, ss, nrm,
+                                         G.V.p + 2 * size_t(j + 1) * n, int64_t(ldv) * n, G.h.p + ((j + 1) & 1) * slot,
+                                         int64_t(4 * (L + 1) + 3) * nrhs));
+      MTF_CUDA(cudaMemcpyAsync(G.h_host + (j & 1) * slot, hA, (4 * L + 2) * nrhs * sizeof(double),
+                               cudaMemcpyDeviceToHost, s));
+      MTF_CUDA(cudaEventRecord(G.ev[j & 1], s));
+    };
+    MTF_CUDA(cudaMemsetAsync(G.h.p, 0, 7 * size_t(nrhs) * sizeof(double), s));  // step 0's accumulators
+    launch_step(0);
+    for (int j = 0; j < m && total < max_iter; ++j) {
+      if (j + 1 < m && total + 1 < max_iter) launch_step(j + 1);
+      MTF_CUDA(cudaEventSynchronize(G.ev[j & 1]));
+      const double* hostA = G.h_host + (j & 1) * slot;
+      const double* hostB = hostA + 2 * size_t(j + 1) * nrhs;
+      const double* hostW = hostB + 2 * size_t(j + 1) * nrhs;
       ++total;
       bool all_done = true;
       for (int c = 0; c < nrhs; ++c) {
         if (!active[c]) continue;
         cd* Hc = &H[size_t(c) * (m + 1) * m + size_t(j) * (m + 1)];
         for (int q = 0; q <= j; ++q)
-          Hc[q] = cd(hostA[2 * (size_t(c) * (m + 1) + q)] + hostB[2 * (size_t(c) * (m + 1) + q)],
-                     hostA[2 * (size_t(c) * (m + 1) + q) + 1] + hostB[2 * (size_t(c) * (m + 1) + q) + 1]);
-        Hc[j + 1] = cd(hostN[2 * c], 0.0);
+          Hc[q] = cd(hostA[2 * (size_t(c) * (j + 1) + q)] + hostB[2 * (size_t(c) * (j + 1) + q)],
+                     hostA[2 * (size_t(c) * (j + 1) + q) + 1] + hostB[2 * (size_t(c) * (j + 1) + q) + 1]);
+        Hc[j + 1] = cd(hostW[2 * c], 0.0);
         // previous rotations
         for (int q = 0; q < j; ++q) {
           const double cq = cs[size_t(c) * m + q];
@@ -476,7 +345,7 @@ static mtf_status gmres_core(mtf_system sys, int nrhs, const double* b_dev, doub
         ++iters[c];
         const double est = std::abs(gc[j + 1]) / bnorm[c];
         if (!std::isfinite(est)) status = MTF_ERR_NAN;
-        if (est <= tol * 0.5 || hostN[2 * c] == 0.0) active[c] = 0;
+        if (est <= tol * 0.5 || hostW[2 * c] == 0.0) active[c] = 0;
         all_done = all_done && !active[c];
       }
       if (status != MTF_OK || all_done) break;
@@ -503,8 +372,7 @@ static mtf_status gmres_core(mtf_system sys, int nrhs, const double* b_dev, doub
     if (jmax > 0) {
       MTF_CUDA(cudaMemcpyAsync(G.y.p, yhost.data(), yhost.size() * sizeof(double), cudaMemcpyHostToDevice, s));
       // x += Z y (flexible) or V y
-      MTF_LAUNCH(KID_AXPY, s, k_axpy_grp<<<dim3(nblk(n, 32), unsigned(nrhs)), 256, size_t(jmax) * sizeof(double2), s>>>(
-          pre ? G.Z.p : G.V.p, G.y.p, jmax, n, pre ? m : ldv, m + 1, 1.0, x_dev, nullptr));
+      launch_axpy(pre ? G.Z.p : G.V.p, G.y.p, jmax, n, pre ? m : ldv, m + 1, 1.0, x_dev, nullptr, nrhs, s);
       MTF_CUDA(cudaStreamSynchronize(s));  // yhost is reused next cycle
     }
   }
@@ -540,10 +408,12 @@ mtf_status solve(mtf_system sys, int nrhs, const double* b_dev, double* x_dev, m
     G.w.alloc(size_t(n) * nrhs * 2);
     G.r.alloc(size_t(n) * nrhs * 2);
     G.y.alloc(size_t(m + 1) * nrhs * 2);
-    G.h.alloc(size_t(2 * (m + 1) + 2) * nrhs * 2);
+    G.h.alloc(2 * size_t(2 * (m + 1) + 2) * nrhs * 2);
     if (G.h_host) cudaFreeHost(G.h_host);
     G.h_host = nullptr;
     MTF_CUDA(cudaMallocHost(&G.h_host, G.h.n * sizeof(double)));
+    for (auto& e : G.ev)
+      if (!e) MTF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     G.nrhs = nrhs;
     G.m = m;
     G.n = n;
