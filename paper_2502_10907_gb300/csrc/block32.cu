@@ -982,7 +982,6 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
     }
     int* kh = B.kept_host + size_t(J & 1) * (2 * s + 1);
     MTF_CUDA(cudaMemcpyAsync(kh, keptR, 2 * size_t(s) * sizeof(int), cudaMemcpyDeviceToHost, st));
-    MTF_CUDA(cudaMemcpyAsync(kh + 2 * s, err_word, sizeof(int), cudaMemcpyDeviceToHost, st));
     MTF_CUDA(cudaEventRecord(B.ev[J & 1], st));
   };
 
@@ -1008,7 +1007,7 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
       ~LsqClock() { acc += std::chrono::duration<double>(clk::now() - t).count(); }
     } lsq_clock{sys->t_lsq, tl};
     const int* kh = B.kept_host + size_t(J & 1) * (2 * s + 1);
-    if (kh[2 * s] != 0) {
+    if (*static_cast<volatile unsigned*>(err_word) != 0) {
       status = MTF_ERR_TIMEOUT;
       break;
     }
@@ -1051,7 +1050,7 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
   }
   MTF_CUDA(cudaStreamSynchronize(st));  // a step queued past the last one has finished
   if (status != MTF_OK) {
-    MTF_CUDA(cudaMemsetAsync(sys->d_mv_ctl.p, 0, 4 * sizeof(unsigned), st));
+    *static_cast<volatile unsigned*>(err_word) = 0;
     return status;
   }
   for (int c = 0; c < s; ++c) iters[c] += steps;

@@ -64,6 +64,23 @@ struct DevBuf {
   }
 };
 
+// Owning array in pinned host memory that kernels write by its host address
+// (error words: the host reads them after a synchronisation, without a copy).
+template <class T>
+struct HostBuf {
+  T* p = nullptr;
+  HostBuf() = default;
+  HostBuf(const HostBuf&) = delete;
+  HostBuf& operator=(const HostBuf&) = delete;
+  ~HostBuf() {
+    if (p) cudaFreeHost(p);
+  }
+  void alloc_zero(size_t count) {
+    MTF_CUDA(cudaHostAlloc(&p, count * sizeof(T), cudaHostAllocMapped | cudaHostAllocPortable));
+    for (size_t q = 0; q < count; ++q) p[q] = T(0);
+  }
+};
+
 // ---------------------------------------------------------------------------
 // quadrature tables (generated on the host from their defining equations)
 // ---------------------------------------------------------------------------
@@ -254,7 +271,7 @@ struct mtf_system_s {
   int32_t ss_npts[3] = {0, 0, 0};
   // streaming matvec: per-row piece sums and the error word (d_mv_ctl[2])
   mtf::DevBuf<float> d_mv_part;
-  mtf::DevBuf<unsigned> d_mv_ctl;
+  mtf::HostBuf<unsigned> d_mv_ctl;           // in mapped host memory
   int32_t mv_grid = 0;
   mtf::GmresWork* gw = nullptr;
   mtf::Gmres32Work* gw32 = nullptr;

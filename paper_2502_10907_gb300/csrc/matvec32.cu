@@ -204,10 +204,8 @@ void tile_stream_operator(const StreamUnits& su, const void* dense, int eb, void
 }
 
 void stream_prepare(mtf_system sys, cudaStream_t s) {
-  if (!sys->d_mv_ctl.p) {
-    sys->d_mv_ctl.alloc(4);
-    MTF_CUDA(cudaMemsetAsync(sys->d_mv_ctl.p, 0, 4 * sizeof(unsigned), s));
-  }
+  (void)s;
+  if (!sys->d_mv_ctl.p) sys->d_mv_ctl.alloc_zero(4);
   if (!sys->mv_grid) {
     int dev = 0, sms = 0;
     MTF_CUDA(cudaGetDevice(&dev));
@@ -325,12 +323,10 @@ void launch_matvec_adj_f32(mtf_system sys, const float* v, int64_t ldv, float* y
 // stream) and clears the error word.
 void check_matvec_stream(mtf_system sys, cudaStream_t s) {
   if (!sys->d_mv_ctl.p) return;
-  unsigned ctl[4];
-  MTF_CUDA(cudaMemcpyAsync(ctl, sys->d_mv_ctl.p, sizeof(ctl), cudaMemcpyDeviceToHost, s));
   MTF_CUDA(cudaStreamSynchronize(s));
-  if (ctl[2] == 0) return;
-  MTF_CUDA(cudaMemsetAsync(sys->d_mv_ctl.p, 0, 4 * sizeof(unsigned), s));
-  MTF_CUDA(cudaStreamSynchronize(s));
+  volatile unsigned* err = sys->d_mv_ctl.p + 2;
+  if (*err == 0) return;
+  *err = 0;
   throw Error{MTF_ERR_TIMEOUT, "a bulk copy of a streaming operator apply did not complete in time"};
 }
 
