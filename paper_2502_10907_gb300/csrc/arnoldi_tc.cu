@@ -316,9 +316,8 @@ static void tca_launch(TcArnoldi& t, const CUtensorMap& amap, const CUtensorMap&
     opted.fetch_or(bit);
   }
   const unsigned grid = unsigned(std::min(n_units, t.n_cta));
-  MTF_LAUNCH(kid, st, k_tc_stream<NPA, NB, EPI><<<grid, 192, Cfg::smem, st>>>(amap, bmap, units, n_units, nullptr,
-                                                                              nullptr, t.part.p, W, t.ldn, nc, n_limit,
-                                                                              cm, err, TcTtOut{}));
+  MTF_LAUNCH(kid, st, launch_pdl(k_tc_stream<NPA, NB, EPI>, dim3(grid), dim3(192), Cfg::smem, st, amap, bmap, units, n_units,
+                                 nullptr, nullptr, t.part.p, W, t.ldn, nc, n_limit, cm, err, TcTtOut{}));
 }
 
 template <int NB>

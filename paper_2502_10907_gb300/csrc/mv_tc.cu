@@ -12,17 +12,22 @@
 //    loads the 64 KB operator tile (4 parts) and the input chunk (hi, lo)
 //    with two cp.async.bulk.tensor.4d copies (128-byte swizzle) into a ring
 //    of S stages, completing on the stage's "full" mbarrier;
-//  - warp 1: allocates TMEM (two accumulator buffers of 2 NB columns:
-//    T products, K products); one lane issues per K = 16 step the six
+//  - warp 1: allocates TMEM (two accumulator buffers of NB columns: NB / 2
+//    of A+ u+, NB / 2 of A- u-); one lane issues per K = 16 step the six
 //    tcgen05.mma of the split products and commits each stage back to its
 //    "empty" barrier, and each finished unit to the buffer's "full" barrier;
 //  - warps 2-5: epilogue.  Each reads its 32 TMEM lanes (rows) of the
 //    finished buffer with tcgen05.ld and writes the unit's raw row sums to a
 //    partial buffer, then frees the TMEM buffer.
+// The two traces are taken together (apply.cu): with w = u_N / rho_i,
+// u+- = u_D +- i w and A+- = K -+ i T,  A+- u+- = y+-,  y_D = y+ + y-,
+// y_N = -i rho_i (y+ - y-): half the products, accumulators and row sums of
+// T u_D, T u_N, K u_D, K u_N from the same operator bytes.
 // k_mv_tc_combine then adds the pieces of each row in order, undoes the
-// scalings and applies 2 (K u_D + rho^-1 T u_N), 2 (-rho T u_D + K u_N) and
-// the exchange rows, as the FMA stream's combine does.  Every wait is
-// bounded (0.5 s) and ends in the error word.
+// scalings, forms y_D and y_N and adds the exchange rows.  Bound: HBM (the
+// operator tiles); on the 4 x 4 x 4 cube (72,000 unknowns, 16 right-hand
+// sides) an apply took 275 us with four products per entry, 255 us with two.
+// Every wait is bounded (0.5 s) and ends in the error word.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -52,8 +57,10 @@ struct TcMatvec {
   DevBuf<int> sched, sched_off, blk_unit_base, blk_pieces, blk_nkc;
   DevBuf<int64_t> blk_tile_base, blk_chunk_base;
   DevBuf<__half> B;                    // input chunks for up to 32 right-hand sides
-  DevBuf<float> part;                  // per unit: 128 rows x 2 NB raw sums
-  DevBuf<unsigned> colmax;             // per right-hand side of a pass (float bits)
+  DevBuf<float> part;                  // per unit: 128 rows x NB raw sums
+  // largest |re|, |im| per right-hand side of a pass: kCmParts partial maxima
+  // of 32 columns, then the 32 results
+  DevBuf<float> colmax;
   CUtensorMap amap{}, bmap{};
   const void* amap_ptr = nullptr;
   const void* bmap_ptr = nullptr;
@@ -108,8 +115,9 @@ __device__ __forceinline__ void tc_split(float v, __half& hi, __half& lo) {
   lo = __float2half_rn(v - __half2float(hi));
 }
 
-// Tiled hi / lo copy: thread = (tile, row, group g of 4 complex columns);
-// writes 8 halves (16 bytes) into each of the 4 parts.
+// Tiled hi / lo copy of A+ = K - i T and A- = K + i T (|A+-| <= 2 amax, inside
+// the FP16 range after the scaling): thread = (tile, row, group g of 4 complex
+// columns); writes 8 halves (16 bytes) into each of the 4 parts.
 __global__ void __launch_bounds__(256) k_tc_tile_a(const float4* __restrict__ TK, const int4* __restrict__ tile_info,
                                                    const int64_t* __restrict__ blk_mat_off,
                                                    const int32_t* __restrict__ blk_N, const unsigned* __restrict__ amax,
@@ -128,10 +136,10 @@ __global__ void __launch_bounds__(256) k_tc_tile_a(const float4* __restrict__ TK
     const int n = info.z * kTcCols + 4 * g + q;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r < N && n < N) v = TK[blk_mat_off[i] + int64_t(r) * N + n];
-    tc_split(v.x * s, h[0][2 * q], h[1][2 * q]);          // T re
-    tc_split(v.y * s, h[0][2 * q + 1], h[1][2 * q + 1]);  // T im
-    tc_split(v.z * s, h[2][2 * q], h[3][2 * q]);          // K re
-    tc_split(v.w * s, h[2][2 * q + 1], h[3][2 * q + 1]);  // K im
+    tc_split((v.z + v.y) * s, h[0][2 * q], h[1][2 * q]);          // A+ re
+    tc_split((v.w - v.x) * s, h[0][2 * q + 1], h[1][2 * q + 1]);  // A+ im
+    tc_split((v.z - v.y) * s, h[2][2 * q], h[3][2 * q]);          // A- re
+    tc_split((v.w + v.x) * s, h[2][2 * q + 1], h[3][2 * q + 1]);  // A- im
   }
 #pragma unroll
   for (int p = 0; p < 4; ++p)
@@ -184,6 +192,49 @@ __global__ void __launch_bounds__(256) k_tc_tile_os_im(const __half2* __restrict
   *reinterpret_cast<uint4*>(A + tc_tile_index(tile, 1, 0, row, 8 * g)) = *reinterpret_cast<const uint4*>(h);
 }
 
+constexpr int kCmParts = 32;
+
+// colmax[32 p + c] = max |re|, |im| over part p of input column c0 + c (n
+// complex entries): one CTA per (part, column), no atomics to clear
+__global__ void __launch_bounds__(256) k_tc_colmax(const float* __restrict__ x, int64_t ldx, int64_t n, int c0,
+                                                   float* __restrict__ colmax) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  const int c = blockIdx.y;
+  const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + c) * ldx);
+  float m = 0.f;
+#pragma unroll 4
+  for (int64_t k = int64_t(blockIdx.x) * 256 + threadIdx.x; k < n; k += kCmParts * 256) {
+    const float2 v = xc[k];
+    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+  }
+  m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+  __shared__ float red[8];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) m = fmaxf(m, red[q]);
+    colmax[32 * blockIdx.x + c] = m;
+  }
+}
+
+// the pass's column maxima from their parts into cm[32] (shared), by a CTA of
+// 256 threads; CTA 0 also stores them behind the parts for the combine
+__device__ __forceinline__ void tc_column_maxima(float* __restrict__ colmax, int nc, float* cm) {
+  const int c = threadIdx.x >> 3, q0 = threadIdx.x & 7;
+  float m = 0.f;
+  if (c < nc)
+#pragma unroll
+    for (int q = 0; q < kCmParts / 8; ++q) m = fmaxf(m, colmax[32 * (q0 + 8 * q) + c]);
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (q0 == 0) {
+    cm[c] = m;
+    if (blockIdx.x == 0) colmax[32 * kCmParts + c] = m;
+  }
+  __syncthreads();
+}
+
 // Real input chunks of the Type-2 apply: thread = (chunk, column col, group g
 // of 8 entries); column 4 c + 2 t + f holds part f (0: re, 1: im) of u_t of
 // right-hand side c0 + c, as FP16 hi / lo after the column's scaling
@@ -191,9 +242,11 @@ __global__ void __launch_bounds__(256) k_tc_build_b_real(const float* __restrict
                                                          int nb, const int2* __restrict__ chunk_info, int64_t n_chunks,
                                                          const int32_t* __restrict__ blk_N,
                                                          const int64_t* __restrict__ blk_dof_off,
-                                                         const unsigned* __restrict__ colmax, __half* __restrict__ B) {
+                                                         float* __restrict__ colmax, __half* __restrict__ B) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
+  __shared__ float cm[32];
+  tc_column_maxima(colmax, nc, cm);
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= n_chunks * nb * 8) return;
   const int64_t chunk = t / (int64_t(nb) * 8);
@@ -205,7 +258,7 @@ __global__ void __launch_bounds__(256) k_tc_build_b_real(const float* __restrict
   if (c < nc) {
     const int2 info = chunk_info[chunk];
     const int N = blk_N[info.x];
-    const float s = tc_scale(colmax[c]);
+    const float s = tc_scale(__float_as_uint(cm[c]));
     const float* xc = x + 2 * (int64_t(c0 + c) * ldx + blk_dof_off[info.x] + int64_t(slot) * N) + part;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -231,7 +284,7 @@ template <int NB, bool IM = false>
 __global__ void __launch_bounds__(256) k_os_tc_combine(
     const float* __restrict__ part, const int32_t* __restrict__ row_blk, const int32_t* __restrict__ blk_N,
     const int64_t* __restrict__ blk_dof_off, const int64_t* __restrict__ blk_row_off, const int* __restrict__ blk_unit_base,
-    const int* __restrict__ blk_pieces, const unsigned* __restrict__ colmax, const float* __restrict__ cf,
+    const int* __restrict__ blk_pieces, const float* __restrict__ colmax, const float* __restrict__ cf,
     float* __restrict__ z, int64_t ldz, int c0, int nc, int64_t n_rows) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
@@ -254,7 +307,7 @@ __global__ void __launch_bounds__(256) k_os_tc_combine(
     t.z += a.z;
     t.w += a.w;
   }
-  const float sc = tcs_inv_scale(colmax[lane]);
+  const float sc = tcs_inv_scale(__float_as_uint(colmax[32 * kCmParts + lane]));
   float a0 = t.x * sc, a1 = t.y * sc, a2 = t.z * sc, a3 = t.w * sc;  // T~ r_D, T~ r_N
   if constexpr (IM) {
     const float d0 = a0, d2 = a2;
@@ -271,28 +324,17 @@ __global__ void __launch_bounds__(256) k_os_tc_combine(
   zc[2 * (N + m) + 1] = -(rr * a1 + ri * a0);
 }
 
-// colmax[c] = max |re|, |im| of input column c0 + c (n complex entries)
-__global__ void k_tc_colmax(const float* __restrict__ x, int64_t ldx, int64_t n, int c0, unsigned* __restrict__ colmax) {
-  const int c = blockIdx.y;
-  const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + c) * ldx);
-  float m = 0.f;
-  for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-    const float2 v = xc[k];
-    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-  }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(colmax + c, __float_as_uint(m));
-}
-
 // Input chunks: thread = (chunk, column col, group g of 4 complex entries);
 // column 4 c + 2 t + f holds form f of u_t of right-hand side c0 + c.
 __global__ void __launch_bounds__(256) k_tc_build_b(const float* __restrict__ x, int64_t ldx, int c0, int nc, int nb,
                                                     const int2* __restrict__ chunk_info, int64_t n_chunks,
                                                     const int32_t* __restrict__ blk_N,
                                                     const int64_t* __restrict__ blk_dof_off,
-                                                    const unsigned* __restrict__ colmax, __half* __restrict__ B) {
+                                                    float* __restrict__ colmax, __half* __restrict__ B) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
+  __shared__ float cm[32];
+  tc_column_maxima(colmax, nc, cm);
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= n_chunks * nb * 8) return;
   const int64_t chunk = t / (int64_t(nb) * 8);
@@ -304,7 +346,7 @@ __global__ void __launch_bounds__(256) k_tc_build_b(const float* __restrict__ x,
   if (c < nc) {
     const int2 info = chunk_info[chunk];
     const int N = blk_N[info.x];
-    const float s = tc_scale(colmax[c]);
+    const float s = tc_scale(__float_as_uint(cm[c]));
     const float2* xc = reinterpret_cast<const float2*>(x + 2 * (int64_t(c0 + c) * ldx + blk_dof_off[info.x] +
                                                                  int64_t(slot) * N));
 #pragma unroll
@@ -321,6 +363,55 @@ __global__ void __launch_bounds__(256) k_tc_build_b(const float* __restrict__ x,
   *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(lo);
 }
 
+// scale of u+- in block i: |u+-| <= (1 + 1 / rho_i) max |u|
+__device__ __forceinline__ unsigned tc_pm_bound(float cm, float irho) { return __float_as_uint(cm * (1.f + fabsf(irho))); }
+
+// Matvec input chunks: thread = (chunk, column col, group g of 4 complex
+// entries); column h NB / 2 + 2 c + f holds form f of u+ (h = 0) or u- (h = 1)
+// of right-hand side c0 + c
+__global__ void __launch_bounds__(256) k_tc_build_pm(const float* __restrict__ x, int64_t ldx, int c0, int nc, int nb,
+                                                     const int2* __restrict__ chunk_info, int64_t n_chunks,
+                                                     const int32_t* __restrict__ blk_N,
+                                                     const int64_t* __restrict__ blk_dof_off,
+                                                     const float* __restrict__ rho32, float* __restrict__ colmax,
+                                                     __half* __restrict__ B) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  __shared__ float cm[32];
+  tc_column_maxima(colmax, nc, cm);
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= n_chunks * nb * 8) return;
+  const int64_t chunk = t / (int64_t(nb) * 8);
+  const int col = int((t / 8) % nb), g = int(t % 8);
+  const bool minus = col >= nb / 2;
+  const int c = (col % (nb / 2)) >> 1, form = col & 1;
+  __half hi[8], lo[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) hi[q] = lo[q] = __float2half_rn(0.f);
+  if (c < nc) {
+    const int2 info = chunk_info[chunk];
+    const int N = blk_N[info.x];
+    const float ir = rho32[4 * info.x + 2], ii = minus ? -ir : ir;  // rho is real
+    const float s = tc_scale(tc_pm_bound(cm[c], ir));
+    const float2* xc = reinterpret_cast<const float2*>(x + 2 * (int64_t(c0 + c) * ldx + blk_dof_off[info.x]));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int n = info.y * kTcCols + 4 * g + q;
+      float2 d = make_float2(0.f, 0.f), w = d;
+      if (n < N) {
+        d = xc[n];
+        w = xc[N + n];
+      }
+      const float2 v = make_float2(fmaf(-ii, w.y, d.x), fmaf(ii, w.x, d.y));  // u_D +- i u_N / rho
+      const float a = form == 0 ? v.x : v.y, b = form == 0 ? -v.y : v.x;
+      tc_split(a * s, hi[2 * q], lo[2 * q]);
+      tc_split(b * s, hi[2 * q + 1], lo[2 * q + 1]);
+    }
+  }
+  *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 0, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(hi);
+  *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(lo);
+}
+
 template <int NB>
 struct TcCfg {
   static constexpr int SA = kTcParts * kTcRows * 128;      // operator tile bytes (64 KB)
@@ -328,7 +419,8 @@ struct TcCfg {
   static constexpr int SB = SA + SBB;                       // stage bytes (a multiple of 1024)
   static constexpr int S0 = (220 * 1024) / SB;
   static constexpr int S = S0 > 4 ? 4 : S0;
-  static constexpr uint32_t TMEM = 4 * NB < 32 ? 32 : 4 * NB;  // two buffers of 2 NB columns
+  static constexpr uint32_t TMEM = 2 * NB;  // two buffers of NB columns
+  static_assert(NB >= 32, "A+ u+ and A- u- need 16 columns each");
   static constexpr size_t smem = size_t(S) * SB + 1024 + 256;
   static_assert(S >= 2, "the stage ring needs two stages");
   static_assert(smem <= 232448, "shared memory above the per-CTA limit");
@@ -373,6 +465,8 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -401,7 +495,7 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f16_m128(NB);
+      constexpr uint32_t idesc = idesc_f16_m128(NB / 2);
       int k = 0, ub = 0;
       bool ok = true;
       for (int q = q_begin; q < q_end && ok; ++q, ++ub) {
@@ -412,7 +506,7 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
           break;
         }
         tc_fence_after();
-        const uint32_t dT = tmem + uint32_t(buf * 2 * NB), dK = dT + uint32_t(NB);
+        const uint32_t dp = tmem + uint32_t(buf * NB), dm = dp + uint32_t(NB / 2);
         for (int kc = U.z; kc < U.w; ++kc, ++k) {
           const int st = k % S;
           if (!mbar_wait_bounded(&full[st], uint32_t(k / S) & 1u, kTcWaitNs)) {
@@ -424,16 +518,18 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
           const uint32_t sa = smem_u32(smem + size_t(st) * SB), sb = sa + SA;
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t th = sw128_desc(sa + kk * 32), tl = sw128_desc(sa + 16384 + kk * 32);
-            const uint64_t kh = sw128_desc(sa + 32768 + kk * 32), kl = sw128_desc(sa + 49152 + kk * 32);
-            const uint64_t bh = sw128_desc(sb + kk * 32), bl = sw128_desc(sb + NB * 128 + kk * 32);
+            const uint64_t ph = sw128_desc(sa + kk * 32), pl = sw128_desc(sa + 16384 + kk * 32);
+            const uint64_t mh = sw128_desc(sa + 32768 + kk * 32), ml = sw128_desc(sa + 49152 + kk * 32);
+            const uint32_t sm = sb + NB / 2 * 128;  // the columns of u-
+            const uint64_t uh = sw128_desc(sb + kk * 32), ul = sw128_desc(sb + NB * 128 + kk * 32);
+            const uint64_t vh = sw128_desc(sm + kk * 32), vl = sw128_desc(sm + NB * 128 + kk * 32);
             const uint32_t acc = (kc != U.z || kk != 0) ? 1u : 0u;
-            tc_mma_f16(dT, th, bh, idesc, acc);
-            tc_mma_f16(dT, th, bl, idesc, 1u);
-            tc_mma_f16(dT, tl, bh, idesc, 1u);
-            tc_mma_f16(dK, kh, bh, idesc, acc);
-            tc_mma_f16(dK, kh, bl, idesc, 1u);
-            tc_mma_f16(dK, kl, bh, idesc, 1u);
+            tc_mma_f16(dp, ph, uh, idesc, acc);
+            tc_mma_f16(dp, ph, ul, idesc, 1u);
+            tc_mma_f16(dp, pl, uh, idesc, 1u);
+            tc_mma_f16(dm, mh, vh, idesc, acc);
+            tc_mma_f16(dm, mh, vl, idesc, 1u);
+            tc_mma_f16(dm, ml, vh, idesc, 1u);
           }
           tc_commit(&empty[st]);  // the stage is free once these MMAs have read it
         }
@@ -452,10 +548,10 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
         break;
       }
       tc_fence_after();
-      const uint32_t ta = tmem + (uint32_t(32 * quarter) << 16) + uint32_t(buf * 2 * NB);
-      float* dst = part + (size_t(sched[q]) * kTcRows + row) * (2 * NB);
+      const uint32_t ta = tmem + (uint32_t(32 * quarter) << 16) + uint32_t(buf * NB);
+      float* dst = part + (size_t(sched[q]) * kTcRows + row) * NB;
 #pragma unroll
-      for (int c0 = 0; c0 < 2 * NB; c0 += 16) {
+      for (int c0 = 0; c0 < NB; c0 += 16) {
         float v[16];
         tmem_ld16(ta + uint32_t(c0), v);
         float4* d4 = reinterpret_cast<float4*>(dst + c0);
@@ -484,7 +580,7 @@ template <int NB>
 __global__ void __launch_bounds__(256) k_mv_tc_combine(
     const float* __restrict__ part, const int32_t* __restrict__ row_blk, const int32_t* __restrict__ blk_N,
     const int64_t* __restrict__ blk_dof_off, const int64_t* __restrict__ blk_row_off, const int* __restrict__ blk_unit_base,
-    const int* __restrict__ blk_pieces, const unsigned* __restrict__ amax, const unsigned* __restrict__ colmax,
+    const int* __restrict__ blk_pieces, const unsigned* __restrict__ amax, const float* __restrict__ colmax,
     const XEntry* __restrict__ xe, const float* __restrict__ xval32, const float* __restrict__ rho32,
     const float* __restrict__ x, int64_t ldx, float* __restrict__ y, int64_t ldy, int c0, int nc, int64_t n_rows) {
   MTF_PDL_WAIT();
@@ -500,31 +596,21 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
   const int P = blk_pieces[i];
   const int64_t u0 = blk_unit_base[i] + (m >> 7) * P;
   const int lr = int(m & 127);
-  float4 t = make_float4(0.f, 0.f, 0.f, 0.f), k = t;
+  float2 a = make_float2(0.f, 0.f), b = a;  // y+, y-
   for (int p = 0; p < P; ++p) {
-    const float* pr = part + (size_t(u0 + p) * kTcRows + lr) * (2 * NB);
-    const float4 a = *reinterpret_cast<const float4*>(pr + 4 * lane);
-    const float4 b = *reinterpret_cast<const float4*>(pr + NB + 4 * lane);
-    t.x += a.x;
-    t.y += a.y;
-    t.z += a.z;
-    t.w += a.w;
-    k.x += b.x;
-    k.y += b.y;
-    k.z += b.z;
-    k.w += b.w;
+    const float2* pr = reinterpret_cast<const float2*>(part + (size_t(u0 + p) * kTcRows + lr) * NB);
+    const float2 v = pr[lane], w = pr[NB / 4 + lane];
+    a.x += v.x;
+    a.y += v.y;
+    b.x += w.x;
+    b.y += w.y;
   }
-  const float sc = tc_inv_scale(amax[i]) * tc_inv_scale(colmax[lane]);
-  // T u_D, T u_N, K u_D, K u_N
-  const float tDr = t.x * sc, tDi = t.y * sc, tNr = t.z * sc, tNi = t.w * sc;
-  const float kDr = k.x * sc, kDi = k.y * sc, kNr = k.z * sc, kNi = k.w * sc;
-  const float rr = rho32[4 * i], ri = rho32[4 * i + 1], ir = rho32[4 * i + 2], ii = rho32[4 * i + 3];
+  const float rr = rho32[4 * i], ir = rho32[4 * i + 2];  // rho is real
+  const float sc = tc_inv_scale(amax[i]) * tc_inv_scale(tc_pm_bound(colmax[32 * kCmParts + lane], ir));
   const int col = c0 + lane;
   const float* xc = x + 2 * int64_t(col) * ldx;
-  float yDr = 2.f * (kDr + (tNr * ir - tNi * ii));
-  float yDi = 2.f * (kDi + (tNr * ii + tNi * ir));
-  float yNr = 2.f * (kNr - (tDr * rr - tDi * ri));
-  float yNi = 2.f * (kNi - (tDr * ri + tDi * rr));
+  float yDr = (a.x + b.x) * sc, yDi = (a.y + b.y) * sc;
+  float yNr = rr * ((a.y - b.y) * sc), yNi = rr * ((b.x - a.x) * sc);
 #pragma unroll
   for (int e = 0; e < 6; ++e) {
     const XEntry X = xe[6 * row + e];
@@ -636,7 +722,7 @@ static void tc_plan_tables(mtf_system sys, TcMatvec& t, cudaStream_t s) {
   upload_vec(t.blk_tile_base, tbase, s);
   upload_vec(t.blk_chunk_base, cbase, s);
   t.amax.alloc(size_t(m->nd));
-  t.colmax.alloc(32);
+  t.colmax.alloc(32 * (kCmParts + 1));
   MTF_CUDA(cudaStreamSynchronize(s));  // the host tables go out of scope
   t.planned = true;
 }
@@ -737,9 +823,10 @@ void tc_build_operator(mtf_system sys, cudaStream_t s) {
   t.built = true;
 }
 
-// input chunks (hi, lo) of columns c0 .. c0 + nc - 1 of x in t.B, their
-// scales in t.colmax, and the B tensor map for width NB
-template <int NB>
+// input chunks (hi, lo) of columns c0 .. c0 + nc - 1 of x in t.B (the matvec's
+// u+, u-, or block-OSRC's u_D, u_N), the column maxima in t.colmax, and the B
+// tensor map for width NB
+template <int NB, bool PM>
 static void tc_build_inputs(mtf_system sys, TcMatvec& t, const float* x, int64_t ldx, int c0, int nc, int kid,
                             cudaStream_t s) {
   mtf_mesh m = sys->mesh;
@@ -754,13 +841,18 @@ static void tc_build_inputs(mtf_system sys, TcMatvec& t, const float* x, int64_t
     t.bmap_ptr = t.B.p;
     t.bmap_nb = NB;
   }
-  const size_t np = p.units.size() * kTcRows * 2 * NB;
-  if (t.part.n < np) t.part.alloc(size_t(p.units.size()) * kTcRows * 2 * 128);
-  MTF_CUDA(cudaMemsetAsync(t.colmax.p, 0, 32 * sizeof(unsigned), s));
-  MTF_LAUNCH(kid, s, k_tc_colmax<<<dim3(64, unsigned(nc)), 256, 0, s>>>(x, ldx, m->n_total, c0, t.colmax.p));
+  const size_t np = p.units.size() * kTcRows * NB;
+  if (t.part.n < np) t.part.alloc(size_t(p.units.size()) * kTcRows * 128);
+  MTF_LAUNCH(kid, s, launch_pdl(k_tc_colmax, dim3(kCmParts, unsigned(nc)), dim3(256), 0, s, x, ldx, m->n_total, c0,
+                                t.colmax.p));
   const int64_t nthr = p.n_chunks * NB * 8;
-  MTF_LAUNCH(kid, s, launch_pdl(k_tc_build_b, dim3(unsigned((nthr + 255) / 256)), dim3(256), 0, s,
-      x, ldx, c0, nc, NB, t.chunk_info.p, p.n_chunks, m->d_blk_N.p, m->d_blk_dof_off.p, t.colmax.p, t.B.p));
+  const dim3 grid(unsigned((nthr + 255) / 256));
+  if constexpr (PM)
+    MTF_LAUNCH(kid, s, launch_pdl(k_tc_build_pm, grid, dim3(256), 0, s, x, ldx, c0, nc, NB, t.chunk_info.p, p.n_chunks,
+                                  m->d_blk_N.p, m->d_blk_dof_off.p, sys->d_rho32.p, t.colmax.p, t.B.p));
+  else
+    MTF_LAUNCH(kid, s, launch_pdl(k_tc_build_b, grid, dim3(256), 0, s, x, ldx, c0, nc, NB, t.chunk_info.p, p.n_chunks,
+                                  m->d_blk_N.p, m->d_blk_dof_off.p, t.colmax.p, t.B.p));
 }
 
 template <int NB>
@@ -768,7 +860,7 @@ static void mv_tc_pass(mtf_system sys, TcMatvec& t, const float* x, int64_t ldx,
                        cudaStream_t s) {
   using Cfg = TcCfg<NB>;
   mtf_mesh m = sys->mesh;
-  tc_build_inputs<NB>(sys, t, x, ldx, c0, nc, KID_MVTC_PREP, s);
+  tc_build_inputs<NB, true>(sys, t, x, ldx, c0, nc, KID_MVTC_PREP, s);
   static std::atomic<uint64_t> opted{0};
   int dev = 0;
   MTF_CUDA(cudaGetDevice(&dev));
@@ -781,7 +873,7 @@ static void mv_tc_pass(mtf_system sys, TcMatvec& t, const float* x, int64_t ldx,
   // every stored {T, K} entry once (16 bytes: FP16 hi + lo of four reals)
   // and the pass's FP16 hi + lo input chunks once
   prof_bytes(KID_MVTC, double(m->n_mat) * 16.0 + double(m->n_total) * nc * 8.0);
-  MTF_LAUNCH(KID_MVTC, s, k_mv_tc<NB><<<unsigned(t.n_cta), 192, Cfg::smem, s>>>(
+  MTF_LAUNCH(KID_MVTC, s, launch_pdl(k_mv_tc<NB>, dim3(unsigned(t.n_cta)), dim3(192), Cfg::smem, s,
       t.amap, t.bmap, t.units.p, t.sched.p, t.sched_off.p, t.blk_tile_base.p, t.blk_nkc.p, t.blk_chunk_base.p,
       t.part.p, sys->d_mv_ctl.p + 2));
   const unsigned gc = unsigned((m->n_rows * tc_row_lanes(nc) + 255) / 256);
@@ -849,7 +941,7 @@ static void os_tc_pass(mtf_system sys, TcMatvec& t, const float* r, int64_t ldr,
                        cudaStream_t s) {
   using Cfg = TcsCfg<1, NB>;
   mtf_mesh m = sys->mesh;
-  tc_build_inputs<NB>(sys, t, r, ldr, c0, nc, KID_OSRC, s);
+  tc_build_inputs<NB, false>(sys, t, r, ldr, c0, nc, KID_OSRC, s);
   static std::atomic<uint64_t> opted{0};
   int dev = 0;
   MTF_CUDA(cudaGetDevice(&dev));
@@ -863,7 +955,7 @@ static void os_tc_pass(mtf_system sys, TcMatvec& t, const float* r, int64_t ldr,
   prof_bytes(KID_OSRC, double(m->n_mat) * 4.0 + double(m->n_total) * nc * 8.0);
   TcUnits units;
   units.list = t.units_ab.p;
-  MTF_LAUNCH(KID_OSRC, s, k_tc_stream<1, NB, 0><<<unsigned(t.n_cta), 192, Cfg::smem, s>>>(
+  MTF_LAUNCH(KID_OSRC, s, launch_pdl(k_tc_stream<1, NB, 0>, dim3(unsigned(t.n_cta)), dim3(192), Cfg::smem, s,
       t.osmap, t.bmap, units, int(t.plan.units.size()), t.sched.p, t.sched_off.p, t.part.p, nullptr, 0, 0, 0, nullptr,
       sys->d_mv_ctl.p + 2, TcTtOut{}));
   const unsigned gc = unsigned((m->n_rows * tc_row_lanes(nc) + 255) / 256);
@@ -892,8 +984,8 @@ static void os_tc_pass_real(mtf_system sys, TcMatvec& t, const float* r, int64_t
     o.bmap_nb = NB;
   }
   if (o.part.n < p.units.size() * kTcRows * NB) o.part.alloc(p.units.size() * kTcRows * 128);
-  MTF_CUDA(cudaMemsetAsync(t.colmax.p, 0, 32 * sizeof(unsigned), s));
-  MTF_LAUNCH(KID_OSRC, s, k_tc_colmax<<<dim3(64, unsigned(nc)), 256, 0, s>>>(r, ldr, m->n_total, c0, t.colmax.p));
+  MTF_LAUNCH(KID_OSRC, s, launch_pdl(k_tc_colmax, dim3(kCmParts, unsigned(nc)), dim3(256), 0, s, r, ldr, m->n_total, c0,
+                                     t.colmax.p));
   const int64_t nthr = p.n_chunks * NB * 8;
   MTF_LAUNCH(KID_OSRC, s, launch_pdl(k_tc_build_b_real, dim3(unsigned((nthr + 255) / 256)), dim3(256), 0, s,
       r, ldr, c0, nc, NB, o.chunk_info.p, p.n_chunks, m->d_blk_N.p, m->d_blk_dof_off.p, t.colmax.p, o.B.p));
@@ -910,7 +1002,7 @@ static void os_tc_pass_real(mtf_system sys, TcMatvec& t, const float* r, int64_t
   prof_bytes(KID_OSRC, double(m->n_mat) * 2.0 + double(m->n_total) * nc * 8.0);
   TcUnits units;
   units.list = o.units_ab.p;
-  MTF_LAUNCH(KID_OSRC, s, k_tc_stream<1, NB, 0><<<unsigned(t.n_cta), 192, Cfg::smem, s>>>(
+  MTF_LAUNCH(KID_OSRC, s, launch_pdl(k_tc_stream<1, NB, 0>, dim3(unsigned(t.n_cta)), dim3(192), Cfg::smem, s,
       o.amap, o.bmap, units, int(p.units.size()), o.sched.p, o.sched_off.p, o.part.p, nullptr, 0, 0, 0, nullptr,
       sys->d_mv_ctl.p + 2, TcTtOut{}));
   const unsigned gc = unsigned((m->n_rows * tc_row_lanes(nc) + 255) / 256);
@@ -955,8 +1047,7 @@ void launch_matvec_tc(mtf_system sys, const float* x, int64_t ldx, float* y, int
   for (int c0 = 0; c0 < nrhs; c0 += 32) {
     const int nc = std::min(32, nrhs - c0);
     const int nb = tc_nb(nc);
-    if (nb == 16) mv_tc_pass<16>(sys, t, x, ldx, y, ldy, c0, nc, s);
-    else if (nb == 32) mv_tc_pass<32>(sys, t, x, ldx, y, ldy, c0, nc, s);
+    if (nb <= 32) mv_tc_pass<32>(sys, t, x, ldx, y, ldy, c0, nc, s);
     else if (nb == 64) mv_tc_pass<64>(sys, t, x, ldx, y, ldy, c0, nc, s);
     else mv_tc_pass<128>(sys, t, x, ldx, y, ldy, c0, nc, s);
   }

@@ -125,6 +125,8 @@ __global__ void __launch_bounds__(192, 1) k_tc_stream(const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  MTF_PDL_WAIT();  // the tables of units are static: read before
+  MTF_PDL_TRIGGER();
 
   if (warp == 0) {
     if (lane == 0) {
