@@ -26,7 +26,7 @@
 // k_mv_tc_combine then adds the pieces of each row in order, undoes the
 // scalings, forms y_D and y_N and adds the exchange rows.  Bound: HBM (the
 // operator tiles); on the 4 x 4 x 4 cube (72,000 unknowns, 16 right-hand
-// sides) an apply took 275 us with four products per entry, 255 us with two.
+// sides) an apply took 275 us with four products per entry, 238 us with two.
 // Every wait is bounded (0.5 s) and ends in the error word.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(256) k_tc_build_b_real(const float* __restrict
   *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(lo);
 }
 
-// lanes per row of the combines: the pass's right-hand sides rounded up to a
+// lanes per row of block-OSRC's combine: the pass's right-hand sides rounded up to a
 // power of two (at least 4), so that one warp takes 32 / lanes rows
 __host__ __device__ constexpr int tc_row_lanes(int nc) { return nc <= 4 ? 4 : nc <= 8 ? 8 : nc <= 16 ? 16 : 32; }
 
@@ -573,9 +573,15 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
   }
 }
 
-// y rows (one warp per global row, lane = right-hand side c < nc): the row's
-// unit pieces summed in order, unscaled, then the epilogue of Eq. 16 with
-// the exchange rows (FP32), as in the FMA stream's combine
+// y rows: the row's unit pieces summed in order, unscaled, y_D and y_N from
+// y+ and y-, and the exchange rows (FP32), as in the FMA stream's combine.  A
+// CTA takes 32 consecutive rows, lane = row, warps over the pass's right-hand
+// sides (8 at a time): consecutive rows of an interface meet nearly
+// consecutive dofs of the neighbour, so a warp's exchange reads and its stores
+// share sectors; with a lane per right-hand side each 8-byte exchange read was
+// a sector of its own.  Matvec of the 4 x 4 x 4 cube with 16 right-hand sides:
+// 255 -> 238 us.  (Block-OSRC's combine, which has no exchange, runs faster
+// with a lane per right-hand side: 85 against 88 us per apply.)
 template <int NB>
 __global__ void __launch_bounds__(256) k_mv_tc_combine(
     const float* __restrict__ part, const int32_t* __restrict__ row_blk, const int32_t* __restrict__ blk_N,
@@ -585,47 +591,50 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
     const float* __restrict__ x, int64_t ldx, float* __restrict__ y, int64_t ldy, int c0, int nc, int64_t n_rows) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
-  const int L = tc_row_lanes(nc);
-  const int64_t gt = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t row = gt / L;
-  const int lane = int(gt % L);
-  if (row >= n_rows || lane >= nc) return;
+  const int64_t row = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
+  if (row >= n_rows) return;
   const int i = row_blk[row];
   const int N = blk_N[i];
-  const int64_t m = row - blk_row_off[i];
+  const int64_t m = row - blk_row_off[i], off = blk_dof_off[i];
   const int P = blk_pieces[i];
-  const int64_t u0 = blk_unit_base[i] + (m >> 7) * P;
-  const int lr = int(m & 127);
-  float2 a = make_float2(0.f, 0.f), b = a;  // y+, y-
-  for (int p = 0; p < P; ++p) {
-    const float2* pr = reinterpret_cast<const float2*>(part + (size_t(u0 + p) * kTcRows + lr) * NB);
-    const float2 v = pr[lane], w = pr[NB / 4 + lane];
-    a.x += v.x;
-    a.y += v.y;
-    b.x += w.x;
-    b.y += w.y;
-  }
+  const float* pr = part + (size_t(blk_unit_base[i] + (m >> 7) * P) * kTcRows + (m & 127)) * NB;
   const float rr = rho32[4 * i], ir = rho32[4 * i + 2];  // rho is real
-  const float sc = tc_inv_scale(amax[i]) * tc_inv_scale(tc_pm_bound(colmax[32 * kCmParts + lane], ir));
-  const int col = c0 + lane;
-  const float* xc = x + 2 * int64_t(col) * ldx;
-  float yDr = (a.x + b.x) * sc, yDi = (a.y + b.y) * sc;
-  float yNr = rr * ((a.y - b.y) * sc), yNi = rr * ((b.x - a.x) * sc);
+  const float sca = tc_inv_scale(amax[i]);
+  int xd[6], xn[6];
+  float xv[6];
 #pragma unroll
   for (int e = 0; e < 6; ++e) {
     const XEntry X = xe[6 * row + e];
-    const float xv = xval32[6 * row + e];
-    const int Nj = X.ab >> 4;
-    yDr += xv * xc[2 * int64_t(X.col)];
-    yDi += xv * xc[2 * int64_t(X.col) + 1];
-    yNr += xv * xc[2 * (int64_t(X.col) + Nj)];
-    yNi += xv * xc[2 * (int64_t(X.col) + Nj) + 1];
+    xd[e] = X.col;
+    xn[e] = X.col + (X.ab >> 4);
+    xv[e] = xval32[6 * row + e];
   }
-  float* yc = y + 2 * (int64_t(col) * ldy + blk_dof_off[i]);
-  yc[2 * m] = yDr;
-  yc[2 * m + 1] = yDi;
-  yc[2 * (N + m)] = yNr;
-  yc[2 * (N + m) + 1] = yNi;
+  for (int c = threadIdx.x >> 5; c < nc; c += 8) {
+    float2 a = make_float2(0.f, 0.f), b = a;  // y+, y-
+    for (int p = 0; p < P; ++p) {
+      const float2* q = reinterpret_cast<const float2*>(pr + size_t(p) * kTcRows * NB);
+      const float2 v = q[c], w = q[NB / 4 + c];
+      a.x += v.x;
+      a.y += v.y;
+      b.x += w.x;
+      b.y += w.y;
+    }
+    const float sc = sca * tc_inv_scale(tc_pm_bound(colmax[32 * kCmParts + c], ir));
+    float yDr = (a.x + b.x) * sc, yDi = (a.y + b.y) * sc;
+    float yNr = rr * ((a.y - b.y) * sc), yNi = rr * ((b.x - a.x) * sc);
+    const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + c) * ldx);
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+      const float2 d = xc[xd[e]], n = xc[xn[e]];
+      yDr = fmaf(xv[e], d.x, yDr);
+      yDi = fmaf(xv[e], d.y, yDi);
+      yNr = fmaf(xv[e], n.x, yNr);
+      yNi = fmaf(xv[e], n.y, yNi);
+    }
+    float2* yc = reinterpret_cast<float2*>(y + 2 * (int64_t(c0 + c) * ldy + off));
+    yc[m] = make_float2(yDr, yDi);
+    yc[N + m] = make_float2(yNr, yNi);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -876,7 +885,7 @@ static void mv_tc_pass(mtf_system sys, TcMatvec& t, const float* x, int64_t ldx,
   MTF_LAUNCH(KID_MVTC, s, launch_pdl(k_mv_tc<NB>, dim3(unsigned(t.n_cta)), dim3(192), Cfg::smem, s,
       t.amap, t.bmap, t.units.p, t.sched.p, t.sched_off.p, t.blk_tile_base.p, t.blk_nkc.p, t.blk_chunk_base.p,
       t.part.p, sys->d_mv_ctl.p + 2));
-  const unsigned gc = unsigned((m->n_rows * tc_row_lanes(nc) + 255) / 256);
+  const unsigned gc = unsigned((m->n_rows + 31) / 32);
   MTF_LAUNCH(KID_MVTC_COMBINE, s, launch_pdl(k_mv_tc_combine<NB>, dim3(gc), dim3(256), 0, s,
       t.part.p, m->d_row_blk.p, m->d_blk_N.p, m->d_blk_dof_off.p, m->d_blk_row_off.p, t.blk_unit_base.p,
       t.blk_pieces.p, t.amax.p, t.colmax.p, m->d_xent.p, sys->d_xval32.p, sys->d_rho32.p, x, ldx, y, ldy, c0, nc,
