@@ -34,6 +34,7 @@
 #include <atomic>
 #include <vector>
 
+#include "arnoldi_tc.h"
 #include "common.h"
 #include "tc.cuh"
 #include "tc_plan.h"
@@ -44,8 +45,6 @@ namespace mtf {
 // tensor-map encoder and helpers of the tensor-core matvec (mv_tc.cu)
 void tc_encode_map(void* map, const void* base, int rows, int parts, int64_t count);
 void tc_encode_map_first(void* map, const void* base, int rows, int parts, int64_t count);
-
-constexpr float kBasisScale = 16384.f;  // 2^14: unit-norm basis entries stay below the FP16 range limit
 
 __device__ __forceinline__ float tca_scale(unsigned bits) {
   const float a = __uint_as_float(bits);
@@ -61,11 +60,6 @@ __device__ __forceinline__ float tca_inv_scale(unsigned bits) {
   frexpf(a, &ex);
   return ldexpf(1.f, ex - 14);
 }
-__device__ __forceinline__ void tca_split(float v, __half& hi, __half& lo) {
-  hi = __float2half_rn(v);
-  lo = __float2half_rn(v - __half2float(hi));
-}
-
 // new basis vectors q0 .. q0 + s - 1 (FP32, stride ldn) into the dots copy:
 // thread = (vector, group of 4 entries), entries fastest
 __global__ void k_tca_store_dots(const float* __restrict__ Vn, int64_t ldn, int q0, int s, int nkc,
@@ -106,39 +100,34 @@ __global__ void k_tca_store_upd(const float* __restrict__ Vn, int64_t ldn, int q
   *reinterpret_cast<__half2*>(Vu + tca_upd_half(qq, k, nbc, 1)) = *reinterpret_cast<const __half2*>(l);
 }
 
-// colmax[c] = max |re|, |im| of FP32 column c (n complex entries, stride ld)
-__global__ void k_tca_colmax32(const float* __restrict__ W, int64_t ld, int64_t n, unsigned* __restrict__ colmax) {
-  const int c = blockIdx.y;
-  const float2* w = reinterpret_cast<const float2*>(W + 2 * int64_t(c) * ld);
+// the column maxima of a pass's nc (<= 64) columns from their kPrepParts
+// partial maxima (stride ncm) into cm[64] (shared), by a CTA of 256 threads;
+// CTA 0 also stores them for the reduction of the sums
+__device__ __forceinline__ void tca_column_maxima(const float* __restrict__ parts, int ncm, int nc, float* cm,
+                                                  unsigned* __restrict__ out) {
+  const int c = threadIdx.x >> 2, q0 = threadIdx.x & 3;
   float m = 0.f;
-  for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
-    const float2 v = w[k];
-    m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+  if (c < nc)
+#pragma unroll
+    for (int q = 0; q < kPrepParts / 4; ++q) m = fmaxf(m, parts[(q0 + 4 * q) * ncm + c]);
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+  if (q0 == 0) {
+    cm[c] = m;
+    if (blockIdx.x == 0) out[c] = __float_as_uint(m);
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(colmax + c, __float_as_uint(m));
-}
-
-// colmax[c] = max over q < nq of |re|, |im| of H[q, c] (FP64, leading dim ldh)
-__global__ void k_tca_colmax64(const double* __restrict__ H, int nq, int ldh, unsigned* __restrict__ colmax) {
-  MTF_PDL_WAIT();
-  MTF_PDL_TRIGGER();
-  const int c = blockIdx.y;
-  float m = 0.f;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
-    const double* h = H + 2 * (int64_t(q) * ldh + c);
-    m = fmaxf(m, fmaxf(fabsf(float(h[0])), fabsf(float(h[1]))));
-  }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(colmax + c, __float_as_uint(m));
+  __syncthreads();
 }
 
 // dots input chunks from W: column 2 c + f, form 0 (w_re, w_im), form 1
 // (w_im, -w_re); thread = (chunk, column, group of 4 entries)
-__global__ void k_tca_w_to_b(const float* __restrict__ W, int64_t ldw, int s, int nkc, int nb,
-                             const unsigned* __restrict__ colmax, __half* __restrict__ Bd) {
+__global__ void __launch_bounds__(256) k_tca_w_to_b(const float* __restrict__ W, int64_t ldw, int s, int nkc, int nb,
+                                                    const float* __restrict__ maxparts, int ncm,
+                                                    unsigned* __restrict__ colmax, __half* __restrict__ Bd) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
+  __shared__ float cm[64];
+  tca_column_maxima(maxparts, ncm, s, cm, colmax);
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= int64_t(nkc) * nb * 8) return;
   const int64_t kc = t / (int64_t(nb) * 8);
@@ -148,7 +137,7 @@ __global__ void k_tca_w_to_b(const float* __restrict__ W, int64_t ldw, int s, in
 #pragma unroll
   for (int i = 0; i < 8; ++i) hi[i] = lo[i] = __float2half_rn(0.f);
   if (c < s) {
-    const float sc = tca_scale(colmax[c]);
+    const float sc = tca_scale(__float_as_uint(cm[c]));
     const float2* w = reinterpret_cast<const float2*>(W + 2 * int64_t(c) * ldw) + kc * kTcCols + 4 * g;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -196,33 +185,43 @@ __global__ void k_tca_h_to_b(const double* __restrict__ H, int nq, int s, int ld
 }
 
 // H[q, c] (at H + 2 (q ldh + c)) = (sum over the P pieces of basis group
-// q / 128 of the raw sums) x the inverse scales, in FP64; thread = (q, c)
-__global__ void k_tca_dots_reduce(const float* __restrict__ part, int nb, int P, int nq, int s,
-                                  const unsigned* __restrict__ colmax, double* __restrict__ H, int ldh) {
+// q / 128 of the raw sums) x the inverse scales, in FP64, threads over (q, c);
+// hmax[c] (cleared before) takes the columns' largest |re|, |im|, the scale of
+// the update's input chunks
+__global__ void __launch_bounds__(256) k_tca_dots_reduce(const float* __restrict__ part, int nb, int P, int nq, int s,
+                                                         const unsigned* __restrict__ colmax, double* __restrict__ H,
+                                                         int ldh, unsigned* __restrict__ hmax) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= int64_t(nq) * s) return;
-  const int q = int(t / s), c = int(t % s);
-  const int g = q / kTcRows, row = q % kTcRows;
-  // FP32 partials added in double-float (two-sum: Knuth's error-free
-  // transformation) on the FP32 pipes, rounded to FP64 once
-  float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-  for (int p = 0; p < P; ++p) {
-    const float2 v = *reinterpret_cast<const float2*>(part + (size_t(g * P + p) * kTcRows + row) * nb + 2 * c);
-    float s1 = rh + v.x, bb = s1 - rh;
-    rl += (rh - (s1 - bb)) + (v.x - bb);
-    rh = s1;
-    s1 = ih + v.y;
-    bb = s1 - ih;
-    il += (ih - (s1 - bb)) + (v.y - bb);
-    ih = s1;
+  __shared__ unsigned mx[64];
+  if (threadIdx.x < 64) mx[threadIdx.x] = 0u;
+  __syncthreads();
+  for (int64_t t = int64_t(blockIdx.x) * 256 + threadIdx.x; t < int64_t(nq) * s; t += int64_t(gridDim.x) * 256) {
+    const int q = int(t / s), c = int(t % s);
+    const int g = q / kTcRows, row = q % kTcRows;
+    // FP32 partials added in double-float (two-sum: Knuth's error-free
+    // transformation) on the FP32 pipes, rounded to FP64 once
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+    for (int p = 0; p < P; ++p) {
+      const float2 v = *reinterpret_cast<const float2*>(part + (size_t(g * P + p) * kTcRows + row) * nb + 2 * c);
+      float s1 = rh + v.x, bb = s1 - rh;
+      rl += (rh - (s1 - bb)) + (v.x - bb);
+      rh = s1;
+      s1 = ih + v.y;
+      bb = s1 - ih;
+      il += (ih - (s1 - bb)) + (v.y - bb);
+      ih = s1;
+    }
+    const double re = double(rh) + double(rl), im = double(ih) + double(il);
+    const float scf = tca_inv_scale(colmax[c]) * (1.f / kBasisScale);  // powers of two
+    const double sc = double(scf);
+    const int64_t o = 2 * (int64_t(q) * ldh + c);
+    H[o] = re * sc;
+    H[o + 1] = im * sc;
+    atomicMax(&mx[c], __float_as_uint(fmaxf(fabsf(rh), fabsf(ih)) * scf));
   }
-  const double re = double(rh) + double(rl), im = double(ih) + double(il);
-  const double sc = double(tca_inv_scale(colmax[c])) / double(kBasisScale);
-  const int64_t o = 2 * (int64_t(q) * ldh + c);
-  H[o] = re * sc;
-  H[o + 1] = im * sc;
+  __syncthreads();
+  if (threadIdx.x < s && mx[threadIdx.x]) atomicMax(hmax + threadIdx.x, mx[threadIdx.x]);
 }
 
 // ---------------------------------------------------------------------------
@@ -236,7 +235,7 @@ struct TcArnoldi {
   int G = 0, nkc = 0, E = 0, nbc = 0;  // basis groups, entry chunks, entry groups, basis chunks
   DevBuf<__half> Vd, Vu, Bd, Bu;
   DevBuf<float> part;
-  DevBuf<unsigned> cm;                 // colmax of W (s) and of H (s)
+  DevBuf<unsigned> cm;                 // column maxima of W (64), of H (64 per pass)
   size_t h_cap = 0;                    // units the partial buffer holds
   int n_cta = 0, b_nb = 0;
   CUtensorMap vd_map{}, vu_map{}, bd_map{}, bu_map{};
@@ -248,6 +247,10 @@ struct TcArnoldi {
 TcArnoldi* tca_create() { return new TcArnoldi(); }
 void tca_destroy(TcArnoldi* t) { delete t; }
 void tca_set_dots_hi(TcArnoldi& t, bool on) { t.dots_hi = on; }
+// the maxima of H's columns of both passes: 2 x 64 words to clear before a projection
+unsigned* tca_hmax(TcArnoldi& t) { return t.cm.p + kTcaMaxCols; }
+// the tiled copies, for a kernel that stores a block's vectors itself
+TcaTiles tca_tiles(const TcArnoldi& t) { return {t.Vd.p, t.Vu.p, t.nkc, t.nbc}; }
 
 static int tca_nb(int nc) { return 2 * nc <= 16 ? 16 : 2 * nc <= 32 ? 32 : 2 * nc <= 64 ? 64 : 128; }
 
@@ -268,7 +271,7 @@ void tca_prepare(TcArnoldi& t, int s, int m, int64_t ldn, cudaStream_t st) {
   MTF_CUDA(cudaMemsetAsync(t.Vu.p, 0, t.Vu.n * sizeof(__half), st));
   t.Bd.alloc(size_t(t.nkc) * 2 * 128 * 64);
   t.Bu.alloc(size_t(t.nbc) * 2 * 128 * 64);
-  t.cm.alloc(size_t(2) * kTcaMaxCols);
+  t.cm.alloc(size_t(3) * kTcaMaxCols);
   int dev = 0;
   MTF_CUDA(cudaGetDevice(&dev));
   MTF_CUDA(cudaDeviceGetAttribute(&t.n_cta, cudaDevAttrMultiProcessorCount, dev));
@@ -321,17 +324,15 @@ static void tca_launch(TcArnoldi& t, const CUtensorMap& amap, const CUtensorMap&
 }
 
 template <int NB>
-static void tca_project_nb(TcArnoldi& t, int nq, float* W, int nc, double* H, int ldh, unsigned* err, cudaStream_t st) {
+static void tca_project_nb(TcArnoldi& t, int nq, float* W, int nc, double* H, int ldh, const float* maxparts, int ncm,
+                           int pass, unsigned* err, cudaStream_t st) {
   tca_bmaps(t, NB);
   unsigned* cmw = t.cm.p;
-  unsigned* cmh = t.cm.p + kTcaMaxCols;
-  MTF_CUDA(cudaMemsetAsync(t.cm.p, 0, size_t(2) * kTcaMaxCols * sizeof(unsigned), st));
+  unsigned* cmh = tca_hmax(t) + pass * kTcaMaxCols;
   // H = V^H W: units (basis group g, a piece of the entry chunks)
-  MTF_LAUNCH(KID_TCA_PREP, st, k_tca_colmax32<<<dim3(64, unsigned(nc)), 256, 0, st>>>(W, t.ldn, t.ldn, cmw));
   const int64_t nthr = int64_t(t.nkc) * NB * 8;
   MTF_LAUNCH(KID_TCA_PREP, st, launch_pdl(k_tca_w_to_b, dim3(unsigned((nthr + 255) / 256)), dim3(256), 0, st,
-      W, t.ldn, nc, t.nkc, NB, cmw,
-                                                                                      t.Bd.p));
+      W, t.ldn, nc, t.nkc, NB, maxparts, ncm, cmw, t.Bd.p));
   const int g_used = (nq + kTcRows - 1) / kTcRows;
   const int P = std::max(1, std::min({t.nkc, 32, (4 * t.n_cta + g_used - 1) / g_used}));
   const int L = (t.nkc + P - 1) / P;
@@ -350,12 +351,10 @@ static void tca_project_nb(TcArnoldi& t, int nq, float* W, int nc, double* H, in
     prof_bytes(KID_DOTS, double(nq + nc) * double(t.ldn) * 8.0);
     tca_launch<2, NB, 0>(t, t.vd_map, t.bd_map, ud, nu, nullptr, nc, 0, cmw, err, KID_DOTS, st);
   }
-  const unsigned gr = unsigned((int64_t(nq) * nc + 255) / 256);
+  const unsigned gr = unsigned(std::min<int64_t>((int64_t(nq) * nc + 255) / 256, 2 * t.n_cta));
   MTF_LAUNCH(KID_TCA_PREP, st, launch_pdl(k_tca_dots_reduce, dim3(gr), dim3(256), 0, st,
-      t.part.p, NB, Pn, nq, nc, cmw, H, ldh));
+      t.part.p, NB, Pn, nq, nc, cmw, H, ldh, cmh));
   // W -= V H: one unit per entry group, over the basis chunks in use
-  MTF_LAUNCH(KID_TCA_PREP, st, launch_pdl(k_tca_colmax64, dim3(8, unsigned(nc)), dim3(256), 0, st,
-      H, nq, ldh, cmh));
   const int nbc_used = (nq + 31) / 32;
   const int64_t nthu = int64_t(nbc_used) * NB * 8;
   MTF_LAUNCH(KID_TCA_PREP, st, launch_pdl(k_tca_h_to_b, dim3(unsigned((nthu + 255) / 256)), dim3(256), 0, st,
@@ -371,19 +370,22 @@ static void tca_project_nb(TcArnoldi& t, int nq, float* W, int nc, double* H, in
 
 // H[q, c] (q < nq, c < nc; complex FP64 at H + 2 (q ldh + c)) = V^H W, then
 // W -= V H, for the first nq basis vectors stored by tca_store and the nc
-// columns of W (stride ldn), in passes of up to 64 columns
-void tca_project(TcArnoldi& t, int nq, float* W, int nc, double* H, int ldh, unsigned* err, cudaStream_t st) {
-  MTF_REQUIRE(nq >= 1 && int64_t(nq) <= int64_t(t.m + 1) * t.s && nc >= 1, MTF_ERR_ARG,
+// columns of W (stride ldn), in passes of up to 64 columns; maxparts:
+// kPrepParts partial maxima of the columns (stride ncm), tca_hmax cleared
+void tca_project(TcArnoldi& t, int nq, float* W, int nc, double* H, int ldh, const float* maxparts, int ncm,
+                 unsigned* err, cudaStream_t st) {
+  MTF_REQUIRE(nq >= 1 && int64_t(nq) <= int64_t(t.m + 1) * t.s && nc >= 1 && nc <= 2 * kTcaMaxCols, MTF_ERR_ARG,
               "tensor-core Arnoldi: basis size");
   for (int c0 = 0; c0 < nc; c0 += kTcaMaxCols) {
-    const int w = std::min(kTcaMaxCols, nc - c0);
+    const int w = std::min(kTcaMaxCols, nc - c0), pass = c0 / kTcaMaxCols;
     float* Wg = W + 2 * int64_t(c0) * t.ldn;
     double* Hg = H + 2 * c0;
+    const float* mg = maxparts + c0;
     const int nb = tca_nb(w);
-    if (nb == 16) tca_project_nb<16>(t, nq, Wg, w, Hg, ldh, err, st);
-    else if (nb == 32) tca_project_nb<32>(t, nq, Wg, w, Hg, ldh, err, st);
-    else if (nb == 64) tca_project_nb<64>(t, nq, Wg, w, Hg, ldh, err, st);
-    else tca_project_nb<128>(t, nq, Wg, w, Hg, ldh, err, st);
+    if (nb == 16) tca_project_nb<16>(t, nq, Wg, w, Hg, ldh, mg, ncm, pass, err, st);
+    else if (nb == 32) tca_project_nb<32>(t, nq, Wg, w, Hg, ldh, mg, ncm, pass, err, st);
+    else if (nb == 64) tca_project_nb<64>(t, nq, Wg, w, Hg, ldh, mg, ncm, pass, err, st);
+    else tca_project_nb<128>(t, nq, Wg, w, Hg, ldh, mg, ncm, pass, err, st);
   }
 }
 

@@ -32,19 +32,13 @@
 #include <cstdlib>
 #include <vector>
 
+#include "arnoldi_tc.h"
 #include "block_krylov.h"
 #include "bulk.h"
 #include "common.h"
+#include "kernel64.cuh"
 
 namespace mtf {
-
-struct TcArnoldi;
-TcArnoldi* tca_create();
-void tca_destroy(TcArnoldi* t);
-void tca_set_dots_hi(TcArnoldi& t, bool on);
-void tca_prepare(TcArnoldi& t, int s, int m, int64_t ldn, cudaStream_t st);
-void tca_store(TcArnoldi& t, const float* Vn, int q0, cudaStream_t st);
-void tca_project(TcArnoldi& t, int nq, float* W, int nc, double* H, int ldh, unsigned* err, cudaStream_t st);
 
 struct BlockWork {
   int s = 0, m = 0;
@@ -52,18 +46,17 @@ struct BlockWork {
   TcArnoldi* tca = nullptr;  // tensor-core projections (arnoldi_tc.cu), with mv_tensor
   DevBuf<float> V, Z, X, D;  // (m + 1) s, m s, 2 s ([V~_J | W]), s vectors
   DevBuf<double> S[2];       // projection coefficients of two steps: (m + 1) s x 2 s, complex
-  DevBuf<double> Gs;         // Gpre (s) | G2 (2s x 2s) | G (s x s) | Hc ((m + 1) s x s) | Rn | R | Rv | Cc (two)
+  DevBuf<double> Gs;         // G2 (2s x 2s) | G (s x s) | R | Rv | Cc (two) | Rn | kept (2 s ints) | Hc ((m + 1) s x s)
+  DevBuf<double> normp;      // kPrepParts partial squared norms of W's columns before the projections
+  DevBuf<float> maxp;        // kPrepParts partial maxima of the columns of X
   DevBuf<double> C;          // s x s (complex, FP64) transform, or the coefficients Y (m s x s)
-  DevBuf<int> kept;          // keptR (s) | keptV (s)
   double* h_host = nullptr;
-  double* pin = nullptr;     // two pinned slots of a step's coefficients
-  int* kept_host = nullptr;  // two pinned slots of kept flags and the error word
+  double* pin = nullptr;     // two pinned slots of a step's Rn | kept | Hc
   cudaEvent_t ev[2] = {nullptr, nullptr};
   BlockLSQ lsq;
   ~BlockWork() {
     if (h_host) cudaFreeHost(h_host);
     if (pin) cudaFreeHost(pin);
-    if (kept_host) cudaFreeHost(kept_host);
     for (auto& e : ev)
       if (e) cudaEventDestroy(e);
     tca_destroy(tca);
@@ -87,6 +80,8 @@ template <int SC, int VW>
 __global__ void __launch_bounds__(256) k_bdots(const float* __restrict__ V, int nq, int64_t ldv,
                                                const float* __restrict__ W, int64_t ldw, int nc, int64_t seg_len,
                                                int64_t n_pad, double* __restrict__ H, int ldh) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
   __shared__ __align__(16) float2 ws[SC][128];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q0 = (int(blockIdx.y) * 8 + warp) * VW;
@@ -288,40 +283,67 @@ __global__ void k_blk_addx(double* __restrict__ x, int64_t n, const float* __res
   *xp = o;
 }
 
-// out[c] += ||W_c||^2 for the s columns of W (FP32 sums per thread and
-// warp, one FP64 atomic per warp and column): the reference norms of the
-// deflation test, read once from the block the operator just produced
-__global__ void __launch_bounds__(256) k_bnorm2(const float* __restrict__ W, int64_t ldw, int64_t n,
-                                                double* __restrict__ out) {
-  const int c = blockIdx.y;
-  const float4* w = reinterpret_cast<const float4*>(W + 2 * int64_t(c) * ldw);
-  float a = 0.f;
-  for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n / 2; k += int64_t(gridDim.x) * blockDim.x) {
-    const float4 v = w[k];  // two complex entries
-    a = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, a))));
+// Everything a step needs before its projections, in one pass over the block's
+// columns: X0 = V~ (copied), the partial maxima of the columns of X = [X0, W]
+// (the scales of their FP16 inputs) and the partial squared norms of W (the
+// reference of the deflation test), one CTA per (part, column); the Gram
+// matrices, and the maxima of H, are cleared.  With W null (the last step) X0
+// alone.  It replaces two reductions, a copy and five clears per step.
+__global__ void __launch_bounds__(256) k_bprep(const float* __restrict__ Vt, float* __restrict__ X0,
+                                               const float* __restrict__ W, int64_t ld, int s, int ncm,
+                                               float* __restrict__ maxp, double* __restrict__ normp,
+                                               double* __restrict__ clear, int nclear, unsigned* __restrict__ hmax) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  const int c = blockIdx.y, p = blockIdx.x;
+  const int64_t nt = int64_t(kPrepParts) * s * 256, me = (int64_t(c) * kPrepParts + p) * 256 + threadIdx.x;
+  for (int64_t q = me; q < nclear; q += nt) clear[q] = 0.0;
+  if (hmax && me < 128) hmax[me] = 0u;
+  const float4* v = reinterpret_cast<const float4*>(Vt + 2 * int64_t(c) * ld);
+  float4* o = reinterpret_cast<float4*>(X0 + 2 * int64_t(c) * ld);
+  const float4* w = W ? reinterpret_cast<const float4*>(W + 2 * int64_t(c) * ld) : nullptr;
+  float mv = 0.f, mw = 0.f, a = 0.f;
+  for (int64_t k = int64_t(p) * 256 + threadIdx.x; k < ld / 2; k += kPrepParts * 256) {
+    const float4 x = v[k];
+    o[k] = x;
+    mv = fmaxf(mv, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+    if (w) {
+      const float4 y = w[k];
+      mw = fmaxf(mw, fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
+      a = fmaf(y.x, y.x, fmaf(y.y, y.y, fmaf(y.z, y.z, fmaf(y.w, y.w, a))));
+    }
   }
-  for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(out + c, double(a));
-}
-
-// 1 / sqrt(d) for d > 0 in FP64: an FP32 seed refined by two Newton steps
-// y <- y (3 - d y^2) / 2 (quadratic convergence: 2^-22 -> 2^-43 -> rounding);
-// the narrow FP64 pipe makes this several times faster than sqrt and a
-// division.  Outside the FP32 range the FP64 library functions are used.
-__device__ __forceinline__ double rsqrt_newton(double d) {
-  if (!(d > 1e-30 && d < 1e30)) return 1.0 / sqrt(d);
-  double y = double(rsqrtf(float(d)));
-  y = y * fma(-0.5 * d, y * y, 1.5);
-  y = y * fma(-0.5 * d, y * y, 1.5);
-  return y;
+  mv = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mv)));
+  mw = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mw)));
+  for (int q = 16; q; q >>= 1) a += __shfl_xor_sync(0xffffffffu, a, q);
+  __shared__ float red[3][8];
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = mv;
+    red[1][threadIdx.x >> 5] = mw;
+    red[2][threadIdx.x >> 5] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int q = 0; q < 8; ++q) {
+      mv = fmaxf(mv, red[0][q]);
+      mw = fmaxf(mw, red[1][q]);
+      t += double(red[2][q]);
+    }
+    maxp[p * ncm + c] = mv;
+    if (w) {
+      maxp[p * ncm + s + c] = mw;
+      normp[p * s + c] = t;
+    }
+  }
 }
 
 // Deflating Cholesky factor of a block's Gram matrix on the device (the
 // rule of deflating_cholesky in block_krylov.h): G (complex FP64, entry
 // [q ldg + c] = <W_q, W_c>) = R^H R with R upper triangular; direction k is
 // dropped (row k of R zero, kept[k] = 0) when its Schur pivot is not above
-// tau^2 ref_k, ref_k = ref[k] (squared norms before the
-// Gram-Schmidt projections) or, with mask, 1 for mask[k] != 0 and 0
+// tau^2 ref_k, ref_k = the sum of its kPrepParts parts in ref (squared norms
+// before the Gram-Schmidt projections) or, with mask, 1 for mask[k] != 0 and 0
 // otherwise.  R complex FP64, column-major (entry (i, c) at [c s + i]).
 // One CTA of 256 threads, s <= 64: per pivot the row of R is formed in
 // parallel and the trailing upper triangle is updated by all threads (the
@@ -349,7 +371,7 @@ struct CxOf<float> {
   using type = float2;
 };
 
-__device__ __forceinline__ double rsqrt_of(double d) { return rsqrt_newton(d); }
+__device__ __forceinline__ double rsqrt_of(double d) { return rsqrt_h(d); }
 __device__ __forceinline__ float rsqrt_of(float d) {
   const float y = rsqrtf(d);
   return y * fmaf(-0.5f * d, y * y, 1.5f);  // one Newton step on the approximate reciprocal square root
@@ -376,7 +398,11 @@ __global__ void __launch_bounds__(256) k_bchol(const double* __restrict__ G, int
     Rs[t] = T2{T(0), T(0)};
   }
   for (int k = tid; k < s; k += nt) {
-    refs[k] = mask ? (mask[k] ? 1.0 : 0.0) : ref[k];
+    double r = 0.0;
+    if (mask) r = mask[k] ? 1.0 : 0.0;
+    else
+      for (int p = 0; p < kPrepParts; ++p) r += ref[p * s + k];
+    refs[k] = r;
     rinv[k] = T(0);
   }
   for (int k = 0; k < s; ++k) {
@@ -435,6 +461,203 @@ __global__ void __launch_bounds__(256) k_bchol(const double* __restrict__ G, int
       C[2 * (i * s + c)] = double(re);
       C[2 * (i * s + c) + 1] = double(im);
     }
+  }
+}
+
+// k_bchol for s <= 16 in one warp: lane (c, h) holds the rows i = 2 j + h of
+// column c in registers; row k goes to the lanes by shuffles, so a pivot costs
+// no block barrier and its few FP64 instructions are those of one warp (eight
+// warps with a sparse update each kept the narrow FP64 pipe of the one SM busy:
+// 23 us for s = 16 in FP64 and 21 us in FP32 with the coefficient solve, now
+// 23 and 12 us).  Same rule, same layouts.
+template <class T2>
+__device__ __forceinline__ T2 shfl2(T2 v, int src) {
+  v.x = __shfl_sync(0xffffffffu, v.x, src);
+  v.y = __shfl_sync(0xffffffffu, v.y, src);
+  return v;
+}
+
+template <class T>
+__global__ void __launch_bounds__(32) k_bchol16(const double* __restrict__ G, int ldg, const double* __restrict__ ref,
+                                                const int* __restrict__ mask, double tau, int s, double* __restrict__ R,
+                                                int* __restrict__ kept, const double* __restrict__ Gwv,
+                                                double* __restrict__ C) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  using T2 = typename CxOf<T>::type;
+  __shared__ T2 Rs[16][17];  // Rs[c][i] = R(i, c)
+  __shared__ T rinv[16];
+  __shared__ int keeps[16];
+  const int lane = threadIdx.x, c = lane & 15, h = lane >> 4;
+  T2 A[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int i = 2 * j + h;
+    A[j] = c < s && i < s ? T2{T(G[2 * (i * ldg + c)]), T(G[2 * (i * ldg + c) + 1])} : T2{T(0), T(0)};
+    Rs[c][i] = T2{T(0), T(0)};
+  }
+  double thr = 0.0;  // tau^2 ref of column c
+  if (c < s) {
+    if (mask) thr = mask[c] && h == 0 ? 1.0 : 0.0;
+    else
+#pragma unroll 4
+      for (int p = h; p < kPrepParts; p += 2) thr += ref[p * s + c];
+  }
+  thr += __shfl_xor_sync(0xffffffffu, thr, 16);
+  thr = tau * tau * fmax(thr, 0.0);
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    if (k < s) {
+      const T2 row = shfl2(A[k >> 1], c + 16 * (k & 1));  // A(k, c)
+      const T d = __shfl_sync(0xffffffffu, row.x, k);
+      const double t = __shfl_sync(0xffffffffu, thr, k);
+      const bool keep = double(d) > t && d > T(0);
+      T y = T(0);
+      if (keep) {
+        y = rsqrt_of(d);
+        const T2 r = c == k ? T2{d * y, T(0)} : T2{row.x * y, row.y * y};
+        if (h == 0 && c >= k) Rs[c][k] = r;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (2 * j + 1 > k) {  // rows i > k (row k itself is no longer needed)
+            const T2 ri = shfl2(r, 2 * j + h);
+            A[j].x -= ri.x * r.x + ri.y * r.y;  // conj(R(k, i)) R(k, c)
+            A[j].y -= ri.x * r.y - ri.y * r.x;
+          }
+      }
+      if (lane == 0) {
+        rinv[k] = y;
+        keeps[k] = keep ? 1 : 0;
+      }
+    }
+  }
+  __syncwarp();
+  for (int t = lane; t < s * s; t += 32) {
+    const T2 r = Rs[t / s][t % s];
+    R[2 * t] = double(r.x);
+    R[2 * t + 1] = double(r.y);
+  }
+  if (lane < s) kept[lane] = keeps[lane];
+  if (C != nullptr && lane < s) {
+    // column c = lane of C = R^-H G_vw by forward substitution
+    T2 g[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      g[i] = i < s ? T2{T(Gwv[2 * (c * s + i)]), -T(Gwv[2 * (c * s + i) + 1])} : T2{T(0), T(0)};
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i < s) {
+        const T f = keeps[i] ? rinv[i] : T(0);
+        const T2 x = T2{g[i].x * f, g[i].y * f};
+#pragma unroll
+        for (int p = i + 1; p < 16; ++p) {
+          const T2 r = Rs[p][i];  // R(i, p); zero past s
+          g[p].x -= r.x * x.x + r.y * x.y;
+          g[p].y -= r.x * x.y - r.y * x.x;
+        }
+        C[2 * (i * s + c)] = double(x.x);
+        C[2 * (i * s + c) + 1] = double(x.y);
+      }
+    }
+  }
+}
+
+// The rest of block J and the correction of W along it, entry by entry
+// (s <= SC): V_J = V~' Rv^-1 on the kept set (forward substitution; with
+// first, V_J as it stands), stored in FP32 and, with tiles, in both tiled
+// copies of the basis (vectors q0 .. q0 + s - 1); then W -= V_J C.  One kernel
+// for a triangular solve, two stores and an update: V_J stays in registers.
+template <int SC>
+__global__ void __launch_bounds__(128) k_bfinish(const float* __restrict__ in, const double* __restrict__ Rv,
+                                                 const int* __restrict__ kept, int s, bool first,
+                                                 float* __restrict__ V, const double* __restrict__ C,
+                                                 float* __restrict__ W, int64_t ld, const TcaTiles tiles, int q0) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  __shared__ float2 rs[SC][SC], cs[SC][SC];  // rs[p][q] = R(p, q), cs[q][c] = C(q, c)
+  __shared__ float2 inv[SC];
+  for (int t = threadIdx.x; t < SC * SC; t += 128) {
+    const int p = t / SC, q = t % SC;
+    const bool ok = p < s && q < s;
+    rs[p][q] = ok ? make_float2(float(Rv[2 * (q * s + p)]), float(Rv[2 * (q * s + p) + 1])) : make_float2(0.f, 0.f);
+    cs[p][q] = ok ? make_float2(float(C[2 * (p * s + q)]), float(C[2 * (p * s + q) + 1])) : make_float2(0.f, 0.f);
+  }
+  for (int q = threadIdx.x; q < SC; q += 128) {
+    float2 v = make_float2(0.f, 0.f);
+    if (q < s && kept[q]) {
+      const double a = Rv[2 * (q * s + q)], b = Rv[2 * (q * s + q) + 1], d = a * a + b * b;
+      v = make_float2(float(a / d), float(-b / d));
+    }
+    inv[q] = v;
+  }
+  __syncthreads();
+  const int64_t k = int64_t(blockIdx.x) * 128 + threadIdx.x;
+  if (k >= ld) return;
+  float2 v[SC];
+#pragma unroll
+  for (int q = 0; q < SC; ++q) {
+    v[q] = make_float2(0.f, 0.f);
+    if (q < s) {
+      float2 a = reinterpret_cast<const float2*>((first ? V : in) + 2 * int64_t(q) * ld)[k];
+      if (!first) {
+#pragma unroll
+        for (int p = 0; p < q; ++p) {
+          const float2 r = rs[p][q];
+          a.x -= v[p].x * r.x - v[p].y * r.y;
+          a.y -= v[p].x * r.y + v[p].y * r.x;
+        }
+        const float2 iv = inv[q];
+        a = make_float2(a.x * iv.x - a.y * iv.y, a.x * iv.y + a.y * iv.x);
+        reinterpret_cast<float2*>(V + 2 * int64_t(q) * ld)[k] = a;
+      }
+      v[q] = a;
+    }
+  }
+  if (tiles.Vd) {
+    const bool by4 = ((q0 | s) & 3) == 0;  // runs of 4 vectors stay 16-byte aligned in the update copy
+#pragma unroll
+    for (int q = 0; q < SC; q += 4) {
+      if (q >= s) break;
+      __half2 hi[4], lo[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        __half h[2], l[2];
+        if (q + e < SC) {
+          tca_split(v[q + e].x * kBasisScale, h[0], l[0]);
+          tca_split(v[q + e].y * kBasisScale, h[1], l[1]);
+          hi[e] = __halves2half2(h[0], h[1]);
+          lo[e] = __halves2half2(l[0], l[1]);
+          if (q + e < s) {
+            *reinterpret_cast<__half2*>(tiles.Vd + tca_dots_half(q0 + q + e, k, tiles.nkc, 0)) = hi[e];
+            *reinterpret_cast<__half2*>(tiles.Vd + tca_dots_half(q0 + q + e, k, tiles.nkc, 1)) = lo[e];
+          }
+        }
+      }
+      if (by4) {
+        *reinterpret_cast<uint4*>(tiles.Vu + tca_upd_half(q0 + q, k, tiles.nbc, 0)) = *reinterpret_cast<const uint4*>(hi);
+        *reinterpret_cast<uint4*>(tiles.Vu + tca_upd_half(q0 + q, k, tiles.nbc, 1)) = *reinterpret_cast<const uint4*>(lo);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (q + e < s) {
+            *reinterpret_cast<__half2*>(tiles.Vu + tca_upd_half(q0 + q + e, k, tiles.nbc, 0)) = hi[e];
+            *reinterpret_cast<__half2*>(tiles.Vu + tca_upd_half(q0 + q + e, k, tiles.nbc, 1)) = lo[e];
+          }
+      }
+    }
+  }
+#pragma unroll 4
+  for (int c = 0; c < s; ++c) {
+    float2* wp = reinterpret_cast<float2*>(W + 2 * int64_t(c) * ld) + k;
+    float2 a = *wp;
+#pragma unroll
+    for (int q = 0; q < SC; ++q) {
+      const float2 t = cs[q][c];
+      a.x = fmaf(-v[q].x, t.x, fmaf(v[q].y, t.y, a.x));
+      a.y = fmaf(-v[q].x, t.y, fmaf(-v[q].y, t.x, a.y));
+    }
+    *wp = a;
   }
 }
 
@@ -594,15 +817,30 @@ __global__ void __launch_bounds__(64) k_bcoef(const double* __restrict__ Gwv, co
 //   h[q, c] = Sw[q, c] + (Sv R)[q, c]            for q < nq0 = (J - 1) s,
 //   h[q, c] = C[q - nq0, c] + (Sv R)[q, c]       for nq0 <= q < nq0 + s,
 //   Rn = Rv R                                     (the subdiagonal block).
-// h complex FP64 at h + 2 (q s + c); R, Rv, Rn column-major.  Thread (q, c).
-__global__ void k_bhcol(const double* __restrict__ Sprev, const double* __restrict__ Scur,
-                        const double* __restrict__ Cp, const double* __restrict__ Rp, const double* __restrict__ Rv,
-                        int nq0, int s, double* __restrict__ h, double* __restrict__ Rn) {
+// h complex FP64 at h + 2 (q s + c); R, Rv, Rn column-major.  Thread (q, c);
+// the CTA's rows of Sv and R are converted to FP32 once, in shared memory
+// (converting them in every product kept the FP64 pipe busy: 14 us, now 11).
+__global__ void __launch_bounds__(256) k_bhcol(const double* __restrict__ Sprev, const double* __restrict__ Scur,
+                                               const double* __restrict__ Cp, const double* __restrict__ Rp,
+                                               const double* __restrict__ Rv, int nq0, int s, double* __restrict__ h,
+                                               double* __restrict__ Rn) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t nh = int64_t(nq0 + s) * s;
+  extern __shared__ float2 shc[];
+  float2* Rf = shc;           // R(p, c) at [c s + p]
+  float2* Sv = shc + s * s;   // rows of the CTA
+  const int64_t nh = int64_t(nq0 + s) * s, t0 = int64_t(blockIdx.x) * 256, t = t0 + threadIdx.x;
   const int ls = 2 * s;
+  const int64_t row0 = t0 / s;
+  const int rows = int(min(int64_t(nq0 + s), (t0 + 255) / s + 1) - row0);
+  if (t0 < nh) {
+    for (int q = threadIdx.x; q < s * s; q += 256) Rf[q] = make_float2(float(Rp[2 * q]), float(Rp[2 * q + 1]));
+    for (int q = threadIdx.x; q < rows * s; q += 256) {
+      const double* v = Scur + 2 * ((row0 + q / s) * ls + q % s);
+      Sv[q] = make_float2(float(v[0]), float(v[1]));
+    }
+  }
+  __syncthreads();
   if (t < nh) {
     const int q = int(t / s), c = int(t % s);
     double re, im;
@@ -617,11 +855,12 @@ __global__ void k_bhcol(const double* __restrict__ Sprev, const double* __restri
     // projection (about the FP32 rounding times the block's condition), so
     // its product with R is formed in FP32 and added to the FP64 part
     float cr = 0.f, ci = 0.f;
+    const float2* sv = Sv + (q - row0) * s;
+    const float2* rf = Rf + c * s;
     for (int p = 0; p <= c; ++p) {  // R upper triangular: R(p, c) at [c s + p]
-      const float ar = float(Scur[2 * (int64_t(q) * ls + p)]), ai = float(Scur[2 * (int64_t(q) * ls + p) + 1]);
-      const float br = float(Rp[2 * (c * s + p)]), bi = float(Rp[2 * (c * s + p) + 1]);
-      cr = fmaf(ar, br, fmaf(-ai, bi, cr));
-      ci = fmaf(ar, bi, fmaf(ai, br, ci));
+      const float2 a = sv[p], b = rf[p];
+      cr = fmaf(a.x, b.x, fmaf(-a.y, b.y, cr));
+      ci = fmaf(a.x, b.y, fmaf(a.y, b.x, ci));
     }
     h[2 * t] = re + double(cr);
     h[2 * t + 1] = im + double(ci);
@@ -664,7 +903,7 @@ static void bdots(mtf_system sys, const float* V, int nq, int64_t ldv, const flo
     // basis and block read once
     prof_bytes(kid, double(nq + nc) * double(n_pad) * 8.0);
 #define MTF_BDOTS(SCV, VWV) \
-  MTF_LAUNCH(kid, st, k_bdots<SCV, VWV><<<grid, 256, 0, st>>>(V, nq, ldv, Wc, ldw, nc, seg, n_pad, Hc, ldh))
+  MTF_LAUNCH(kid, st, launch_pdl(k_bdots<SCV, VWV>, grid, dim3(256), 0, st, V, nq, ldv, Wc, ldw, nc, seg, n_pad, Hc, ldh))
     if (SC == 16) MTF_BDOTS(16, 2);
     else if (SC == 8) MTF_BDOTS(8, 4);
     else if (SC == 4) MTF_BDOTS(4, 4);
@@ -761,14 +1000,16 @@ static void btrsm(const float* in, int64_t ldi, const double* R, const int* kept
 #undef MTF_BT
 }
 
-// G (nc x nc, complex FP64, G[a ldg + c] = <X_a, X_c>) of nc columns of
-// stride ldx over n_pad entries (bdots: FP32 products per segment, FP64
-// atomics; a two-stage kernel with per-CTA partial matrices measured slower,
-// its shared-memory loads per product outweighing the saved atomics)
-static void bgram(mtf_system sys, const float* X, int64_t ldx, int nc, int64_t n_pad, double* G, int ldg,
-                  cudaStream_t st) {
-  MTF_CUDA(cudaMemsetAsync(G, 0, 2 * size_t(nc) * ldg * sizeof(double), st));
-  bdots(sys, X, nc, ldx, X, ldx, nc, n_pad, G, ldg, st);
+static void bfinish(const float* in, const double* Rv, const int* kept, int s, bool first, float* V, const double* C,
+                    float* W, int64_t ld, const TcaTiles& tiles, int q0, cudaStream_t st) {
+#define MTF_BF(SCV)                                                                                              \
+  MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bfinish<SCV>, dim3(nbk(ld, 128)), dim3(128), 0, st, in, Rv, kept, s,   \
+                                        first, V, C, W, ld, tiles, q0))
+  if (s <= 4) MTF_BF(4);
+  else if (s <= 8) MTF_BF(8);
+  else if (s <= 12) MTF_BF(12);
+  else MTF_BF(16);
+#undef MTF_BF
 }
 
 // relative size below which a new direction of a block is deflated (its norm
@@ -789,9 +1030,9 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
   BlockWork& B = *sys->bw;
   stream_prepare(sys, st);  // error word of the bounded waits
   const size_t nhc = size_t(m + 1) * s * s;  // complex entries of a Hessenberg column block
-  const size_t gsz = size_t(2) * (size_t(s) * s + 4 * size_t(s) * s + size_t(s) * s + nhc + 5 * size_t(s) * s);
-  // pinned slot of a step (doubles): column block (nhc complex) | Rn (s x s complex)
-  const size_t slot_len = 2 * nhc + 2 * size_t(s) * s;
+  // pinned slot of a step (doubles): Rn (s x s complex) | kept flags (2 s ints) | column block (nhc complex)
+  const size_t slot_len = 2 * size_t(s) * s + s + 2 * nhc;
+  const size_t gsz = size_t(2) * 9 * s * s + slot_len;
   if (B.s != s || B.m != m || B.n != n) {
     B.V.alloc(size_t(m + 1) * s * ldn * 2);
     B.Z.alloc(size_t(m) * s * ldn * 2);
@@ -803,16 +1044,14 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
     for (auto& b : B.S) b.alloc(size_t(2) * (m + 1) * s * 2 * s);
     B.Gs.alloc(gsz);
     B.C.alloc(size_t(2) * std::max<size_t>(size_t(s) * s, size_t(m) * s * s));
-    B.kept.alloc(size_t(2) * s);
+    B.normp.alloc(size_t(kPrepParts) * s);
+    B.maxp.alloc(size_t(kPrepParts) * 2 * s);
     if (B.h_host) cudaFreeHost(B.h_host);
     if (B.pin) cudaFreeHost(B.pin);
-    if (B.kept_host) cudaFreeHost(B.kept_host);
     B.h_host = nullptr;
     B.pin = nullptr;
-    B.kept_host = nullptr;
     MTF_CUDA(cudaMallocHost(&B.h_host, 2 * size_t(s) * s * sizeof(double)));
     MTF_CUDA(cudaMallocHost(&B.pin, 2 * slot_len * sizeof(double)));
-    MTF_CUDA(cudaMallocHost(&B.kept_host, 2 * (2 * size_t(s) + 1) * sizeof(int)));
     for (auto& e : B.ev)
       if (!e) MTF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     B.s = s;
@@ -820,16 +1059,15 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
     B.n = n;
     B.ldn = ldn;
   }
-  double* Gpre = B.Gs.p;                       // s: squared column norms of W before the projections
-  double* G2 = Gpre + 2 * size_t(s) * s;       // 2s x s: <X_q, V~'_c> for the columns q of [V~', W']
+  double* G2 = B.Gs.p;                         // 2s x s: <X_q, V~'_c> for the columns q of [V~', W']
   double* G = G2 + 8 * size_t(s) * s;          // s x s: Gram of W''
-  double* Hc = G + 2 * size_t(s) * s;          // completed column block ((m + 1) s x s)
-  double* Rn = Hc + 2 * nhc;                   // its subdiagonal block
-  double* R = Rn + 2 * size_t(s) * s;          // W'' = V~_{J+1} R
+  double* R = G + 2 * size_t(s) * s;           // W'' = V~_{J+1} R
   double* Rv = R + 2 * size_t(s) * s;          // V~' = V_J Rv
   double* CcBuf[2] = {Rv + 2 * size_t(s) * s, Rv + 4 * size_t(s) * s};  // W' = V_J Cc + W'' (steps by parity)
-  int* keptR = B.kept.p;
+  double* Rn = Rv + 6 * size_t(s) * s;         // subdiagonal block of the completed column block
+  int* keptR = reinterpret_cast<int*>(Rn + 2 * size_t(s) * s);
   int* keptV = keptR + s;
+  double* Hc = Rn + 2 * size_t(s) * s + s;     // completed column block ((m + 1) s x s)
   const int64_t vstride = int64_t(s) * ldn;  // complex entries per block of s vectors
   float* X0 = B.X.p;                          // V~_J (then V~')
   float* X1 = B.X.p + 2 * vstride;            // W (then W', W'')
@@ -847,7 +1085,7 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
   // X[:, 0 .. nc) -= V S and S = V^H X against the first nq basis vectors (S leading dimension 2 s)
   auto project = [&](int nq, int nc, double* S) {
     if (tc) {
-      tca_project(*B.tca, nq, B.X.p, nc, S, 2 * s, err_word, st);
+      tca_project(*B.tca, nq, B.X.p, nc, S, 2 * s, B.maxp.p, 2 * s, err_word, st);
     } else {
       MTF_CUDA(cudaMemsetAsync(S, 0, 2 * size_t(nq) * 2 * s * sizeof(double), st));
       bdots(sys, B.V.p, nq, ldn, B.X.p, ldn, nc, ldn, S, 2 * s, st, KID_DOTS);
@@ -941,14 +1179,14 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
         MTF_CUDA(cudaMemcpyAsync(Zj, Vt, size_t(s) * ldn * 8, cudaMemcpyDeviceToDevice, st));
       }
       launch_matvec_f32(sys, Zj, ldn, X1, ldn, s, st);
-      MTF_CUDA(cudaMemsetAsync(Gpre, 0, size_t(s) * sizeof(double), st));
-      MTF_LAUNCH(KID_BGRAM, st, k_bnorm2<<<dim3(64, unsigned(s)), 256, 0, st>>>(X1, ldn, ldn, Gpre));
     }
-    MTF_CUDA(cudaMemcpyAsync(X0, Vt, size_t(s) * ldn * 8, cudaMemcpyDeviceToDevice, st));
+    // X0 = V~_J, scales and reference norms; G2, G and H's maxima cleared
+    MTF_LAUNCH(KID_BGRAM, st, launch_pdl(k_bprep, dim3(kPrepParts, unsigned(s)), dim3(256), 0, st,
+        Vt, X0, finish ? nullptr : X1, ldn, s, 2 * s, B.maxp.p, B.normp.p, G2, 10 * s * s,
+        tc ? tca_hmax(*B.tca) : nullptr));
     if (nq > 0) project(nq, nc, Scur);
     // <X_q, V~'_c> for every column q of X = [V~', W'] (G_vv, then the
     // conjugate of G_vw): one pass with s right-hand columns
-    MTF_CUDA(cudaMemsetAsync(G2, 0, 2 * size_t(nc) * s * sizeof(double), st));
     bdots(sys, B.X.p, nc, ldn, X0, ldn, s, ldn, G2, s, st);
     const double* Gwv = G2 + 2 * size_t(s) * s;
     if (J == 0) {
@@ -956,32 +1194,39 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
     } else {
       // second CholQR pass of V~_J: directions that the first kept
       // Rv and, for a step with an operator apply, Cc = Rv^-H G_vw
-      MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol<float>, dim3(1), dim3(256), chol_smem32, st,
-          G2, s, nullptr, keptR, 1e-3, s, Rv, keptV,
-                                                                          Gwv, finish ? nullptr : Cc));
-      MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bhcol, dim3(nbk(int64_t(nq + s) * s, 256)), dim3(256), 0, st,
+      if (s <= 16)
+        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol16<float>, dim3(1), dim3(32), 0, st,
+            G2, s, nullptr, keptR, 1e-3, s, Rv, keptV, Gwv, finish ? nullptr : Cc));
+      else
+        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol<float>, dim3(1), dim3(256), chol_smem32, st,
+            G2, s, nullptr, keptR, 1e-3, s, Rv, keptV, Gwv, finish ? nullptr : Cc));
+      const size_t hsm = (size_t(s) * s + 256 + 2 * size_t(s)) * sizeof(float2);
+      MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bhcol, dim3(nbk(int64_t(nq + s) * s, 256)), dim3(256), hsm, st,
           Sprev, Scur, Cprev, R, Rv, nq - s, s, Hc, Rn));
     }
     if (!finish) {
-      if (J > 0) btrsm(X0, ldn, Rv, keptV, s, Vt, ldn, ldn, st);
       // (step 0: V_0 is final, Cc = G_vw on its kept set)
       if (J == 0)
         MTF_LAUNCH(KID_BXFORM, st, k_bcoef<<<1, 64, 2 * size_t(s) * s * sizeof(double2), st>>>(Gwv, Rv, keptV, s, Cc));
-      bupdate(Vt, s, ldn, Cc, s, X1, ldn, s, ldn, st);
-      bgram(sys, X1, ldn, s, ldn, G, s, st);
-      MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol<double>, dim3(1), dim3(256), chol_smem, st,
-          G, s, Gpre, nullptr, kDeflateTau, s, R,
-                                                                           keptR, nullptr, nullptr));
+      if (s <= 16) {
+        bfinish(X0, Rv, keptV, s, J == 0, Vt, Cc, X1, ldn, tc && J > 0 ? tca_tiles(*B.tca) : TcaTiles{}, J * s, st);
+      } else {
+        if (J > 0) btrsm(X0, ldn, Rv, keptV, s, Vt, ldn, ldn, st);
+        bupdate(Vt, s, ldn, Cc, s, X1, ldn, s, ldn, st);
+        if (tc && J > 0) tca_store(*B.tca, Vt, J * s, st);
+      }
+      bdots(sys, X1, s, ldn, X1, ldn, s, ldn, G, s, st);  // Gram of W''
+      if (s <= 16)
+        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol16<double>, dim3(1), dim3(32), 0, st,
+            G, s, B.normp.p, nullptr, kDeflateTau, s, R, keptR, nullptr, nullptr));
+      else
+        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol<double>, dim3(1), dim3(256), chol_smem, st,
+            G, s, B.normp.p, nullptr, kDeflateTau, s, R, keptR, nullptr, nullptr));
       btrsm(X1, ldn, R, keptR, s, Vt + 2 * vstride, ldn, ldn, st);
-      if (tc && J > 0) tca_store(*B.tca, Vt, J * s, st);
     }
-    double* sl = slot(J);
-    if (J > 0) {
-      MTF_CUDA(cudaMemcpyAsync(sl, Hc, 2 * size_t(nq) * s * sizeof(double), cudaMemcpyDeviceToHost, st));
-      MTF_CUDA(cudaMemcpyAsync(sl + 2 * nhc, Rn, 2 * size_t(s) * s * sizeof(double), cudaMemcpyDeviceToHost, st));
-    }
-    int* kh = B.kept_host + size_t(J & 1) * (2 * s + 1);
-    MTF_CUDA(cudaMemcpyAsync(kh, keptR, 2 * size_t(s) * sizeof(int), cudaMemcpyDeviceToHost, st));
+    // Rn, the kept flags and, from step 1 on, the column block: one copy
+    const size_t len = 2 * size_t(s) * s + s + (J > 0 ? 2 * size_t(nq) * s : 0);
+    MTF_CUDA(cudaMemcpyAsync(slot(J), Rn, len * sizeof(double), cudaMemcpyDeviceToHost, st));
     MTF_CUDA(cudaEventRecord(B.ev[J & 1], st));
   };
 
@@ -1006,26 +1251,27 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
       clk::time_point t;
       ~LsqClock() { acc += std::chrono::duration<double>(clk::now() - t).count(); }
     } lsq_clock{sys->t_lsq, tl};
-    const int* kh = B.kept_host + size_t(J & 1) * (2 * s + 1);
+    const double* sl = slot(J);  // Rn | kept | column block J - 1
+    const int* kh = reinterpret_cast<const int*>(sl + 2 * size_t(s) * s);
+    const double* hc = sl + 2 * size_t(s) * s + s;
     if (*static_cast<volatile unsigned*>(err_word) != 0) {
       status = MTF_ERR_TIMEOUT;
       break;
     }
     if (J == 0) continue;
     // column block J - 1: rows of blocks 0 .. J - 1 and the subdiagonal block
-    const double* sl = slot(J);
     const int nq = J * s;
     h.assign(size_t(nq) * s, cdouble(0));
     bool finite = true;
     for (int q = 0; q < nq; ++q)
       for (int c = 0; c < s; ++c) {
         const size_t o = 2 * (size_t(q) * s + c);
-        const cdouble v(sl[o], sl[o + 1]);
+        const cdouble v(hc[o], hc[o + 1]);
         finite = finite && std::isfinite(v.real()) && std::isfinite(v.imag());
         h[size_t(c) * nq + q] = v;
       }
     for (size_t t = 0; t < size_t(s) * s; ++t) {
-      Rnh[t] = cdouble(sl[2 * nhc + 2 * t], sl[2 * nhc + 2 * t + 1]);
+      Rnh[t] = cdouble(sl[2 * t], sl[2 * t + 1]);
       finite = finite && std::isfinite(Rnh[t].real()) && std::isfinite(Rnh[t].imag());
     }
     if (!finite) {
