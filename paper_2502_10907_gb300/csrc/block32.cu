@@ -48,6 +48,7 @@ struct BlockWork {
   DevBuf<double> S[2];       // projection coefficients of two steps: (m + 1) s x 2 s, complex
   DevBuf<double> Gs;         // G2 (2s x 2s) | G (s x s) | R | Rv | Cc (two) | Rn | kept (2 s ints) | Hc ((m + 1) s x s)
   DevBuf<double> normp;      // kPrepParts partial squared norms of W's columns before the projections
+  DevBuf<float> fac;         // FP32 copies: R, 1 / diag of Rv | of R | C
   DevBuf<float> maxp;        // kPrepParts partial maxima of the columns of X
   DevBuf<double> C;          // s x s (complex, FP64) transform, or the coefficients Y (m s x s)
   double* h_host = nullptr;
@@ -360,6 +361,14 @@ __global__ void __launch_bounds__(256) k_bprep(const float* __restrict__ Vt, flo
 // pass, whose Gram matrix is the identity to the FP32 rounding of the
 // once-normalised block (its factor is I + O(2^-24) and FP32 keeps that),
 // on the FP32 pipes instead of the narrow FP64 one.
+// FP32 copies of a factor for the kernels over the vectors: R column-major,
+// 1 / R(k, k) (0 for dropped directions), C row-major
+struct BlockFactors {
+  float2* R = nullptr;
+  float* rinv = nullptr;
+  float2* C = nullptr;
+};
+
 template <class T>
 struct CxOf;
 template <>
@@ -381,7 +390,7 @@ template <class T>
 __global__ void __launch_bounds__(256) k_bchol(const double* __restrict__ G, int ldg, const double* __restrict__ ref,
                                                const int* __restrict__ mask, double tau, int s, double* __restrict__ R,
                                                int* __restrict__ kept, const double* __restrict__ Gwv,
-                                               double* __restrict__ C) {
+                                               double* __restrict__ C, const BlockFactors F) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
   using T2 = typename CxOf<T>::type;
@@ -439,8 +448,12 @@ __global__ void __launch_bounds__(256) k_bchol(const double* __restrict__ G, int
   for (int t = tid; t < s * s; t += nt) {
     R[2 * t] = double(Rs[t].x);
     R[2 * t + 1] = double(Rs[t].y);
+    F.R[t] = make_float2(float(Rs[t].x), float(Rs[t].y));
   }
-  for (int k = tid; k < s; k += nt) kept[k] = keeps[k];
+  for (int k = tid; k < s; k += nt) {
+    kept[k] = keeps[k];
+    F.rinv[k] = float(rinv[k]);
+  }
   if (C != nullptr && tid < s) {
     const int c = tid;
     T2* Cs = A;  // the Schur complement is no longer needed
@@ -464,102 +477,131 @@ __global__ void __launch_bounds__(256) k_bchol(const double* __restrict__ G, int
   }
 }
 
-// k_bchol for s <= 16 in one warp: lane (c, h) holds the rows i = 2 j + h of
-// column c in registers; row k goes to the lanes by shuffles, so a pivot costs
-// no block barrier and its few FP64 instructions are those of one warp (eight
-// warps with a sparse update each kept the narrow FP64 pipe of the one SM busy:
-// 23 us for s = 16 in FP64 and 21 us in FP32 with the coefficient solve, now
-// 23 and 12 us).  Same rule, same layouts.
-template <class T2>
-__device__ __forceinline__ T2 shfl2(T2 v, int src) {
-  v.x = __shfl_sync(0xffffffffu, v.x, src);
-  v.y = __shfl_sync(0xffffffffu, v.y, src);
-  return v;
+// k_bchol for s <= 16 on 128 threads: thread (c, r) holds the rows i = r and
+// r + 8 of column c in registers.  Each quarter of an SM has its own narrow
+// FP64 pipe (about 70 cycles per warp instruction), so the four warps share
+// the rows and a pivot's chain is kept short: the row as it stands, 1 / d by
+// one third-order Newton (Householder) step from the hardware's approximation
+// (y <- y (1 + e + e^2), e = 1 - d y), one barrier; the square roots of all pivots are taken
+// together at the end (R(k, c) = a_kc / sqrt(d_k), the Schur complement loses
+// conj(a_ki) a_kc / d_k).  Same rule and layouts; also R, 1 / R(k, k) and C in
+// FP32 for the kernels that use them so.  s = 16, a step's two factorisations:
+// 2 x 20.6 us with one warp, 2 x 14.3 us so.
+__device__ __forceinline__ double rcp_of(double d) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float rcp_of(float d) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+  return fmaf(y, fmaf(-d, y, 1.f), y);
 }
 
 template <class T>
-__global__ void __launch_bounds__(32) k_bchol16(const double* __restrict__ G, int ldg, const double* __restrict__ ref,
-                                                const int* __restrict__ mask, double tau, int s, double* __restrict__ R,
-                                                int* __restrict__ kept, const double* __restrict__ Gwv,
-                                                double* __restrict__ C) {
+__global__ void __launch_bounds__(128) k_bchol16(const double* __restrict__ G, int ldg, const double* __restrict__ ref,
+                                                 const int* __restrict__ mask, double tau, int s, double* __restrict__ R,
+                                                 int* __restrict__ kept, const double* __restrict__ Gwv,
+                                                 double* __restrict__ C, const BlockFactors F) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
   using T2 = typename CxOf<T>::type;
-  __shared__ T2 Rs[16][17];  // Rs[c][i] = R(i, c)
-  __shared__ T rinv[16];
-  __shared__ int keeps[16];
-  const int lane = threadIdx.x, c = lane & 15, h = lane >> 4;
-  T2 A[8];
+  __shared__ T2 row[2][16];   // row k of the Schur complement (by the parity of k)
+  __shared__ T2 Rs[16][17];   // Rs[c][k] = a_kc, then R(k, c)
+  __shared__ T2 gs[16][17];   // G_vw, then C
+  __shared__ double thr[16];  // tau^2 ref of column c
+  __shared__ T sq[16];        // 1 / sqrt(d_k), 0 for dropped directions
+  const int tid = threadIdx.x, c = tid & 15, r = tid >> 4;
+  T2 A[2];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int i = 2 * j + h;
+  for (int j = 0; j < 2; ++j) {
+    const int i = r + 8 * j;
     A[j] = c < s && i < s ? T2{T(G[2 * (i * ldg + c)]), T(G[2 * (i * ldg + c) + 1])} : T2{T(0), T(0)};
     Rs[c][i] = T2{T(0), T(0)};
+    if (C != nullptr)
+      gs[c][i] = c < s && i < s ? T2{T(Gwv[2 * (c * s + i)]), -T(Gwv[2 * (c * s + i) + 1])} : T2{T(0), T(0)};
   }
-  double thr = 0.0;  // tau^2 ref of column c
-  if (c < s) {
-    if (mask) thr = mask[c] && h == 0 ? 1.0 : 0.0;
-    else
-#pragma unroll 4
-      for (int p = h; p < kPrepParts; p += 2) thr += ref[p * s + c];
-  }
-  thr += __shfl_xor_sync(0xffffffffu, thr, 16);
-  thr = tau * tau * fmax(thr, 0.0);
-  __syncwarp();
+  {
+    double t = 0.0;
+    if (c < s) {
+      if (mask) t = r == 0 && mask[c] ? 1.0 : 0.0;
+      else
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    if (k < s) {
-      const T2 row = shfl2(A[k >> 1], c + 16 * (k & 1));  // A(k, c)
-      const T d = __shfl_sync(0xffffffffu, row.x, k);
-      const double t = __shfl_sync(0xffffffffu, thr, k);
-      const bool keep = double(d) > t && d > T(0);
-      T y = T(0);
-      if (keep) {
-        y = rsqrt_of(d);
-        const T2 r = c == k ? T2{d * y, T(0)} : T2{row.x * y, row.y * y};
-        if (h == 0 && c >= k) Rs[c][k] = r;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (2 * j + 1 > k) {  // rows i > k (row k itself is no longer needed)
-            const T2 ri = shfl2(r, 2 * j + h);
-            A[j].x -= ri.x * r.x + ri.y * r.y;  // conj(R(k, i)) R(k, c)
-            A[j].y -= ri.x * r.y - ri.y * r.x;
-          }
-      }
-      if (lane == 0) {
-        rinv[k] = y;
-        keeps[k] = keep ? 1 : 0;
-      }
+        for (int p = 0; p < kPrepParts / 8; ++p) t += ref[(8 * p + r) * s + c];
     }
+    // r = 2 warp + (lane >> 4): the halves of a warp, then the warps
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+    __shared__ double parts[4][16];
+    if ((tid & 31) < 16) parts[tid >> 5][c] = t;
+    __syncthreads();
+    if (tid < 16) thr[c] = tau * tau * fmax(parts[0][c] + parts[1][c] + parts[2][c] + parts[3][c], 0.0);
   }
-  __syncwarp();
-  for (int t = lane; t < s * s; t += 32) {
-    const T2 r = Rs[t / s][t % s];
-    R[2 * t] = double(r.x);
-    R[2 * t + 1] = double(r.y);
+  for (int k = 0; k < s; ++k) {
+    if (r == (k & 7)) row[k & 1][c] = k < 8 ? A[0] : A[1];
+    __syncthreads();
+    const T2* rk = row[k & 1];
+    const T d = rk[k].x;
+    const bool keep = double(d) > thr[k] && d > T(0);
+    if (keep) {
+      const T y = rcp_of(d);
+      const T2 a = rk[c], t = T2{a.x * y, a.y * y};
+      if (r == 0 && c >= k) Rs[c][k] = a;
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        if (r + 8 * j > k) {
+          const T2 b = rk[r + 8 * j];  // conj(a_ki) a_kc / d_k
+          A[j].x = fma(-b.x, t.x, fma(-b.y, t.y, A[j].x));
+          A[j].y = fma(-b.x, t.y, fma(b.y, t.x, A[j].y));
+        }
+    }
+    if (tid == 0) sq[k] = keep ? d : T(0);
   }
-  if (lane < s) kept[lane] = keeps[lane];
-  if (C != nullptr && lane < s) {
-    // column c = lane of C = R^-H G_vw by forward substitution
+  __syncthreads();
+  if (tid < s) {
+    const T d = sq[tid];
+    sq[tid] = d > T(0) ? rsqrt_of(d) : T(0);
+    kept[tid] = d > T(0) ? 1 : 0;
+  }
+  __syncthreads();
+  for (int t = tid; t < s * s; t += 128) {
+    const int cc = t / s, i = t % s;
+    T2 v = Rs[cc][i];
+    v.x *= sq[i];
+    v.y = i == cc ? T(0) : v.y * sq[i];
+    Rs[cc][i] = v;
+    R[2 * t] = double(v.x);
+    R[2 * t + 1] = double(v.y);
+    F.R[t] = make_float2(float(v.x), float(v.y));
+  }
+  if (tid < s) F.rinv[tid] = float(sq[tid]);
+  if (C == nullptr) return;
+  __syncthreads();
+  if (tid < s) {
+    // column tid of C = R^-H G_vw by forward substitution
     T2 g[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      g[i] = i < s ? T2{T(Gwv[2 * (c * s + i)]), -T(Gwv[2 * (c * s + i) + 1])} : T2{T(0), T(0)};
+    for (int i = 0; i < 16; ++i) g[i] = gs[tid][i];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       if (i < s) {
-        const T f = keeps[i] ? rinv[i] : T(0);
-        const T2 x = T2{g[i].x * f, g[i].y * f};
+        const T2 x = T2{g[i].x * sq[i], g[i].y * sq[i]};
 #pragma unroll
         for (int p = i + 1; p < 16; ++p) {
-          const T2 r = Rs[p][i];  // R(i, p); zero past s
-          g[p].x -= r.x * x.x + r.y * x.y;
-          g[p].y -= r.x * x.y - r.y * x.x;
+          const T2 q = Rs[p][i];  // R(i, p); zero past s
+          g[p].x = fma(-q.x, x.x, fma(-q.y, x.y, g[p].x));
+          g[p].y = fma(-q.x, x.y, fma(q.y, x.x, g[p].y));
         }
-        C[2 * (i * s + c)] = double(x.x);
-        C[2 * (i * s + c) + 1] = double(x.y);
+        gs[tid][i] = x;
       }
     }
+  }
+  __syncthreads();
+  for (int t = tid; t < s * s; t += 128) {
+    const T2 v = gs[t % s][t / s];  // C(i, c) at [i s + c]
+    C[2 * t] = double(v.x);
+    C[2 * t + 1] = double(v.y);
+    F.C[t] = make_float2(float(v.x), float(v.y));
   }
 }
 
@@ -569,28 +611,20 @@ __global__ void __launch_bounds__(32) k_bchol16(const double* __restrict__ G, in
 // copies of the basis (vectors q0 .. q0 + s - 1); then W -= V_J C.  One kernel
 // for a triangular solve, two stores and an update: V_J stays in registers.
 template <int SC>
-__global__ void __launch_bounds__(128) k_bfinish(const float* __restrict__ in, const double* __restrict__ Rv,
-                                                 const int* __restrict__ kept, int s, bool first,
-                                                 float* __restrict__ V, const double* __restrict__ C,
-                                                 float* __restrict__ W, int64_t ld, const TcaTiles tiles, int q0) {
+__global__ void __launch_bounds__(128) k_bfinish(const float* __restrict__ in, const BlockFactors F, int s, bool first,
+                                                 float* __restrict__ V, float* __restrict__ W, int64_t ld,
+                                                 const TcaTiles tiles, int q0) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
   __shared__ float2 rs[SC][SC], cs[SC][SC];  // rs[p][q] = R(p, q), cs[q][c] = C(q, c)
-  __shared__ float2 inv[SC];
+  __shared__ float inv[SC];
   for (int t = threadIdx.x; t < SC * SC; t += 128) {
     const int p = t / SC, q = t % SC;
     const bool ok = p < s && q < s;
-    rs[p][q] = ok ? make_float2(float(Rv[2 * (q * s + p)]), float(Rv[2 * (q * s + p) + 1])) : make_float2(0.f, 0.f);
-    cs[p][q] = ok ? make_float2(float(C[2 * (p * s + q)]), float(C[2 * (p * s + q) + 1])) : make_float2(0.f, 0.f);
+    rs[p][q] = ok && !first ? F.R[q * s + p] : make_float2(0.f, 0.f);
+    cs[p][q] = ok ? F.C[p * s + q] : make_float2(0.f, 0.f);
   }
-  for (int q = threadIdx.x; q < SC; q += 128) {
-    float2 v = make_float2(0.f, 0.f);
-    if (q < s && kept[q]) {
-      const double a = Rv[2 * (q * s + q)], b = Rv[2 * (q * s + q) + 1], d = a * a + b * b;
-      v = make_float2(float(a / d), float(-b / d));
-    }
-    inv[q] = v;
-  }
+  for (int q = threadIdx.x; q < SC; q += 128) inv[q] = q < s && !first ? F.rinv[q] : 0.f;
   __syncthreads();
   const int64_t k = int64_t(blockIdx.x) * 128 + threadIdx.x;
   if (k >= ld) return;
@@ -607,8 +641,7 @@ __global__ void __launch_bounds__(128) k_bfinish(const float* __restrict__ in, c
           a.x -= v[p].x * r.x - v[p].y * r.y;
           a.y -= v[p].x * r.y + v[p].y * r.x;
         }
-        const float2 iv = inv[q];
-        a = make_float2(a.x * iv.x - a.y * iv.y, a.x * iv.y + a.y * iv.x);
+        a = make_float2(a.x * inv[q], a.y * inv[q]);
         reinterpret_cast<float2*>(V + 2 * int64_t(q) * ld)[k] = a;
       }
       v[q] = a;
@@ -663,28 +696,19 @@ __global__ void __launch_bounds__(128) k_bfinish(const float* __restrict__ in, c
 
 // out_q[k] = (in_q[k] - sum_{p < q} out_p[k] R(p, q)) / R(q, q) for kept q,
 // 0 otherwise: V = W R^-1 on the kept set by forward substitution, entry by
-// entry (R complex FP64, column-major, used in FP32)
+// entry (the factor's FP32 copies; the diagonal of R is real)
 template <int SC>
-__global__ void __launch_bounds__(128) k_btrsm(const float* __restrict__ in, int64_t ldi, const double* __restrict__ R,
-                                               const int* __restrict__ kept, int s, float* __restrict__ out, int64_t ldo,
-                                               int64_t n_pad) {
+__global__ void __launch_bounds__(128) k_btrsm(const float* __restrict__ in, int64_t ldi, const BlockFactors F, int s,
+                                               float* __restrict__ out, int64_t ldo, int64_t n_pad) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
   __shared__ float2 rs[SC][SC];  // rs[p][q] = R(p, q)
-  __shared__ float2 inv[SC];     // 1 / R(q, q), 0 for dropped q
+  __shared__ float inv[SC];      // 1 / R(q, q), 0 for dropped q
   for (int t = threadIdx.x; t < SC * SC; t += blockDim.x) {
     const int p = t / SC, q = t % SC;
-    rs[p][q] = (p < s && q < s) ? make_float2(float(R[2 * (q * s + p)]), float(R[2 * (q * s + p) + 1]))
-                                : make_float2(0.f, 0.f);
+    rs[p][q] = (p < s && q < s) ? F.R[q * s + p] : make_float2(0.f, 0.f);
   }
-  for (int q = threadIdx.x; q < SC; q += blockDim.x) {
-    float2 v = make_float2(0.f, 0.f);
-    if (q < s && kept[q]) {
-      const double a = R[2 * (q * s + q)], b = R[2 * (q * s + q) + 1], d = a * a + b * b;
-      v = make_float2(float(a / d), float(-b / d));
-    }
-    inv[q] = v;
-  }
+  for (int q = threadIdx.x; q < SC; q += blockDim.x) inv[q] = q < s ? F.rinv[q] : 0.f;
   __syncthreads();
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= n_pad) return;
@@ -699,8 +723,7 @@ __global__ void __launch_bounds__(128) k_btrsm(const float* __restrict__ in, int
       a.x -= v[p].x * r.x - v[p].y * r.y;
       a.y -= v[p].x * r.y + v[p].y * r.x;
     }
-    const float2 iv = inv[q];
-    v[q] = make_float2(a.x * iv.x - a.y * iv.y, a.x * iv.y + a.y * iv.x);
+    v[q] = make_float2(a.x * inv[q], a.y * inv[q]);
     reinterpret_cast<float2*>(out + 2 * int64_t(q) * ldo)[k] = v[q];
   }
 }
@@ -710,28 +733,19 @@ __global__ void __launch_bounds__(128) k_btrsm(const float* __restrict__ in, int
 // (SC complex values per thread would spill), R and the reciprocals staged
 // as in k_btrsm.  Dynamic shared memory: SC^2 + SC x 128 complex FP32.
 template <int SC>
-__global__ void __launch_bounds__(128) k_btrsm_wide(const float* __restrict__ in, int64_t ldi,
-                                                    const double* __restrict__ R, const int* __restrict__ kept, int s,
+__global__ void __launch_bounds__(128) k_btrsm_wide(const float* __restrict__ in, int64_t ldi, const BlockFactors F, int s,
                                                     float* __restrict__ out, int64_t ldo, int64_t n_pad) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
   extern __shared__ float2 shw[];
   float2* rs = shw;             // rs[p * SC + q] = R(p, q)
   float2* vs = shw + SC * SC;   // vs[q * 128 + thread]
-  __shared__ float2 inv[SC];
+  __shared__ float inv[SC];
   for (int t = threadIdx.x; t < SC * SC; t += blockDim.x) {
     const int p = t / SC, q = t % SC;
-    rs[t] = (p < s && q < s) ? make_float2(float(R[2 * (q * s + p)]), float(R[2 * (q * s + p) + 1]))
-                             : make_float2(0.f, 0.f);
+    rs[t] = (p < s && q < s) ? F.R[q * s + p] : make_float2(0.f, 0.f);
   }
-  for (int q = threadIdx.x; q < SC; q += blockDim.x) {
-    float2 v = make_float2(0.f, 0.f);
-    if (q < s && kept[q]) {
-      const double a = R[2 * (q * s + q)], b = R[2 * (q * s + q) + 1], d = a * a + b * b;
-      v = make_float2(float(a / d), float(-b / d));
-    }
-    inv[q] = v;
-  }
+  for (int q = threadIdx.x; q < SC; q += blockDim.x) inv[q] = q < s ? F.rinv[q] : 0.f;
   __syncthreads();
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= n_pad) return;
@@ -742,8 +756,7 @@ __global__ void __launch_bounds__(128) k_btrsm_wide(const float* __restrict__ in
       a.x -= v.x * r.x - v.y * r.y;
       a.y -= v.x * r.y + v.y * r.x;
     }
-    const float2 iv = inv[q];
-    const float2 o = make_float2(a.x * iv.x - a.y * iv.y, a.x * iv.y + a.y * iv.x);
+    const float2 o = make_float2(a.x * inv[q], a.y * inv[q]);
     vs[q * 128 + threadIdx.x] = o;
     reinterpret_cast<float2*>(out + 2 * int64_t(q) * ldo)[k] = o;
   }
@@ -769,7 +782,8 @@ __global__ void k_beye(const int* __restrict__ kept_in, int s, double* __restric
 // forward substitution of column c (no reductions across threads: the
 // narrow FP64 pipe makes warp-shuffle sums the slower form).
 __global__ void __launch_bounds__(64) k_bcoef(const double* __restrict__ Gwv, const double* __restrict__ R,
-                                              const int* __restrict__ kept, int s, double* __restrict__ C) {
+                                              const int* __restrict__ kept, int s, double* __restrict__ C,
+                                              float2* __restrict__ Cf) {
   extern __shared__ double2 sh[];
   double2* Rs = sh;              // Rs[i * s + p] = R(p, i)
   double2* Cs = sh + s * s;      // Cs[i * s + c]; first G_vw(i, c)
@@ -806,6 +820,7 @@ __global__ void __launch_bounds__(64) k_bcoef(const double* __restrict__ Gwv, co
   for (int t = threadIdx.x; t < s * s; t += blockDim.x) {
     C[2 * t] = Cs[t].x;
     C[2 * t + 1] = Cs[t].y;
+    Cf[t] = make_float2(float(Cs[t].x), float(Cs[t].y));
   }
 }
 
@@ -816,14 +831,13 @@ __global__ void __launch_bounds__(64) k_bcoef(const double* __restrict__ Gwv, co
 // step J - 1 and Rv of step J,
 //   h[q, c] = Sw[q, c] + (Sv R)[q, c]            for q < nq0 = (J - 1) s,
 //   h[q, c] = C[q - nq0, c] + (Sv R)[q, c]       for nq0 <= q < nq0 + s,
-//   Rn = Rv R                                     (the subdiagonal block).
+//   Rn = Rv R                                     (the subdiagonal block, k_brn).
 // h complex FP64 at h + 2 (q s + c); R, Rv, Rn column-major.  Thread (q, c);
 // the CTA's rows of Sv and R are converted to FP32 once, in shared memory
 // (converting them in every product kept the FP64 pipe busy: 14 us, now 11).
 __global__ void __launch_bounds__(256) k_bhcol(const double* __restrict__ Sprev, const double* __restrict__ Scur,
-                                               const double* __restrict__ Cp, const double* __restrict__ Rp,
-                                               const double* __restrict__ Rv, int nq0, int s, double* __restrict__ h,
-                                               double* __restrict__ Rn) {
+                                               const double* __restrict__ Cp, const float2* __restrict__ Rp, int nq0,
+                                               int s, double* __restrict__ h) {
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
   extern __shared__ float2 shc[];
@@ -834,7 +848,7 @@ __global__ void __launch_bounds__(256) k_bhcol(const double* __restrict__ Sprev,
   const int64_t row0 = t0 / s;
   const int rows = int(min(int64_t(nq0 + s), (t0 + 255) / s + 1) - row0);
   if (t0 < nh) {
-    for (int q = threadIdx.x; q < s * s; q += 256) Rf[q] = make_float2(float(Rp[2 * q]), float(Rp[2 * q + 1]));
+    for (int q = threadIdx.x; q < s * s; q += 256) Rf[q] = Rp[q];
     for (int q = threadIdx.x; q < rows * s; q += 256) {
       const double* v = Scur + 2 * ((row0 + q / s) * ls + q % s);
       Sv[q] = make_float2(float(v[0]), float(v[1]));
@@ -864,15 +878,31 @@ __global__ void __launch_bounds__(256) k_bhcol(const double* __restrict__ Sprev,
     }
     h[2 * t] = re + double(cr);
     h[2 * t + 1] = im + double(ci);
-  } else if (t < nh + int64_t(s) * s) {
-    const int u = int(t - nh), c = u / s, i = u % s;
-    double re = 0.0, im = 0.0;
-    for (int p = i; p <= c; ++p) {  // Rv(i, p) R(p, c)
+  }
+}
+
+// Rn = Rv R of k_bhcol (FP64): 4 lanes per entry, 64 entries per CTA, so that
+// the products are spread over several SMs' FP64 pipes
+__global__ void __launch_bounds__(256) k_brn(const double* __restrict__ Rp, const double* __restrict__ Rv, int s,
+                                             double* __restrict__ Rn) {
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+  const int u = blockIdx.x * 64 + (threadIdx.x >> 2), l = threadIdx.x & 3;
+  const int c = u / s, i = u % s;
+  double re = 0.0, im = 0.0;
+  if (u < s * s)
+    for (int p = i + l; p <= c; p += 4) {  // Rv(i, p) R(p, c)
       const double ar = Rv[2 * (p * s + i)], ai = Rv[2 * (p * s + i) + 1];
       const double br = Rp[2 * (c * s + p)], bi = Rp[2 * (c * s + p) + 1];
-      re += ar * br - ai * bi;
-      im += ar * bi + ai * br;
+      re = fma(ar, br, fma(-ai, bi, re));
+      im = fma(ar, bi, fma(ai, br, im));
     }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, o);
+    im += __shfl_xor_sync(0xffffffffu, im, o);
+  }
+  if (u < s * s && l == 0) {
     Rn[2 * (c * s + i)] = re;
     Rn[2 * (c * s + i) + 1] = im;
   }
@@ -965,11 +995,11 @@ static void bxform(const float* in, int64_t ldi, const double* T, int s, float* 
 #undef MTF_BX
 }
 
-static void btrsm(const float* in, int64_t ldi, const double* R, const int* kept, int s, float* out, int64_t ldo,
-                  int64_t n_pad, cudaStream_t st) {
+static void btrsm(const float* in, int64_t ldi, const BlockFactors& F, int s, float* out, int64_t ldo, int64_t n_pad,
+                  cudaStream_t st) {
   const unsigned g = nbk(n_pad, 128);
 #define MTF_BT(SCV) \
-  MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_btrsm<SCV>, dim3(g), dim3(128), 0, st, in, ldi, R, kept, s, out, ldo, n_pad))
+  MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_btrsm<SCV>, dim3(g), dim3(128), 0, st, in, ldi, F, s, out, ldo, n_pad))
   if (s <= 1) MTF_BT(1);
   else if (s <= 2) MTF_BT(2);
   else if (s <= 4) MTF_BT(4);
@@ -992,19 +1022,19 @@ static void btrsm(const float* in, int64_t ldi, const double* R, const int* kept
     }
     if (SC == 32)
       MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_btrsm_wide<32>, dim3(g), dim3(128), smem, st,
-          in, ldi, R, kept, s, out, ldo, n_pad));
+          in, ldi, F, s, out, ldo, n_pad));
     else
       MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_btrsm_wide<64>, dim3(g), dim3(128), smem, st,
-          in, ldi, R, kept, s, out, ldo, n_pad));
+          in, ldi, F, s, out, ldo, n_pad));
   }
 #undef MTF_BT
 }
 
-static void bfinish(const float* in, const double* Rv, const int* kept, int s, bool first, float* V, const double* C,
-                    float* W, int64_t ld, const TcaTiles& tiles, int q0, cudaStream_t st) {
-#define MTF_BF(SCV)                                                                                              \
-  MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bfinish<SCV>, dim3(nbk(ld, 128)), dim3(128), 0, st, in, Rv, kept, s,   \
-                                        first, V, C, W, ld, tiles, q0))
+static void bfinish(const float* in, const BlockFactors& F, int s, bool first, float* V, float* W, int64_t ld,
+                    const TcaTiles& tiles, int q0, cudaStream_t st) {
+#define MTF_BF(SCV)                                                                                                  \
+  MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bfinish<SCV>, dim3(nbk(ld, 128)), dim3(128), 0, st, in, F, s, first, V, W, \
+                                        ld, tiles, q0))
   if (s <= 4) MTF_BF(4);
   else if (s <= 8) MTF_BF(8);
   else if (s <= 12) MTF_BF(12);
@@ -1045,6 +1075,7 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
     B.Gs.alloc(gsz);
     B.C.alloc(size_t(2) * std::max<size_t>(size_t(s) * s, size_t(m) * s * s));
     B.normp.alloc(size_t(kPrepParts) * s);
+    B.fac.alloc(size_t(6) * s * s + 2 * size_t(s));
     B.maxp.alloc(size_t(kPrepParts) * 2 * s);
     if (B.h_host) cudaFreeHost(B.h_host);
     if (B.pin) cudaFreeHost(B.pin);
@@ -1068,6 +1099,10 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
   int* keptR = reinterpret_cast<int*>(Rn + 2 * size_t(s) * s);
   int* keptV = keptR + s;
   double* Hc = Rn + 2 * size_t(s) * s + s;     // completed column block ((m + 1) s x s)
+  float2* fac = reinterpret_cast<float2*>(B.fac.p);
+  float* frinv = B.fac.p + 6 * size_t(s) * s;
+  const BlockFactors FV{fac, frinv, fac + 2 * size_t(s) * s};                           // of Rv, with Cc
+  const BlockFactors FR{fac + size_t(s) * s, frinv + s, nullptr};                       // of R
   const int64_t vstride = int64_t(s) * ldn;  // complex entries per block of s vectors
   float* X0 = B.X.p;                          // V~_J (then V~')
   float* X1 = B.X.p + 2 * vstride;            // W (then W', W'')
@@ -1195,34 +1230,36 @@ mtf_status fgmres_block32(mtf_system sys, int s, const double* r_dev, double* x_
       // second CholQR pass of V~_J: directions that the first kept
       // Rv and, for a step with an operator apply, Cc = Rv^-H G_vw
       if (s <= 16)
-        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol16<float>, dim3(1), dim3(32), 0, st,
-            G2, s, nullptr, keptR, 1e-3, s, Rv, keptV, Gwv, finish ? nullptr : Cc));
+        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol16<float>, dim3(1), dim3(128), 0, st,
+            G2, s, nullptr, keptR, 1e-3, s, Rv, keptV, Gwv, finish ? nullptr : Cc, FV));
       else
         MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol<float>, dim3(1), dim3(256), chol_smem32, st,
-            G2, s, nullptr, keptR, 1e-3, s, Rv, keptV, Gwv, finish ? nullptr : Cc));
+            G2, s, nullptr, keptR, 1e-3, s, Rv, keptV, Gwv, finish ? nullptr : Cc, FV));
       const size_t hsm = (size_t(s) * s + 256 + 2 * size_t(s)) * sizeof(float2);
-      MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bhcol, dim3(nbk(int64_t(nq + s) * s, 256)), dim3(256), hsm, st,
-          Sprev, Scur, Cprev, R, Rv, nq - s, s, Hc, Rn));
+      // (before this step's R replaces the last one's)
+      MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_bhcol, dim3(nbk(int64_t(nq) * s, 256)), dim3(256), hsm, st,
+          Sprev, Scur, Cprev, FR.R, nq - s, s, Hc));
+      MTF_LAUNCH(KID_BXFORM, st, launch_pdl(k_brn, dim3(nbk(int64_t(s) * s, 64)), dim3(256), 0, st, R, Rv, s, Rn));
     }
     if (!finish) {
       // (step 0: V_0 is final, Cc = G_vw on its kept set)
       if (J == 0)
-        MTF_LAUNCH(KID_BXFORM, st, k_bcoef<<<1, 64, 2 * size_t(s) * s * sizeof(double2), st>>>(Gwv, Rv, keptV, s, Cc));
+        MTF_LAUNCH(KID_BXFORM, st, k_bcoef<<<1, 64, 2 * size_t(s) * s * sizeof(double2), st>>>(Gwv, Rv, keptV, s, Cc, FV.C));
       if (s <= 16) {
-        bfinish(X0, Rv, keptV, s, J == 0, Vt, Cc, X1, ldn, tc && J > 0 ? tca_tiles(*B.tca) : TcaTiles{}, J * s, st);
+        bfinish(X0, FV, s, J == 0, Vt, X1, ldn, tc && J > 0 ? tca_tiles(*B.tca) : TcaTiles{}, J * s, st);
       } else {
-        if (J > 0) btrsm(X0, ldn, Rv, keptV, s, Vt, ldn, ldn, st);
+        if (J > 0) btrsm(X0, ldn, FV, s, Vt, ldn, ldn, st);
         bupdate(Vt, s, ldn, Cc, s, X1, ldn, s, ldn, st);
         if (tc && J > 0) tca_store(*B.tca, Vt, J * s, st);
       }
       bdots(sys, X1, s, ldn, X1, ldn, s, ldn, G, s, st);  // Gram of W''
       if (s <= 16)
-        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol16<double>, dim3(1), dim3(32), 0, st,
-            G, s, B.normp.p, nullptr, kDeflateTau, s, R, keptR, nullptr, nullptr));
+        MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol16<double>, dim3(1), dim3(128), 0, st,
+            G, s, B.normp.p, nullptr, kDeflateTau, s, R, keptR, nullptr, nullptr, FR));
       else
         MTF_LAUNCH(KID_BCHOL, st, launch_pdl(k_bchol<double>, dim3(1), dim3(256), chol_smem, st,
-            G, s, B.normp.p, nullptr, kDeflateTau, s, R, keptR, nullptr, nullptr));
-      btrsm(X1, ldn, R, keptR, s, Vt + 2 * vstride, ldn, ldn, st);
+            G, s, B.normp.p, nullptr, kDeflateTau, s, R, keptR, nullptr, nullptr, FR));
+      btrsm(X1, ldn, FR, s, Vt + 2 * vstride, ldn, ldn, st);
     }
     // Rn, the kept flags and, from step 1 on, the column block: one copy
     const size_t len = 2 * size_t(s) * s + s + (J > 0 ? 2 * size_t(nq) * s : 0);
