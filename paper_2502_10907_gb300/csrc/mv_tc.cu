@@ -465,14 +465,25 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  MTF_PDL_WAIT();
-  MTF_PDL_TRIGGER();
 
   if (warp == 0) {
     if (lane == 0) {
       tma_prefetch_map(&amap);
       tma_prefetch_map(&bmap);
       const uint64_t pol_a = l2_policy_evict_first(), pol_b = l2_policy_evict_last();
+      // the operator tiles of the first S stages, before the wait for the
+      // kernel that makes the inputs (the tiles are older)
+      int ahead = 0;
+      for (int q = q_begin; q < q_end && ahead < S; ++q) {
+        const int4 U = units[sched[q]];
+        const int64_t tb = blk_tile_base[U.x] + int64_t(U.y) * blk_nkc[U.x];
+        for (int kc = U.z; kc < U.w && ahead < S; ++kc, ++ahead) {
+          mbar_arrive_expect_tx(&full[ahead], uint32_t(SB));
+          tma_load_4d(smem + size_t(ahead) * SB, &amap, 0, 0, 0, int(tb + kc), &full[ahead], pol_a);
+        }
+      }
+      MTF_PDL_WAIT();
+      MTF_PDL_TRIGGER();
       int k = 0;
       bool ok = true;
       for (int q = q_begin; q < q_end && ok; ++q) {
@@ -481,6 +492,10 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
         const int64_t cb = blk_chunk_base[U.x];
         for (int kc = U.z; kc < U.w; ++kc, ++k) {
           const int st = k % S;
+          if (k < ahead) {
+            tma_load_4d(smem + size_t(st) * SB + SA, &bmap, 0, 0, 0, int(cb + kc), &full[st], pol_b);
+            continue;
+          }
           if (!mbar_wait_bounded(&empty[st], (uint32_t(k / S) & 1u) ^ 1u, kTcWaitNs)) {
             atomicExch(err, 1u);
             ok = false;
@@ -495,6 +510,8 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
     }
   } else if (warp == 1) {
     if (lane == 0) {
+      MTF_PDL_WAIT();
+      MTF_PDL_TRIGGER();
       constexpr uint32_t idesc = idesc_f16_m128(NB / 2);
       int k = 0, ub = 0;
       bool ok = true;
@@ -538,6 +555,8 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
     }
   } else {
     // epilogue: warps 2..5 cover the four TMEM lane quarters
+    MTF_PDL_WAIT();
+    MTF_PDL_TRIGGER();
     const int quarter = warp & 3;
     const int row = 32 * quarter + lane;
     int ub = 0;

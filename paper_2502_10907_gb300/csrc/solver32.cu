@@ -87,7 +87,7 @@ constexpr int kDtR = kDtRW * kDtCons;     // basis vectors per unit
 constexpr int kDtSliceB = kDtL * 8;       // bytes of one slice
 constexpr int kDtSB = (kDtR + 2) * kDtSliceB;
 constexpr int kDtS = MTF_DT_S;
-static_assert(kDtL % 64 == 0 && (kDtRW == 1 || kDtRW == 2 || kDtRW == 4), "unsupported dot-kernel tiling");
+static_assert(kDtS <= kDtCons && kDtL % 64 == 0 && (kDtRW == 1 || kDtRW == 2 || kDtRW == 4), "unsupported dot-kernel tiling");
 constexpr size_t kDtSmem = size_t(kDtS) * kDtSB + size_t(kDtS) * 2 * sizeof(uint64_t);
 static_assert(kDtSmem <= 232448, "stage ring above the per-CTA shared-memory limit");
 constexpr uint64_t kDtWaitNs = 500000000ull;
@@ -95,8 +95,6 @@ constexpr uint64_t kDtWaitNs = 500000000ull;
 __global__ void __launch_bounds__((kDtCons + 1) * 32, 1)
     k_dots_tma(const float* __restrict__ V, const float* __restrict__ w, int64_t ldn, int64_t ldv, int rows, int jq,
                double* __restrict__ t, double* __restrict__ sq, int hst, int nrhs, unsigned* __restrict__ err) {
-  MTF_PDL_WAIT();
-  MTF_PDL_TRIGGER();
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + size_t(kDtS) * kDtSB);
   uint64_t* empty = full + kDtS;
@@ -111,26 +109,54 @@ __global__ void __launch_bounds__((kDtCons + 1) * 32, 1)
     mbar_fence_init();
   }
   __syncthreads();
+  auto slice = [&](int u, int& c, int& i0, int64_t& k0) {
+    const int seg = u % nseg, rg = (u / nseg) % nrg;
+    c = u / (nseg * nrg);
+    i0 = rg * kDtR;
+    k0 = int64_t(seg) * kDtL;
+    return uint32_t(min(int64_t(kDtL), ldn - k0)) * 8u;
+  };
+  // the basis vectors of a unit, the stage's barrier armed for all of it
+  auto load_v = [&](int u, int st) {
+    int c, i0;
+    int64_t k0;
+    const uint32_t bytes = slice(u, c, i0, k0);
+    const int nr = min(kDtR, rows - i0);
+    mbar_arrive_expect_tx(&full[st], uint32_t(nr + 2) * bytes);
+    unsigned char* sb = smem + size_t(st) * kDtSB;
+    const float* Vc = V + 2 * (int64_t(c) * ldv + k0);
+    for (int r = 0; r < nr; ++r) bulk_g2s(sb + r * kDtSliceB, Vc + 2 * int64_t(i0 + r) * ldn, bytes, &full[st]);
+    bulk_g2s(sb + (kDtR + 1) * kDtSliceB, Vc + 2 * int64_t(jq) * ldn, bytes, &full[st]);
+  };
+  auto load_w = [&](int u, int st) {
+    int c, i0;
+    int64_t k0;
+    const uint32_t bytes = slice(u, c, i0, k0);
+    bulk_g2s(smem + size_t(st) * kDtSB + kDtR * kDtSliceB, w + 2 * (int64_t(c) * ldn + k0), bytes, &full[st]);
+  };
+  // the first units by one warp each; the basis is older than the kernel that
+  // makes w: its vectors are fetched before the wait for it
+  {
+    const int u = int(blockIdx.x) + warp * int(gridDim.x);
+    const bool first = lane == 0 && warp < kDtS && u < n_units;
+    if (first) load_v(u, warp);
+    MTF_PDL_WAIT();
+    MTF_PDL_TRIGGER();
+    if (first) load_w(u, warp);
+    __syncwarp();
+  }
   if (warp == kDtCons) {
-    // producer: one lane issues every copy
+    // producer of the other units: one lane issues every copy
     if (lane != 0) return;
-    int k = 0;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++k) {
-      const int seg = u % nseg, rg = (u / nseg) % nrg, c = u / (nseg * nrg);
+    int k = kDtS;
+    for (int u = int(blockIdx.x) + kDtS * int(gridDim.x); u < n_units; u += gridDim.x, ++k) {
       const int st = k % kDtS;
       if (!mbar_wait_bounded(&empty[st], (uint32_t(k / kDtS) & 1u) ^ 1u, kDtWaitNs)) {
         atomicExch(err, 1u);
         return;
       }
-      const int64_t k0 = int64_t(seg) * kDtL;
-      const uint32_t bytes = uint32_t(min(int64_t(kDtL), ldn - k0)) * 8u;
-      const int i0 = rg * kDtR, nr = min(kDtR, rows - i0);
-      mbar_arrive_expect_tx(&full[st], uint32_t(nr + 2) * bytes);
-      unsigned char* sb = smem + size_t(st) * kDtSB;
-      const float* Vc = V + 2 * (int64_t(c) * ldv + k0);
-      for (int r = 0; r < nr; ++r) bulk_g2s(sb + r * kDtSliceB, Vc + 2 * int64_t(i0 + r) * ldn, bytes, &full[st]);
-      bulk_g2s(sb + kDtR * kDtSliceB, w + 2 * (int64_t(c) * ldn + k0), bytes, &full[st]);
-      bulk_g2s(sb + (kDtR + 1) * kDtSliceB, Vc + 2 * int64_t(jq) * ldn, bytes, &full[st]);
+      load_v(u, st);
+      load_w(u, st);
     }
     return;
   }
@@ -217,8 +243,6 @@ __global__ void __launch_bounds__(256) k_axpy2_32(float* __restrict__ V, const d
                                                   const double* __restrict__ sq, double* __restrict__ coef,
                                                   int j, int j0, int nrhs, int64_t ldn, int64_t ldv,
                                                   float* __restrict__ w, double* __restrict__ ss) {
-  MTF_PDL_WAIT();
-  MTF_PDL_TRIGGER();
   const int c = blockIdx.y;
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int64_t q = int64_t(blockIdx.x) * 32 + lane;  // float4 index within a vector
@@ -228,8 +252,8 @@ __global__ void __launch_bounds__(256) k_axpy2_32(float* __restrict__ V, const d
   __shared__ float cf[3];
   extern __shared__ float2 hs[];  // t_i at hs[i], s_i at hs[j + i]
   const bool lead = blockIdx.x == 0;
-  // the first 8 basis columns of this group are loaded before the
-  // coefficients are formed, so that their latency overlaps the prologue
+  // the first 8 basis columns of this group (older than the reduction before
+  // this kernel) are loaded before the wait for the coefficients
   const int64_t ldq = ldn >> 1;
   float4* vb = reinterpret_cast<float4*>(V + 2 * int64_t(c) * ldv) + q;
   float4 pre[8];
@@ -238,6 +262,8 @@ __global__ void __launch_bounds__(256) k_axpy2_32(float* __restrict__ V, const d
     const int i = grp + 8 * u;
     pre[u] = (q < ldq && i < j) ? vb[int64_t(i) * ldq] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
   float s2 = 0.f, pr = 0.f, pi = 0.f;
   double s2d = 0, prd = 0, pid = 0;
   for (int u = threadIdx.x; u < j; u += blockDim.x) {

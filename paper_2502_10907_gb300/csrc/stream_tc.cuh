@@ -48,7 +48,7 @@ struct StreamTC {
   static constexpr int S0 = (kStSmemBudget - RED) / SB;
   static constexpr int S = S0 < kStMaxStages ? S0 : kStMaxStages;
   static constexpr size_t smem = size_t(S) * SB + RED + size_t(S) * (2 * sizeof(uint64_t) + sizeof(int4));
-  static_assert(S >= 2, "the stage ring needs at least two stages");
+  static_assert(S >= 2 && S <= 8, "the stage ring needs two stages, filled at first by as many consumer warps");
   static_assert(smem <= 232448, "shared memory above the per-CTA limit");
   static_assert(st_unit_rows<3>() == ROWS && st_consumers<3>() == 8, "units of 16 rows, 8 consumer warps");
 };
@@ -66,8 +66,6 @@ __global__ void __launch_bounds__(9 * 32, 1) k_stream_tc(const void* __restrict_
                                                         float* __restrict__ part, unsigned* __restrict__ err) {
   using TC = StreamTC<NC>;
   constexpr int S = TC::S, SB = TC::SB, RBP = TC::RBP, XB = TC::XB, ROWS = TC::ROWS, NT = TC::NT, K = TC::K;
-  MTF_PDL_WAIT();
-  MTF_PDL_TRIGGER();
   extern __shared__ __align__(128) unsigned char smem[];
   float* red = reinterpret_cast<float*>(smem + size_t(S) * SB);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + size_t(S) * SB + TC::RED);
@@ -83,13 +81,51 @@ __global__ void __launch_bounds__(9 * 32, 1) k_stream_tc(const void* __restrict_
   }
   __syncthreads();
 
+  const unsigned char* ent = static_cast<const unsigned char*>(tiled);
+  const uint64_t stream_pol = l2_policy_evict_first();
+  auto load_op = [&](const int4 rec, int64_t src, int s) {
+    const int N = rec.x, len = rec.w & 0xfff, nrows = (rec.w >> 24) & 0xff;
+    const uint32_t rows_bytes = uint32_t(nrows * st_tile_pitch(4, len));  // the unit's contiguous run
+    uint32_t total = rows_bytes;
+#pragma unroll
+    for (int q = 0; q < 2 * NC; ++q) {
+      const int64_t a = int64_t(c0 + (q >> 1)) * ld32 + rec.z + (q & 1) * N, xa = a & ~int64_t(1);
+      total += uint32_t((((a + len + 1) & ~int64_t(1)) - xa) * 8);
+    }
+    meta[s] = rec;
+    mbar_arrive_expect_tx(&full[s], total);
+    bulk_g2s_hint(smem + size_t(s) * SB, ent + src, rows_bytes, &full[s], stream_pol);
+  };
+  auto load_x = [&](const int4 rec, int s) {
+    const int N = rec.x, len = rec.w & 0xfff;
+    unsigned char* st = smem + size_t(s) * SB;
+#pragma unroll
+    for (int q = 0; q < 2 * NC; ++q) {
+      const int64_t a = int64_t(c0 + (q >> 1)) * ld32 + rec.z + (q & 1) * N, xa = a & ~int64_t(1);
+      bulk_g2s(st + ROWS * RBP + q * XB, x32 + 2 * xa, uint32_t((((a + len + 1) & ~int64_t(1)) - xa) * 8), &full[s]);
+    }
+  };
+  // the first S units by one warp each, the operator part before the wait for
+  // the input, as in k_stream_tiles
+  {
+    const int u = int(blockIdx.x) + warp * int(gridDim.x);
+    const bool first = lane == 0 && warp < S && u < n_units;
+    int4 rec;
+    if (first) {
+      rec = units[u];
+      load_op(rec, toff[u], warp);
+    }
+    MTF_PDL_WAIT();  // (part is read by the kernels before)
+    MTF_PDL_TRIGGER();
+    if (first) load_x(rec, warp);
+    __syncwarp();
+  }
+
   if (warp == 8) {
-    // producer: one lane issues every copy
+    // producer of the other units: one lane issues every copy
     if (lane != 0) return;
-    const unsigned char* ent = static_cast<const unsigned char*>(tiled);
-    const uint64_t stream_pol = l2_policy_evict_first();
-    int k = 0;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++k) {
+    int k = S;
+    for (int u = int(blockIdx.x) + S * int(gridDim.x); u < n_units; u += gridDim.x, ++k) {
       const int4 rec = units[u];
       const int64_t src = toff[u];
       const int s = k % S;
@@ -97,24 +133,8 @@ __global__ void __launch_bounds__(9 * 32, 1) k_stream_tc(const void* __restrict_
         atomicExch(err, 1u);
         return;
       }
-      const int N = rec.x, len = rec.w & 0xfff, nrows = (rec.w >> 24) & 0xff;
-      const uint32_t rows_bytes = uint32_t(nrows * st_tile_pitch(4, len));  // the unit's contiguous run
-      uint32_t total = rows_bytes;
-      int64_t xa[2 * NC];
-      uint32_t xbytes[2 * NC];
-#pragma unroll
-      for (int q = 0; q < 2 * NC; ++q) {
-        const int64_t a = int64_t(c0 + (q >> 1)) * ld32 + rec.z + (q & 1) * N;
-        xa[q] = a & ~int64_t(1);
-        xbytes[q] = uint32_t((((a + len + 1) & ~int64_t(1)) - xa[q]) * 8);
-        total += xbytes[q];
-      }
-      meta[s] = rec;
-      mbar_arrive_expect_tx(&full[s], total);
-      unsigned char* st = smem + size_t(s) * SB;
-      bulk_g2s_hint(st, ent + src, rows_bytes, &full[s], stream_pol);
-#pragma unroll
-      for (int q = 0; q < 2 * NC; ++q) bulk_g2s(st + ROWS * RBP + q * XB, x32 + 2 * xa[q], xbytes[q], &full[s]);
+      load_op(rec, src, s);
+      load_x(rec, s);
     }
     return;
   }

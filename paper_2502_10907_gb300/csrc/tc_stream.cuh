@@ -125,20 +125,35 @@ __global__ void __launch_bounds__(192, 1) k_tc_stream(const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  MTF_PDL_WAIT();  // the tables of units are static: read before
-  MTF_PDL_TRIGGER();
 
   if (warp == 0) {
     if (lane == 0) {
       tma_prefetch_map(&amap);
       tma_prefetch_map(&bmap);
       const uint64_t pol_a = l2_policy_evict_first(), pol_b = l2_policy_evict_last();
+      // the A tiles of the first S stages, before the wait for the kernel that
+      // packs B: under a programmatic launch A (an operator, or basis vectors
+      // stored in an earlier step) was written before that kernel began
+      int ahead = 0;
+      for (int q = q0; q < q1 && ahead < S; q += qs) {
+        const int4 U = units.get(listed ? sched[q] : q);
+        for (int kc = U.z; kc < U.w && ahead < S; ++kc, ++ahead) {
+          mbar_arrive_expect_tx(&full[ahead], uint32_t(SB));
+          tma_load_4d(smem + size_t(ahead) * SB, &amap, 0, 0, 0, U.x + kc, &full[ahead], pol_a);
+        }
+      }
+      MTF_PDL_WAIT();
+      MTF_PDL_TRIGGER();
       int k = 0;
       bool ok = true;
       for (int q = q0; q < q1 && ok; q += qs) {
         const int4 U = units.get(listed ? sched[q] : q);
         for (int kc = U.z; kc < U.w; ++kc, ++k) {
           const int st = k % S;
+          if (k < ahead) {
+            tma_load_4d(smem + size_t(st) * SB + SA, &bmap, 0, 0, 0, U.y + kc, &full[st], pol_b);
+            continue;
+          }
           if (!mbar_wait_bounded(&empty[st], (uint32_t(k / S) & 1u) ^ 1u, kTcsWaitNs)) {
             atomicExch(err, 1u);
             ok = false;
@@ -153,6 +168,8 @@ __global__ void __launch_bounds__(192, 1) k_tc_stream(const __grid_constant__ CU
     }
   } else if (warp == 1) {
     if (lane == 0) {
+      MTF_PDL_WAIT();
+      MTF_PDL_TRIGGER();
       constexpr uint32_t idesc = idesc_f16_m128(NB);
       int k = 0, ub = 0;
       bool ok = true;
@@ -189,6 +206,8 @@ __global__ void __launch_bounds__(192, 1) k_tc_stream(const __grid_constant__ CU
       }
     }
   } else {
+    MTF_PDL_WAIT();
+    MTF_PDL_TRIGGER();
     const int quarter = warp & 3;
     const int row = 32 * quarter + lane;
     int ub = 0;
