@@ -599,7 +599,9 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
 // consecutive dofs of the neighbour, so a warp's exchange reads and its stores
 // share sectors; with a lane per right-hand side each 8-byte exchange read was
 // a sector of its own.  Matvec of the 4 x 4 x 4 cube with 16 right-hand sides:
-// 255 -> 238 us.  (Block-OSRC's combine, which has no exchange, runs faster
+// 255 -> 238 us; 236 -> 231 us with the exchange rows read while the stream
+// before this kernel still runs.  (The same in the FMA stream's combine gave
+// nothing.)  (Block-OSRC's combine, which has no exchange, runs faster
 // with a lane per right-hand side: 85 against 88 us per apply.)
 template <int NB>
 __global__ void __launch_bounds__(256) k_mv_tc_combine(
@@ -608,8 +610,6 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
     const int* __restrict__ blk_pieces, const unsigned* __restrict__ amax, const float* __restrict__ colmax,
     const XEntry* __restrict__ xe, const float* __restrict__ xval32, const float* __restrict__ rho32,
     const float* __restrict__ x, int64_t ldx, float* __restrict__ y, int64_t ldy, int c0, int nc, int64_t n_rows) {
-  MTF_PDL_WAIT();
-  MTF_PDL_TRIGGER();
   const int64_t row = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
   if (row >= n_rows) return;
   const int i = row_blk[row];
@@ -628,7 +628,31 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
     xn[e] = X.col + (X.ab >> 4);
     xv[e] = xval32[6 * row + e];
   }
-  for (int c = threadIdx.x >> 5; c < nc; c += 8) {
+  // the exchange rows of this warp's columns, while the stream before this
+  // kernel still runs (x is older than it)
+  constexpr int CW = NB / 4 > 8 ? NB / 32 : 1;
+  const int w8 = threadIdx.x >> 5;
+  float4 ex[CW];
+#pragma unroll
+  for (int k = 0; k < CW; ++k) {
+    ex[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (w8 + 8 * k >= nc) break;
+    const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + w8 + 8 * k) * ldx);
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+      const float2 d = xc[xd[e]], n = xc[xn[e]];
+      ex[k].x = fmaf(xv[e], d.x, ex[k].x);
+      ex[k].y = fmaf(xv[e], d.y, ex[k].y);
+      ex[k].z = fmaf(xv[e], n.x, ex[k].z);
+      ex[k].w = fmaf(xv[e], n.y, ex[k].w);
+    }
+  }
+  MTF_PDL_WAIT();
+  MTF_PDL_TRIGGER();
+#pragma unroll
+  for (int k = 0; k < CW; ++k) {
+    const int c = w8 + 8 * k;
+    if (c >= nc) break;
     float2 a = make_float2(0.f, 0.f), b = a;  // y+, y-
     for (int p = 0; p < P; ++p) {
       const float2* q = reinterpret_cast<const float2*>(pr + size_t(p) * kTcRows * NB);
@@ -639,17 +663,8 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
       b.y += w.y;
     }
     const float sc = sca * tc_inv_scale(tc_pm_bound(colmax[32 * kCmParts + c], ir));
-    float yDr = (a.x + b.x) * sc, yDi = (a.y + b.y) * sc;
-    float yNr = rr * ((a.y - b.y) * sc), yNi = rr * ((b.x - a.x) * sc);
-    const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + c) * ldx);
-#pragma unroll
-    for (int e = 0; e < 6; ++e) {
-      const float2 d = xc[xd[e]], n = xc[xn[e]];
-      yDr = fmaf(xv[e], d.x, yDr);
-      yDi = fmaf(xv[e], d.y, yDi);
-      yNr = fmaf(xv[e], n.x, yNr);
-      yNi = fmaf(xv[e], n.y, yNi);
-    }
+    const float yDr = fmaf(a.x + b.x, sc, ex[k].x), yDi = fmaf(a.y + b.y, sc, ex[k].y);
+    const float yNr = fmaf(rr, (a.y - b.y) * sc, ex[k].z), yNi = fmaf(rr, (b.x - a.x) * sc, ex[k].w);
     float2* yc = reinterpret_cast<float2*>(y + 2 * (int64_t(c0 + c) * ldy + off));
     yc[m] = make_float2(yDr, yDi);
     yc[N + m] = make_float2(yNr, yNi);
