@@ -142,10 +142,11 @@ typedef struct {
                            (residual_df).  Default 0                         */
   double inner_tol_min; /* mixed mode: lower bound of the relative tolerance
                            given to an inner FP32 FGMRES cycle (the cycle's
-                           target is 0.3 tol / (current FP64 residual),
-                           clamped to [inner_tol_min, 0.5]); a smaller bound
-                           lets the first cycle run further before the FP64
-                           residual is taken, a larger one restarts sooner.
+                           target is 0.3 tol / (current FP64 residual), 0.15
+                           tol for a block cycle, clamped to
+                           [inner_tol_min, 0.5]); a smaller bound lets the
+                           first cycle run further before the FP64 residual
+                           is taken, a larger one restarts sooner.
                            0 selects the default 1e-5; otherwise in
                            [1e-9, 0.5]                                       */
   int32_t gs_dots_half; /* mixed mode, block_krylov with mv_tensor: 1: the
