@@ -47,6 +47,25 @@ FP64_PEAK_TFLOPS = 1.25                                # GB300 nominal dense FP6
 # FP32 operations per kernel evaluation of the regular-pair kernel's
 # moment-form inner loop (distance, G and grad G, the moment updates)
 FLOPS_PER_EVAL = 57
+# FP64 operations per hat point of the singular-pair kernel, by kind: at least
+# 136 (the distance and 8 Horner chains of 6 or more steps, shared by the n_ss
+# radial points) and 2 per moment sum
+FLOPS_PER_HAT = (160, 196, 204)
+
+
+def regular_flops(counts):
+    """Operations of one regular-pair launch: unordered pairs (counts[3] is of
+    ordered ones), 36 evaluations each."""
+    return counts[3] // 2 * 36 * FLOPS_PER_EVAL
+
+
+def singular_flops(counts, n_ss):
+    """(operations of one assembly's singular pairs, its launches): 6, 5 and 2
+    subdomains of n_ss^3 hat points per coincident, edge and vertex pair,
+    adjacent pairs once per unordered pair, one launch per kind."""
+    npts, per = (6, 5, 2), (1, 2, 2)
+    fl = sum(int(counts[c]) // per[c] * npts[c] * n_ss ** 3 * FLOPS_PER_HAT[c] for c in range(3))
+    return fl, sum(1 for c in range(3) if counts[c] > 0)
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from one ncu capture
@@ -408,13 +427,12 @@ def roofline_of(prof, counts, n_ss, hbm, src):
     per_launch_s = tms / max(1, nl) / 1e3
     if name in ("regular64", "regular32"):
         peak = FP64_PEAK_TFLOPS if name == "regular64" else FP32_PEAK_TFLOPS
-        ach = counts[3] * 36 * FLOPS_PER_EVAL / per_launch_s / 1e12
+        ach = regular_flops(counts) / per_launch_s / 1e12
         roof = {"kernel": name, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": None, "peak_source": "derived from unit counts and max SM clock"}
     elif name == "singular64":
-        npts, per = {0: 6, 1: 5, 2: 2}, {0: 1, 1: 2, 2: 2}
-        evals = sum(int(counts[c]) // per[c] * npts[c] * n_ss ** 4 for c in range(3))
-        ach = evals * 75 / per_launch_s / 1e12
+        fl, kinds = singular_flops(counts, n_ss)
+        ach = fl / (per_launch_s * kinds) / 1e12
         roof = {"kernel": name, "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": ach / FP64_PEAK_TFLOPS, "traffic": None, "peak_source": "derived (FP64 1.25 TF/s)"}
     else:
@@ -757,11 +775,10 @@ def main():
             continue
         per = tms / nl / 1e3
         if name.startswith("regular"):
-            fl, pk = counts[3] * 36 * FLOPS_PER_EVAL, peaks[0 if name == "regular32" else 1]
+            fl, pk = regular_flops(counts), peaks[0 if name == "regular32" else 1]
         else:
-            npts, per_pair = {0: 6, 1: 5, 2: 2}, {0: 1, 1: 2, 2: 2}
-            fl = sum(int(counts[c]) // per_pair[c] * npts[c] * sysg.opt.n_ss ** 4 for c in range(3)) * 75
-            pk = peaks[1]
+            fl, kinds = singular_flops(counts, sysg.opt.n_ss)
+            pk, per = peaks[1], per * kinds
         asm_roof.append({"kernel": name, "bound": "alu", "achieved": fl / per / 1e12, "peak": pk / 1e12,
                          "unit": "TFLOP/s", "frac": fl / per / pk, "ms_per_launch": per * 1e3,
                          "peak_source": "measured (mtf_probe_peaks: FP32 / FP64 FMA chains)"})
