@@ -12,21 +12,29 @@
 //    loads the 64 KB operator tile (4 parts) and the input chunk (hi, lo)
 //    with two cp.async.bulk.tensor.4d copies (128-byte swizzle) into a ring
 //    of S stages, completing on the stage's "full" mbarrier;
-//  - warp 1: allocates TMEM (two accumulator buffers of NB columns: NB / 2
-//    of A+ u+, NB / 2 of A- u-); one lane issues per K = 16 step the six
-//    tcgen05.mma of the split products and commits each stage back to its
-//    "empty" barrier, and each finished unit to the buffer's "full" barrier;
+//  - warp 1: allocates TMEM (two accumulator buffers of 2 NB columns); one
+//    lane issues per K = 16 step the six tcgen05.mma of the split products
+//    and commits each stage back to its "empty" barrier, and each finished
+//    unit to the buffer's "full" barrier;
 //  - warps 2-5: epilogue.  Each reads its 32 TMEM lanes (rows) of the
-//    finished buffer with tcgen05.ld and writes the unit's raw row sums to a
-//    partial buffer, then frees the TMEM buffer.
-// The two traces are taken together (apply.cu): with w = u_N / rho_i,
-// u+- = u_D +- i w and A+- = K -+ i T,  A+- u+- = y+-,  y_D = y+ + y-,
-// y_N = -i rho_i (y+ - y-): half the products, accumulators and row sums of
-// T u_D, T u_N, K u_D, K u_N from the same operator bytes.
+//    finished buffer with tcgen05.ld, adds the hi x lo sums to the hi x hi
+//    ones and writes the unit's raw row sums to a partial buffer, then frees
+//    the TMEM buffer.
+// The four products of a row meet in NB columns: with w = u_N / rho_i,
+//   y_D = 2 (K u_D + T w),   y_N = 2 rho_i (K w - T u_D),
+// K against the input columns [u_D | w] and T against [w | -u_D]: half the
+// accumulators and row sums of four separate products.  T and K keep
+// their own FP16 hi + lo parts: |T| exceeds |K| by about 1 / (k h), and a
+// combination such as K -+ i T, which would need half the products, keeps K
+// to 2^-22 of |T| only (error of the D rows for u_N = 0 at k = 0.1: 4.6e-5
+// instead of 8e-8).  Every addition to an accumulator is truncated to FP32, so
+// the small hi x lo products have columns of their own: two additions per
+// step reach the large sums (with six the error against FP64 on the 4 x 4 x 4
+// cube is 6.4e-6, so 2.5e-6).
 // k_mv_tc_combine then adds the pieces of each row in order, undoes the
 // scalings, forms y_D and y_N and adds the exchange rows.  Bound: HBM (the
 // operator tiles); on the 4 x 4 x 4 cube (72,000 unknowns, 16 right-hand
-// sides) an apply took 275 us with four products per entry, 238 us with two.
+// sides) an apply took 275 us with four products apart, 231 us so.
 // Every wait is bounded (0.5 s) and ends in the error word.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -115,8 +123,7 @@ __device__ __forceinline__ void tc_split(float v, __half& hi, __half& lo) {
   lo = __float2half_rn(v - __half2float(hi));
 }
 
-// Tiled hi / lo copy of A+ = K - i T and A- = K + i T (|A+-| <= 2 amax, inside
-// the FP16 range after the scaling): thread = (tile, row, group g of 4 complex
+// Tiled hi / lo copy of T and K: thread = (tile, row, group g of 4 complex
 // columns); writes 8 halves (16 bytes) into each of the 4 parts.
 __global__ void __launch_bounds__(256) k_tc_tile_a(const float4* __restrict__ TK, const int4* __restrict__ tile_info,
                                                    const int64_t* __restrict__ blk_mat_off,
@@ -136,10 +143,10 @@ __global__ void __launch_bounds__(256) k_tc_tile_a(const float4* __restrict__ TK
     const int n = info.z * kTcCols + 4 * g + q;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r < N && n < N) v = TK[blk_mat_off[i] + int64_t(r) * N + n];
-    tc_split((v.z + v.y) * s, h[0][2 * q], h[1][2 * q]);          // A+ re
-    tc_split((v.w - v.x) * s, h[0][2 * q + 1], h[1][2 * q + 1]);  // A+ im
-    tc_split((v.z - v.y) * s, h[2][2 * q], h[3][2 * q]);          // A- re
-    tc_split((v.w + v.x) * s, h[2][2 * q + 1], h[3][2 * q + 1]);  // A- im
+    tc_split(v.x * s, h[0][2 * q], h[1][2 * q]);          // T re
+    tc_split(v.y * s, h[0][2 * q + 1], h[1][2 * q + 1]);  // T im
+    tc_split(v.z * s, h[2][2 * q], h[3][2 * q]);          // K re
+    tc_split(v.w * s, h[2][2 * q + 1], h[3][2 * q + 1]);  // K im
   }
 #pragma unroll
   for (int p = 0; p < 4; ++p)
@@ -363,13 +370,16 @@ __global__ void __launch_bounds__(256) k_tc_build_b(const float* __restrict__ x,
   *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(lo);
 }
 
-// scale of u+- in block i: |u+-| <= (1 + 1 / rho_i) max |u|
-__device__ __forceinline__ unsigned tc_pm_bound(float cm, float irho) { return __float_as_uint(cm * (1.f + fabsf(irho))); }
+// what u_D and w = u_N / rho_i of block i are scaled by: their bound
+__device__ __forceinline__ unsigned tc_dw_bound(float cm, float irho) { return __float_as_uint(cm * fmaxf(1.f, fabsf(irho))); }
 
-// Matvec input chunks: thread = (chunk, column col, group g of 4 complex
-// entries); column h NB / 2 + 2 c + f holds form f of u+ (h = 0) or u- (h = 1)
-// of right-hand side c0 + c
-__global__ void __launch_bounds__(256) k_tc_build_pm(const float* __restrict__ x, int64_t ldx, int c0, int nc, int nb,
+// columns of a matvec input chunk: u_D, w = u_N / rho and -u_D, NB / 2 each
+__host__ __device__ constexpr int tc_dw_columns(int nb) { return nb / 2 * 3; }
+
+// Matvec input chunks: thread = (chunk, column col < NB, group g of 4 complex
+// entries); column h NB / 2 + 2 c + f holds form f of u_D (h = 0), w (h = 1) or
+// -u_D (h = 2) of right-hand side c0 + c
+__global__ void __launch_bounds__(256) k_tc_build_dw(const float* __restrict__ x, int64_t ldx, int c0, int nc, int nb,
                                                      const int2* __restrict__ chunk_info, int64_t n_chunks,
                                                      const int32_t* __restrict__ blk_N,
                                                      const int64_t* __restrict__ blk_dof_off,
@@ -383,7 +393,7 @@ __global__ void __launch_bounds__(256) k_tc_build_pm(const float* __restrict__ x
   if (t >= n_chunks * nb * 8) return;
   const int64_t chunk = t / (int64_t(nb) * 8);
   const int col = int((t / 8) % nb), g = int(t % 8);
-  const bool minus = col >= nb / 2;
+  const bool slot_n = col >= nb / 2;
   const int c = (col % (nb / 2)) >> 1, form = col & 1;
   __half hi[8], lo[8];
 #pragma unroll
@@ -391,36 +401,44 @@ __global__ void __launch_bounds__(256) k_tc_build_pm(const float* __restrict__ x
   if (c < nc) {
     const int2 info = chunk_info[chunk];
     const int N = blk_N[info.x];
-    const float ir = rho32[4 * info.x + 2], ii = minus ? -ir : ir;  // rho is real
-    const float s = tc_scale(tc_pm_bound(cm[c], ir));
-    const float2* xc = reinterpret_cast<const float2*>(x + 2 * (int64_t(c0 + c) * ldx + blk_dof_off[info.x]));
+    const float ir = rho32[4 * info.x + 2], f = slot_n ? ir : 1.f;  // rho is real
+    const float s = tc_scale(tc_dw_bound(cm[c], ir));
+    const float2* xc = reinterpret_cast<const float2*>(x + 2 * (int64_t(c0 + c) * ldx + blk_dof_off[info.x] +
+                                                                 (slot_n ? int64_t(N) : 0)));
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int n = info.y * kTcCols + 4 * g + q;
-      float2 d = make_float2(0.f, 0.f), w = d;
-      if (n < N) {
-        d = xc[n];
-        w = xc[N + n];
-      }
-      const float2 v = make_float2(fmaf(-ii, w.y, d.x), fmaf(ii, w.x, d.y));  // u_D +- i u_N / rho
+      float2 v = make_float2(0.f, 0.f);
+      if (n < N) v = xc[n];
+      v = make_float2(v.x * f, v.y * f);
       const float a = form == 0 ? v.x : v.y, b = form == 0 ? -v.y : v.x;
       tc_split(a * s, hi[2 * q], lo[2 * q]);
       tc_split(b * s, hi[2 * q + 1], lo[2 * q + 1]);
     }
   }
-  *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 0, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(hi);
-  *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, col, 8 * g, nb)) = *reinterpret_cast<const uint4*>(lo);
+  const int cols = tc_dw_columns(nb);
+  const uint4 h = *reinterpret_cast<const uint4*>(hi), l = *reinterpret_cast<const uint4*>(lo);
+  *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 0, col, 8 * g, cols)) = h;
+  *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, col, 8 * g, cols)) = l;
+  if (!slot_n) {
+    constexpr unsigned sign = 0x80008000u;
+    *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 0, nb + col, 8 * g, cols)) =
+        make_uint4(h.x ^ sign, h.y ^ sign, h.z ^ sign, h.w ^ sign);
+    *reinterpret_cast<uint4*>(B + tc_b_index(chunk, 1, nb + col, 8 * g, cols)) =
+        make_uint4(l.x ^ sign, l.y ^ sign, l.z ^ sign, l.w ^ sign);
+  }
 }
 
 template <int NB>
 struct TcCfg {
   static constexpr int SA = kTcParts * kTcRows * 128;      // operator tile bytes (64 KB)
-  static constexpr int SBB = 2 * NB * 128;                  // input chunk bytes (hi + lo)
+  static constexpr int NC = tc_dw_columns(NB);              // input columns
+  static constexpr int SBB = 2 * NC * 128;                  // input chunk bytes (hi + lo)
   static constexpr int SB = SA + SBB;                       // stage bytes (a multiple of 1024)
-  static constexpr int S0 = (220 * 1024) / SB;
+  static constexpr int S0 = (232448 - 1280) / SB;
   static constexpr int S = S0 > 4 ? 4 : S0;
-  static constexpr uint32_t TMEM = 2 * NB;  // two buffers of NB columns
-  static_assert(NB >= 32, "A+ u+ and A- u- need 16 columns each");
+  static constexpr uint32_t TMEM = 4 * NB;  // two buffers of NB columns, hi x hi and hi x lo products
+  static_assert(NB >= 32, "the D and N rows need 16 columns each");
   static constexpr size_t smem = size_t(S) * SB + 1024 + 256;
   static_assert(S >= 2, "the stage ring needs two stages");
   static_assert(smem <= 232448, "shared memory above the per-CTA limit");
@@ -512,7 +530,7 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
     if (lane == 0) {
       MTF_PDL_WAIT();
       MTF_PDL_TRIGGER();
-      constexpr uint32_t idesc = idesc_f16_m128(NB / 2);
+      constexpr uint32_t idesc = idesc_f16_m128(NB);
       int k = 0, ub = 0;
       bool ok = true;
       for (int q = q_begin; q < q_end && ok; ++q, ++ub) {
@@ -523,7 +541,7 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
           break;
         }
         tc_fence_after();
-        const uint32_t dp = tmem + uint32_t(buf * NB), dm = dp + uint32_t(NB / 2);
+        const uint32_t y = tmem + uint32_t(buf * 2 * NB), yl = y + uint32_t(NB);  // hi x hi, hi x lo
         for (int kc = U.z; kc < U.w; ++kc, ++k) {
           const int st = k % S;
           if (!mbar_wait_bounded(&full[st], uint32_t(k / S) & 1u, kTcWaitNs)) {
@@ -535,18 +553,18 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
           const uint32_t sa = smem_u32(smem + size_t(st) * SB), sb = sa + SA;
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t ph = sw128_desc(sa + kk * 32), pl = sw128_desc(sa + 16384 + kk * 32);
-            const uint64_t mh = sw128_desc(sa + 32768 + kk * 32), ml = sw128_desc(sa + 49152 + kk * 32);
-            const uint32_t sm = sb + NB / 2 * 128;  // the columns of u-
-            const uint64_t uh = sw128_desc(sb + kk * 32), ul = sw128_desc(sb + NB * 128 + kk * 32);
-            const uint64_t vh = sw128_desc(sm + kk * 32), vl = sw128_desc(sm + NB * 128 + kk * 32);
+            const uint64_t th = sw128_desc(sa + kk * 32), tl = sw128_desc(sa + 16384 + kk * 32);
+            const uint64_t kh = sw128_desc(sa + 32768 + kk * 32), kl = sw128_desc(sa + 49152 + kk * 32);
+            const uint32_t sw = sb + NB / 2 * 128;  // columns [w | -u_D]
+            const uint64_t uh = sw128_desc(sb + kk * 32), ul = sw128_desc(sb + C::NC * 128 + kk * 32);
+            const uint64_t wh = sw128_desc(sw + kk * 32), wl = sw128_desc(sw + C::NC * 128 + kk * 32);
             const uint32_t acc = (kc != U.z || kk != 0) ? 1u : 0u;
-            tc_mma_f16(dp, ph, uh, idesc, acc);
-            tc_mma_f16(dp, ph, ul, idesc, 1u);
-            tc_mma_f16(dp, pl, uh, idesc, 1u);
-            tc_mma_f16(dm, mh, vh, idesc, acc);
-            tc_mma_f16(dm, mh, vl, idesc, 1u);
-            tc_mma_f16(dm, ml, vh, idesc, 1u);
+            tc_mma_f16(y, kh, uh, idesc, acc);  // K [u_D | w] + T [w | -u_D]
+            tc_mma_f16(y, th, wh, idesc, 1u);
+            tc_mma_f16(yl, kh, ul, idesc, acc);
+            tc_mma_f16(yl, kl, uh, idesc, 1u);
+            tc_mma_f16(yl, th, wl, idesc, 1u);
+            tc_mma_f16(yl, tl, wh, idesc, 1u);
           }
           tc_commit(&empty[st]);  // the stage is free once these MMAs have read it
         }
@@ -567,12 +585,15 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
         break;
       }
       tc_fence_after();
-      const uint32_t ta = tmem + (uint32_t(32 * quarter) << 16) + uint32_t(buf * NB);
+      const uint32_t ta = tmem + (uint32_t(32 * quarter) << 16) + uint32_t(buf * 2 * NB);
       float* dst = part + (size_t(sched[q]) * kTcRows + row) * NB;
 #pragma unroll
       for (int c0 = 0; c0 < NB; c0 += 16) {
-        float v[16];
+        float v[16], l[16];
         tmem_ld16(ta + uint32_t(c0), v);
+        tmem_ld16(ta + uint32_t(NB + c0), l);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] += l[e];
         float4* d4 = reinterpret_cast<float4*>(dst + c0);
         d4[0] = make_float4(v[0], v[1], v[2], v[3]);
         d4[1] = make_float4(v[4], v[5], v[6], v[7]);
@@ -592,8 +613,8 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
   }
 }
 
-// y rows: the row's unit pieces summed in order, unscaled, y_D and y_N from
-// y+ and y-, and the exchange rows (FP32), as in the FMA stream's combine.  A
+// y rows: the row's unit pieces summed in order, unscaled, as y_D and y_N
+// with the exchange rows (FP32), as in the FMA stream's combine.  A
 // CTA takes 32 consecutive rows, lane = row, warps over the pass's right-hand
 // sides (8 at a time): consecutive rows of an interface meet nearly
 // consecutive dofs of the neighbour, so a warp's exchange reads and its stores
@@ -653,7 +674,7 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
   for (int k = 0; k < CW; ++k) {
     const int c = w8 + 8 * k;
     if (c >= nc) break;
-    float2 a = make_float2(0.f, 0.f), b = a;  // y+, y-
+    float2 a = make_float2(0.f, 0.f), b = a;  // K u_D + T w, K w - T u_D
     for (int p = 0; p < P; ++p) {
       const float2* q = reinterpret_cast<const float2*>(pr + size_t(p) * kTcRows * NB);
       const float2 v = q[c], w = q[NB / 4 + c];
@@ -662,9 +683,9 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
       b.x += w.x;
       b.y += w.y;
     }
-    const float sc = sca * tc_inv_scale(tc_pm_bound(colmax[32 * kCmParts + c], ir));
-    const float yDr = fmaf(a.x + b.x, sc, ex[k].x), yDi = fmaf(a.y + b.y, sc, ex[k].y);
-    const float yNr = fmaf(rr, (a.y - b.y) * sc, ex[k].z), yNi = fmaf(rr, (b.x - a.x) * sc, ex[k].w);
+    const float sc = 2.f * sca * tc_inv_scale(tc_dw_bound(colmax[32 * kCmParts + c], ir));
+    const float yDr = fmaf(a.x, sc, ex[k].x), yDi = fmaf(a.y, sc, ex[k].y);
+    const float yNr = fmaf(rr, b.x * sc, ex[k].z), yNi = fmaf(rr, b.y * sc, ex[k].w);
     float2* yc = reinterpret_cast<float2*>(y + 2 * (int64_t(c0 + c) * ldy + off));
     yc[m] = make_float2(yDr, yDi);
     yc[N + m] = make_float2(yNr, yNi);
@@ -867,22 +888,23 @@ void tc_build_operator(mtf_system sys, cudaStream_t s) {
 }
 
 // input chunks (hi, lo) of columns c0 .. c0 + nc - 1 of x in t.B (the matvec's
-// u+, u-, or block-OSRC's u_D, u_N), the column maxima in t.colmax, and the B
-// tensor map for width NB
-template <int NB, bool PM>
+// [u_D | w | -u_D], or block-OSRC's u_D, u_N), the column maxima in t.colmax,
+// and the B tensor map
+template <int NB, bool MV>
 static void tc_build_inputs(mtf_system sys, TcMatvec& t, const float* x, int64_t ldx, int c0, int nc, int kid,
                             cudaStream_t s) {
   mtf_mesh m = sys->mesh;
   const TcPlan& p = t.plan;
-  const size_t bh = size_t(p.n_chunks) * 2 * NB * 64;
+  constexpr int cols = MV ? tc_dw_columns(NB) : NB;
+  const size_t bh = size_t(p.n_chunks) * 2 * cols * 64;
   if (t.B.n < bh) {
-    t.B.alloc(size_t(p.n_chunks) * 2 * 128 * 64);  // room for the widest pass
+    t.B.alloc(size_t(p.n_chunks) * 2 * tc_dw_columns(128) * 64);  // room for the widest pass
     t.bmap_ptr = nullptr;
   }
-  if (t.bmap_ptr != t.B.p || t.bmap_nb != NB) {
-    tc_encode_map(&t.bmap, t.B.p, NB, 2, p.n_chunks);
+  if (t.bmap_ptr != t.B.p || t.bmap_nb != cols) {
+    tc_encode_map(&t.bmap, t.B.p, cols, 2, p.n_chunks);
     t.bmap_ptr = t.B.p;
-    t.bmap_nb = NB;
+    t.bmap_nb = cols;
   }
   const size_t np = p.units.size() * kTcRows * NB;
   if (t.part.n < np) t.part.alloc(size_t(p.units.size()) * kTcRows * 128);
@@ -890,8 +912,8 @@ static void tc_build_inputs(mtf_system sys, TcMatvec& t, const float* x, int64_t
                                 t.colmax.p));
   const int64_t nthr = p.n_chunks * NB * 8;
   const dim3 grid(unsigned((nthr + 255) / 256));
-  if constexpr (PM)
-    MTF_LAUNCH(kid, s, launch_pdl(k_tc_build_pm, grid, dim3(256), 0, s, x, ldx, c0, nc, NB, t.chunk_info.p, p.n_chunks,
+  if constexpr (MV)
+    MTF_LAUNCH(kid, s, launch_pdl(k_tc_build_dw, grid, dim3(256), 0, s, x, ldx, c0, nc, NB, t.chunk_info.p, p.n_chunks,
                                   m->d_blk_N.p, m->d_blk_dof_off.p, sys->d_rho32.p, t.colmax.p, t.B.p));
   else
     MTF_LAUNCH(kid, s, launch_pdl(k_tc_build_b, grid, dim3(256), 0, s, x, ldx, c0, nc, NB, t.chunk_info.p, p.n_chunks,

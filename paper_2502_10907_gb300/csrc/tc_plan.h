@@ -2,23 +2,23 @@
 // can be tested on its own.
 //
 // Formulation.  For block i with dense complex operators (N_i x N_i; the
-// matvec's A+- = K_i -+ i T_i against u+- = u_D +- i u_N / rho_i, block-OSRC's
-// T~_i against u_D, u_N) every product is one real matrix product: a row of
-// an operator stored as interleaved (re, im)
+// matvec's T_i and K_i against u_D and w = u_N / rho_i, block-OSRC's T~_i
+// against u_D, u_N) every product is one real matrix product: a row of an
+// operator stored as interleaved (re, im)
 // pairs is a real row of length 2 N_i, and a complex input v becomes two real
 // columns of the same length,
 //   form 0: (v_re, -v_im) per entry -> Re(A v),   form 1: (v_im, v_re) -> Im(A v).
 // The B operand has NB = 4 nc columns rounded up to 16, 32, 64 or 128 (up to
 // 32 right-hand sides per pass).  Matvec: column 2 c + f of its first half
-// holds form f of u+ of right-hand side c, of its second half of u-
-// (multiplied with A+ and A-).  Block-OSRC: column 4 c + 2 t + f holds form f
+// holds form f of u_D of right-hand side c, of its second half of w.
+// Block-OSRC: column 4 c + 2 t + f holds form f
 // of u_t (t = 0: D slot, t = 1: N slot).  Both operands are FP16 after a power-of-two scaling (per block
 // for the operators, per right-hand side and block for the inputs) and are split into an FP16
 // value and the FP16 rounding of its remainder (hi + lo, about 22 significant
 // bits); a product is hi*hi + hi*lo + lo*hi with FP32 accumulation.
 //
 // Layout.  A tile is (block i, row tile mt of 128 rows, chunk kc of 32
-// complex columns = 64 FP16 per row): four parts A+ hi, A+ lo, A- hi, A- lo of
+// complex columns = 64 FP16 per row): four parts T hi, T lo, K hi, K lo of
 // 128 rows x 64 FP16 (128 bytes per row), 64 KB, tiles of a block in
 // (mt, kc) order.  An input chunk is (block i, kc): two parts (hi, lo) of NB
 // columns x 64 FP16.  Rows and columns past N_i are zero.  A work unit is
@@ -38,7 +38,7 @@ namespace mtf {
 
 constexpr int kTcRows = 128;  // rows per tile (M of the MMA)
 constexpr int kTcCols = 32;   // complex columns per chunk (64 FP16, 128 bytes)
-constexpr int kTcParts = 4;   // A+ hi, A+ lo, A- hi, A- lo
+constexpr int kTcParts = 4;   // T hi, T lo, K hi, K lo
 constexpr int64_t kTcPartHalves = int64_t(kTcRows) * 64;
 constexpr int64_t kTcTileHalves = kTcParts * kTcPartHalves;
 
@@ -51,7 +51,7 @@ inline int tc_nb(int nc) { return nc <= 4 ? 16 : nc <= 8 ? 32 : nc <= 16 ? 64 : 
 constexpr int64_t tc_tile_index(int64_t tile, int parts, int part, int row, int e) {
   return ((tile * parts + part) * kTcRows + row) * 64 + e;
 }
-// the matvec's operator tiles (4 parts: A+ hi, A+ lo, A- hi, A- lo)
+// the matvec's operator tiles (4 parts: T hi, T lo, K hi, K lo)
 constexpr int64_t tc_a_index(int64_t tile, int part, int row, int e) {
   return tc_tile_index(tile, kTcParts, part, row, e);
 }
