@@ -614,25 +614,31 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
 }
 
 // y rows: the row's unit pieces summed in order, unscaled, as y_D and y_N
-// with the exchange rows (FP32), as in the FMA stream's combine.  A
-// CTA takes 32 consecutive rows, lane = row, warps over the pass's right-hand
-// sides (8 at a time): consecutive rows of an interface meet nearly
-// consecutive dofs of the neighbour, so a warp's exchange reads and its stores
-// share sectors; with a lane per right-hand side each 8-byte exchange read was
-// a sector of its own.  Matvec of the 4 x 4 x 4 cube with 16 right-hand sides:
-// 255 -> 238 us; 236 -> 231 us with the exchange rows read while the stream
-// before this kernel still runs.  (The same in the FMA stream's combine gave
-// nothing.)  (Block-OSRC's combine, which has no exchange, runs faster
-// with a lane per right-hand side: 85 against 88 us per apply.)
+// with the exchange rows (FP32), as in the FMA stream's combine.  Lane = row,
+// warp = 4 right-hand sides of a CTA's 32 consecutive rows: consecutive rows of an
+// interface meet nearly consecutive dofs of the neighbour, so a warp's
+// exchange reads and its stores share sectors, and the 4 right-hand sides of a
+// row's sums are one 32-byte sector.  The exchange rows are read while the
+// stream before this kernel still runs; a CTA that starts then has only the
+// L1 that the stream's stage ring leaves, so nothing here counts on L1: with
+// one right-hand side per lane, whose sector four warps shared, 16 right-hand
+// sides on the split sphere of 11 rings took 125 us and on the 4 x 4 x 4 cube
+// 231, now 90 and 222.  Beside the 32-right-hand-side ring only one CTA per SM
+// finds room before the stream ends, and those that follow it keep the small
+// L1: that width is launched after the stream (split sphere 162 -> 122 us,
+// 190 us with one right-hand side per lane; cube 279 -> 270).
+// (Block-OSRC's combine, which has no exchange, runs faster with a lane per
+// right-hand side: 85 against 88 us per apply.)
 template <int NB>
-__global__ void __launch_bounds__(256) k_mv_tc_combine(
+__global__ void __launch_bounds__(2 * NB) k_mv_tc_combine(
     const float* __restrict__ part, const int32_t* __restrict__ row_blk, const int32_t* __restrict__ blk_N,
     const int64_t* __restrict__ blk_dof_off, const int64_t* __restrict__ blk_row_off, const int* __restrict__ blk_unit_base,
     const int* __restrict__ blk_pieces, const unsigned* __restrict__ amax, const float* __restrict__ colmax,
     const XEntry* __restrict__ xe, const float* __restrict__ xval32, const float* __restrict__ rho32,
     const float* __restrict__ x, int64_t ldx, float* __restrict__ y, int64_t ldy, int c0, int nc, int64_t n_rows) {
+  const int cq = 4 * (threadIdx.x >> 5);
   const int64_t row = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
-  if (row >= n_rows) return;
+  if (row >= n_rows || cq >= nc) return;
   const int i = row_blk[row];
   const int N = blk_N[i];
   const int64_t m = row - blk_row_off[i], off = blk_dof_off[i];
@@ -649,16 +655,14 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
     xn[e] = X.col + (X.ab >> 4);
     xv[e] = xval32[6 * row + e];
   }
-  // the exchange rows of this warp's columns, while the stream before this
-  // kernel still runs (x is older than it)
-  constexpr int CW = NB / 4 > 8 ? NB / 32 : 1;
-  const int w8 = threadIdx.x >> 5;
-  float4 ex[CW];
+  // the exchange rows of the warp's columns, before the wait for the stream
+  // (x is older than the kernel that packed the stream's inputs)
+  float4 ex[4];
 #pragma unroll
-  for (int k = 0; k < CW; ++k) {
+  for (int k = 0; k < 4; ++k) {
     ex[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (w8 + 8 * k >= nc) break;
-    const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + w8 + 8 * k) * ldx);
+    if (cq + k >= nc) continue;
+    const float2* xc = reinterpret_cast<const float2*>(x + 2 * int64_t(c0 + cq + k) * ldx);
 #pragma unroll
     for (int e = 0; e < 6; ++e) {
       const float2 d = xc[xd[e]], n = xc[xn[e]];
@@ -670,25 +674,33 @@ __global__ void __launch_bounds__(256) k_mv_tc_combine(
   }
   MTF_PDL_WAIT();
   MTF_PDL_TRIGGER();
+  float d[8], n[8];  // K u_D + T w, K w - T u_D (re, im of 4 right-hand sides)
 #pragma unroll
-  for (int k = 0; k < CW; ++k) {
-    const int c = w8 + 8 * k;
-    if (c >= nc) break;
-    float2 a = make_float2(0.f, 0.f), b = a;  // K u_D + T w, K w - T u_D
-    for (int p = 0; p < P; ++p) {
-      const float2* q = reinterpret_cast<const float2*>(pr + size_t(p) * kTcRows * NB);
-      const float2 v = q[c], w = q[NB / 4 + c];
-      a.x += v.x;
-      a.y += v.y;
-      b.x += w.x;
-      b.y += w.y;
+  for (int q = 0; q < 8; ++q) d[q] = n[q] = 0.f;
+#pragma unroll 2
+  for (int p = 0; p < P; ++p) {
+    const float4* q = reinterpret_cast<const float4*>(pr + size_t(p) * kTcRows * NB + 2 * cq);
+    const float4 v[4] = {q[0], q[1], q[NB / 8], q[NB / 8 + 1]};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      d[4 * k] += v[k].x;
+      d[4 * k + 1] += v[k].y;
+      d[4 * k + 2] += v[k].z;
+      d[4 * k + 3] += v[k].w;
+      n[4 * k] += v[2 + k].x;
+      n[4 * k + 1] += v[2 + k].y;
+      n[4 * k + 2] += v[2 + k].z;
+      n[4 * k + 3] += v[2 + k].w;
     }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int c = cq + k;
+    if (c >= nc) break;
     const float sc = 2.f * sca * tc_inv_scale(tc_dw_bound(colmax[32 * kCmParts + c], ir));
-    const float yDr = fmaf(a.x, sc, ex[k].x), yDi = fmaf(a.y, sc, ex[k].y);
-    const float yNr = fmaf(rr, b.x * sc, ex[k].z), yNi = fmaf(rr, b.y * sc, ex[k].w);
     float2* yc = reinterpret_cast<float2*>(y + 2 * (int64_t(c0 + c) * ldy + off));
-    yc[m] = make_float2(yDr, yDi);
-    yc[N + m] = make_float2(yNr, yNi);
+    yc[m] = make_float2(fmaf(d[2 * k], sc, ex[k].x), fmaf(d[2 * k + 1], sc, ex[k].y));
+    yc[N + m] = make_float2(fmaf(rr, n[2 * k] * sc, ex[k].z), fmaf(rr, n[2 * k + 1] * sc, ex[k].w));
   }
 }
 
@@ -942,10 +954,17 @@ static void mv_tc_pass(mtf_system sys, TcMatvec& t, const float* x, int64_t ldx,
       t.amap, t.bmap, t.units.p, t.sched.p, t.sched_off.p, t.blk_tile_base.p, t.blk_nkc.p, t.blk_chunk_base.p,
       t.part.p, sys->d_mv_ctl.p + 2));
   const unsigned gc = unsigned((m->n_rows + 31) / 32);
-  MTF_LAUNCH(KID_MVTC_COMBINE, s, launch_pdl(k_mv_tc_combine<NB>, dim3(gc), dim3(256), 0, s,
-      t.part.p, m->d_row_blk.p, m->d_blk_N.p, m->d_blk_dof_off.p, m->d_blk_row_off.p, t.blk_unit_base.p,
-      t.blk_pieces.p, t.amax.p, t.colmax.p, m->d_xent.p, sys->d_xval32.p, sys->d_rho32.p, x, ldx, y, ldy, c0, nc,
-      m->n_rows));
+  // (why the widest one is an ordinary launch: k_mv_tc_combine)
+  const auto combine = [&](auto launch) {
+    MTF_LAUNCH(KID_MVTC_COMBINE, s, launch(
+        t.part.p, m->d_row_blk.p, m->d_blk_N.p, m->d_blk_dof_off.p, m->d_blk_row_off.p, t.blk_unit_base.p,
+        t.blk_pieces.p, t.amax.p, t.colmax.p, m->d_xent.p, sys->d_xval32.p, sys->d_rho32.p, x, ldx, y, ldy, c0, nc,
+        m->n_rows));
+  };
+  if constexpr (NB < 128)
+    combine([&](auto... a) { launch_pdl(k_mv_tc_combine<NB>, dim3(gc), dim3(2 * NB), 0, s, a...); });
+  else
+    combine([&](auto... a) { k_mv_tc_combine<NB><<<gc, 2 * NB, 0, s>>>(a...); });
 }
 
 // FP16 T~ tiles of the block-OSRC apply, rebuilt from the FP16 copy of T~
