@@ -226,7 +226,12 @@ void mtf_mesh_destroy(mtf_mesh mesh);
  * at k_i (Eqs. 7-9) tested with the x-pairing (Eq. 5) -- regular pairs with
  * the 6x6-point tensor rule, coincident / common-edge / common-vertex pairs
  * with Sauter-Schwab rules -- and the sparse transmission Grams of Eq. (18)
- * for the exchange X (Eqs. 11-13).  All data stays on the device. */
+ * for the exchange X (Eqs. 11-13).  All data stays on the device: 32 bytes per
+ * entry (T, K) of the blocks in FP64, 16 in mixed precision beside the options'
+ * copies.  An FP64 system keeps 32 bytes per entry more, a copy that makes its
+ * matvec faster, while seven eighths of the device's memory stay free beside
+ * it; where an allocation for the system fails, the copy is given back first
+ * (results do not depend on it). */
 mtf_status mtf_assemble(mtf_mesh mesh, double k0, const double* eps_r, const double* mu_r,
                         const mtf_options* opt, void* stream, mtf_system* out);
 

@@ -9,8 +9,9 @@
 //   y_D = y+ + y-,   y_N = -i rho_i (y+ - y-),
 // two complex products per entry and right-hand side instead of the four of
 // K x_D, K x_N, T x_D, T x_N.  FP64 systems keep the entries in this form
-// (d_rot64, written with the mirrored blocks); FP32-stored entries (the
-// residual_df = 0 residual) are rotated as they are read.
+// (d_rot64, written with the mirrored blocks) while memory is plentiful
+// (rotated_copy.h); otherwise they, and FP32-stored entries (the residual_df =
+// 0 residual), are rotated as they are read, with the same results.
 //
 // Bound: the FP64 pipe (8 instructions per entry and right-hand side; the
 // 32-byte entries would stream in an eighth of that time).  A CTA of 8 warps
@@ -18,7 +19,8 @@
 // once per CTA in shared memory; the exchange entries join the lanes' sums
 // before the reduction.  Rows per CTA (8, 16, 32) are chosen for the fewest
 // rounds of CTAs over the SMs.  Measured on the split sphere of 11 rings (3
-// blocks of 2,178 rows), 2 right-hand sides: 1,503 -> 470 us.
+// blocks of 2,178 rows), 2 right-hand sides: 1,503 -> 470 us (588 us without
+// the rotated copy).
 #include <algorithm>
 
 #include "common.h"
@@ -41,15 +43,25 @@ struct MvArgs {
   int nblk;
 };
 
-template <class MatT>
+// what an entry is stored as: (K - i T, K + i T) or (T, K)
+enum class Ent { kRotated64, kBlocks64, kBlocks32 };
+
+template <Ent E>
 __device__ __forceinline__ void load_rotated(const void* entries, int64_t e, double* a) {
-  if constexpr (sizeof(MatT) == 8) {
+  if constexpr (E == Ent::kRotated64) {
     const double2 p = __ldg(static_cast<const double2*>(entries) + 2 * e);
     const double2 m = __ldg(static_cast<const double2*>(entries) + 2 * e + 1);
     a[0] = p.x; a[1] = p.y; a[2] = m.x; a[3] = m.y;
   } else {
-    const float4 v = __ldg(static_cast<const float4*>(entries) + e);  // T, K
-    const double tr = v.x, ti = v.y, kr = v.z, ki = v.w;
+    double tr, ti, kr, ki;
+    if constexpr (E == Ent::kBlocks64) {
+      const double2 t = __ldg(static_cast<const double2*>(entries) + 2 * e);
+      const double2 k = __ldg(static_cast<const double2*>(entries) + 2 * e + 1);
+      tr = t.x; ti = t.y; kr = k.x; ki = k.y;
+    } else {
+      const float4 v = __ldg(static_cast<const float4*>(entries) + e);
+      tr = v.x; ti = v.y; kr = v.z; ki = v.w;
+    }
     a[0] = kr + ti; a[1] = ki - tr; a[2] = kr - ti; a[3] = ki + tr;
   }
 }
@@ -102,7 +114,7 @@ __device__ __forceinline__ void mv_finish(const MvArgs& A, int i, int m0, int la
 }
 
 // y = M x for right-hand sides c0 .. c0 + NC - 1; R rows per warp
-template <class MatT, int NC, int R>
+template <Ent E, int NC, int R>
 __global__ void __launch_bounds__(256, R * NC >= 4 ? 2 : 4) k_matvec(const MvArgs A, const double* __restrict__ x, int64_t ldx,
                                                 double* __restrict__ y, int64_t ldy, int c0) {
   MTF_PDL_WAIT();
@@ -142,7 +154,7 @@ __global__ void __launch_bounds__(256, R * NC >= 4 ? 2 : 4) k_matvec(const MvArg
     for (int n = lane; n < min(kMvCols, N - n0); n += 32) {
       double a[R][4];
 #pragma unroll
-      for (int r = 0; r < R; ++r) load_rotated<MatT>(A.entries, row[r] + n0 + n, a[r]);
+      for (int r = 0; r < R; ++r) load_rotated<E>(A.entries, row[r] + n0 + n, a[r]);
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const double2 p = us[c][n][0], m = us[c][n][1];
@@ -160,14 +172,14 @@ __global__ void __launch_bounds__(256, R * NC >= 4 ? 2 : 4) k_matvec(const MvArg
   mv_finish<NC, R>(A, i, m0, lane, off, x, ldx, y, ldy, c0, acc, sums[warp]);
 }
 
-template <class MatT, int NC, int R>
+template <Ent E, int NC, int R>
 static void mv64_launch(mtf_system sys, const MvArgs& A, unsigned grid, const double* x, int64_t ldx, double* y,
                         int64_t ldy, int c0, cudaStream_t s) {
-  MTF_LAUNCH(KID_MATVEC64, s, launch_pdl(k_matvec<MatT, NC, R>, dim3(grid), dim3(256), 0, s, A, x, ldx, y, ldy, c0));
+  MTF_LAUNCH(KID_MATVEC64, s, launch_pdl(k_matvec<E, NC, R>, dim3(grid), dim3(256), 0, s, A, x, ldx, y, ldy, c0));
 }
 
 // passes of up to 4 right-hand sides
-template <class MatT>
+template <Ent E>
 static void matvec64(mtf_system sys, const void* entries, const double* x, int64_t ldx, double* y, int64_t ldy, int nrhs,
                      cudaStream_t s) {
   mtf_mesh m = sys->mesh;
@@ -192,7 +204,7 @@ static void matvec64(mtf_system sys, const void* entries, const double* x, int64
     }
     A.prefix = m->d_mv_cta_prefix[best].p;
     const unsigned grid = unsigned(m->mv_cta_prefix[best].back());
-#define MTF_MV(NCV, RV) mv64_launch<MatT, NCV, RV>(sys, A, grid, x, ldx, y, ldy, c0, s)
+#define MTF_MV(NCV, RV) mv64_launch<E, NCV, RV>(sys, A, grid, x, ldx, y, ldy, c0, s)
     if (nc == 1) best == 0 ? MTF_MV(1, 1) : best == 1 ? MTF_MV(1, 2) : MTF_MV(1, 4);
     else if (nc == 2) best == 0 ? MTF_MV(2, 1) : best == 1 ? MTF_MV(2, 2) : MTF_MV(2, 4);
     else if (nc == 3) best == 0 ? MTF_MV(3, 1) : MTF_MV(3, 2);
@@ -370,7 +382,8 @@ void launch_matvec_kind(mtf_system sys, int kind, const double* x, int64_t ldx, 
     // mixed path with residual_fp64: the FP64 blocks as FP32 pairs, double-float sums
     matvec_df<true>(sys, sys->d_TK64hl.p, sys->d_TK64hl.p + size_t(m->n_mat) * 4, x, ldx, y, ldy, nrhs, s);
   } else if (kind == MV_FP64) {
-    matvec64<double>(sys, sys->d_rot64.p, x, ldx, y, ldy, nrhs, s);
+    if (sys->d_rot64.p) matvec64<Ent::kRotated64>(sys, sys->d_rot64.p, x, ldx, y, ldy, nrhs, s);
+    else matvec64<Ent::kBlocks64>(sys, sys->d_TK64.p, x, ldx, y, ldy, nrhs, s);
   } else if (kind == MV_FP32) {
     const int64_t n2 = 2 * m->n_total;
     if (sys->d_x32.n < size_t(n2) * nrhs) sys->d_x32.alloc(size_t(n2) * nrhs);
@@ -380,7 +393,7 @@ void launch_matvec_kind(mtf_system sys, int kind, const double* x, int64_t ldx, 
     // FP32 storage, double-float sums of the split input
     matvec_df<false>(sys, sys->d_TK32.p, nullptr, x, ldx, y, ldy, nrhs, s);
   } else {
-    matvec64<float>(sys, sys->d_TK32.p, x, ldx, y, ldy, nrhs, s);
+    matvec64<Ent::kBlocks32>(sys, sys->d_TK32.p, x, ldx, y, ldy, nrhs, s);
   }
 }
 

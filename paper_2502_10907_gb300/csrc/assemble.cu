@@ -24,6 +24,7 @@
 #include "common.h"
 #include "kernel64.cuh"
 #include "pair_tile.cuh"
+#include "rotated_copy.h"
 
 namespace mtf {
 
@@ -787,6 +788,24 @@ __global__ void k_split_pairs(const double* __restrict__ v, int64_t n, float* __
   out[n + t] = float(a - double(h));
 }
 
+// room for the rotated copy of the FP64 blocks, where it may be kept
+static void alloc_rotated_copy(mtf_system sys) {
+  if (sys->d_rot64.p || sys->rot64_off) return;
+  const size_t n = size_t(sys->mesh->n_mat) * 4;
+  size_t free_bytes = 0, total_bytes = 0;
+  MTF_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
+  sys->rot64_off = !keep_rotated_copy(n * sizeof(double), free_bytes, total_bytes);
+  if (sys->rot64_off) return;
+  try {
+    sys->d_rot64.alloc(n);
+  } catch (const Error& e) {
+    if (e.status != MTF_ERR_OOM) throw;
+    cudaGetLastError();  // (the matvec does without)
+    sys->d_rot64.p = nullptr;
+    sys->rot64_off = true;
+  }
+}
+
 void launch_assemble(mtf_system sys, cudaStream_t s) {
   mtf_mesh m = sys->mesh;
   upload_rule_constants(s);
@@ -804,7 +823,7 @@ void launch_assemble(mtf_system sys, cudaStream_t s) {
   if (fp64_blocks) {
     sys->d_TK64.alloc(size_t(m->n_mat) * 4);
     MTF_CUDA(cudaMemsetAsync(sys->d_TK64.p, 0, size_t(m->n_mat) * 4 * sizeof(double), s));
-    if (sys->opt.precision == MTF_PREC_FP64) sys->d_rot64.alloc(size_t(m->n_mat) * 4);
+    if (sys->opt.precision == MTF_PREC_FP64) alloc_rotated_copy(sys);
     const int64_t nct = m->reg_cta_prefix.back();
     MTF_LAUNCH(KID_REGULAR64, s, k_regular64<<<unsigned(nct), 128, 0, s>>>(A, m->d_reg_cta_prefix.p, sys->d_TK64.p));
     launch_singular(sys, A, sys->d_TK64.p, s);

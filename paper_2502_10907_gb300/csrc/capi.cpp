@@ -36,6 +36,28 @@ static mtf_status guarded(Fn&& fn) {
   }
 }
 
+// fn; if it runs out of device memory while the system keeps the copy of its
+// blocks that it can do without, once more without that copy
+template <class Fn>
+static void retry_without_copy(mtf_system sys, Fn&& fn) {
+  try {
+    fn();
+    return;
+  } catch (const Error& e) {
+    if (e.status != MTF_ERR_OOM || !sys || !sys->d_rot64.p) throw;
+  }
+  cudaGetLastError();
+  MTF_CUDA(cudaDeviceSynchronize());
+  sys->d_rot64.release();
+  sys->rot64_off = true;
+  fn();
+}
+
+template <class Fn>
+static mtf_status guarded(mtf_system sys, Fn&& fn) {
+  return guarded([&] { retry_without_copy(sys, fn); });
+}
+
 static void upload_small(DevBuf<double>& buf, const double* h, size_t n, cudaStream_t s) {
   if (buf.n < n) buf.alloc(n);
   MTF_CUDA(cudaMemcpyAsync(buf.p, h, n * sizeof(double), cudaMemcpyHostToDevice, s));
@@ -176,7 +198,7 @@ mtf_status mtf_assemble(mtf_mesh mesh, double k0, const double* eps_r, const dou
       if (sys->opt.osrc_type == 0) sys->opt.osrc_type = 1;
       MTF_REQUIRE(sys->opt.osrc_type == 1 || sys->opt.osrc_type == 2, MTF_ERR_ARG, "osrc_type must be 1 or 2");
       MTF_REQUIRE(sys->opt.osrc_np >= 1 && sys->opt.osrc_np <= 16, MTF_ERR_ARG, "osrc_np out of range 1..16");
-      assemble_into(sys, k0, eps_r, mu_r, s);
+      retry_without_copy(sys, [&] { assemble_into(sys, k0, eps_r, mu_r, s); });
     } catch (...) {
       delete sys;
       throw;
@@ -186,7 +208,7 @@ mtf_status mtf_assemble(mtf_mesh mesh, double k0, const double* eps_r, const dou
 }
 
 mtf_status mtf_reassemble(mtf_system sys, double k0, const double* eps_r, const double* mu_r, void* stream) {
-  return guarded([&] {
+  return guarded(sys, [&] {
     MTF_REQUIRE(sys && eps_r && mu_r, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(k0 > 0 && std::isfinite(k0), MTF_ERR_ARG, "k0 must be positive");
     assemble_into(sys, k0, eps_r, mu_r, static_cast<cudaStream_t>(stream));
@@ -225,7 +247,7 @@ mtf_status mtf_get_block(mtf_system sys, int32_t i, void* t_out, void* k_out, vo
 }
 
 mtf_status mtf_matvec(mtf_system sys, const void* x, void* y, int32_t nrhs, void* stream) {
-  return guarded([&] {
+  return guarded(sys, [&] {
     MTF_REQUIRE(sys && x && y, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(nrhs >= 1, MTF_ERR_ARG, "nrhs must be >= 1");
     MTF_REQUIRE(x != y, MTF_ERR_ARG, "x and y must not overlap");
@@ -236,7 +258,7 @@ mtf_status mtf_matvec(mtf_system sys, const void* x, void* y, int32_t nrhs, void
 }
 
 mtf_status mtf_precond_apply(mtf_system sys, const void* r, void* z, int32_t nrhs, void* stream) {
-  return guarded([&] {
+  return guarded(sys, [&] {
     MTF_REQUIRE(sys && r && z, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(nrhs >= 1, MTF_ERR_ARG, "nrhs must be >= 1");
     MTF_REQUIRE(r != z, MTF_ERR_ARG, "r and z must not overlap");
@@ -303,7 +325,7 @@ static void upload_waves(DevBuf<double>& d_dirs, DevBuf<double>& d_pols, int32_t
 
 mtf_status mtf_rhs(mtf_system sys, int32_t nrhs, const double* dirs, const double* pols, void* b_out,
                    void* stream) {
-  return guarded([&] {
+  return guarded(sys, [&] {
     MTF_REQUIRE(sys && b_out, MTF_ERR_ARG, "null argument");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     DevBuf<double> dd, dp;
@@ -316,7 +338,7 @@ mtf_status mtf_rhs(mtf_system sys, int32_t nrhs, const double* dirs, const doubl
 mtf_status mtf_solve(mtf_system sys, int32_t nrhs, const double* dirs, const double* pols, void* x_out,
                      mtf_solve_stats* stats, void* stream) {
   mtf_status st = MTF_OK;
-  mtf_status g = guarded([&] {
+  mtf_status g = guarded(sys, [&] {
     MTF_REQUIRE(sys && x_out, MTF_ERR_ARG, "null argument");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // the buffers stay with the system (no allocation, and no implicit
@@ -336,7 +358,7 @@ mtf_status mtf_solve(mtf_system sys, int32_t nrhs, const double* dirs, const dou
 mtf_status mtf_solve_rhs(mtf_system sys, int32_t nrhs, const void* b, void* x_out, mtf_solve_stats* stats,
                          void* stream) {
   mtf_status st = MTF_OK;
-  mtf_status g = guarded([&] {
+  mtf_status g = guarded(sys, [&] {
     MTF_REQUIRE(sys && b && x_out, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(nrhs >= 1, MTF_ERR_ARG, "nrhs must be >= 1");
     MTF_REQUIRE(b != x_out, MTF_ERR_ARG, "b and x_out must not overlap");
@@ -658,7 +680,7 @@ mtf_status mtf_learned_apply(mtf_system sys, const void* r, void* z, int32_t nrh
 
 mtf_status mtf_nearfield(mtf_system sys, const void* x, int32_t nrhs, const double* points, const int32_t* domains,
                          int32_t n_pts, void* f_out, void* stream) {
-  return guarded([&] {
+  return guarded(sys, [&] {
     MTF_REQUIRE(sys && x && points && domains && f_out, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(nrhs >= 1 && n_pts >= 1, MTF_ERR_ARG, "nrhs and n_pts must be >= 1");
     const int nd = sys->mesh->nd;
@@ -673,7 +695,7 @@ mtf_status mtf_nearfield(mtf_system sys, const void* x, int32_t nrhs, const doub
 
 mtf_status mtf_farfield(mtf_system sys, const void* x, int32_t nrhs, const double* obs_dirs, int32_t n_obs,
                         void* f_out, void* stream) {
-  return guarded([&] {
+  return guarded(sys, [&] {
     MTF_REQUIRE(sys && x && obs_dirs && f_out, MTF_ERR_ARG, "null argument");
     MTF_REQUIRE(nrhs >= 1 && n_obs >= 1, MTF_ERR_ARG, "need nrhs >= 1 and n_obs >= 1");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
