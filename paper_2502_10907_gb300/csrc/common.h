@@ -309,12 +309,22 @@ const char* kernel_name(int kid);
   } while (0)
 
 // Programmatic dependent launch for the chains of short kernels of the
-// inner solver: a kernel launched by launch_pdl may be scheduled before its
-// predecessor on the stream has finished; its first statements must be
-// MTF_PDL_WAIT() (returns once the predecessor grid has completed and its
-// memory is visible, so stream order holds for every access) and
-// MTF_PDL_TRIGGER() (lets the next such kernel be scheduled once all CTAs of
-// this one have started).  Both are no-ops for ordinary launches.
+// inner solver: a kernel launched by launch_pdl may start before its
+// predecessor on the stream has finished, as soon as every CTA of it has
+// triggered or ended.  MTF_PDL_WAIT() returns once the predecessor has
+// completed and its memory is visible; MTF_PDL_TRIGGER() lets the next such
+// kernel start.  Both are no-ops for ordinary launches.  Rules for every
+// kernel launched so:
+//  1. A thread triggers only after its wait, and every CTA has a thread that
+//     waits before the CTA ends.  Then, when a kernel starts, all kernels but
+//     the one just before it have completed, visibly.
+//  2. Before its wait a thread writes no global memory, and reads only what
+//     the kernel just before does not write: data at least two kernels old.
+//     A kernel that reads so names there what it reads and who writes it;
+//     whoever fuses, drops or adds a kernel in front of it checks that.
+// The operator copies are two ordinary kernels old when the first apply after
+// an assembly starts (launch_assemble ends in launch_exchange_values) or, with
+// block-OSRC, older than a synchronisation (osrc_setup).
 #define MTF_PDL_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
 #define MTF_PDL_TRIGGER() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
 

@@ -490,7 +490,8 @@ __global__ void __launch_bounds__(192, 1) k_mv_tc(const __grid_constant__ CUtens
       tma_prefetch_map(&bmap);
       const uint64_t pol_a = l2_policy_evict_first(), pol_b = l2_policy_evict_last();
       // the operator tiles of the first S stages, before the wait for the
-      // kernel that makes the inputs (the tiles are older)
+      // kernel that makes the inputs (k_tc_build_dw; the tiles are k_tc_tile_a's,
+      // of the assembly)
       int ahead = 0;
       for (int q = q_begin; q < q_end && ahead < S; ++q) {
         const int4 U = units[sched[q]];
@@ -656,7 +657,8 @@ __global__ void __launch_bounds__(2 * NB) k_mv_tc_combine(
     xv[e] = xval32[6 * row + e];
   }
   // the exchange rows of the warp's columns, before the wait for the stream
-  // (x is older than the kernel that packed the stream's inputs)
+  // (k_mv_tc; x, the largest entries and the tables are older: x was complete
+  // before k_tc_colmax and k_tc_build_dw, which read it ahead of the stream)
   float4 ex[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {

@@ -134,8 +134,9 @@ __global__ void __launch_bounds__((kDtCons + 1) * 32, 1)
     const uint32_t bytes = slice(u, c, i0, k0);
     bulk_g2s(smem + size_t(st) * kDtSB + kDtR * kDtSliceB, w + 2 * (int64_t(c) * ldn + k0), bytes, &full[st]);
   };
-  // the first units by one warp each; the basis is older than the kernel that
-  // makes w: its vectors are fetched before the wait for it
+  // the first units by one warp each; the basis (k_axpy2_32 and k_scale32 of
+  // the step before, k_start32) is older than the two kernels of the matvec
+  // whose second makes w: its vectors are fetched before the wait for that one
   {
     const int u = int(blockIdx.x) + warp * int(gridDim.x);
     const bool first = lane == 0 && warp < kDtS && u < n_units;
@@ -252,8 +253,9 @@ __global__ void __launch_bounds__(256) k_axpy2_32(float* __restrict__ V, const d
   __shared__ float cf[3];
   extern __shared__ float2 hs[];  // t_i at hs[i], s_i at hs[j + i]
   const bool lead = blockIdx.x == 0;
-  // the first 8 basis columns of this group (older than the reduction before
-  // this kernel) are loaded before the wait for the coefficients
+  // the first 8 basis columns of this group, i < j (written two steps back at
+  // the latest; the reduction just before writes t and sq only), are loaded
+  // before the wait for the coefficients
   const int64_t ldq = ldn >> 1;
   float4* vb = reinterpret_cast<float4*>(V + 2 * int64_t(c) * ldv) + q;
   float4 pre[8];

@@ -243,8 +243,8 @@ __global__ void __launch_bounds__(st_threads<ENT>(), 1) k_stream_tiles(
     }
   };
   // the first S units, one by each of the first S warps: the operator part
-  // before the wait for the kernel that makes x (the operator is older:
-  // written before that kernel began), x after it.  The ramp of the stream
+  // before the wait for the kernel that makes x (the unit tables and the
+  // operator are the mesh's and the assembly's), x after it.  The ramp of the stream
   // hides behind the previous kernel: split sphere, 2 right-hand sides, a
   // solve of 464 steps 48.5 -> 47.7 ms with the reduction's basis fetched the
   // same way.

@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(9 * 32, 1) k_stream_tc(const void* __restrict_
       bulk_g2s(st + ROWS * RBP + q * XB, x32 + 2 * xa, uint32_t((((a + len + 1) & ~int64_t(1)) - xa) * 8), &full[s]);
     }
   };
-  // the first S units by one warp each, the operator part before the wait for
-  // the input, as in k_stream_tiles
+  // the first S units by one warp each, the operator part (the assembly's)
+  // before the wait for the kernel that makes x, as in k_stream_tiles
   {
     const int u = int(blockIdx.x) + warp * int(gridDim.x);
     const bool first = lane == 0 && warp < S && u < n_units;

@@ -132,8 +132,11 @@ __global__ void __launch_bounds__(192, 1) k_tc_stream(const __grid_constant__ CU
       tma_prefetch_map(&bmap);
       const uint64_t pol_a = l2_policy_evict_first(), pol_b = l2_policy_evict_last();
       // the A tiles of the first S stages, before the wait for the kernel that
-      // packs B: under a programmatic launch A (an operator, or basis vectors
-      // stored in an earlier step) was written before that kernel began
+      // packs B.  Under a programmatic launch that kernel is k_tc_build_b(_real)
+      // with A the block-OSRC tiles of the assembly, or k_tca_w_to_b or
+      // k_tca_h_to_b with A the basis: k_bfinish or k_tca_store_dots / _upd wrote
+      // its last vectors before that step's Gram matrix and triangular solve.
+      // (k_tc_stream of the T~ formation is an ordinary launch.)
       int ahead = 0;
       for (int q = q0; q < q1 && ahead < S; q += qs) {
         const int4 U = units.get(listed ? sched[q] : q);
