@@ -34,7 +34,7 @@ def _sources():
 
 
 def _headers_mtime():
-    hs = [os.path.join(SRC, f) for f in os.listdir(SRC) if f.endswith(".h")]
+    hs = [os.path.join(SRC, f) for f in os.listdir(SRC) if f.endswith((".h", ".cuh"))]
     hs.append(os.path.join(ROOT, "include", "mtf.h"))
     return max(os.path.getmtime(h) for h in hs)
 
