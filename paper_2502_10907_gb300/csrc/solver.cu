@@ -33,6 +33,7 @@ struct GmresWork {
   DevBuf<double> h;
   double* h_host = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
+  int sms = 0;
   ~GmresWork() {
     if (h_host) cudaFreeHost(h_host);
     for (auto& e : ev)
@@ -114,9 +115,9 @@ __global__ void __launch_bounds__(256) k_dots64(const double* __restrict__ V, co
 }
 
 static void launch_dots(const double* V, const double* w, int64_t n, int ldv, int rows, double* h, int ldh, int nrhs,
-                        cudaStream_t s) {
+                        int sms, cudaStream_t s) {
   const int64_t pairs = (rows + 1) / 2;
-  const int64_t nseg = std::max<int64_t>(1, std::min<int64_t>((n + 63) / 64, 2432 / (pairs * nrhs)));
+  const int64_t nseg = std::max<int64_t>(1, std::min<int64_t>((n + 63) / 64, 16 * sms / (pairs * nrhs)));
   const int64_t seg = (n + nseg - 1) / nseg;
   MTF_LAUNCH(KID_DOTS, s, launch_pdl(k_dots64, dim3(nblk(pairs * nseg * nrhs, 8)), dim3(256), 0, s, V, w, n, ldv, rows,
                                      int(nseg), seg, nrhs, h, ldh));
@@ -282,9 +283,9 @@ static mtf_status gmres_core(mtf_system sys, int nrhs, const double* b_dev, doub
       double* hB = hA + 2 * L * nrhs;
       double* nrm = hB + 2 * L * nrhs;
       double* ss = nrm + 2 * nrhs;  // sum of squares scratch after the norms
-      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hA, j + 1, nrhs, s);
+      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hA, j + 1, nrhs, G.sms, s);
       launch_axpy(G.V.p, hA, j + 1, n, ldv, j + 1, -1.0, G.r.p, nullptr, nrhs, s);
-      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hB, j + 1, nrhs, s);
+      launch_dots(G.V.p, G.r.p, n, ldv, j + 1, hB, j + 1, nrhs, G.sms, s);
       launch_axpy(G.V.p, hB, j + 1, n, ldv, j + 1, -1.0, G.r.p, ss, nrhs, s);
       MTF_LAUNCH(KID_NORM, s, launch_pdl(k_scale, dim3(nblk(n, 256), unsigned(nrhs)), dim3(256), 0, s, G.r.p, n, ss, nrm,
                                          G.V.p + 2 * size_t(j + 1) * n, int64_t(ldv) * n, G.h.p + ((j + 1) & 1) * slot,
@@ -414,6 +415,9 @@ mtf_status solve(mtf_system sys, int nrhs, const double* b_dev, double* x_dev, m
     MTF_CUDA(cudaMallocHost(&G.h_host, G.h.n * sizeof(double)));
     for (auto& e : G.ev)
       if (!e) MTF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    int dev = 0;
+    MTF_CUDA(cudaGetDevice(&dev));
+    MTF_CUDA(cudaDeviceGetAttribute(&G.sms, cudaDevAttrMultiProcessorCount, dev));
     G.nrhs = nrhs;
     G.m = m;
     G.n = n;
