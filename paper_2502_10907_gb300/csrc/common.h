@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
 #include <mutex>
 #include <string>
 #include <utility>
@@ -61,6 +62,40 @@ struct DevBuf {
   void upload(const std::vector<T>& h, cudaStream_t s) {
     alloc(h.size());
     if (!h.empty()) MTF_CUDA(cudaMemcpyAsync(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, s));
+  }
+};
+
+// A table inside another buffer (TableUpload).
+template <class T>
+struct DevView {
+  T* p = nullptr;
+};
+
+// Tables copied to the device as one allocation and one copy: a small mesh has
+// about thirty, and an allocation costs more than its data.
+struct TableUpload {
+  struct Item {
+    void* view;  // the view's pointer
+    const void* data;
+    size_t bytes, at;
+  };
+  std::vector<Item> items;
+  size_t total = 0;
+  template <class T>
+  void add(DevView<T>& v, const std::vector<T>& h) {  // (h is read by run)
+    items.push_back({&v.p, h.data(), h.size() * sizeof(T), total});
+    total += (h.size() * sizeof(T) + 255) / 256 * 256;
+  }
+  void run(DevBuf<unsigned char>& buf, cudaStream_t s) {
+    std::vector<unsigned char> host(total);
+    buf.alloc(total);
+    for (const Item& t : items) {
+      if (t.bytes) std::memcpy(host.data() + t.at, t.data, t.bytes);
+      const void* at = t.bytes ? buf.p + t.at : nullptr;
+      std::memcpy(t.view, &at, sizeof(at));
+    }
+    if (total) MTF_CUDA(cudaMemcpyAsync(buf.p, host.data(), total, cudaMemcpyHostToDevice, s));
+    MTF_CUDA(cudaStreamSynchronize(s));  // the host copy goes out of scope
   }
 };
 
@@ -180,29 +215,30 @@ struct mtf_mesh_s {
   std::vector<mtf::SingPair> sing;
   std::vector<mtf::XEntry> xent;
   std::vector<int32_t> dof_bt;               // per exchange row: 2 x (bt*3 + a)
-  // device copies
-  mtf::DevBuf<double> d_bt_v, d_bt_c, d_bt_area;
-  mtf::DevBuf<int32_t> d_bt_dof, d_bt_vid, d_bt_blk, d_dof_bt;
-  mtf::DevBuf<int8_t> d_bt_swap;
-  mtf::DevBuf<mtf::SingPair> d_sing;
-  mtf::DevBuf<mtf::XEntry> d_xent;
-  mtf::DevBuf<int64_t> d_blk_mat_off;        // per block
-  mtf::DevBuf<int32_t> d_blk_N, d_blk_T;
-  mtf::DevBuf<int64_t> d_blk_bt_off, d_blk_dof_off, d_blk_row_off;
+  // device copies, one allocation (upload_mesh)
+  mtf::DevBuf<unsigned char> d_tables;
+  mtf::DevView<double> d_bt_v, d_bt_c, d_bt_area;
+  mtf::DevView<int32_t> d_bt_dof, d_bt_vid, d_bt_blk, d_dof_bt;
+  mtf::DevView<int8_t> d_bt_swap;
+  mtf::DevView<mtf::SingPair> d_sing;
+  mtf::DevView<mtf::XEntry> d_xent;
+  mtf::DevView<int64_t> d_blk_mat_off;        // per block
+  mtf::DevView<int32_t> d_blk_N, d_blk_T;
+  mtf::DevView<int64_t> d_blk_bt_off, d_blk_dof_off, d_blk_row_off;
   // CTA prefixes over blocks of the regular-pair tiles (16 triangles per side)
   // and of the mirror tiles (32 rows per side)
   std::vector<int64_t> reg_cta_prefix, mirror_cta_prefix;
-  mtf::DevBuf<int64_t> d_reg_cta_prefix, d_mirror_cta_prefix;
-  mtf::DevBuf<int32_t> d_row_blk;            // exchange row -> block
+  mtf::DevView<int64_t> d_reg_cta_prefix, d_mirror_cta_prefix;
+  mtf::DevView<int32_t> d_row_blk;            // exchange row -> block
   // first CTA of every block of the FP64 matvec with 8, 16, 32 rows per CTA
   std::vector<int32_t> mv_cta_prefix[3];
-  mtf::DevBuf<int32_t> d_mv_cta_prefix[3];
+  mtf::DevView<int32_t> d_mv_cta_prefix[3];
   // field evaluation: chunks of kFieldTris triangles of a block (first chunk
   // of every block, and the end) and the dofs of each: {corner (3 t + a) |
   // second corner << 8 (0xff: outside the chunk), local dof}
   std::vector<int32_t> fld_chunk;
-  mtf::DevBuf<int32_t> d_fld_first;
-  mtf::DevBuf<int2> d_fld_dofs;
+  mtf::DevView<int32_t> d_fld_first;
+  mtf::DevView<int2> d_fld_dofs;
   // streaming work units of the FP32 matvec ({T, K} entries) and of the
   // OSRC apply (T~ entries)
   mtf::StreamUnits mv_units, os_units;
@@ -223,9 +259,9 @@ struct mtf_mesh_s {
   std::vector<int32_t> bt_lv;                            // local vertex index per triangle corner
   std::vector<int32_t> edge_lohi;                        // per exchange row: local (lo, hi) vertex
   std::vector<double> edge_len;                          // per exchange row: edge length
-  mtf::DevBuf<int32_t> d_bt_lv, d_p1_n, d_edge_lohi;
-  mtf::DevBuf<int64_t> d_p1_off;
-  mtf::DevBuf<double> d_edge_len;
+  mtf::DevView<int32_t> d_bt_lv, d_p1_n, d_edge_lohi;
+  mtf::DevView<int64_t> d_p1_off;
+  mtf::DevView<double> d_edge_len;
 };
 
 namespace mtf {

@@ -266,21 +266,22 @@ mtf_mesh build_mesh(const double* V, int32_t nv, const int32_t* F, int32_t nt, c
 }
 
 void upload_mesh(mtf_mesh m, cudaStream_t s) {
-  m->d_bt_v.upload(m->bt_v, s);
-  m->d_bt_c.upload(m->bt_c, s);
-  m->d_bt_area.upload(m->bt_area, s);
-  m->d_bt_dof.upload(m->bt_dof, s);
-  m->d_bt_vid.upload(m->bt_vid, s);
-  m->d_bt_blk.upload(m->bt_blk, s);
-  m->d_bt_swap.upload(m->bt_swap, s);
-  m->d_sing.upload(m->sing, s);
-  m->d_xent.upload(m->xent, s);
-  m->d_dof_bt.upload(m->dof_bt, s);
-  m->d_bt_lv.upload(m->bt_lv, s);
-  m->d_p1_n.upload(m->p1_n, s);
-  m->d_p1_off.upload(m->p1_off_h, s);
-  m->d_edge_lohi.upload(m->edge_lohi, s);
-  m->d_edge_len.upload(m->edge_len, s);
+  TableUpload up;
+  up.add(m->d_bt_v, m->bt_v);
+  up.add(m->d_bt_c, m->bt_c);
+  up.add(m->d_bt_area, m->bt_area);
+  up.add(m->d_bt_dof, m->bt_dof);
+  up.add(m->d_bt_vid, m->bt_vid);
+  up.add(m->d_bt_blk, m->bt_blk);
+  up.add(m->d_bt_swap, m->bt_swap);
+  up.add(m->d_sing, m->sing);
+  up.add(m->d_xent, m->xent);
+  up.add(m->d_dof_bt, m->dof_bt);
+  up.add(m->d_bt_lv, m->bt_lv);
+  up.add(m->d_p1_n, m->p1_n);
+  up.add(m->d_p1_off, m->p1_off_h);
+  up.add(m->d_edge_lohi, m->edge_lohi);
+  up.add(m->d_edge_len, m->edge_len);
   std::vector<int64_t> mo, bo, dofo, rowo;
   std::vector<int32_t> N, T, row_blk;
   m->reg_cta_prefix.assign(1, 0);
@@ -301,38 +302,42 @@ void upload_mesh(mtf_mesh m, cudaStream_t s) {
     m->mv_cta_prefix[q].assign(1, 0);
     for (int i = 0; i < m->nd; ++i)
       m->mv_cta_prefix[q].push_back(m->mv_cta_prefix[q].back() + (m->blk[i].N + (8 << q) - 1) / (8 << q));
-    m->d_mv_cta_prefix[q].upload(m->mv_cta_prefix[q], s);
+    up.add(m->d_mv_cta_prefix[q], m->mv_cta_prefix[q]);
   }
   // chunks of the field kernels
   std::vector<int2> fdofs;
   std::vector<int32_t> ffirst(1, 0);
   m->fld_chunk.assign(1, 0);
   for (int i = 0; i < m->nd; ++i) {
+    std::vector<int32_t> at(size_t(m->blk[i].N), -1);  // entry of a dof's first corner
     for (int t0 = 0; t0 < m->blk[i].T; t0 += mtf::kFieldTris) {
-      std::vector<int2> d;
+      const int32_t first = ffirst.back();
       for (int c = 0; c < 3 * std::min(mtf::kFieldTris, m->blk[i].T - t0); ++c) {
         const int32_t dof = m->bt_dof[size_t(3 * (m->blk[i].bt_off + t0) + c)];
-        auto e = std::find_if(d.begin(), d.end(), [&](const int2& v) { return v.y == dof; });
-        if (e == d.end()) d.push_back(make_int2(c | 0xff << 8, dof));
-        else e->x = (e->x & 0xff) | c << 8;
+        int32_t& e = at[size_t(dof)];
+        if (e < first) {
+          e = int32_t(fdofs.size());
+          fdofs.push_back(make_int2(c | 0xff << 8, dof));
+        } else {
+          fdofs[size_t(e)].x = (fdofs[size_t(e)].x & 0xff) | c << 8;
+        }
       }
-      fdofs.insert(fdofs.end(), d.begin(), d.end());
       ffirst.push_back(int32_t(fdofs.size()));
     }
     m->fld_chunk.push_back(int32_t(ffirst.size()) - 1);
   }
-  m->d_fld_first.upload(ffirst, s);
-  m->d_fld_dofs.upload(fdofs, s);
-  m->d_blk_mat_off.upload(mo, s);
-  m->d_blk_bt_off.upload(bo, s);
-  m->d_blk_dof_off.upload(dofo, s);
-  m->d_blk_row_off.upload(rowo, s);
-  m->d_blk_N.upload(N, s);
-  m->d_blk_T.upload(T, s);
-  m->d_reg_cta_prefix.upload(m->reg_cta_prefix, s);
-  m->d_mirror_cta_prefix.upload(m->mirror_cta_prefix, s);
-  m->d_row_blk.upload(row_blk, s);
-  MTF_CUDA(cudaStreamSynchronize(s));
+  up.add(m->d_fld_first, ffirst);
+  up.add(m->d_fld_dofs, fdofs);
+  up.add(m->d_blk_mat_off, mo);
+  up.add(m->d_blk_bt_off, bo);
+  up.add(m->d_blk_dof_off, dofo);
+  up.add(m->d_blk_row_off, rowo);
+  up.add(m->d_blk_N, N);
+  up.add(m->d_blk_T, T);
+  up.add(m->d_reg_cta_prefix, m->reg_cta_prefix);
+  up.add(m->d_mirror_cta_prefix, m->mirror_cta_prefix);
+  up.add(m->d_row_blk, row_blk);
+  up.run(m->d_tables, s);
 }
 
 }  // namespace mtf
