@@ -265,7 +265,12 @@ mtf_status mtf_get_block(mtf_system sys, int32_t i, void* t_out, void* k_out, vo
  * sum_j G^{ij} u_j in both trace slots (Remark 2).  x, y: device complex128,
  * n_total x nrhs, must not overlap.  Mixed-precision systems apply their
  * FP32-stored blocks with double-float sums (opt.residual_df, default) or
- * FP64 sums: the refinement residual. */
+ * FP64 sums: the refinement residual.
+ * Accuracy: the two traces are multiplied together (as K -+ i T), so a row of
+ * block i is exact to a few e times 2 sum_n (|K| + |T|) (|u_D| + |u_N| / rho_i)
+ * (times rho_i in the N rows), e = 2^-53, or 2^-46 with double-float sums.
+ * |T| exceeds |K| by about 1 / (k h): the rows that hold K alone, for an input
+ * with one trace zero, are exact to e / (k h) of themselves. */
 mtf_status mtf_matvec(mtf_system sys, const void* x, void* y, int32_t nrhs, void* stream);
 
 /* z = A~ r: the block-OSRC preconditioner of Sec. 4.4 (Eq. 19),

@@ -8,7 +8,10 @@
 //   (K -+ i T) u+- = (K x_D + T w) +- i (K w - T x_D) =: y+-,
 //   y_D = y+ + y-,   y_N = -i rho_i (y+ - y-),
 // two complex products per entry and right-hand side instead of the four of
-// K x_D, K x_N, T x_D, T x_N.  FP64 systems keep the entries in this form
+// K x_D, K x_N, T x_D, T x_N.  A row is then exact to 2^-53 of (|K| + |T|)
+// (|x_D| + |w|), as with four products where both traces are filled; K x_D
+// alone (x_N = 0) is exact to 2^-53 of |T| |x_D| only, about 1 / (k h) more
+// (mtf.h; the tensor-core matvec, whose unit is 2^-22, keeps K apart).  FP64 systems keep the entries in this form
 // (d_rot64, written with the mirrored blocks) while memory is plentiful
 // (rotated_copy.h); otherwise they, and FP32-stored entries (the residual_df =
 // 0 residual), are rotated as they are read, with the same results.

@@ -42,10 +42,14 @@ def dense_part(sk, blocks, rho, x):
     return y
 
 
-def check(api, m, k0, contrast, nrhs, apply, dtype, eps, factor, **opts):
+def errors(api, m, k0, contrast, nrhs, apply, dtype, **opts):
+    """For one trace empty, then the other, and every block and slot: the
+    error of the rows against FP64, their dense part and exchange part, and
+    (|K| + |T|) (|u_D| + |w|) as the rows' products add it up, w = u_N / rho."""
     epsr, mur = materials(m, contrast)
     sk = skeleton_of(m)
-    s = api.System(api.Mesh.from_inputs(m), k0, epsr, mur, **opts)
+    mesh = api.Mesh.from_inputs(m)
+    s = api.System(mesh, k0, epsr, mur, **opts)
     blocks = [tuple(t.cpu().numpy() for t in s.block(i)) for i in range(m.n_domains)]
     ref = MTFSystem(sk, k0, epsr, mur, assemble=False)
     ref.T, ref.K = [b[0] for b in blocks], [b[1] for b in blocks]
@@ -59,12 +63,13 @@ def check(api, m, k0, contrast, nrhs, apply, dtype, eps, factor, **opts):
         xd = x.astype(np.complex128)
         yr = ref.matvec(xd.T).T
         dense = dense_part(sk, blocks, rho, xd)
-        for i in range(m.n_domains):
-            for slot, sl in enumerate(sk.block_slices(i)):
-                err = np.linalg.norm(y[:, sl] - yr[:, sl])
-                exchange = np.linalg.norm(yr[:, sl] - dense[:, sl])
-                bound = eps * (factor(blocks[i], rho[i], slot, empty, np.linalg.norm(dense[:, sl])) + 4 * exchange)
-                assert err < bound, (i, slot, empty, err / np.linalg.norm(dense[:, sl]))
+        for i, (T, K) in enumerate(blocks):
+            d, n = sk.block_slices(i)
+            sums = 2 * (np.abs(xd[:, d]) + np.abs(xd[:, n]) / rho[i]) @ (np.abs(K) + np.abs(T)).T
+            for slot, sl in enumerate((d, n)):
+                nrm = np.linalg.norm
+                yield ((i, slot, empty), nrm(y[:, sl] - yr[:, sl]), nrm(dense[:, sl]), nrm(yr[:, sl] - dense[:, sl]),
+                       nrm(sums) * (rho[i] if slot else 1.0))
 
 
 # every width of the tensor-core kernel (32, 64, 128 columns) and the FMA stream (4)
@@ -74,5 +79,19 @@ def test_matvec_f32_keeps_both_traces(api, mesh, nrhs, k0, contrast):
     """Operands of 22 significant bits (rounding, dropped lo x lo: 3 x 2^-22)
     and FP32 sums of up to 2 x 480 products: 8 x 2^-22 of the dense part,
     2^-22 of the exchange part's FP32 sums."""
-    check(api, MESHES[mesh](), k0, contrast, nrhs, lambda s: s.matvec_f32, np.complex64, 2.0 ** -24,
-          lambda block, rho, slot, empty, dense: 32 * dense, precision=1)
+    for where, err, dense, exchange, _ in errors(api, MESHES[mesh](), k0, contrast, nrhs, lambda s: s.matvec_f32,
+                                                 np.complex64, precision=1):
+        assert err < 2.0 ** -22 * (8 * dense + exchange), (where, err / dense)
+
+
+@pytest.mark.parametrize("mesh, nrhs", [("ico2", 1), ("cubes", 2), ("uv", 5)])
+@pytest.mark.parametrize("k0, contrast", [(0.05, 1.0), (0.3, 0.1), (0.3, 10.0), (1.3, 1.0)])
+@pytest.mark.parametrize("opts, unit", [({}, 2.0 ** -53), (dict(precision=1), 2.0 ** -46),
+                                        (dict(precision=1, residual_df=0), 2.0 ** -53)])
+def test_matvec_within_the_stated_bound(api, mesh, nrhs, k0, contrast, opts, unit):
+    """mtf_matvec's rows, each trace by itself, to the bound of mtf.h: its unit
+    times (|K| + |T|) (|u_D| + |w|) summed over the row, with 16 for the
+    roundings of up to 2 x 480 products per row in chains of at most 60."""
+    for where, err, _, exchange, sums in errors(api, MESHES[mesh](), k0, contrast, nrhs, lambda s: s.matvec,
+                                                np.complex128, **opts):
+        assert err < unit * 16 * sums + 2.0 ** -51 * exchange, (where, err / sums)
