@@ -332,7 +332,11 @@ __global__ void __launch_bounds__(kFieldThreads) k_field(const FieldMesh A, cons
         for (int q = 0; q < CO; ++q) cw[CO * (e & 0xff) + q] += cw[CO * (e >> 8) + q];
     }
     __syncwarp();
-    // ---- products: lane = (right-hand side, slice of the dofs) -------------
+    // ---- products: lane = (right-hand side, slice of the dofs), the chunk's
+    // sum by itself (one running sum over thousands of dofs loses a digit)
+    double sum[OUT];
+#pragma unroll
+    for (int q = 0; q < OUT; ++q) sum[q] = 0.0;
     for (int d = slice; d < nd; d += nslice) {
       const double2* w = reinterpret_cast<const double2*>(cw + CO * (A.dofs[d0 + d].x & 0xff));
       const double2 uD = u[(2 * d) * L + col], uN = u[(2 * d + 1) * L + col];
@@ -340,21 +344,23 @@ __global__ void __launch_bounds__(kFieldThreads) k_field(const FieldMesh A, cons
         const double pr = fma(h, uN.x, -uD.y), pi = fma(h, uN.y, uD.x);  // h u_N + i u_D
         const double mr = fma(h, uN.x, uD.y), mi = fma(h, uN.y, -uD.x);  // h u_N - i u_D
         const double2 qp = w[0], qm = w[1];
-        acc[0] = fma(qp.x, pr, fma(-qp.y, pi, acc[0]));
-        acc[1] = fma(qp.x, pi, fma(qp.y, pr, acc[1]));
-        acc[2] = fma(qm.x, mr, fma(-qm.y, mi, acc[2]));
-        acc[3] = fma(qm.x, mi, fma(qm.y, mr, acc[3]));
+        sum[0] = fma(qp.x, pr, fma(-qp.y, pi, sum[0]));
+        sum[1] = fma(qp.x, pi, fma(qp.y, pr, sum[1]));
+        sum[2] = fma(qm.x, mr, fma(-qm.y, mi, sum[2]));
+        sum[3] = fma(qm.x, mi, fma(qm.y, mr, sum[3]));
       } else {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const double2 H = w[c], N = w[3 + c];
-          acc[2 * c] = fma(H.x, uD.x, fma(-H.y, uD.y, acc[2 * c]));
-          acc[2 * c + 1] = fma(H.x, uD.y, fma(H.y, uD.x, acc[2 * c + 1]));
-          acc[2 * c] = fma(N.x, uN.x, fma(-N.y, uN.y, acc[2 * c]));
-          acc[2 * c + 1] = fma(N.x, uN.y, fma(N.y, uN.x, acc[2 * c + 1]));
+          sum[2 * c] = fma(H.x, uD.x, fma(-H.y, uD.y, sum[2 * c]));
+          sum[2 * c + 1] = fma(H.x, uD.y, fma(H.y, uD.x, sum[2 * c + 1]));
+          sum[2 * c] = fma(N.x, uN.x, fma(-N.y, uN.y, sum[2 * c]));
+          sum[2 * c + 1] = fma(N.x, uN.y, fma(N.y, uN.x, sum[2 * c + 1]));
         }
       }
     }
+#pragma unroll
+    for (int q = 0; q < OUT; ++q) acc[q] += sum[q];
   }
   if (!mine) return;
 #pragma unroll
