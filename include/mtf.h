@@ -229,9 +229,10 @@ void mtf_mesh_destroy(mtf_mesh mesh);
  * for the exchange X (Eqs. 11-13).  All data stays on the device: 32 bytes per
  * entry (T, K) of the blocks in FP64, 16 in mixed precision beside the options'
  * copies.  An FP64 system keeps 32 bytes per entry more, a copy that makes its
- * matvec faster, while seven eighths of the device's memory stay free beside
- * it; where an allocation for the system fails, the copy is given back first
- * (results do not depend on it). */
+ * matvec faster, where that takes at most an eighth of the free memory and
+ * all such copies at most a sixteenth of the device; where an allocation for
+ * the system fails, its copy is given back first (results do not depend on
+ * it). */
 mtf_status mtf_assemble(mtf_mesh mesh, double k0, const double* eps_r, const double* mu_r,
                         const mtf_options* opt, void* stream, mtf_system* out);
 

@@ -12,7 +12,7 @@
 // (|x_D| + |w|), as with four products where both traces are filled; K x_D
 // alone (x_N = 0) is exact to 2^-53 of |T| |x_D| only, about 1 / (k h) more
 // (mtf.h; the tensor-core matvec, whose unit is 2^-22, keeps K apart).  FP64 systems keep the entries in this form
-// (d_rot64, written with the mirrored blocks) while memory is plentiful
+// (d_rot64, written with the mirrored blocks) where memory is plentiful
 // (rotated_copy.h); otherwise they, and FP32-stored entries (the residual_df =
 // 0 residual), are rotated as they are read, with the same results.
 //

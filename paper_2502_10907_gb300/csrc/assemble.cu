@@ -792,9 +792,13 @@ __global__ void k_split_pairs(const double* __restrict__ v, int64_t n, float* __
 static void alloc_rotated_copy(mtf_system sys) {
   if (sys->d_rot64.p || sys->rot64_off) return;
   const size_t n = size_t(sys->mesh->n_mat) * 4;
+  static RotatedBudget budgets[64];  // per device
+  int dev = 0;
   size_t free_bytes = 0, total_bytes = 0;
+  MTF_CUDA(cudaGetDevice(&dev));
   MTF_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
-  sys->rot64_off = !keep_rotated_copy(n * sizeof(double), free_bytes, total_bytes);
+  sys->rot64_off = dev >= 64 || !rotated_copy_fits(n * sizeof(double), free_bytes) ||
+                   !sys->rot64_share.take(budgets[dev], n * sizeof(double), total_bytes);
   if (sys->rot64_off) return;
   try {
     sys->d_rot64.alloc(n);
@@ -802,6 +806,7 @@ static void alloc_rotated_copy(mtf_system sys) {
     if (e.status != MTF_ERR_OOM) throw;
     cudaGetLastError();  // (the matvec does without)
     sys->d_rot64.p = nullptr;
+    sys->rot64_share.give();
     sys->rot64_off = true;
   }
 }

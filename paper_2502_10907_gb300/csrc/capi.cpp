@@ -49,6 +49,7 @@ static void retry_without_copy(mtf_system sys, Fn&& fn) {
   cudaGetLastError();
   MTF_CUDA(cudaDeviceSynchronize());
   sys->d_rot64.release();
+  sys->rot64_share.give();
   sys->rot64_off = true;
   fn();
 }

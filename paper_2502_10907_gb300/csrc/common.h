@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/mtf.h"
+#include "rotated_copy.h"
 #include "stream_plan.h"
 
 namespace mtf {
@@ -284,7 +285,8 @@ struct mtf_system_s {
   mtf::DevBuf<double> d_wdir, d_wpol, d_brhs;  // mtf_solve: wave parameters and right-hand sides (kept)
   mtf::DevBuf<double> d_TK64;                // FP64: 4 doubles per dense entry
   mtf::DevBuf<double> d_rot64;               // FP64 systems: the entries as (K - i T, K + i T) for the matvec
-  bool rot64_off = false;                    // not kept (rotated_copy.h, or memory ran out)
+  mtf::RotatedShare rot64_share;             // its part of the device's budget (rotated_copy.h)
+  bool rot64_off = false;                    // not kept (no room, or memory ran out)
   mtf::DevBuf<float> d_TK64hl;               // residual_fp64: the FP64 entries as FP32 pairs (all hi, then all lo)
   mtf::DevBuf<float> d_TK32;                 // mixed: 4 floats per dense entry
   mtf::DevBuf<float> d_TK32t;                // the same, tiled per stream unit (streaming matvec)

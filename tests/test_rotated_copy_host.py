@@ -13,7 +13,7 @@ def test_rule(tmp_path):
     if cxx is None:
         pytest.skip("needs g++")
     exe = tmp_path / "rotated_copy"
-    subprocess.run([cxx, "-O2", "-std=c++17", "-I", os.path.join(ROOT, "paper_2502_10907_gb300", "csrc"),
+    subprocess.run([cxx, "-O2", "-std=c++17", "-pthread", "-I", os.path.join(ROOT, "paper_2502_10907_gb300", "csrc"),
                     os.path.join(ROOT, "tests", "host_src", "rotated_copy.cpp"), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
