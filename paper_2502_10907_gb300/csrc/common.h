@@ -160,6 +160,7 @@ struct BlockInfo {
 };
 
 constexpr int kFieldTris = 32;  // triangles per chunk of the field kernels
+constexpr size_t kFieldKeep = size_t(4) << 20;
 
 // Singular pair record (device): block-triangle ids and the Sauter-Schwab
 // vertex orders (local vertex indices 0..2 packed in 2 bits each).
@@ -307,6 +308,7 @@ struct mtf_system_s {
   mtf::DevBuf<float> d_os_part;              // per-row piece sums of the OSRC apply
   mtf::DevBuf<double> d_cen;
   mtf::DevBuf<float> d_qx, d_pv, d_cc;
+  mtf::DevBuf<unsigned char> d_field;        // small field calls' workspace (up to kFieldKeep bytes)
   int32_t ss_npts[3] = {0, 0, 0};
   // streaming matvec: per-row piece sums and the error word (d_mv_ctl[2])
   mtf::DevBuf<float> d_mv_part;

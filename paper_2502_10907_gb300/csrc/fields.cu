@@ -18,10 +18,11 @@
 // per rule point; moments over the rule's orbits); the two halves of a dof
 // whose triangles are both in the chunk are added; then the lanes turn to the
 // right-hand sides (up to 32) and slices of the chunk's dofs.  Work items are
-// (8 points of one block) x (a range of chunks), about two per SM; their sums
-// are added in order by k_field_sum.  Before, every right-hand side
-// re-evaluated the kernel at every rule point: 16 right-hand sides on the
-// 2 x 2 x 2 cube (181 directions and 584 points) took 96.0 ms, now 7.8 ms.
+// (8 points of one block) x (a range of chunks), about two per SM, times
+// passes of up to 32 right-hand sides; fewer points and narrower passes where
+// that would leave SMs idle; their sums are added in order by k_field_sum.
+// Before, every right-hand side re-evaluated the kernel at every rule point: 16
+// right-hand sides on the 2 x 2 x 2 cube (181 directions and 584 points) took 96.0 ms, now 7.5 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -30,7 +31,7 @@
 
 namespace mtf {
 
-constexpr int kFieldPts = 8;   // points per work item (one per warp)
+constexpr int kFieldPts = 8;   // points per work item (one per warp), at most
 constexpr int kFieldThreads = 32 * kFieldPts;
 constexpr int kFieldBatch = 4096;  // point groups per launch (bounds the workspace)
 
@@ -134,13 +135,15 @@ __global__ void __launch_bounds__(kFieldThreads) k_field(const FieldMesh A, cons
                                                          const FieldItem* __restrict__ items,
                                                          const FieldGroup* __restrict__ groups,
                                                          const double* __restrict__ pts, const double* __restrict__ x,
-                                                         int64_t n_total, int c0, int nc, int L,
+                                                         int64_t n_total, int c0, int nrhs, int L, int group_pts,
                                                          double* __restrict__ part) {
   constexpr int CO = FieldCfg<FAR>::co, OUT = FieldCfg<FAR>::out;
   extern __shared__ __align__(16) unsigned char raw[];
   FieldGeom& S = *reinterpret_cast<FieldGeom*>(raw);
   double* coef = reinterpret_cast<double*>(raw + sizeof(FieldGeom));            // [point][corner][CO]
   double2* u = reinterpret_cast<double2*>(coef + kFieldPts * 3 * kFieldTris * CO);  // [dof][slot][L]
+  c0 += int(blockIdx.y) * L;  // the pass
+  const int nc = min(L, nrhs - c0);
   const FieldItem it = items[blockIdx.x];
   const FieldGroup g = groups[it.group];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -367,7 +370,7 @@ __global__ void __launch_bounds__(kFieldThreads) k_field(const FieldMesh A, cons
   for (int q = 0; q < OUT; ++q)
     for (int o = L; o < 32; o <<= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
   if (lane < nc) {
-    double* o = part + ((size_t(it.part) * kFieldPts + warp) * nc + lane) * OUT;
+    double* o = part + (((size_t(blockIdx.y) * gridDim.x + it.part) * group_pts + warp) * L + lane) * OUT;
 #pragma unroll
     for (int q = 0; q < OUT; ++q) o[q] = acc[q];
   }
@@ -377,20 +380,21 @@ __global__ void __launch_bounds__(kFieldThreads) k_field(const FieldMesh A, cons
 // thread = (point, right-hand side); point order[p] of the call
 template <bool FAR>
 __global__ void k_field_sum(const double* __restrict__ part, const FieldGroup* __restrict__ groups, int n_groups,
-                            const double* __restrict__ pts, const int32_t* __restrict__ order, int nc, int c0, int npts,
-                            double* __restrict__ fout) {
+                            const double* __restrict__ pts, const int32_t* __restrict__ order, int n_items, int c0,
+                            int nrhs, int L, int group_pts, int npts, double* __restrict__ fout) {
   constexpr int OUT = FieldCfg<FAR>::out;
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int c = int(t % nc), p = int((t / nc) % kFieldPts);
-  const int64_t gi = t / (int64_t(nc) * kFieldPts);
-  if (gi >= n_groups) return;
+  c0 += int(blockIdx.y) * L;
+  const int c = int(t % L), p = int((t / L) % group_pts);
+  const int64_t gi = t / (int64_t(L) * group_pts);
+  if (gi >= n_groups || c0 + c >= nrhs) return;
   const FieldGroup g = groups[gi];
   if (p >= g.n) return;
   double s[OUT];
 #pragma unroll
   for (int q = 0; q < OUT; ++q) s[q] = 0.0;
   for (int i = 0; i < g.items; ++i) {
-    const double* v = part + ((size_t(g.item0 + i) * kFieldPts + p) * nc + c) * OUT;
+    const double* v = part + (((size_t(blockIdx.y) * n_items + g.item0 + i) * group_pts + p) * L + c) * OUT;
 #pragma unroll
     for (int q = 0; q < OUT; ++q) s[q] += v[q];
   }
@@ -412,7 +416,7 @@ __global__ void k_field_sum(const double* __restrict__ part, const FieldGroup* _
   }
 }
 
-// points (host, 3 per point) in blocks dom (host; null: block 0): groups of 8
+// points (host, 3 per point) in blocks dom (host; null: block 0): groups of 4 or 8
 // points of one block, items of about equal chunk counts, in batches
 template <bool FAR>
 static void run_fields(mtf_system sys, const double* x, int nrhs, const double* pts, const int32_t* dom, int npts,
@@ -436,8 +440,32 @@ static void run_fields(mtf_system sys, const double* x, int nrhs, const double* 
   std::vector<int32_t> order(static_cast<size_t>(npts));
   for (int p = 0; p < npts; ++p) order[size_t(p)] = p;
   if (dom) std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return dom[a] < dom[b]; });
+  // Points per item (8 or 4) and right-hand sides per pass (32 to 4): 8 points
+  // share a chunk's geometry and fill each quarter of an SM with two warps, and
+  // wide passes form the coefficients least often.  A call with fewer items
+  // than SMs is a chain of FP64 operations (about 600 a chunk for the
+  // coefficients and 36 per right-hand side of the pass, 64 cycles each, times
+  // the warps of a quarter): both are halved while the items still fit one per
+  // SM.  Near field of 64 solutions at 2 points, 80 triangles: 223 us with 8
+  // points and passes of 32 in turn, 84 us so; 100 points, one solution, 20
+  // triangles: 115 -> 87 us.
+  std::vector<int64_t> count(size_t(m->nd), 0);
+  for (int p = 0; p < npts; ++p) ++count[dom ? size_t(dom[p]) : 0];
+  const auto n_items = [&](int pts_per) {
+    int64_t n = 0;
+    for (int i = 0; i < m->nd; ++i)
+      n += (count[size_t(i)] + pts_per - 1) / pts_per * (m->fld_chunk[size_t(i) + 1] - m->fld_chunk[size_t(i)]);
+    return n;
+  };
+  const int group_pts = n_items(kFieldPts / 2) <= sms ? kFieldPts / 2 : kFieldPts;
+  int L = 1;
+  while (L < std::min(nrhs, 32)) L *= 2;
+  bool narrow = false;
+  while (L > 4 && n_items(group_pts) * ((nrhs + L / 2 - 1) / (L / 2)) <= sms) {
+    L /= 2;
+    narrow = true;
+  }
   const FieldMesh A{m->d_bt_v.p, m->d_bt_c.p, m->d_bt_area.p, m->d_fld_dofs.p, m->d_fld_first.p};
-  const int ncmax = std::min(nrhs, 32);
   int at = 0;
   while (at < npts) {
     std::vector<FieldGroup> groups;
@@ -448,7 +476,7 @@ static void run_fields(mtf_system sys, const double* x, int nrhs, const double* 
       const int i = dom ? dom[order[size_t(at)]] : 0;
       FieldGroup g{};
       g.point0 = at - p_begin;
-      while (g.n < kFieldPts && at < npts && (!dom || dom[order[size_t(at)]] == i)) {
+      while (g.n < group_pts && at < npts && (!dom || dom[order[size_t(at)]] == i)) {
         const double* p = pts + 3 * int64_t(order[size_t(at)]);
         sorted.insert(sorted.end(), p, p + 3);
         ++g.n;
@@ -488,8 +516,16 @@ static void run_fields(mtf_system sys, const double* x, int nrhs, const double* 
     std::copy_n(reinterpret_cast<const unsigned char*>(order.data() + p_begin), sizeof(int32_t) * size_t(at - p_begin),
                 host.data() + bg + bi);
     std::copy_n(reinterpret_cast<const unsigned char*>(sorted.data()), bp, host.data() + bg + bi + bo);
-    DevBuf<unsigned char> ws;
-    ws.alloc(head + items.size() * kFieldPts * size_t(ncmax) * FieldCfg<FAR>::out * sizeof(double));
+    // partial sums of a pass; passes per launch within 64 MB
+    const size_t pass_doubles = items.size() * size_t(group_pts) * size_t(L) * FieldCfg<FAR>::out;
+    const int per_launch = int(std::min({size_t(nrhs + L - 1) / size_t(L), size_t(65535),
+                                         std::max<size_t>(1, (size_t(8) << 20) / pass_doubles)}));
+    // a workspace of up to 4 MB stays with the system: an allocation that the
+    // driver has no mapped room for takes 0.15 ms, as long as such a call
+    const size_t need = head + size_t(per_launch) * pass_doubles * sizeof(double);
+    DevBuf<unsigned char> own;
+    DevBuf<unsigned char>& ws = need <= kFieldKeep ? sys->d_field : own;
+    if (ws.n < need) ws.alloc(need);
     MTF_CUDA(cudaMemcpyAsync(ws.p, host.data(), head, cudaMemcpyHostToDevice, s));
     const auto* dg = reinterpret_cast<const FieldGroup*>(ws.p);
     const auto* di = reinterpret_cast<const FieldItem*>(ws.p + bg);
@@ -497,15 +533,22 @@ static void run_fields(mtf_system sys, const double* x, int nrhs, const double* 
     const auto* dp = reinterpret_cast<const double*>(ws.p + bg + bi + bo);
     auto* part = reinterpret_cast<double*>(ws.p + head);
     MTF_CUDA(cudaFuncSetAttribute(k_field<FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(field_smem<FAR>(32))));
-    for (int c0 = 0; c0 < nrhs; c0 += 32) {
-      const int nc = std::min(32, nrhs - c0);
-      int L = 1;
-      while (L < nc) L *= 2;
-      MTF_LAUNCH(KID_FARFIELD, s, k_field<FAR><<<unsigned(items.size()), kFieldThreads, field_smem<FAR>(L), s>>>(
-          A, R, di, dg, dp, x, m->n_total, c0, nc, L, part));
-      const int64_t nt = int64_t(groups.size()) * kFieldPts * nc;
-      MTF_LAUNCH(KID_FARFIELD, s, k_field_sum<FAR><<<unsigned((nt + 127) / 128), 128, 0, s>>>(
-          part, dg, int(groups.size()), dp, dord, nc, c0, npts, f));
+    for (int c0 = 0; c0 < nrhs;) {
+      // whole passes together, then the rest in a pass of its own width (narrow
+      // passes run side by side: the last one may be partly empty)
+      int Lq = L, np = narrow ? (nrhs - c0 + L - 1) / L : (nrhs - c0) / L;
+      if (np == 0) {
+        np = 1;
+        while (Lq / 2 >= nrhs - c0) Lq /= 2;
+      }
+      np = std::min(np, per_launch);
+      MTF_LAUNCH(KID_FARFIELD, s,
+                 k_field<FAR><<<dim3(unsigned(items.size()), unsigned(np)), kFieldThreads, field_smem<FAR>(Lq), s>>>(
+                     A, R, di, dg, dp, x, m->n_total, c0, nrhs, Lq, group_pts, part));
+      const int64_t nt = int64_t(groups.size()) * group_pts * Lq;
+      MTF_LAUNCH(KID_FARFIELD, s, k_field_sum<FAR><<<dim3(unsigned((nt + 127) / 128), unsigned(np)), 128, 0, s>>>(
+          part, dg, int(groups.size()), dp, dord, int(items.size()), c0, nrhs, Lq, group_pts, npts, f));
+      c0 += np * Lq;
     }
     MTF_CUDA(cudaStreamSynchronize(s));  // the workspace and the host tables are released
   }

@@ -55,3 +55,26 @@ def test_close_points(api, mesh, k0, distance):
     # and point by point, on the scale of the field there
     err = np.linalg.norm(u - ur, axis=2).max(axis=0)
     assert (err < 1e-11 * np.linalg.norm(ur, axis=2).max(axis=0)).all(), err.max()
+
+
+@pytest.mark.parametrize("npts, nrhs", [(1, 2), (1, 33), (3, 40), (37, 1), (40, 19), (120, 2), (300, 1), (700, 2), (700, 70)])
+def test_points_per_work_item(api, npts, nrhs):
+    """4 or 8 points per work item and passes of 4 to 32 right-hand sides, by the
+    size of the call: sums of a few
+    thousand FP64 products per value, 1e-12 norm-wise."""
+    m = mi.split_sphere(2)
+    eps = np.array([1.0, 2.0, 3.0])
+    ref = MTFSystem(skeleton_of(m), 1.5, eps, np.ones(3), assemble=False)
+    s = api.System(api.Mesh.from_inputs(m), 1.5, eps, np.ones(3))
+    rng = np.random.default_rng(npts)
+    x = rng.standard_normal((nrhs, s.mesh.n_total)) + 1j * rng.standard_normal((nrhs, s.mesh.n_total))
+    xt = torch.from_numpy(x).cuda()
+    d = rng.standard_normal((npts, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    f = s.farfield(xt, d).cpu().numpy()
+    fr = ref.farfield(x.T, d).transpose(2, 0, 1)
+    assert np.linalg.norm(f - fr) < 1e-12 * np.linalg.norm(fr)
+    dom = rng.integers(0, 3, npts).astype(np.int32)
+    u = s.nearfield(xt, 2.0 * d, dom).cpu().numpy()
+    ur = representation(ref, x.T, 2.0 * d, dom).transpose(2, 0, 1)
+    assert np.linalg.norm(u - ur) < 1e-12 * np.linalg.norm(ur)
