@@ -81,12 +81,14 @@ __device__ __forceinline__ void cross3f(const float* a, const float* b, float* c
 // vertex distance in FP32.  The RWG factors scale whole rows and columns, and
 // on structured meshes their rounding is the same everywhere: they carry their
 // residues (K of a cube of 8 x 8 squares per face: error 1.7e-7 without, 7e-8
-// with them).
+// with them), and the rule's weight sum in FP32 over the exact one, 7e-9 that
+// every entry would share.
 struct Geom32Args {
   const double* bt_v;
   const double* bt_c;
   const double* bt_area;
   int64_t n_bt;
+  double wsum;   // sum of the FP32 weights over the exact sum
   double* cen;   // 3 per bt
   float* qx;     // 18 per bt
   float* pv;     // 24 per bt: vertices, v_1 - v_0, v_2 - v_0, the vertices' rounding
@@ -115,7 +117,7 @@ __global__ void k_geom32(Geom32Args G) {
       d2 = fmaf(d, d, d2);
     }
     rad = fmaxf(rad, d2);
-    const double ca = G.bt_c[3 * q + a] * (2.0 * INV_SQRT_FOUR_PI * G.bt_area[q]);
+    const double ca = G.bt_c[3 * q + a] * (2.0 * INV_SQRT_FOUR_PI * G.bt_area[q]) / G.wsum;
     G.cc[8 * q + a] = float(ca);
     G.cc[8 * q + 4 + a] = float(ca - double(float(ca)));
   }
@@ -402,7 +404,12 @@ void launch_assemble_regular32(mtf_system sys, cudaStream_t s) {
     sys->d_pv.alloc(size_t(m->n_bt) * 24);
     sys->d_cc.alloc(size_t(m->n_bt) * 8);
   }
-  Geom32Args G{m->d_bt_v.p, m->d_bt_c.p, m->d_bt_area.p, m->n_bt, sys->d_cen.p, sys->d_qx.p, sys->d_pv.p, sys->d_cc.p};
+  double wsum = 0.0, w32 = 0.0;
+  for (int p = 0; p < 6; ++p) {
+    wsum += rule.w[p];
+    w32 += double(float(rule.w[p]));
+  }
+  Geom32Args G{m->d_bt_v.p, m->d_bt_c.p, m->d_bt_area.p, m->n_bt, w32 / wsum, sys->d_cen.p, sys->d_qx.p, sys->d_pv.p, sys->d_cc.p};
   MTF_LAUNCH(KID_MISC, s, k_geom32<<<unsigned((m->n_bt + 127) / 128), 128, 0, s>>>(G));
   Reg32Args A{sys->d_cen.p, sys->d_qx.p, sys->d_pv.p, sys->d_cc.p, m->d_bt_dof.p, m->d_bt_vid.p,
               m->d_blk_T.p, m->d_blk_N.p, m->d_blk_bt_off.p, m->d_blk_mat_off.p, sys->d_k.p, m->nd};
