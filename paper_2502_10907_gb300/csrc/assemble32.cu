@@ -137,6 +137,7 @@ struct Reg32Args {
   const int64_t* blk_bt_off;
   const int64_t* blk_mat_off;
   const double* k;
+  const float4* k32;  // per block: k, its residue, -4 / k^2, its residue
   int nblk;
 };
 
@@ -196,7 +197,8 @@ __global__ void __launch_bounds__(128, 4) k_regular32(Reg32Args A, const int64_t
   load_side(A, A.blk_bt_off[i] + P.s0, min(kPairTile, T - P.s0), Y);
   __syncthreads();
   const double kr = A.k[2 * i];
-  const float k = float(kr), m4k2 = -4.0f / (k * k);
+  const float4 k32 = A.k32[i];
+  const float k = k32.x;
   const int N = A.blk_N[i];
   float4* M = reinterpret_cast<float4*>(TK) + A.blk_mat_off[i];
   const int b = threadIdx.x & (kPairTile - 1);
@@ -270,14 +272,15 @@ __global__ void __launch_bounds__(128, 4) k_regular32(Reg32Args A, const int64_t
           }
         }
     }
-    // rotate every moment by exp(i k R0)
+    // rotate every moment by exp(i k R0), those of G by k exp(i k R0)
+    const float ck0 = fmaf(c0, k, c0 * k32.y), sk0 = fmaf(s0, k, s0 * k32.y);
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         const float gr = G[p][q][0], hr = H[p][q][0];
-        G[p][q][0] = gr * c0 - G[p][q][1] * s0;
-        G[p][q][1] = gr * s0 + G[p][q][1] * c0;
+        G[p][q][0] = gr * ck0 - G[p][q][1] * sk0;
+        G[p][q][1] = gr * sk0 + G[p][q][1] * ck0;
         H[p][q][0] = hr * c0 - H[p][q][1] * s0;
         H[p][q][1] = hr * s0 + H[p][q][1] * c0;
       }
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(128, 4) k_regular32(Reg32Args A, const int64_t
 #pragma unroll
       for (int q = 0; q < 3; ++q) q3[q][c] = Y.v[3 * q + c][b];
     }
+    const float Q0[2] = {fmaf(k32.z, G[0][0][0], k32.w * G[0][0][0]), fmaf(k32.z, G[0][0][1], k32.w * G[0][0][1])};
     float Sx[3][2], Sy[3][2], Hx[3][2], Hy[3][2], Hc[3][2], Sxy[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
@@ -361,19 +365,21 @@ __global__ void __launch_bounds__(128, 4) k_regular32(Reg32Args A, const int64_t
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           xc[c] = base[c] - fmaf(q3[q][0], B3[0][c], fmaf(q3[q][1], B3[1][c], q3[q][2] * B3[2][c]));
-          // the -4 / (i k) S0 term of T last: it is the large one (first, it made
-          // every later addition round at its size: T 2.9e-7, so 2.3e-7)
-          xc[c] = fmaf(m4k2, G[0][0][c], xc[c]);
           kk[c] = kap[c] - fmaf(q3[q][0], L3[0][c], fmaf(q3[q][1], L3[1][c], q3[q][2] * L3[2][c]));
           kk[c] -= fmaf(Y.v[15 + 3 * q][b], L3[0][c], fmaf(Y.v[16 + 3 * q][b], L3[1][c], Y.v[17 + 3 * q][b] * L3[2][c]));
         }
-        // c_a c_b = cc + cl
+        // c_a c_b = cc + cl; T = -i c_a c_b (k X - 4 / k S0): the S0 term is the
+        // large one, and combinations without divergence cancel it, but not the
+        // entries' own roundings.  So it is rounded once per pair (Q0) and each
+        // entry once, at the end (with S0 at the head of X's sums: T 2.9e-7
+        // and a solve near a resonance 4.7e-6, so 2.3e-7 and 4.2e-6)
         const float cq = Y.c[q][b], cc = cp * cq, cl = fmaf(cp, cq, -cc) + fmaf(cp, Y.c[4 + q][b], cpl * cq);
-        const float tr = k * xc[1], ti = -k * xc[0];
+        float tv[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) tv[c] = fmaf(cc, Q0[c], fmaf(cc, xc[c], fmaf(cl, Q0[c], cl * xc[c])));
         const int ncol = Y.dof[q][b];
         const int64_t at = mrow < ncol ? int64_t(mrow) * N + ncol : int64_t(ncol) * N + mrow;
-        atomicAdd(M + at, make_float4(fmaf(cc, tr, cl * tr), fmaf(cc, ti, cl * ti), fmaf(cc, kk[0], cl * kk[0]),
-                                      fmaf(cc, kk[1], cl * kk[1])));
+        atomicAdd(M + at, make_float4(tv[1], -tv[0], fmaf(cc, kk[0], cl * kk[0]), fmaf(cc, kk[1], cl * kk[1])));
       }
     }
   }
@@ -412,7 +418,8 @@ void launch_assemble_regular32(mtf_system sys, cudaStream_t s) {
   Geom32Args G{m->d_bt_v.p, m->d_bt_c.p, m->d_bt_area.p, m->n_bt, w32 / wsum, sys->d_cen.p, sys->d_qx.p, sys->d_pv.p, sys->d_cc.p};
   MTF_LAUNCH(KID_MISC, s, k_geom32<<<unsigned((m->n_bt + 127) / 128), 128, 0, s>>>(G));
   Reg32Args A{sys->d_cen.p, sys->d_qx.p, sys->d_pv.p, sys->d_cc.p, m->d_bt_dof.p, m->d_bt_vid.p,
-              m->d_blk_T.p, m->d_blk_N.p, m->d_blk_bt_off.p, m->d_blk_mat_off.p, sys->d_k.p, m->nd};
+              m->d_blk_T.p, m->d_blk_N.p, m->d_blk_bt_off.p, m->d_blk_mat_off.p, sys->d_k.p,
+              reinterpret_cast<const float4*>(sys->d_rho32.p) + m->nd, m->nd};
   const int64_t nct = m->reg_cta_prefix.back();
   MTF_LAUNCH(KID_REGULAR32, s, k_regular32<<<unsigned(nct), 128, 0, s>>>(A, m->d_reg_cta_prefix.p, sys->d_TK32.p));
 }

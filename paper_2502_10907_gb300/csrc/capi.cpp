@@ -93,13 +93,20 @@ void assemble_into(mtf_system sys, double k0, const double* eps_r, const double*
   upload_small(sys->d_k, kk.data(), kk.size(), s);
   upload_small(sys->d_rho, rr.data(), rr.size(), s);
   // FP32 (rho, 1 / rho) per block for the FP32 epilogues
-  std::vector<float> r32(4 * mesh->nd);
+  std::vector<float> r32(8 * mesh->nd);
   for (int i = 0; i < mesh->nd; ++i) {
     const std::complex<double> r(rr[2 * i], rr[2 * i + 1]), ri = 1.0 / r;
     r32[4 * i] = float(r.real());
     r32[4 * i + 1] = float(r.imag());
     r32[4 * i + 2] = float(ri.real());
     r32[4 * i + 3] = float(ri.imag());
+    // and k, -4 / k^2 with their residues for the FP32 pair kernel
+    float* k32 = r32.data() + 4 * (mesh->nd + i);
+    const double m4k2 = -4.0 / (sys->k_re[size_t(i)] * sys->k_re[size_t(i)]);
+    k32[0] = float(sys->k_re[size_t(i)]);
+    k32[1] = float(sys->k_re[size_t(i)] - double(k32[0]));
+    k32[2] = float(m4k2);
+    k32[3] = float(m4k2 - double(k32[2]));
   }
   sys->d_rho32.alloc(r32.size());
   MTF_CUDA(cudaMemcpyAsync(sys->d_rho32.p, r32.data(), r32.size() * sizeof(float), cudaMemcpyHostToDevice, s));

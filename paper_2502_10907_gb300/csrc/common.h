@@ -293,7 +293,7 @@ struct mtf_system_s {
   mtf::DevBuf<float> d_TK32t;                // the same, tiled per stream unit (streaming matvec)
   mtf::DevBuf<double> d_xval;                // exchange values (6 per row)
   mtf::DevBuf<float> d_xval32;               // FP32 copy of the exchange values
-  mtf::DevBuf<float> d_rho32;                // per block: rho (re, im), 1 / rho (re, im)
+  mtf::DevBuf<float> d_rho32;                // per block: rho (re, im), 1 / rho (re, im); then k, -4 / k^2 (value, residue)
   mtf::DevBuf<double> d_ss_pts[3];           // Sauter-Schwab hat tables
   mtf::SingRadial ss_radial{};               // and their radial sums
   // FP32 geometry of the mixed regular-pair kernel (per block-triangle)
