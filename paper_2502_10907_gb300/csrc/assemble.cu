@@ -7,24 +7,21 @@
 // (Eq. 7 potentials, Eq. 9 operators; the normal cancels in the pairing).
 // Entries are stored row-major per block as (T.re, T.im, K.re, K.im).
 //
-// Each triangle pair (tau test, sigma trial) contributes a 3x3 block.  The
-// kernels never form the 9 products per quadrature point: with local origins
-// o_tau, o_sigma, x' = x - o_tau, y' = y - o_sigma, Delta = o_tau - o_sigma,
-// and RWG functions c_a (x - p_a), c_b (y - q_b), all 18 entries follow from
-// 16 complex moments of the kernel over the pair's points,
-//   S0 = sum W G, Sx = sum W G x', Sy = sum W G y', Sxy = sum W G x'.y',
-//   Q = sum W g, Gx = sum W g x', Gy = sum W g y', C = sum W g (x' x y'),
-// g = G (i k - 1/r) / r, through
-//   T_ab = c_a c_b [ -ik (Sxy - q'.Sx - p'.Sy + (p'.q') S0) - 4/(ik) S0 ]
-//   K_ab = -c_a c_b [ (q' - p' - Delta).C - p'.(Delta x Gy) - q'.(Gx x Delta)
-//                     + (q' x p').(Gx - Gy + Delta Q) ]
-// (expansion of (x - y).((y - q_b) x (x - p_a)) by the triple product).
+// Each triangle pair (tau test, sigma trial) contributes a 3x3 block, with RWG
+// functions c_a (x - v_a) and c_b (y - u_b):
+//   T_ab = c_a c_b [ -ik sum W G (x - v_a).(y - u_b) - 4/(ik) sum W G ]
+//   K_ab = -c_a c_b (v_a - u_b) . sum W g (y - u_b) x (x - v_a),
+// g = G (i k - 1/r) / r ((x - y).((y - u_b) x (x - v_a)) by the triple
+// product).  x and y are linear in their triangles' coordinates, so the kernels
+// never form the 9 products per quadrature point: all 18 entries follow from
+// the sums of G and of g times (1, s, t) of x and (1, s', t') of y, nine
+// complex sums each (k_regular64), or from the monomials in the coordinates of
+// the singular rules (k_singular64).
 #include <cmath>
 
 #include "common.h"
 #include "kernel64.cuh"
 #include "pair_tile.cuh"
-#include "rotated_copy.h"
 
 namespace mtf {
 

@@ -520,8 +520,8 @@ static void run_fields(mtf_system sys, const double* x, int nrhs, const double* 
     const size_t pass_doubles = items.size() * size_t(group_pts) * size_t(L) * FieldCfg<FAR>::out;
     const int per_launch = int(std::min({size_t(nrhs + L - 1) / size_t(L), size_t(65535),
                                          std::max<size_t>(1, (size_t(8) << 20) / pass_doubles)}));
-    // a workspace of up to 4 MB stays with the system: an allocation that the
-    // driver has no mapped room for takes 0.15 ms, as long as such a call
+    // a workspace of up to 4 MB stays with the system: an allocation that needs
+    // new mapped memory takes 0.15 ms, as long as such a call
     const size_t need = head + size_t(per_launch) * pass_doubles * sizeof(double);
     DevBuf<unsigned char> own;
     DevBuf<unsigned char>& ws = need <= kFieldKeep ? sys->d_field : own;
